@@ -1,9 +1,11 @@
 // C ABI of librsd (declared in include/rsd.h), verification half: rsd_verify_tree, rsd_verify_tree_rule and
 // rsd_resample_residual.  Argument checks and kernel launches, nothing else.
 #include <atomic>
+#include <cstring>
 
 #include "rsd_api_common.h"
 #include "rsd_verify.cuh"
+#include "rsd_walk_cluster.cuh"
 #include "rsd_walk_ring.cuh"
 
 using namespace rsd_host;
@@ -35,6 +37,62 @@ void launch_ring_walk(const rsd::VerifyArgs& a, int B, cudaStream_t s) {
         if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
     }
     verify_tree_ring_kernel<T><<<B, kThreads, kRingBytes, s>>>(a);
+}
+
+// Shape of a cluster walk (rsd_walk_cluster.cuh): C blocks of W working warps with NT tiles of 512 entries each.
+struct ClusterShape {
+    int C, W, NT;
+    float waves;   // sequences asked for over sequences resident at a time
+};
+// The smallest cluster that holds a row, with one tile per warp (three blocks an SM) as long as all sequences are
+// resident at once, else with two (two blocks an SM), which costs a sequence about 10 % more time and 25 % fewer SM-cycles
+// (V = 32,000, bf16: 42 against 47 us at 64 sequences, 122 against 102 us at 256).  Rows beyond 65,536 entries take
+// sixteen warps, one block an SM; beyond 131,072 no cluster holds them (C = 0).
+ClusterShape cluster_shape(int B, int V) {
+    auto blocks = [&](int per_block) {
+        int c = 1;
+        while (c * per_block < V) c *= 2;
+        return c;
+    };
+    const float sms = (float)sm_count();
+    int c = blocks(8 * 512);
+    if (c <= 8 && (float)B * (float)c <= 3.0f * sms) return {c, 8, 1, (float)B * (float)c / (3.0f * sms)};
+    c = blocks(16 * 512);
+    if (c <= 8) return {c, 8, 2, (float)B * (float)c / (2.0f * sms)};
+    c = blocks(32 * 512);
+    if (c <= 8) return {c, 16, 2, (float)B * (float)c / sms};
+    return {0, 0, 0, 0.0f};
+}
+
+template <typename T, int NT, int WARPS, bool EXTRA>
+void launch_cluster(const rsd::walk_cluster::ClusterArgs& a, int B, int C, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * C));
+    cfg.blockDim = dim3((WARPS + 1) * 32);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, rsd::walk_cluster::walk_cluster_kernel<T, NT, WARPS, EXTRA>, a);   // (an error stays pending for check_launch())
+}
+template <typename T, bool EXTRA>
+void launch_cluster_shape(const rsd::walk_cluster::ClusterArgs& a, int B, const ClusterShape& c, cudaStream_t s) {
+    if (c.W == 16) launch_cluster<T, 2, 16, EXTRA>(a, B, c.C, s);
+    else if (c.NT == 2) launch_cluster<T, 2, 8, EXTRA>(a, B, c.C, s);
+    else launch_cluster<T, 1, 8, EXTRA>(a, B, c.C, s);
+}
+void launch_cluster_walk(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const ClusterShape& c, cudaStream_t s) {
+    if (dtype == RSD_F32) {
+        if (extra) launch_cluster_shape<float, true>(a, B, c, s);
+        else launch_cluster_shape<float, false>(a, B, c, s);
+    } else {
+        if (extra) launch_cluster_shape<__nv_bfloat16, true>(a, B, c, s);
+        else launch_cluster_shape<__nv_bfloat16, false>(a, B, c, s);
+    }
 }
 }  // namespace
 
@@ -80,33 +138,38 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
     a.last_token = last_token; a.stop_reason = stop_reason; a.dbg_theta = dbg_theta; a.status = status;
     cudaStream_t s = (cudaStream_t)stream;
     const bool aligned = rows_aligned(draft) && rows_aligned(target);
-    // at most one sequence per SM: blocks of 512 threads; otherwise blocks of 256
-#define RSD_LAUNCH_WALK(NS, BASELINES)                                                                                   \
-    do {                                                                                                                 \
-        using namespace rsd::NS;                                                                                         \
-        if (draft->dtype == RSD_F32) {                                                                                   \
-            if (aligned) verify_tree_kernel<float, true, BASELINES><<<B, kVerifyThreads, 0, s>>>(a);                     \
-            else verify_tree_kernel<float, false, BASELINES><<<B, kVerifyThreads, 0, s>>>(a);                            \
-        } else {                                                                                                         \
-            if (aligned) verify_tree_kernel<__nv_bfloat16, true, BASELINES><<<B, kVerifyThreads, 0, s>>>(a);             \
-            else verify_tree_kernel<__nv_bfloat16, false, BASELINES><<<B, kVerifyThreads, 0, s>>>(a);                    \
-        }                                                                                                                \
-    } while (0)
-    const bool wide_blocks = B <= sm_count();
-    if (rule == RSD_RULE_RRS && final_sampler == RSD_FINAL_INVERSE_CDF) {
-        // rows on 16-byte boundaries, of at most 64 chunks (the ring keeps its chunks as bits of one word): the walk
-        // whose passes are fed by the copy engine
-        const size_t row_bytes = (size_t)V * (draft->dtype == RSD_F32 ? 4 : 2);
-        if (aligned && (row_bytes + rsd::walk_ring::kRowChunkBytes - 1) / rsd::walk_ring::kRowChunkBytes <= 64) {
-            if (draft->dtype == RSD_F32) launch_ring_walk<float>(a, B, s);
-            else launch_ring_walk<__nv_bfloat16>(a, B, s);
-        }
-        else if (wide_blocks) RSD_LAUNCH_WALK(walk_wide, false);
-        else RSD_LAUNCH_WALK(walk_narrow, false);
+    const bool plain = rule == RSD_RULE_RRS && final_sampler == RSD_FINAL_INVERSE_CDF;
+    // the ring walk: rows on 16-byte boundaries, of at most 64 chunks (it keeps its chunks as bits of one word)
+    const size_t row_bytes = (size_t)V * (draft->dtype == RSD_F32 ? 4 : 2);
+    const bool ring = plain && aligned && (row_bytes + rsd::walk_ring::kRowChunkBytes - 1) / rsd::walk_ring::kRowChunkBytes <= 64;
+    // A cluster per sequence while there are few: its passes are two to three times as short (V = 32,000 bf16: 30 -> 16 us
+    // for one sequence, 94 -> 42 for 64), but it takes more SM time per walk.  The kernels with one block per sequence are
+    // ahead from about 2.5 waves of clusters on with rows on 16-byte boundaries (192 / 320 sequences: ring 104 / 116 us,
+    // cluster 79 / 119; V = 50,272: 64 / 128 sequences 59 / 61 against 49 / 81), from about 3 for the baseline rules (128 /
+    // 256 sequences: 73 / 79 against 49 / 84), from about 8 where the last token is drawn by Gumbel-Top-1 (256 / 1024
+    // sequences: 147 / 348 against 128 / 392).  For plain walks over other rows the cluster is ahead at every size (32,001
+    // entries, 64 / 512 / 1000 sequences: 110 / 296 / 444 against 32 / 180 / 329).
+    const ClusterShape shape = cluster_shape(B, V);
+    const float most = ring ? 2.0f : plain ? 1e30f : final_sampler == RSD_FINAL_GUMBEL_TOP1 ? 8.0f : 3.0f;
+    if (shape.C > 0 && shape.waves <= most) {
+        rsd::walk_cluster::ClusterArgs ca;
+        memset(&ca, 0, sizeof(ca));
+        ca.v = a;
+        launch_cluster_walk(ca, draft->dtype, !plain, B, shape, s);
+    } else if (ring) {
+        if (draft->dtype == RSD_F32) launch_ring_walk<float>(a, B, s);
+        else launch_ring_walk<__nv_bfloat16>(a, B, s);
     } else {
-        RSD_LAUNCH_WALK(walk_narrow, true);
+        using namespace rsd::walk_narrow;
+        auto launch = [&](auto kernel) { kernel<<<B, kVerifyThreads, 0, s>>>(a); };
+        if (draft->dtype == RSD_F32) {
+            if (plain) launch(aligned ? verify_tree_kernel<float, true, false> : verify_tree_kernel<float, false, false>);
+            else launch(aligned ? verify_tree_kernel<float, true, true> : verify_tree_kernel<float, false, true>);
+        } else {
+            if (plain) launch(verify_tree_kernel<__nv_bfloat16, false, false>);   // (2-byte rows on 16-byte boundaries fit the ring)
+            else launch(aligned ? verify_tree_kernel<__nv_bfloat16, true, true> : verify_tree_kernel<__nv_bfloat16, false, true>);
+        }
     }
-#undef RSD_LAUNCH_WALK
     return check_launch("rsd_verify_tree_rule");
 }
 
@@ -131,6 +194,19 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     a.seed_lo = (uint32_t)seed; a.seed_hi = (uint32_t)(seed >> 32); a.step = step; a.seq_base = seq_base;
     a.out_token = out_token; a.out_residual = out_residual; a.status = status;
     cudaStream_t s = (cudaStream_t)stream;
+    // rows that fit a cluster take it at every batch size (V = 32,000, three rejected tokens: 137 -> 75 us for 256 sequences)
+    const ClusterShape shape = cluster_shape(B, V);
+    if (shape.C > 0) {
+        rsd::walk_cluster::ClusterArgs ca;
+        memset(&ca, 0, sizeof(ca));
+        ca.r = a;
+        ca.resample = 1;
+        ca.v.draft = a.draft; ca.v.target = a.target;
+        ca.v.V = V; ca.v.num_nodes = 1;
+        ca.v.seed_lo = a.seed_lo; ca.v.seed_hi = a.seed_hi; ca.v.step = step; ca.v.seq_base = seq_base;
+        launch_cluster_walk(ca, target_row->dtype, true, B, shape, s);
+        return check_launch("rsd_resample_residual");
+    }
     const bool aligned = rows_aligned(target_row) && (!rejected || rows_aligned(draft_row));
     using namespace rsd::walk_narrow;
     if (target_row->dtype == RSD_F32) {

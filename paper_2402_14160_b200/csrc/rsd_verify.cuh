@@ -171,29 +171,6 @@ __device__ __forceinline__ float load_clean(const char* row, int g, int V, float
     return clean<T>(pk, v, saw_nan);
 }
 
-// The walk itself is compiled twice (rsd_verify_walk.inc): for blocks of 256 threads, three (2-byte rows) or two
-// (4-byte rows) per SM, and for blocks of 512 threads, one per SM with all its registers.  A launch with at most one
-// sequence per SM has every SM to spare, and there the wider block shortens each pass of a walk's chain.
-#define RSD_WALK_NS walk_narrow
-#define RSD_WALK_THREADS 256
-#define RSD_WALK_MIN_BLOCKS_2B 3
-#define RSD_WALK_MIN_BLOCKS_4B 2
-#define RSD_WALK_WITH_RESAMPLE
 #include "rsd_verify_walk.inc"
-#undef RSD_WALK_WITH_RESAMPLE
-#undef RSD_WALK_NS
-#undef RSD_WALK_THREADS
-#undef RSD_WALK_MIN_BLOCKS_2B
-#undef RSD_WALK_MIN_BLOCKS_4B
-
-#define RSD_WALK_NS walk_wide
-#define RSD_WALK_THREADS 512
-#define RSD_WALK_MIN_BLOCKS_2B 1
-#define RSD_WALK_MIN_BLOCKS_4B 1
-#include "rsd_verify_walk.inc"
-#undef RSD_WALK_NS
-#undef RSD_WALK_THREADS
-#undef RSD_WALK_MIN_BLOCKS_2B
-#undef RSD_WALK_MIN_BLOCKS_4B
 
 }  // namespace rsd

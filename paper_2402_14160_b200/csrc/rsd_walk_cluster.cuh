@@ -1,0 +1,1010 @@
+// Recursive rejection sampling along the draft tree (Eqs. 1-4, Algorithm 1; Section 3.2.2, Algorithm 6), its two
+// baseline rules and the stand-alone residual draw, by a thread block cluster per sequence that holds the weights of the
+// node it is at on chip.
+//
+// A walk is a chain of dependent passes (open a node, one residual pass per rejected child), so with one block per
+// sequence its latency is the number of passes times a sweep over two rows by one SM.  Here the vocabulary is dealt out
+// to the blocks of a cluster, 512-element tiles in turn (tile t to block t mod C), and within a block to its working
+// warps, NT tiles each.  Opening a node loads both rows once, turns them into exponentials and leaves these in registers;
+// a rejected child then costs a fused multiply-add, a clamp and a sum per element, nothing is read or exponentiated
+// again.  The blocks' partial sums travel to all blocks through distributed shared memory (st.async onto an mbarrier),
+// and the control warp of every block takes the same decisions from the same numbers.  A control warp is one warp running
+// dependent scalar code (5-6 cycles per instruction), so whatever does not depend on the running pass is done while it
+// runs, one child per lane: tokens, row values, uniforms, the next node's children.
+//
+// Sums are taken in the order of the ring walk (rsd_walk_ring.cuh): per lane over the tiles of equal index modulo 8, in
+// pass direction, then over the lanes, then a tree over the eight classes in double.  The two walks give the same
+// bits, so which of them runs (a matter of batch size and vocabulary) does not show in any result.
+// Every wait on an mbarrier is bounded (about a second); a wait that runs out abandons the walk with RSD_ST_TIMEOUT.
+#pragma once
+#include "rsd_verify.cuh"
+#include "rsd_walk_ring.cuh"
+
+namespace rsd {
+namespace walk_cluster {
+
+using walk_ring::kSumFloor;
+using walk_ring::kTileElems;
+using walk_ring::warp_sum_f32;
+
+constexpr int kClasses = 8;              // summation classes: tiles of equal index modulo 8
+constexpr int kMaxListed = 64;           // rejected tokens remembered per node
+
+// Cmd::flags: what a pass does (low four bits) and options
+enum {
+    kEnd = 0,
+    kOpen = 1,           // load both rows of a node; sums of exp(lt k_q - c_q) and exp(ld k_p - c_p)
+    kOpenTarget = 2,     // load its target row; sum of exp(lt k_q - c_q)
+    kResidualPass = 3,   // sum of (q - a p)+
+    kPlainPass = 4,      // sum of q
+    kRestPass = 5,       // sum of p without the listed tokens
+    kOverlapPass = 6,    // K-SEQ: sum of min(a_hi p, a_lo q)
+    kSeqPass = 7,        // K-SEQ: sum of (q - c min(a_hi p, a_lo q))+
+    kDump = 8,           // the weights of one tile in token order
+    kTop1 = 9,           // Gumbel-Top-1 over the weights
+    kWrite = 10,         // the normalised weights to global memory
+    kKindMask = 15,
+    kClean = 16,         // kOpen, kOpenTarget: NaN counts as -inf; the rows' maxima are reported
+    kRelative = 32,      // kOpen, kOpenTarget: exponentials relative to sm.ref_q, sm.ref_p (else to 0)
+    kStoreTiles = 64,    // the sum of every tile goes to every block's tile_sum
+    kBackward = 128,     // order of the lanes' sums
+    kBuffer = 256,       // which half of class_sum / red_bar the pass reports to
+    kFreeze = 512,       // kResidualPass: first sm.freeze_x leaves the draft and keeps its weight
+    kModeShift = 12      // kDump, kTop1, kWrite: weights are 0 q, kResidual (q - a p)+, kSeqResidual K-SEQ's residual
+};
+
+struct __align__(16) Cmd {
+    int flags;
+    int node;            // kOpen, kOpenTarget: the node; kDump: the tile; kTop1: the node of the random stream
+    float a_hi, a_lo;
+};
+
+struct ClusterArgs {
+    VerifyArgs v;
+    ResampleArgs r;      // resample != 0: the stand-alone draw (v: rows, V and random stream only)
+    int resample;
+};
+
+template <int WARPS, int NT>
+struct Smem {
+    unsigned long long red_bar[2];
+    Cmd cmd;
+    float ref_q, ref_p;                      // references of the exponentials, in units of log2
+    float c_seq;                             // K-SEQ's factor of its residual
+    int freeze_x;
+    float freeze_hi, freeze_lo;              // the coefficient under which the frozen token's weight is taken
+    double inv_total;                        // kWrite
+    float class_sum[2][2 * kClasses];        // [buffer][target or only sum: 8 classes, draft sum: 8 classes]
+    float extra[2][3][kClasses];             // [buffer][maxima of target and draft, NaN seen][block]
+    unsigned long long top1[kClasses];       // [block] smallest key of the Gumbel draw with its token
+    unsigned long long warp_key[WARPS];
+    float lane_sum[2][WARPS * NT][32];       // [target / only sum, draft][local tile][lane]
+    float warp_top[2][WARPS];
+    int nan_seen;
+    int abort;
+    float tile_sum[kClasses * WARPS * NT];   // of all blocks' tiles
+    __align__(16) float tile_w[kTileElems];  // (read as float4)
+    int par[kMaxCachedNodes], tok[kMaxCachedNodes];
+    int kid_node[32];
+    int gone_tok[kMaxListed];
+    int n_gone_tok;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t remote_addr(const void* p, uint32_t rank) {   // p: this block's shared memory
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+// store a word in a block's shared memory and count its four bytes on that block's mbarrier
+__device__ __forceinline__ void send_word(uint32_t addr, float v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// the command barrier: the control warp arrives, the working warps wait
+template <int THREADS>
+__device__ __forceinline__ void cmd_arrive() { asm volatile("barrier.cta.arrive 1, %0;" ::"n"(THREADS) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void cmd_sync() { asm volatile("barrier.cta.sync 1, %0;" ::"n"(THREADS) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void dump_sync() { asm volatile("barrier.cta.sync 3, %0;" ::"n"(THREADS) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void workers_sync() { asm volatile("barrier.cta.sync 2, %0;" ::"n"(THREADS) : "memory"); }
+
+// A lane's 16 values of a tile: the 16-byte pieces lane, lane + 32, ... (the order of the ring walk), -inf beyond the
+// row's end.  Rows on 16-byte boundaries take one load a piece.  Others take the two aligned words around it, shifted;
+// tiles at the ends of such a row, and every row's partial tile, are put together from single elements.
+template <typename T>
+__device__ __forceinline__ void load_tile(Packed<T>& pk, const char* row, int tile, int lane, int V) {
+    constexpr int kElem = (int)sizeof(T), kPer = 16 / kElem, kPieces = 16 / kPer;
+    const char* at = row + ((int64_t)tile * kTileElems + lane * kPer) * kElem;
+    const uint32_t m = (uint32_t)(uintptr_t)row & 15u;
+    const int after = V - (tile + 1) * kTileElems;      // elements behind the tile
+    if (m == 0 && after >= 0) {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) pk.w[i] = ld_stream(at + 512 * i);
+    } else if (tile > 0 && after >= kPer) {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            const uint4 a = *(const uint4*)(at + 512 * i - m), b = *(const uint4*)(at + 512 * i - m + 16);
+            uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z, w7 = b.w;
+            if (m & 8u) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = w7; }
+            if (m & 4u) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
+            const uint32_t s = (m & 3u) * 8u;
+            pk.w[i] = make_uint4(__funnelshift_r(w0, w1, s), __funnelshift_r(w1, w2, s), __funnelshift_r(w2, w3, s), __funnelshift_r(w3, w4, s));
+        }
+    } else {
+        const int x0 = tile * kTileElems + lane * kPer;
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (kElem == 4) {
+                    const int x = x0 + i * 32 * kPer + j;
+                    w[j] = x < V ? ((const uint32_t*)row)[x] : 0xFF800000u;
+                } else {
+                    const int x = x0 + i * 32 * kPer + 2 * j;
+                    const uint32_t lo = x < V ? ((const uint16_t*)row)[x] : 0xFF80u, hi = x + 1 < V ? ((const uint16_t*)row)[x + 1] : 0xFF80u;
+                    w[j] = lo | (hi << 16);
+                }
+            }
+            pk.w[i] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+
+// weights of a lane's 16 values under the mode of a drawing pass
+template <bool EXTRA>
+__device__ __forceinline__ void mode_weights(int mode, const float (&q)[16], const float (&p)[16], float a_hi, float a_lo, float c, float (&w)[16]) {
+    if (mode == kResidual) {
+        residual16(q, p, a_hi, a_lo, w);
+    } else if (EXTRA && mode == kSeqResidual) {
+        weights16<kSeqResidual>(q, p, a_hi, a_lo, c, w);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) w[j] = q[j];
+    }
+}
+
+// A block's place in its cluster and the row's tiles.
+struct Place {
+    int rank, C, V, n_tiles, n_local;   // n_local: tiles rank, rank + C, ...
+};
+
+// What the working warps need to know about the sequence.
+struct WorkRows {
+    const char* q;               // its rows of node 0 ...
+    const char* p;
+    int64_t stride_q, stride_p;  // ... and the bytes from node to node
+    float kq, kp;                // log2(e) / temperature
+    bool with_draft;             // the first node probably needs its draft row as well
+    RngKey key;                  // kTop1
+    float* out_residual;         // kWrite
+};
+
+// Gumbel-Top-1 draw (Algorithm 6's last step, see gumbel_top1_pick() in rsd_verify_walk.inc): arg min of E(y) / w(y),
+// E(y) = t(U_M) / 16 + [y mod 16 != a] t(U_y).  E >= t(U_M) / 16 with equality at position a: the smallest exact key at
+// the positions a of the block's groups bounds the winner, and only entries whose own lower bound reaches it (a few per
+// cent) need their word of the fine stream.  The result is that of taking every entry.
+template <typename T, int NT, int WARPS>
+__device__ __forceinline__ void top1_pass(Smem<WARPS, NT>& sm, const Place& pl, const RngKey& key, uint32_t node, int flags, float a_hi, float a_lo,
+                                          const float (&q)[NT][16], const float (&p)[NT][16]) {
+    constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float inf = __int_as_float(0x7F800000);
+    unsigned long long best = ~0ull;             // key bits << 32 | token: keys are >= 0, so the order is that of (key, token)
+    auto offer = [&](float k, int x) {
+        if (k < inf) best = min(best, ((unsigned long long)__float_as_uint(k) << 32) | (uint32_t)x);
+    };
+#pragma unroll 1
+    for (int turn = 0; turn < 2; ++turn) {       // turn 0: positions a; turn 1: the rest below the block's bound
+        const float bound = best == ~0ull ? inf : __uint_as_float((uint32_t)(best >> 32));
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            const int tile = pl.rank + pl.C * (warp + WARPS * k);
+            if (tile >= pl.n_tiles) continue;
+            float w[16];
+            mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+#pragma unroll
+            for (int i = 0; i < kRuns; ++i) {
+                const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
+                const uint32_t g = (uint32_t)x0 >> 4;
+                const uint32_t cw = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
+                const float tg = neg_log_group_uniform_f32(cw) * 0.0625f;
+                const int ja = (int)(cw & 15u) - (x0 & 15);
+                if (turn == 0) {
+#pragma unroll
+                    for (int j = 0; j < kPer; ++j)
+                        if (j == ja && w[i * kPer + j] > 0.0f) offer(tg / w[i * kPer + j], x0 + j);
+                } else {
+                    uint32_t todo = 0;
+#pragma unroll
+                    for (int j = 0; j < kPer; ++j)
+                        if (w[i * kPer + j] > 0.0f && j != ja && tg <= bound * w[i * kPer + j] * 1.00001f) todo |= 1u << j;
+                    while (todo) {
+                        const int j = __ffs(todo) - 1;
+                        todo &= todo - 1;
+                        float wj = 0.0f;
+#pragma unroll
+                        for (int jj = 0; jj < kPer; ++jj)
+                            if (jj == j) wj = w[i * kPer + jj];
+                        const uint4 fw = rng_draw(key, node, kTagFinalGumbelFine, (uint32_t)(x0 + j) >> 2);
+                        const uint32_t sel = (uint32_t)(x0 + j) & 3u;
+                        const uint32_t word = sel < 2 ? (sel == 0 ? fw.x : fw.y) : (sel == 2 ? fw.z : fw.w);
+                        offer((tg + neg_log_uniform_f32(word)) / wj, x0 + j);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
+        if (lane == 0) sm.warp_key[warp] = best;
+        workers_sync<WARPS * 32>();
+        for (int w = 0; w < WARPS; ++w) best = min(best, sm.warp_key[w]);
+        workers_sync<WARPS * 32>();
+    }
+    if (warp == 0 && lane < pl.C) {
+        const uint32_t bar = remote_addr(&sm.red_bar[flags & kBuffer ? 1 : 0], lane), at = remote_addr(&sm.top1[pl.rank], lane);
+        send_word(at, __uint_as_float((uint32_t)best), bar);
+        send_word(at + 4u, __uint_as_float((uint32_t)(best >> 32)), bar);
+    }
+}
+
+// The working warps: the passes they are told to run.  The root's rows are asked for before the first command is there.
+// EXTRA: also the passes that only the baseline rules, the Gumbel-Top-1 draw and the stand-alone residual draw need.
+template <typename T, int NT, int WARPS, bool EXTRA>
+__device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const WorkRows& rows) {
+    constexpr int kAll = (WARPS + 1) * 32, kWorkers = WARPS * 32;
+    constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int C = pl.C, V = pl.V, n_tiles = pl.n_tiles;
+    const int tile0 = pl.rank + C * warp, tile_step = C * WARPS;   // this warp's tiles: tile0, tile0 + tile_step, ...
+    const int per_block = kClasses / C;                            // summation classes of this block
+    float q[NT][16], p[NT][16];
+#pragma unroll
+    for (int k = 0; k < NT; ++k)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) q[k][j] = p[k][j] = 0.0f;
+    int flags = rows.with_draft ? kOpen : kOpenTarget, node = 0;
+    float a_hi = 0.0f, a_lo = 0.0f;
+    bool first = true;
+    for (;;) {
+        int kind = flags & kKindMask;
+        float s[NT];
+        if (kind == kOpen || kind == kOpenTarget) {
+            Packed<T> rq[NT], rp[NT];
+            const char* rowq = rows.q + (int64_t)node * rows.stride_q;
+            const char* rowp = rows.p + (int64_t)node * rows.stride_p;
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                const int tile = tile0 + tile_step * k;
+                rq[k].fill_neg_inf();
+                rp[k].fill_neg_inf();
+                if (tile < n_tiles) {
+                    load_tile<T>(rq[k], rowq, tile, lane, V);
+                    if (kind == kOpen) load_tile<T>(rp[k], rowp, tile, lane, V);
+                }
+            }
+            if (first) {
+                first = false;
+                cluster_wait();         // every block's mbarriers are in place
+                cmd_sync<kAll>();
+                flags = sm.cmd.flags;   // the root's rows, with or without the draft row
+                kind = flags & kKindMask;
+            }
+            float cq = 0.0f, cp = 0.0f;
+            if (flags & (kClean | kRelative)) {
+                if (flags & kRelative) { cq = sm.ref_q; cp = sm.ref_p; }
+                if (flags & kClean) {
+                    float mq = kNegInf, mp = kNegInf;
+                    bool saw_nan = false;
+#pragma unroll
+                    for (int k = 0; k < NT; ++k) {
+                        float m = group_max_nan(rq[k]);
+                        if (m != m) { saw_nan = true; rq[k].clean_nan(); m = group_max_nan(rq[k]); }
+                        mq = fmaxf(mq, m);
+                        if (kind == kOpen) {
+                            m = group_max_nan(rp[k]);
+                            if (m != m) { saw_nan = true; rp[k].clean_nan(); m = group_max_nan(rp[k]); }
+                            mp = fmaxf(mp, m);
+                        }
+                    }
+                    mq = warp_max(mq);
+                    mp = warp_max(mp);
+                    if (lane == 0) { sm.warp_top[0][warp] = mq; sm.warp_top[1][warp] = mp; }
+                    if (saw_nan) sm.nan_seen = 1;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                rq[k].unpack(q[k]);
+                exp16(q[k], rows.kq, cq, q[k]);
+                s[k] = tree_sum16(q[k]);
+            }
+            if (kind == kOpen) {
+#pragma unroll
+                for (int k = 0; k < NT; ++k) {
+                    rp[k].unpack(p[k]);
+                    exp16(p[k], rows.kp, cp, p[k]);
+                    sm.lane_sum[1][warp + WARPS * k][lane] = tree_sum16(p[k]);
+                }
+            }
+        } else if (kind == kResidualPass) {
+            if (EXTRA && (flags & kFreeze)) {
+                const int x = sm.freeze_x;
+                int l_, j_;
+                walk_ring::piece_of<T>(x % kTileElems, l_, j_);
+#pragma unroll
+                for (int k = 0; k < NT; ++k)
+                    if (tile0 + tile_step * k == x / kTileElems && l_ == lane) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j == j_) { q[k][j] = residual_weight(q[k][j], p[k][j], sm.freeze_hi, sm.freeze_lo); p[k][j] = 0.0f; }
+                    }
+            }
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                float w[16];
+                residual16(q[k], p[k], a_hi, a_lo, w);
+                s[k] = tree_sum16(w);
+            }
+        } else if (kind == kPlainPass) {
+#pragma unroll
+            for (int k = 0; k < NT; ++k) s[k] = tree_sum16(q[k]);
+        } else if (kind == kRestPass) {
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                uint32_t gone = 0;
+                for (int i = 0; i < sm.n_gone_tok; ++i) {
+                    const int o = sm.gone_tok[i] - (tile0 + tile_step * k) * kTileElems;
+                    if (o < 0 || o >= kTileElems) continue;
+                    int l_, j_;
+                    walk_ring::piece_of<T>(o, l_, j_);
+                    if (l_ == lane) gone |= 1u << j_;
+                }
+                float w[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) w[j] = ((gone >> j) & 1u) ? 0.0f : p[k][j];
+                s[k] = tree_sum16(w);
+            }
+        } else if (EXTRA && (kind == kOverlapPass || kind == kSeqPass)) {
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                float w[16];
+                if (kind == kOverlapPass) weights16<kSeqOverlap>(q[k], p[k], a_hi, a_lo, 0.0f, w);
+                else weights16<kSeqResidual>(q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+                s[k] = tree_sum16(w);
+            }
+        } else if (kind == kDump) {
+#pragma unroll
+            for (int k = 0; k < NT; ++k)
+                if (tile0 + tile_step * k == node) {
+                    float w[16];
+                    mode_weights<EXTRA>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, EXTRA ? sm.c_seq : 0.0f, w);
+#pragma unroll
+                    for (int i = 0; i < kRuns; ++i)
+#pragma unroll
+                        for (int j = 0; j < kPer; ++j) sm.tile_w[(i * 32 + lane) * kPer + j] = w[i * kPer + j];
+                }
+            dump_sync<kAll>();
+        } else if (EXTRA && kind == kWrite) {
+            dump_sync<kAll>();                  // everyone has read the command
+            const double inv = sm.inv_total;
+            float* out = rows.out_residual;
+            const bool vec = ((uintptr_t)out & 15u) == 0;
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                const int tile = tile0 + tile_step * k;
+                if (tile >= n_tiles) continue;
+                float w[16];
+                mode_weights<EXTRA>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, 0.0f, w);
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                    const int x = tile * kTileElems + ((i / kPer) * 32 + lane) * kPer + i % kPer;
+                    float o[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[j] = (float)((double)w[i + j] * inv);
+                    if (vec && x + 4 <= V) {
+                        *(float4*)(out + x) = make_float4(o[0], o[1], o[2], o[3]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (x + j < V) out[x + j] = o[j];
+                    }
+                }
+            }
+        } else if (EXTRA && kind == kTop1) {
+            top1_pass<T, NT, WARPS>(sm, pl, rows.key, (uint32_t)node, flags, a_hi, a_lo, q, p);
+        } else {
+            return;                             // kEnd
+        }
+        if (kind < kDump) {                     // the pass reports sums
+#pragma unroll
+            for (int k = 0; k < NT; ++k) sm.lane_sum[0][warp + WARPS * k][lane] = s[k];
+            workers_sync<kWorkers>();           // the lanes' sums are in place
+            const int buf = flags & kBuffer ? 1 : 0;
+            for (int i = warp; i < (kind == kOpen ? 2 * per_block : per_block); i += WARPS) {
+                const int which = i >= per_block ? 1 : 0, cl = i - which * per_block;
+                const int n = pl.n_local > cl ? (pl.n_local - cl + per_block - 1) / per_block : 0;
+                const int step = flags & kBackward ? -per_block : per_block, at = flags & kBackward ? cl + per_block * (n - 1) : cl;
+                float acc = 0.0f;
+                for (int m0 = 0; m0 < n; m0 += 8) {
+                    float v[8];
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) v[m] = m0 + m < n ? sm.lane_sum[which][at + step * (m0 + m)][lane] : 0.0f;
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) acc += v[m];
+                }
+                acc = warp_sum_f32(acc);
+                if (lane < C)
+                    send_word(remote_addr(&sm.class_sum[buf][which * kClasses + pl.rank + C * cl], lane), acc, remote_addr(&sm.red_bar[buf], lane));
+            }
+            if (flags & kStoreTiles) {
+#pragma unroll
+                for (int k = 0; k < NT; ++k) {
+                    const int tile = tile0 + tile_step * k;
+                    const float ts = warp_sum_f32(s[k]);
+                    if (lane < C && tile < n_tiles) send_word(remote_addr(&sm.tile_sum[tile], lane), ts, remote_addr(&sm.red_bar[buf], lane));
+                }
+            }
+            if ((flags & kClean) && warp == WARPS - 1) {
+                const float mq = warp_max(lane < WARPS ? sm.warp_top[0][lane] : kNegInf), mp = warp_max(lane < WARPS ? sm.warp_top[1][lane] : kNegInf);
+                if (lane < C) {
+                    const uint32_t bar = remote_addr(&sm.red_bar[buf], lane);
+                    send_word(remote_addr(&sm.extra[buf][0][pl.rank], lane), mq, bar);
+                    send_word(remote_addr(&sm.extra[buf][1][pl.rank], lane), mp, bar);
+                    send_word(remote_addr(&sm.extra[buf][2][pl.rank], lane), sm.nan_seen ? 1.0f : 0.0f, bar);
+                }
+            }
+        }
+        cmd_sync<kAll>();
+        const Cmd cmd = sm.cmd;
+        flags = cmd.flags;
+        node = cmd.node;
+        a_hi = cmd.a_hi;
+        a_lo = cmd.a_lo;
+    }
+}
+
+// Sum over the eight classes in lanes 8 i .. 8 i + 7 as ((0+1)+(2+3))+((4+5)+(6+7)), on each of those lanes.
+__device__ __forceinline__ double class_tree(double v) {
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+// The control warp: the walk itself, the same in every block of the cluster.
+template <typename T, int NT, int WARPS, bool EXTRA>
+struct Control {
+    static constexpr int kAll = (WARPS + 1) * 32;
+    Smem<WARPS, NT>& sm;
+    const ClusterArgs& ca;
+    const VerifyArgs& a;
+    const Place& pl;
+    const int b, lane;
+    const RngKey key;
+    int pass_no, backward;
+    bool aborted;
+    float kq, kp, mq, mp;           // log2(e) / temperature; references of the exponentials (raw units)
+    double Sq, Sp, inv_Sq, inv_Sp, ratio;
+    double A, Z;                    // closed-form chain (see rsd_verify.cuh)
+    float a_hi, a_lo;               // A Sq / Sp as a two-float sum
+    int status;
+
+    __device__ __forceinline__ Control(Smem<WARPS, NT>& sm_, const ClusterArgs& ca_, const Place& pl_, int b_)
+        : sm(sm_), ca(ca_), a(ca_.v), pl(pl_), b(b_), lane(threadIdx.x & 31),
+          key{ca_.v.seed_lo, ca_.v.seed_hi, ca_.v.step, ca_.v.seq_base + (uint32_t)b_}, pass_no(0), backward(0), aborted(false),
+          kq(kLog2e * ca_.v.target.inv_temp), kp(kLog2e * ca_.v.draft.inv_temp), mq(0.0f), mp(0.0f), A(0.0), Z(1.0), a_hi(0.0f), a_lo(0.0f),
+          status(0) {}
+
+    // publish a command; the pass reports `words` words to every block
+    __device__ __forceinline__ void issue(int flags, int node, int words) {
+        const int buf = pass_no & 1;
+        ++pass_no;
+        if (lane == 0) {
+            Cmd cmd;
+            cmd.flags = flags | (buf ? kBuffer : 0) | (backward ? kBackward : 0);
+            cmd.node = node;
+            cmd.a_hi = a_hi;
+            cmd.a_lo = a_lo;
+            sm.cmd = cmd;
+            mbar_expect_tx(&sm.red_bar[buf], 4u * (uint32_t)words);
+        }
+        __syncwarp();
+        cmd_arrive<kAll>();
+        backward ^= 1;
+    }
+    // wait for the words of the latest pass; sets `aborted` when they do not come
+    __device__ __forceinline__ int land() {
+        const int n = pass_no - 1, buf = n & 1;
+        int late = 0;
+        wait_bar(&sm.red_bar[buf], (uint32_t)(n >> 1) & 1u, &late);
+        if (__any_sync(0xFFFFFFFFu, late)) aborted = true;
+        return buf;
+    }
+    __device__ __forceinline__ double collect() {        // one sum
+        const int buf = land();
+        return __shfl_sync(0xFFFFFFFFu, class_tree((double)sm.class_sum[buf][lane & (kClasses - 1)]), 0);
+    }
+    __device__ __forceinline__ void collect2(double& s0, double& s1) {
+        const int buf = land();
+        const double v = class_tree((double)sm.class_sum[buf][lane & (2 * kClasses - 1)]);
+        s0 = __shfl_sync(0xFFFFFFFFu, v, 0);
+        s1 = __shfl_sync(0xFFFFFFFFu, v, kClasses);
+    }
+    __device__ __forceinline__ static bool usable(double s) { return s >= (double)kSumFloor && s < 1e300; }
+
+    __device__ __forceinline__ void issue_open(int node, bool with_draft, int options) {
+        issue((with_draft ? kOpen : kOpenTarget | kStoreTiles) | options, node,
+              (with_draft ? 2 * kClasses : kClasses + pl.n_tiles) + (options & kClean ? 3 * pl.C : 0));
+    }
+    // The sums of a node whose first pass, relative to 0, has been issued.  If they are not finite, or so small that
+    // underflow may have eaten them, a cleaning pass finds the rows' maxima and the pass is run again relative to them.
+    __device__ __forceinline__ void open_sums(int node, bool with_draft) {
+        A = 0.0; Z = 1.0; a_hi = a_lo = 0.0f; mq = mp = 0.0f;
+        double s0, s1;
+        collect2(s0, s1);
+        if (!with_draft) s1 = 1.0;
+        if (!(usable(s0) && usable(s1)) && !aborted) {
+            issue_open(node, with_draft, kClean);
+            collect2(s0, s1);
+            if (!with_draft) s1 = 1.0;
+            const int buf = (pass_no - 1) & 1;
+            float top_q = kNegInf, top_p = kNegInf;
+            bool saw_nan = false;
+            for (int i = 0; i < pl.C; ++i) {
+                top_q = fmaxf(top_q, sm.extra[buf][0][i]);
+                top_p = fmaxf(top_p, sm.extra[buf][1][i]);
+                saw_nan |= sm.extra[buf][2][i] != 0.0f;
+            }
+            if (saw_nan) status |= 1;              // RSD_ST_NAN_INPUT
+            if (!(usable(s0) && usable(s1)) && !aborted) {
+                if (top_q > kNegInf) mq = top_q;
+                if (with_draft && top_p > kNegInf) mp = top_p;
+                if (lane == 0) { sm.ref_q = mq * kq; sm.ref_p = mp * kp; }
+                issue_open(node, with_draft, (saw_nan ? kClean : 0) | kRelative);
+                collect2(s0, s1);
+                if (!with_draft) s1 = 1.0;
+            }
+            if (lane == 0) sm.nan_seen = 0;        // (published with the next command)
+        }
+        Sq = s0;
+        Sp = s1;
+    }
+    __device__ __forceinline__ void set_a(double A_) {
+        A = A_;
+        const double aa = A * ratio;
+        a_hi = (float)aa;
+        a_lo = (float)(aa - (double)a_hi);
+    }
+    __device__ __forceinline__ void take_in(double Z_new, double A_old, bool& kept) {
+        if (Z_new > 0.0 && Z_new < 1.7e308) {
+            Z = Z_new;
+            kept = true;
+        } else {
+            status |= 4;   // RSD_ST_ZERO_RESIDUAL: keep the previous residual
+            set_a(A_old);
+            kept = false;
+        }
+    }
+
+    // a node's first 32 children after node `after`, in stored order, one per lane (-1: none)
+    __device__ __forceinline__ int children(int of, int after, const int32_t* par, const int32_t* tok, bool cached) {
+        int found = 0;
+        sm.kid_node[lane] = -1;
+        __syncwarp();
+        for (int c0 = after + 1; c0 < a.num_nodes && found < 32; c0 += 32) {
+            const int cc = c0 + lane;
+            bool ok = false;
+            if (cc < a.num_nodes) {
+                const int pn = cached ? sm.par[cc] : par[cc];
+                const int t = cached ? sm.tok[cc] : tok[cc];
+                ok = pn == of && t >= 0 && t < pl.V;
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, ok);
+            const int at = found + __popc(m & ((1u << lane) - 1u));
+            if (ok && at < 32) sm.kid_node[at] = cc;
+            found += __popc(m);
+        }
+        __syncwarp();
+        const int r = sm.kid_node[lane];
+        __syncwarp();
+        return r;
+    }
+
+    // The last token under the weights of `mode` and its block's outputs.  Every block knows the tile sums; the block
+    // that holds the crossing's tile ends the draw.  Returns true on the block that has the token in `last`.
+    __device__ __forceinline__ bool draw(int mode, uint32_t node, int& last) {
+        const uint4 rw = rng_draw(key, node, kTagResample, 0u);
+        const double u = ((double)rw.x + 0.5) * (1.0 / 4294967296.0);
+        walk_ring::TilePick t;
+        walk_ring::pick_tile(sm.tile_sum, pl.n_tiles, u, t);
+        if (t.tile < 0) { last = -1; return pl.rank == 0; }
+        if (t.tile % pl.C != pl.rank) return false;
+        if (lane == 0) {
+            Cmd cmd;
+            cmd.flags = kDump | (mode << kModeShift);
+            cmd.node = t.tile;
+            cmd.a_hi = a_hi;
+            cmd.a_lo = a_lo;
+            sm.cmd = cmd;
+        }
+        __syncwarp();
+        cmd_arrive<kAll>();
+        dump_sync<kAll>();
+        float w[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 f = *(const float4*)&sm.tile_w[16 * lane + 4 * i];
+            w[4 * i] = f.x; w[4 * i + 1] = f.y; w[4 * i + 2] = f.z; w[4 * i + 3] = f.w;
+        }
+        last = walk_ring::pick_in_tile(w, t);
+        return true;
+    }
+    __device__ __forceinline__ bool draw_top1(int mode, uint32_t node, int& last) {
+        issue(kTop1 | (mode << kModeShift), (int)node, 2 * pl.C);
+        land();
+        unsigned long long best = ~0ull;
+        for (int i = 0; i < pl.C; ++i) best = min(best, sm.top1[i]);
+        last = aborted || best == ~0ull ? -1 : (int)(uint32_t)best;
+        return pl.rank == 0;
+    }
+    // after a walk whose latest pass does not hold the tile sums of what the last token is drawn from
+    __device__ __forceinline__ double refresh_tiles(bool residual) {
+        issue((residual ? kResidualPass : kPlainPass) | kStoreTiles, 0, kClasses + pl.n_tiles);
+        return collect();
+    }
+    __device__ __forceinline__ void end_work() {
+        if (lane == 0) sm.cmd.flags = kEnd;
+        __syncwarp();
+        cmd_arrive<kAll>();
+        if (aborted) status |= 32;   // RSD_ST_TIMEOUT
+    }
+
+    // What is left of the draft once subtraction has lost its accuracy: summed anew without the rejected tokens.
+    __device__ __forceinline__ double rest(int n_removed) {
+        if (lane == 0) sm.n_gone_tok = n_removed;
+        issue(kRestPass, 0, kClasses);
+        return collect() * inv_Sp;
+    }
+
+    __device__ __forceinline__ void walk() {
+        const int32_t* par = a.parent + (a.shared_topology ? 0 : (int64_t)b * a.num_nodes);
+        const int32_t* tok = a.token + (int64_t)b * a.num_nodes;
+        const bool cached = a.num_nodes <= kMaxCachedNodes;
+        const int rule = EXTRA ? a.rule : 0;
+        const int64_t out0 = (int64_t)b * a.L;
+        if (cached) {
+#pragma unroll 4
+            for (int n = lane; n < a.num_nodes; n += 32) { sm.par[n] = par[n]; sm.tok[n] = tok[n]; }
+            __syncwarp();
+        }
+        int cur = 0, len = 0, reason = 0, seq_kids = 0;
+        bool tiles_valid = false, with_draft;
+        int child_node = children(0, 0, par, tok, cached);
+        unsigned kids = __ballot_sync(0xFFFFFFFFu, child_node >= 0);
+        with_draft = kids != 0u && a.L > 0;
+        cluster_wait();                               // every block's mbarriers are in place
+        issue_open(0, with_draft, 0);
+        if (pl.rank == 0) {
+            for (int i = lane; i < a.L; i += 32) {
+                a.accepted_node[out0 + i] = -1;
+                a.accepted_token[out0 + i] = -1;
+            }
+            if (a.dbg_theta)
+                for (int n = lane; n < a.num_nodes; n += 32) a.dbg_theta[(int64_t)b * a.num_nodes + n] = __int_as_float(0x7FC00000);
+            __syncwarp();
+        }
+        for (;;) {
+            // ---- the node `cur` is being opened: what its children need, one child per lane ---------------------------------
+            if (!with_draft) {
+                open_sums(cur, false);
+                tiles_valid = true;
+                reason = len >= a.L ? 2 : 1;          // RSD_STOP_LEAF : RSD_STOP_NO_CHILDREN
+                break;
+            }
+            const char* rowq = row_ptr<T>(a.target, b, cur);
+            const char* rowp = row_ptr<T>(a.draft, b, cur);
+            int j0 = 0, n_removed = 0;                // children are looked at 32 at a time: j0 is the rank of lane 0's
+            int child_x;
+            float lq, lp;
+            double Ud;
+            bool repeated, p_none;
+            auto fetch_children = [&] {
+                child_x = -1;
+                lq = lp = 0.0f;
+                if (child_node >= 0) {
+                    child_x = cached ? sm.tok[child_node] : tok[child_node];
+                    lq = RowIO<T>::scalar(rowq, child_x);
+                    lp = RowIO<T>::scalar(rowp, child_x);
+                }
+                const uint4 rw = rng_draw(key, (uint32_t)cur, kTagAccept, (uint32_t)(j0 + lane));
+                Ud = (double)(rw.x >> 8) * (1.0 / 16777216.0);
+                // an earlier sibling with the same token: rejected by the time this one is tested, its draft mass is gone (Eq. 1)
+                repeated = (__match_any_sync(0xFFFFFFFFu, child_x) & ((1u << lane) - 1u)) != 0u;
+                for (int i = 0; i < n_removed && j0 > 0; ++i) repeated |= sm.gone_tok[i] == child_x;
+                if (rule != 0) repeated = false;      // (the baselines never change the draft)
+            };
+            fetch_children();
+            int next_kid = children(__shfl_sync(0xFFFFFFFFu, child_node, 0), 0, par, tok, cached);
+            open_sums(cur, true);
+            if (aborted) break;
+            inv_Sq = 1.0 / Sq;
+            inv_Sp = 1.0 / Sp;
+            ratio = Sq * inv_Sp;
+            const float lg_inv_ratio = lg2_approx((float)fmin(fmax(Sp * inv_Sq, 1e-37), 1e37));
+            double qpd, px_row, qxd;                  // q(x) / p(x), p(x), q(x)
+            auto weigh_children = [&] {
+                const float eq = fmaf(lq, kq, -mq * kq), ep = fmaf(lp, kp, -mp * kp);
+                const float qh = (lq == lq) ? ex2_approx(eq) : 0.0f, ph = (lp == lp) ? ex2_approx(ep) : 0.0f;
+                // q(x) / p(x) from the difference of the exponents survives probabilities below the fp32 range
+                p_none = !(lp == lp) || !(lp > kNegInf);
+                qpd = (double)((lq == lq && !p_none) ? ex2_approx((eq - ep) + lg_inv_ratio) : 0.0f);
+                px_row = (double)ph * inv_Sp;
+                qxd = (double)qh * inv_Sq;
+            };
+            weigh_children();
+            // 1 - P of the closed form (see the ring walk: summed anew once subtraction loses accuracy)
+            double one_mP = 1.0, one_mP_err = 0.0, inv_1mP = 1.0;
+            int j = 0, accepted_lane = -1;            // j: lane of the child under test
+            for (;;) {
+                // Eq. 3 in closed form: accept iff U < min(1, (q/p - A)+ (1 - P) / Z); a child the draft cannot produce any more
+                // is taken iff it has residual mass (RSD_ST_ZERO_DRAFT_PROB).  Every lane tests its own child, lane j's counts.
+                const bool no_draft = repeated || p_none;
+                double g;
+                bool take;
+                if (EXTRA && rule == 2) {             // K-SEQ: min(1, q / (gamma p))
+                    g = no_draft ? (qxd > 0.0 ? 1.0 : 0.0) : qpd / (double)a.gamma;
+                    take = Ud < g;
+                } else if (!no_draft) {
+                    g = fmax(qpd - A, 0.0) * one_mP;
+                    take = Ud * Z < g;
+                } else {
+                    take = fmax(qxd - A * px_row, 0.0) > 0.0;
+                    g = take ? Z : 0.0;
+                }
+                const unsigned taken = __ballot_sync(0xFFFFFFFFu, take), none_left = __ballot_sync(0xFFFFFFFFu, no_draft);
+                if ((none_left >> j) & 1u) status |= 8;
+                if (a.dbg_theta && pl.rank == 0 && lane == j)
+                    a.dbg_theta[(int64_t)b * a.num_nodes + child_node] = (float)fmin(1.0, (EXTRA && rule == 2) ? g : g / Z);
+                if ((taken >> j) & 1u) { accepted_lane = j; break; }
+                // rejected.  Eqs. 1-2 in closed form: A_{j+1} = A_j + Z_j / (1 - P_j), Z_{j+1} = sum (q - A_{j+1} p)+
+                const bool more_here = j < 31 && ((kids >> (j + 1)) & 1u);
+                const int more_nodes = (j == 31 && kids == 0xFFFFFFFFu) ? children(cur, __shfl_sync(0xFFFFFFFFu, child_node, 31), par, tok, cached) : -1;
+                const bool more = more_here || __any_sync(0xFFFFFFFFu, more_nodes >= 0);
+                const double A_old = A;
+                if (!(EXTRA && rule == 2)) {
+                    set_a(fma(Z, inv_1mP, A));
+                    issue(kResidualPass | (more ? 0 : kStoreTiles), 0, kClasses + (more ? 0 : pl.n_tiles));
+                }
+                const int x = __shfl_sync(0xFFFFFFFFu, child_x, j);
+                const bool rep = (__ballot_sync(0xFFFFFFFFu, repeated) >> j) & 1u;
+                const double px = (EXTRA && rule != 0) ? 0.0 : __shfl_sync(0xFFFFFFFFu, no_draft ? 0.0 : px_row, j);
+                double one_mP_new = one_mP - px, err_new = one_mP_err + 4e-7 * px;   // (px = 0 for a repeated token)
+                if (!rep && n_removed < kMaxListed) {
+                    if (lane == 0) sm.gone_tok[n_removed] = x;
+                    ++n_removed;
+                    __syncwarp();
+                }
+                inv_1mP = 1.0 / one_mP_new;
+                if (more) {
+                    if (more_here) {
+                        ++j;
+                    } else {                          // the next 32 children
+                        child_node = more_nodes;
+                        kids = __ballot_sync(0xFFFFFFFFu, child_node >= 0);
+                        j0 += 32;
+                        j = 0;
+                        fetch_children();
+                        weigh_children();
+                    }
+                    next_kid = children(__shfl_sync(0xFFFFFFFFu, child_node, j), 0, par, tok, cached);
+                }
+                if (!(EXTRA && rule == 2)) {
+                    const double Z_new = collect() * inv_Sq;
+                    if (aborted) break;
+                    bool kept;
+                    take_in(Z_new, A_old, kept);
+                    tiles_valid = kept && !more;
+                }
+                if (!(EXTRA && rule != 0)) {
+                    if (more && err_new > 2e-6 * one_mP_new && n_removed < kMaxListed) {   // (every rejected token is listed)
+                        one_mP_new = rest(n_removed);
+                        if (aborted) break;
+                        err_new = 4e-7 * one_mP_new;
+                        inv_1mP = 1.0 / one_mP_new;
+                    }
+                    one_mP = one_mP_new;
+                    one_mP_err = err_new;
+                    if (!(one_mP > 0.0)) { status |= 16; break; }   // RSD_ST_DRAFT_EXHAUSTED
+                }
+                if (!more) { ++j; break; }
+            }
+            if (aborted) break;
+            if (accepted_lane < 0) {   // RSD_STOP_ALL_REJECTED: the last token comes from the residual in force
+                reason = 0;
+                seq_kids = j0 + j;
+                break;
+            }
+            const int x = __shfl_sync(0xFFFFFFFFu, child_x, accepted_lane);
+            cur = __shfl_sync(0xFFFFFFFFu, child_node, accepted_lane);
+            child_node = next_kid;
+            kids = __ballot_sync(0xFFFFFFFFu, child_node >= 0);
+            with_draft = kids != 0u && len + 1 < a.L;
+            backward = 0;
+            tiles_valid = false;
+            issue_open(cur, with_draft, 0);
+            if (lane == 0 && pl.rank == 0) {
+                a.accepted_node[out0 + len] = cur;
+                a.accepted_token[out0 + len] = x;
+            }
+            ++len;
+        }
+        int mode = with_draft && A != 0.0 ? (int)kResidual : 0;
+        if (EXTRA && !aborted && rule == 2 && with_draft) {
+            // K-SEQ after all K children were rejected: beta = sum min{p, q / gamma}, then the residual
+            // (q - min{p, q / gamma} (1 - (1 - beta)^K) / beta)+
+            a_hi = (float)(Sq / Sp);
+            a_lo = (float)(1.0 / (double)a.gamma);
+            issue(kOverlapPass, 0, kClasses);
+            const double beta = collect() / Sq;
+            double miss = 1.0;
+            for (int i = 0; i < seq_kids; ++i) miss *= 1.0 - beta;
+            const float c = (float)(beta > 0.0 ? (1.0 - miss) / beta : (double)seq_kids);
+            if (lane == 0) sm.c_seq = c;
+            issue(kSeqPass | kStoreTiles, 0, kClasses + pl.n_tiles);
+            const double t = collect();
+            tiles_valid = t > 0.0 && t < 1.7e308;
+            if (tiles_valid) mode = kSeqResidual;
+            else status |= 4;                         // RSD_ST_ZERO_RESIDUAL: draw from the target row itself
+        }
+        const bool top1 = EXTRA && a.final_sampler == 1;
+        if (!aborted && !tiles_valid && !top1) refresh_tiles(mode == kResidual);
+        int last = -1;
+        bool mine = pl.rank == 0;
+        if (!aborted) mine = top1 ? draw_top1(mode, (uint32_t)cur, last) : draw(mode, (uint32_t)cur, last);
+        end_work();
+        if (mine && lane == 0) {
+            a.accepted_len[b] = len;
+            a.last_token[b] = last;
+            a.stop_reason[b] = reason;
+            a.status[b] = status;
+        }
+    }
+
+    // The stand-alone residual draw: the tokens of a list are rejected in order, then one token is drawn.  A listed token
+    // keeps the residual mass it has when it is removed (its draft probability is 0 afterwards): the pass after freezes it.
+    __device__ __forceinline__ void resample() {
+        const ResampleArgs& r = ca.r;
+        int tok = -1;
+        if (r.rejected && lane < r.max_k) tok = r.rejected[(int64_t)b * r.max_k + lane];
+        if (tok < 0 || tok >= pl.V) tok = -1;
+        unsigned left = __ballot_sync(0xFFFFFFFFu, tok >= 0);
+        const bool with_draft = left != 0u;
+        cluster_wait();
+        issue_open(0, with_draft, 0);
+        const char* rowp = row_ptr<T>(a.draft, b, 0);
+        const float lp = tok >= 0 ? RowIO<T>::scalar(rowp, tok) : 0.0f;
+        const bool repeated = (__match_any_sync(0xFFFFFFFFu, tok) & ((1u << lane) - 1u)) != 0u;   // listed twice
+        const uint32_t node = (uint32_t)r.rng_node[b];
+        open_sums(0, with_draft);
+        inv_Sq = 1.0 / Sq;
+        inv_Sp = 1.0 / Sp;
+        ratio = Sq * inv_Sp;
+        double total = Sq;
+        bool tiles_valid = !with_draft;
+        const double px_row = (lp == lp) ? (double)ex2_approx(fmaf(lp, kp, -mp * kp)) * inv_Sp : 0.0;
+        double one_mP = 1.0, one_mP_err = 0.0;
+        int n_removed = 0, freeze = 0;
+        while (left && !aborted) {
+            const int j = __ffs(left) - 1;
+            left &= left - 1u;
+            const double A_old = A;
+            set_a(A + Z / one_mP);
+            issue(kResidualPass | freeze | (left ? 0 : kStoreTiles), 0, kClasses + (left ? 0 : pl.n_tiles));
+            freeze = 0;
+            const bool rep = (__ballot_sync(0xFFFFFFFFu, repeated) >> j) & 1u;
+            const int x = __shfl_sync(0xFFFFFFFFu, tok, j);
+            const double px = rep ? 0.0 : __shfl_sync(0xFFFFFFFFu, px_row, j);
+            const double zhat = collect();
+            if (aborted) break;
+            bool kept;
+            take_in(zhat * inv_Sq, A_old, kept);
+            if (kept) total = zhat;
+            tiles_valid = kept && !left;
+            if (!rep) {
+                if (lane == 0) { sm.gone_tok[n_removed] = x; sm.freeze_x = x; sm.freeze_hi = a_hi; sm.freeze_lo = a_lo; }
+                ++n_removed;
+                freeze = kFreeze;
+            }
+            one_mP -= px;
+            one_mP_err += 4e-7 * px;
+            if (one_mP_err > 2e-6 * one_mP && left) {
+                one_mP = rest(n_removed);
+                one_mP_err = 4e-7 * one_mP;
+            }
+            if (!(one_mP > 0.0)) { status |= 16; break; }   // RSD_ST_DRAFT_EXHAUSTED
+        }
+        const int mode = with_draft && A != 0.0 ? (int)kResidual : 0;
+        if (!aborted && !tiles_valid) total = refresh_tiles(mode == kResidual);
+        int last = -1;
+        bool mine = pl.rank == 0;
+        if (!aborted) {
+            mine = draw(mode, node, last);
+            if (r.out_residual) {
+                if (lane == 0) {
+                    sm.inv_total = total > 0.0 ? 1.0 / total : 0.0;
+                    Cmd cmd;
+                    cmd.flags = kWrite | (mode << kModeShift);
+                    cmd.node = 0;
+                    cmd.a_hi = a_hi;
+                    cmd.a_lo = a_lo;
+                    sm.cmd = cmd;
+                }
+                __syncwarp();
+                cmd_arrive<kAll>();
+                dump_sync<kAll>();   // (the command has been read: its place may take the next one)
+            }
+        }
+        end_work();
+        if (mine && lane == 0) {
+            r.out_token[b] = last;
+            r.status[b] = status;
+        }
+    }
+};
+
+template <typename T, int NT, int WARPS, bool EXTRA>
+__global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 2) : 1) walk_cluster_kernel(const __grid_constant__ ClusterArgs ca) {
+    __shared__ Smem<WARPS, NT> sm;
+    const VerifyArgs& a = ca.v;
+    Place pl;
+    pl.rank = (int)cluster_rank();
+    pl.C = (int)cluster_size();
+    pl.V = a.V;
+    pl.n_tiles = (a.V + kTileElems - 1) / kTileElems;
+    pl.n_local = pl.n_tiles > pl.rank ? (pl.n_tiles - pl.rank + pl.C - 1) / pl.C : 0;
+    const int b = blockIdx.x / pl.C;
+    if (threadIdx.x == WARPS * 32) {
+        mbar_init(&sm.red_bar[0], 1);
+        mbar_init(&sm.red_bar[1], 1);
+        sm.nan_seen = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_arrive();
+    if (threadIdx.x < WARPS * 32) {
+        WorkRows rows;
+        rows.q = row_ptr<T>(a.target, b, 0);
+        rows.p = row_ptr<T>(a.draft, b, 0);
+        rows.stride_q = a.target.row_stride * RowIO<T>::kBytes;
+        rows.stride_p = a.draft.row_stride * RowIO<T>::kBytes;
+        rows.kq = kLog2e * a.target.inv_temp;
+        rows.kp = kLog2e * a.draft.inv_temp;
+        rows.with_draft = EXTRA && ca.resample ? ca.r.max_k > 0 : (a.L > 0 && a.num_nodes > 1);
+        rows.key = RngKey{a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
+        rows.out_residual = EXTRA && ca.resample && ca.r.out_residual ? ca.r.out_residual + (int64_t)b * a.V : nullptr;
+        work<T, NT, WARPS, EXTRA>(sm, pl, rows);
+    } else {
+        Control<T, NT, WARPS, EXTRA> control(sm, ca, pl, b);
+        if (EXTRA && ca.resample) control.resample();
+        else control.walk();
+    }
+    cluster_arrive();   // nothing is on its way to a block that has left
+    cluster_wait();
+}
+
+}  // namespace walk_cluster
+}  // namespace rsd

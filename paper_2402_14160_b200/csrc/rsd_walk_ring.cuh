@@ -372,6 +372,90 @@ __device__ __forceinline__ void group_weights(const char* rowq, const char* rowp
     }
 }
 
+// The last token's draw, by one warp: inverse CDF over the tile sums of the last pass, the smallest y whose running sum
+// exceeds u * total; if rounding leaves none, the largest y with positive weight; -1 if there is no weight at all.
+struct TilePick {
+    int tile;            // the tile that holds the crossing, or failing that the last one with weight; -1: no weight
+    bool take_last;
+    double before, target;
+};
+template <typename S>
+__device__ __forceinline__ void pick_tile(const S* tile_sum, int n_tiles, double u, TilePick& r) {
+    const int lane = threadIdx.x & 31;
+    // lanes take consecutive runs of tiles; running sums in tile order
+    const int per = (n_tiles + 31) / 32;
+    const int t_lo = lane * per, t_hi = min(n_tiles, t_lo + per);
+    double mine = 0.0;
+    for (int t = t_lo; t < t_hi; ++t) mine += (double)tile_sum[t];
+    double incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const double total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    r.tile = -1;
+    r.take_last = false;
+    r.before = 0.0;
+    r.target = u * total;
+    if (!(total > 0.0 && total < 1.7e308)) return;   // (uniform over the warp)
+    const unsigned crossing = __ballot_sync(0xFFFFFFFFu, incl > r.target);
+    const unsigned positive = __ballot_sync(0xFFFFFFFFu, mine > 0.0);
+    r.take_last = crossing == 0u;
+    const int src = r.take_last ? 31 - __clz(positive) : __ffs(crossing) - 1;
+    int tile = -1;
+    double before = 0.0;
+    if (lane == src) {
+        double cum = incl - mine;
+        for (int t = t_lo; t < t_hi; ++t) {
+            const double s = (double)tile_sum[t];
+            if (r.take_last) { if (s > 0.0) { tile = t; before = cum; } }
+            else if (cum + s > r.target) { tile = t; before = cum; break; }
+            cum += s;
+        }
+        if (tile < 0) {   // rounding: the lane's total crossed, no tile did: its last tile with weight
+            cum = incl - mine;
+            for (int t = t_lo; t < t_hi; ++t) {
+                const double s = (double)tile_sum[t];
+                if (s > 0.0) { tile = t; before = cum; }
+                cum += s;
+            }
+        }
+    }
+    r.tile = __shfl_sync(0xFFFFFFFFu, tile, src);
+    r.before = __shfl_sync(0xFFFFFFFFu, before, src);
+}
+// w: the weights of tokens 16 lane .. 16 lane + 15 of the picked tile
+__device__ __forceinline__ int pick_in_tile(const float (&w)[16], const TilePick& r) {
+    const int lane = threadIdx.x & 31;
+    double gs = 0.0;
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) gs += (double)w[jj];
+    double gincl = gs;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(0xFFFFFFFFu, gincl, o);
+        if (lane >= o) gincl += t;
+    }
+    const unsigned cross = __ballot_sync(0xFFFFFFFFu, !r.take_last && (r.before + gincl > r.target));
+    const unsigned pos = __ballot_sync(0xFFFFFFFFu, gs > 0.0);
+    const bool last_mode = cross == 0u;
+    const int src = last_mode ? (pos ? 31 - __clz(pos) : 0) : __ffs(cross) - 1;
+    int y = -1;
+    if (lane == src) {
+        int last_pos = -1;
+        double cacc = r.before + (gincl - gs);
+#pragma unroll
+        for (int jj = 0; jj < 16; ++jj) {
+            cacc += (double)w[jj];
+            if (w[jj] > 0.0f) last_pos = r.tile * kTileElems + 16 * lane + jj;
+            if (!last_mode && y < 0 && cacc > r.target) y = r.tile * kTileElems + 16 * lane + jj;
+        }
+        if (y < 0) y = last_pos;
+    }
+    return __shfl_sync(0xFFFFFFFFu, y, src);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const VerifyArgs a) {
     extern __shared__ __align__(128) unsigned char ring_mem[];
@@ -721,85 +805,19 @@ __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const Ver
     }
     __syncthreads();
     if (!aborted) {
-        // Inverse CDF over the tile sums of the last pass: the smallest y whose running sum exceeds u * total; if
-        // rounding leaves none, the largest y with positive weight; -1 if there is no weight at all.
         const uint4 rw = rng_draw(key, (uint32_t)cur, kTagResample, 0u);
         const double u = ((double)rw.x + 0.5) * (1.0 / 4294967296.0);
-        const int n_tiles = ring.n_tiles;
-        // lanes take consecutive runs of tiles; running sums in tile order
-        const int per = (n_tiles + 31) / 32;
-        const int t_lo = lane * per, t_hi = min(n_tiles, t_lo + per);
-        double mine = 0.0;
-        for (int t = t_lo; t < t_hi; ++t) mine += sm.tile_sum[t];
-        double incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        const double total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-        int y = -1;
-        if (total > 0.0 && total < 1.7e308) {   // (uniform over the warp)
-            const double target = u * total;
-            // the tile that holds the crossing, or failing that the last tile with weight
-            const unsigned crossing = __ballot_sync(0xFFFFFFFFu, incl > target);
-            const unsigned positive = __ballot_sync(0xFFFFFFFFu, mine > 0.0);
-            const bool take_last = crossing == 0u;
-            const int src = take_last ? 31 - __clz(positive) : __ffs(crossing) - 1;
-            int tile = -1;
-            double before = 0.0;
-            if (lane == src) {
-                double cum = incl - mine;
-                for (int t = t_lo; t < t_hi; ++t) {
-                    const double s = sm.tile_sum[t];
-                    if (take_last) { if (s > 0.0) { tile = t; before = cum; } }
-                    else if (cum + s > target) { tile = t; before = cum; break; }
-                    cum += s;
-                }
-                if (tile < 0) {   // rounding: the lane's total crossed, no tile did: its last tile with weight
-                    cum = incl - mine;
-                    for (int t = t_lo; t < t_hi; ++t) {
-                        const double s = sm.tile_sum[t];
-                        if (s > 0.0) { tile = t; before = cum; }
-                        cum += s;
-                    }
-                }
-            }
-            tile = __shfl_sync(0xFFFFFFFFu, tile, src);
-            before = __shfl_sync(0xFFFFFFFFu, before, src);
+        TilePick t;
+        pick_tile(sm.tile_sum, ring.n_tiles, u, t);
+        if (t.tile >= 0) {
             // the tile's weights once more, in token order: lane owns tokens 16 lane .. 16 lane + 15 of the tile
             float w[16];
-            const int g = tile * 32 + lane;
+            const int g = t.tile * 32 + lane;
 #pragma unroll
             for (int jj = 0; jj < 16; ++jj) w[jj] = 0.0f;
-            if (tile >= 0 && g * 16 < a.V) group_weights<T>(rowq, rowp, g, a.V, st, residual, w);
-            double gs = 0.0;
-#pragma unroll
-            for (int jj = 0; jj < 16; ++jj) gs += (double)w[jj];
-            double gincl = gs;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const double t = __shfl_up_sync(0xFFFFFFFFu, gincl, o);
-                if (lane >= o) gincl += t;
-            }
-            const unsigned cross2 = __ballot_sync(0xFFFFFFFFu, !take_last && (before + gincl > target));
-            const unsigned pos2 = __ballot_sync(0xFFFFFFFFu, gs > 0.0);
-            const bool last_mode = cross2 == 0u;
-            const int src2 = last_mode ? (pos2 ? 31 - __clz(pos2) : 0) : __ffs(cross2) - 1;
-            if (lane == src2) {
-                int last_pos = -1;
-                double cacc = before + (gincl - gs);
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) {
-                    cacc += (double)w[jj];
-                    if (w[jj] > 0.0f) last_pos = g * 16 + jj;
-                    if (!last_mode && y < 0 && cacc > target) y = g * 16 + jj;
-                }
-                if (y < 0) y = last_pos;
-            }
-            y = __shfl_sync(0xFFFFFFFFu, y, src2);
+            if (g * 16 < a.V) group_weights<T>(rowq, rowp, g, a.V, st, residual, w);
+            last = pick_in_tile(w, t);
         }
-        last = y;
     }
     if (lane == 0) {
         a.accepted_len[b] = len;
