@@ -721,7 +721,15 @@ struct Control {
             int child_x;
             float lq, lp;
             double Ud;
-            bool repeated, p_none;
+            bool repeated, p_none;                    // p_none: the draft row gives the token no mass (-inf or NaN)
+            float qh, ph;                             // the token's weights under the two rows
+            walk_ring::WeightRatio qp_rows;
+            auto child_weights = [&] {
+                qh = (lq == lq) ? ex2_approx(fmaf(lq, kq, -mq * kq)) : 0.0f;
+                ph = (lp == lp) ? ex2_approx(fmaf(lp, kp, -mp * kp)) : 0.0f;
+                p_none = !(lp > kNegInf);
+                qp_rows = walk_ring::WeightRatio(lq, kq, mq * kq, lp, kp, mp * kp);
+            };
             auto fetch_children = [&] {
                 child_x = -1;
                 lq = lp = 0.0f;
@@ -738,23 +746,22 @@ struct Control {
                 if (rule != 0) repeated = false;      // (the baselines never change the draft)
             };
             fetch_children();
+            mq = mp = 0.0f;
+            child_weights();
             int next_kid = children(__shfl_sync(0xFFFFFFFFu, child_node, 0), 0, par, tok, cached);
             open_sums(cur, true);
             if (aborted) break;
             inv_Sq = 1.0 / Sq;
             inv_Sp = 1.0 / Sp;
             ratio = Sq * inv_Sp;
-            const float lg_inv_ratio = lg2_approx((float)fmin(fmax(Sp * inv_Sq, 1e-37), 1e37));
+            const double sp_over_sq = Sp * inv_Sq;
             double qpd, px_row, qxd;                  // q(x) / p(x), p(x), q(x)
             auto weigh_children = [&] {
-                const float eq = fmaf(lq, kq, -mq * kq), ep = fmaf(lp, kp, -mp * kp);
-                const float qh = (lq == lq) ? ex2_approx(eq) : 0.0f, ph = (lp == lp) ? ex2_approx(ep) : 0.0f;
-                // q(x) / p(x) from the difference of the exponents survives probabilities below the fp32 range
-                p_none = !(lp == lp) || !(lp > kNegInf);
-                qpd = (double)((lq == lq && !p_none) ? ex2_approx((eq - ep) + lg_inv_ratio) : 0.0f);
+                qpd = qp_rows.times(sp_over_sq);
                 px_row = (double)ph * inv_Sp;
                 qxd = (double)qh * inv_Sq;
             };
+            if (mq != 0.0f || mp != 0.0f) child_weights();   // (the references have moved)
             weigh_children();
             // 1 - P of the closed form (see the ring walk: summed anew once subtraction loses accuracy)
             double one_mP = 1.0, one_mP_err = 0.0, inv_1mP = 1.0;
@@ -808,6 +815,7 @@ struct Control {
                         j0 += 32;
                         j = 0;
                         fetch_children();
+                        child_weights();
                         weigh_children();
                     }
                     next_kid = children(__shfl_sync(0xFFFFFFFFu, child_node, j), 0, par, tok, cached);

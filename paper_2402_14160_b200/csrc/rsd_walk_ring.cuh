@@ -123,6 +123,30 @@ struct NodeState {
     bool has_nan;       // a NaN was seen in the node's rows: the passes clean their inputs
 };
 
+// q(x) / p(x) of a token = 2^d S_p / S_q with d = (lq kq - cq) - (lp kp - cp), taken in double: an exponent rounded to fp32
+// would be off by up to 1e-6, which q/p - A scales up where it cancels.  The powers of two are kept apart from the
+// factors, so that the quotient survives weights below the fp32 range (children drafted from the far tail of a peaked row).
+struct WeightRatio {
+    float factor;
+    int exponent;
+    __device__ __forceinline__ WeightRatio() : factor(0.0f), exponent(0) {}
+    __device__ __forceinline__ WeightRatio(float lq, float kq, float cq, float lp, float kp, float cp) : factor(0.0f), exponent(0) {
+        if (lq > kNegInf && lp > kNegInf) {   // (a token without weight: 0)
+            const double d = ((double)lq * (double)kq - (double)cq) - ((double)lp * (double)kp - (double)cp);
+            const double whole = rint(d);
+            factor = exp2f((float)(d - whole));
+            exponent = __double2int_rn(whole);
+        }
+    }
+    // S_p / S_q as a factor in [1, 2) and a power of two
+    __device__ __forceinline__ double times(double sp_over_sq) const {
+        const double r = fmin(fmax(sp_over_sq, 1e-37), 1e37);
+        const int hi = __double2hiint(r), e_sums = (hi >> 20) - 1023;
+        const int e = min(max(min(max(exponent, -100000), 100000) + e_sums, -1000), 1000);
+        return (double)factor * __hiloint2double(hi - (e_sums << 20), __double2loint(r)) * __hiloint2double((e + 1023) << 20, 0);
+    }
+};
+
 template <typename T>
 struct Ring {
     RingSmem& sm;
@@ -651,11 +675,11 @@ __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const Ver
         // What the test of child j needs and no pass changes: its token, its probabilities under the node's two rows,
         // whether an earlier sibling with the same token was rejected, and its uniform.
         int j = 0, x = -1;
-        float qh_x = 0.0f, ph_x = 0.0f, qp = 0.0f;          // weights of x under the two rows; q(x) / p(x)
+        float qh_x = 0.0f, ph_x = 0.0f;                     // weights of x under the two rows
+        double qp = 0.0;                                    // q(x) / p(x)
         uint32_t U24 = 0u;                                 // the uniform, as 24 bits
         bool repeated = false, p_none = false;             // p_none: the draft row gives the token no mass (-inf or NaN)
-        // log2(S_p / S_q) for the exponent of q(x)/p(x), by the fast logarithm (absolute error 2^-22)
-        const float lg_inv_ratio = lg2_approx((float)fmin(fmax(st.Sp * inv_Sq, 1e-37), 1e37));
+        const double sp_over_sq = st.Sp * inv_Sq;
         auto prepare = [&](int child) {
             float lq, lp;
             if (j < 32) {
@@ -670,10 +694,8 @@ __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const Ver
             const float eq = fmaf(lq, st.kq, -st.mq * st.kq), ep = fmaf(lp, st.kp, -st.mp * st.kp);
             qh_x = (lq == lq) ? ex2_approx(eq) : 0.0f;
             ph_x = (lp == lp) ? ex2_approx(ep) : 0.0f;
-            // The test needs q(x) / p(x) only: taken from the difference of the exponents it survives probabilities
-            // below the fp32 range (children drafted from the far tail of a peaked row), where q(x) and p(x) are both 0.
-            p_none = !(lp == lp) || !(lp > kNegInf);
-            qp = (lq == lq && !p_none) ? ex2_approx((eq - ep) + lg_inv_ratio) : 0.0f;
+            p_none = !(lp > kNegInf);
+            qp = WeightRatio(lq, st.kq, st.mq * st.kq, lp, st.kp, st.mp * st.kp).times(sp_over_sq);
             bool mine = false;
 #pragma unroll
             for (int i = 0; i < 4; ++i) mine |= rem_x[i] == x;
@@ -711,7 +733,7 @@ __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const Ver
             bool take;
             double g;   // the threshold times Z; with no draft mass: 1 or 0 times Z
             if (!no_draft) {   // U < min(1, (q/p - A)+ (1 - P) / Z)
-                g = fmax((double)qp - st.A, 0.0) * one_mP;
+                g = fmax(qp - st.A, 0.0) * one_mP;
                 take = U * st.Z < g;
             } else {           // RSD_ST_ZERO_DRAFT_PROB
                 const double r = fmax((double)qh_x * inv_Sq - st.A * px_row, 0.0);
