@@ -155,6 +155,7 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
         rsd::walk_cluster::ClusterArgs ca;
         memset(&ca, 0, sizeof(ca));
         ca.v = a;
+        ca.off_boundaries = aligned ? 0 : 1;
         launch_cluster_walk(ca, draft->dtype, !plain, B, shape, s);
     } else if (ring) {
         if (draft->dtype == RSD_F32) launch_ring_walk<float>(a, B, s);

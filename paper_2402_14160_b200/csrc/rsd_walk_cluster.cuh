@@ -63,6 +63,7 @@ struct ClusterArgs {
     VerifyArgs v;
     ResampleArgs r;      // resample != 0: the stand-alone draw (v: rows, V and random stream only)
     int resample;
+    int off_boundaries;  // a base or stride of the rows is not a multiple of 16 bytes
 };
 
 template <int WARPS, int NT>
@@ -165,6 +166,27 @@ __device__ __forceinline__ void load_tile(Packed<T>& pk, const char* row, int ti
     }
 }
 
+// exp16() relative to 0 with the exponents' rounding put back in: v k = x + d with x = fl(v k), 2^(v k) = 2^x (1 + d ln 2).
+// Relative to 0 an exponent of ten or so is rounded by 5e-7, where one relative to the row's maximum would be exact for
+// the entries that matter.  (-inf would make d a NaN: it enters as -1e30, whose weight is 0 as well.)
+__device__ __forceinline__ void exp16_precise(const float (&v)[16], float k, float (&e)[16]) {
+    const unsigned long long k2 = f32x2(k, k), zero = f32x2(0.0f, 0.0f), minus = f32x2(-1.0f, -1.0f), ln2 = f32x2(0.69314718f, 0.69314718f);
+#pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+        const unsigned long long vv = f32x2(max_nan(v[j], -1e30f), max_nan(v[j + 1], -1e30f));
+        const unsigned long long x = fma_f32x2(vv, k2, zero), d = fma_f32x2(vv, k2, fma_f32x2(x, minus, zero));
+        float a, b;
+        split_f32x2(x, a, b);
+        const unsigned long long w = f32x2(ex2_approx(a), ex2_approx(b));
+        split_f32x2(fma_f32x2(fma_f32x2(w, ln2, zero), d, w), e[j], e[j + 1]);
+    }
+}
+__device__ __forceinline__ float weight_precise(float l, float k) {
+    if (!(l > -1e30f)) return 0.0f;
+    const float x = l * k, w = ex2_approx(x);
+    return fmaf(w * 0.69314718f, fmaf(l, k, -x), w);
+}
+
 // weights of a lane's 16 values under the mode of a drawing pass
 template <bool EXTRA>
 __device__ __forceinline__ void mode_weights(int mode, const float (&q)[16], const float (&p)[16], float a_hi, float a_lo, float c, float (&w)[16]) {
@@ -190,6 +212,7 @@ struct WorkRows {
     int64_t stride_q, stride_p;  // ... and the bytes from node to node
     float kq, kp;                // log2(e) / temperature
     bool with_draft;             // the first node probably needs its draft row as well
+    bool precise;                // exponentials by exp16_precise() while they are relative to 0
     RngKey key;                  // kTop1
     float* out_residual;         // kWrite
 };
@@ -305,6 +328,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                 kind = flags & kKindMask;
             }
             float cq = 0.0f, cp = 0.0f;
+            const bool precise = rows.precise && !(flags & kRelative);
             if (flags & (kClean | kRelative)) {
                 if (flags & kRelative) { cq = sm.ref_q; cp = sm.ref_p; }
                 if (flags & kClean) {
@@ -330,14 +354,16 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
                 rq[k].unpack(q[k]);
-                exp16(q[k], rows.kq, cq, q[k]);
+                if (precise) exp16_precise(q[k], rows.kq, q[k]);
+                else exp16(q[k], rows.kq, cq, q[k]);
                 s[k] = tree_sum16(q[k]);
             }
             if (kind == kOpen) {
 #pragma unroll
                 for (int k = 0; k < NT; ++k) {
                     rp[k].unpack(p[k]);
-                    exp16(p[k], rows.kp, cp, p[k]);
+                    if (precise) exp16_precise(p[k], rows.kp, p[k]);
+                    else exp16(p[k], rows.kp, cp, p[k]);
                     sm.lane_sum[1][warp + WARPS * k][lane] = tree_sum16(p[k]);
                 }
             }
@@ -493,7 +519,9 @@ struct Control {
     const ClusterArgs& ca;
     const VerifyArgs& a;
     const Place& pl;
-    const int b, lane;
+    const int b;
+    const bool precise;
+    const int lane;
     const RngKey key;
     int pass_no, backward;
     bool aborted;
@@ -503,8 +531,8 @@ struct Control {
     float a_hi, a_lo;               // A Sq / Sp as a two-float sum
     int status;
 
-    __device__ __forceinline__ Control(Smem<WARPS, NT>& sm_, const ClusterArgs& ca_, const Place& pl_, int b_)
-        : sm(sm_), ca(ca_), a(ca_.v), pl(pl_), b(b_), lane(threadIdx.x & 31),
+    __device__ __forceinline__ Control(Smem<WARPS, NT>& sm_, const ClusterArgs& ca_, const Place& pl_, int b_, bool precise_)
+        : sm(sm_), ca(ca_), a(ca_.v), pl(pl_), b(b_), precise(precise_), lane(threadIdx.x & 31),
           key{ca_.v.seed_lo, ca_.v.seed_hi, ca_.v.step, ca_.v.seq_base + (uint32_t)b_}, pass_no(0), backward(0), aborted(false),
           kq(kLog2e * ca_.v.target.inv_temp), kp(kLog2e * ca_.v.draft.inv_temp), mq(0.0f), mp(0.0f), A(0.0), Z(1.0), a_hi(0.0f), a_lo(0.0f),
           status(0) {}
@@ -588,6 +616,11 @@ struct Control {
         const double aa = A * ratio;
         a_hi = (float)aa;
         a_lo = (float)(aa - (double)a_hi);
+    }
+    // weight of a token with row value l as the working warps take it (NaN: 0)
+    __device__ __forceinline__ float weight(float l, float k, float m) const {
+        if (precise && m == 0.0f) return weight_precise(l, k);
+        return l == l ? ex2_approx(fmaf(l, k, -m * k)) : 0.0f;
     }
     __device__ __forceinline__ void take_in(double Z_new, double A_old, bool& kept) {
         if (Z_new > 0.0 && Z_new < 1.7e308) {
@@ -725,8 +758,8 @@ struct Control {
             float qh, ph;                             // the token's weights under the two rows
             walk_ring::WeightRatio qp_rows;
             auto child_weights = [&] {
-                qh = (lq == lq) ? ex2_approx(fmaf(lq, kq, -mq * kq)) : 0.0f;
-                ph = (lp == lp) ? ex2_approx(fmaf(lp, kp, -mp * kp)) : 0.0f;
+                qh = weight(lq, kq, mq);
+                ph = weight(lp, kp, mp);
                 p_none = !(lp > kNegInf);
                 qp_rows = walk_ring::WeightRatio(lq, kq, mq * kq, lp, kp, mp * kp);
             };
@@ -913,7 +946,7 @@ struct Control {
         ratio = Sq * inv_Sp;
         double total = Sq;
         bool tiles_valid = !with_draft;
-        const double px_row = (lp == lp) ? (double)ex2_approx(fmaf(lp, kp, -mp * kp)) * inv_Sp : 0.0;
+        const double px_row = (double)weight(lp, kp, mp) * inv_Sp;
         double one_mP = 1.0, one_mP_err = 0.0;
         int n_removed = 0, freeze = 0;
         while (left && !aborted) {
@@ -985,6 +1018,8 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
     pl.n_tiles = (a.V + kTileElems - 1) / kTileElems;
     pl.n_local = pl.n_tiles > pl.rank ? (pl.n_tiles - pl.rank + pl.C - 1) / pl.C : 0;
     const int b = blockIdx.x / pl.C;
+    // Rows off 16-byte boundaries, the baseline rules and the residual draw never take the ring walk: no bits to match.
+    const bool precise = EXTRA || ca.off_boundaries;
     if (threadIdx.x == WARPS * 32) {
         mbar_init(&sm.red_bar[0], 1);
         mbar_init(&sm.red_bar[1], 1);
@@ -1002,11 +1037,12 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         rows.kq = kLog2e * a.target.inv_temp;
         rows.kp = kLog2e * a.draft.inv_temp;
         rows.with_draft = EXTRA && ca.resample ? ca.r.max_k > 0 : (a.L > 0 && a.num_nodes > 1);
+        rows.precise = precise;
         rows.key = RngKey{a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
         rows.out_residual = EXTRA && ca.resample && ca.r.out_residual ? ca.r.out_residual + (int64_t)b * a.V : nullptr;
         work<T, NT, WARPS, EXTRA>(sm, pl, rows);
     } else {
-        Control<T, NT, WARPS, EXTRA> control(sm, ca, pl, b);
+        Control<T, NT, WARPS, EXTRA> control(sm, ca, pl, b, precise);
         if (EXTRA && ca.resample) control.resample();
         else control.walk();
     }
