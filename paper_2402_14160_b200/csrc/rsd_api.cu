@@ -19,49 +19,34 @@ namespace {
 
 thread_local cudaEvent_t g_scan_before = nullptr, g_scan_after = nullptr;  // one-shot, see rsd_profile_next_scan
 
-template <typename T, bool ALIGNED, bool WIDE, bool NEED_LSE, bool TEMP>
-void launch_scan_temp(int blocks, const rsd::ScanArgs& a, cudaStream_t s) {
-    const size_t smem = sizeof(float) * (size_t)((((a.V + 15) / 16) + 3) / 4 * 4);  // one bound per group of 16 elements, padded to fours
-    if (smem > 48 * 1024) {
-        // The attribute belongs to the (function, device) pair; it is only needed beyond 48 KB (V > 196,608), so it
-        // is simply set on every such launch instead of being remembered per device.
-        if (cudaFuncSetAttribute(rsd::scan_topk_kernel<T, ALIGNED, WIDE, NEED_LSE, TEMP>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(sizeof(float) * (RSD_MAX_VOCAB / 16))) != cudaSuccess)
-            return;   // the error stays pending: the caller's check_launch() reports it
-    }
-    rsd::scan_topk_kernel<T, ALIGNED, WIDE, NEED_LSE, TEMP><<<blocks, rsd::kScanThreads, smem, s>>>(a);
-}
-
-template <typename T, bool ALIGNED, bool WIDE, bool NEED_LSE>
-void launch_scan_one(int blocks, const rsd::ScanArgs& a, cudaStream_t s) {
-    if (a.temp != 1.0f) launch_scan_temp<T, ALIGNED, WIDE, NEED_LSE, true>(blocks, a, s);
-    else launch_scan_temp<T, ALIGNED, WIDE, NEED_LSE, false>(blocks, a, s);
-}
-
-template <bool NEED_LSE>
-void launch_scan_lse(const rsd_rows* rows, int align, int blocks, const rsd::ScanArgs& a, cudaStream_t s) {
-    if (rows->dtype == RSD_F32) {
-        if (align == 32) launch_scan_one<float, true, true, NEED_LSE>(blocks, a, s);
-        else if (align == 16) launch_scan_one<float, true, false, NEED_LSE>(blocks, a, s);
-        else launch_scan_one<float, false, false, NEED_LSE>(blocks, a, s);
-    } else {
-        if (align == 32) launch_scan_one<__nv_bfloat16, true, true, NEED_LSE>(blocks, a, s);
-        else if (align == 16) launch_scan_one<__nv_bfloat16, true, false, NEED_LSE>(blocks, a, s);
-        else launch_scan_one<__nv_bfloat16, false, false, NEED_LSE>(blocks, a, s);
-    }
+// Threads per row.  A block is a row; 128 threads give the most rows in flight and the least work per row (the stages after
+// the streaming loop cost a row the same whatever its threads), but a row then takes 16 us at 32,000 entries, and with few
+// rows most of the chip waits for it.  Measured (us, 32,000 bf16 with log-sum-exp; 128 / 256 / 512 threads): 4 rows 10.0 /
+// 9.0 / 8.0, 192 rows 16.0 / 12.1 / 12.0, 320 rows 16.4 / 14.1 / 18.4, 640 rows 20.2 / 22.3 / 26.4.  Rows of more than
+// 49,152 entries carry over 12 KB of bounds, so that blocks of 128 threads no longer fill an SM: 128,000 bf16, 5000 rows
+// 370 / 247 / 286, 4-byte rows 3000 rows 321 / 284 / 268.
+int scan_threads(int rows, int V, bool f32) {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        return (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 148;
+    }();
+    if (V >= 16384 && rows <= sms + sms / 2) return 512;
+    if (V > 65536) return f32 ? 512 : 256;
+    if (V >= 16384 && rows <= 5 * sms / 2) return 256;
+    if (V >= 4096 && rows <= sms + sms / 2) return 256;
+    return 128;
 }
 
 void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs& a, cudaStream_t s) {
-    // vector paths: rows made of whole groups that start on 32- or 16-byte boundaries
-    const int aligned = a.V % 16 != 0 ? 0 : rows_aligned(rows, 32) ? 32 : rows_aligned(rows, 16) ? 16 : 0;
+    const bool aligned = a.V % 16 == 0 && rows_aligned(rows, 32);   // rows made of whole groups that start on 32-byte boundaries
     for (int r = 0; r < 10; ++r) {
         a.rk0[r] = a.seed_lo + (uint32_t)r * 0x9E3779B9u;
         a.rk1[r] = a.seed_hi + (uint32_t)r * 0xBB67AE85u;
     }
     if (g_scan_before) cudaEventRecord(g_scan_before, s);
-    if (need_lse) launch_scan_lse<true>(rows, aligned, blocks, a, s);
-    else launch_scan_lse<false>(rows, aligned, blocks, a, s);
+    const int threads = scan_threads(blocks, a.V, rows->dtype == RSD_F32);
+    if (rows->dtype == RSD_F32) rsd::launch_scan_f32(threads, aligned, need_lse, blocks, a, s);
+    else rsd::launch_scan_bf16(threads, aligned, need_lse, blocks, a, s);
     if (g_scan_after) cudaEventRecord(g_scan_after, s);
     g_scan_before = g_scan_after = nullptr;
 }

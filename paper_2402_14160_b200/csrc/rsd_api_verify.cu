@@ -5,7 +5,7 @@
 
 #include "rsd_api_common.h"
 #include "rsd_verify.cuh"
-#include "rsd_walk_cluster.cuh"
+#include "rsd_walk_cluster_args.h"
 #include "rsd_walk_ring.cuh"
 
 using namespace rsd_host;
@@ -39,16 +39,11 @@ void launch_ring_walk(const rsd::VerifyArgs& a, int B, cudaStream_t s) {
     verify_tree_ring_kernel<T><<<B, kThreads, kRingBytes, s>>>(a);
 }
 
-// Shape of a cluster walk (rsd_walk_cluster.cuh): C blocks of W working warps with NT tiles of 512 entries each.
-struct ClusterShape {
-    int C, W, NT;
-    float waves;   // sequences asked for over sequences resident at a time
-};
 // The smallest cluster that holds a row, with one tile per warp (three blocks an SM) as long as all sequences are
 // resident at once, else with two (two blocks an SM), which costs a sequence about 10 % more time and 25 % fewer SM-cycles
 // (V = 32,000, bf16: 42 against 47 us at 64 sequences, 122 against 102 us at 256).  Rows beyond 65,536 entries take
 // sixteen warps, one block an SM; beyond 131,072 no cluster holds them (C = 0).
-ClusterShape cluster_shape(int B, int V) {
+rsd::walk_cluster::Shape cluster_shape(int B, int V) {
     auto blocks = [&](int per_block) {
         int c = 1;
         while (c * per_block < V) c *= 2;
@@ -64,35 +59,9 @@ ClusterShape cluster_shape(int B, int V) {
     return {0, 0, 0, 0.0f};
 }
 
-template <typename T, int NT, int WARPS, bool EXTRA>
-void launch_cluster(const rsd::walk_cluster::ClusterArgs& a, int B, int C, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(B * C));
-    cfg.blockDim = dim3((WARPS + 1) * 32);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, rsd::walk_cluster::walk_cluster_kernel<T, NT, WARPS, EXTRA>, a);   // (an error stays pending for check_launch())
-}
-template <typename T, bool EXTRA>
-void launch_cluster_shape(const rsd::walk_cluster::ClusterArgs& a, int B, const ClusterShape& c, cudaStream_t s) {
-    if (c.W == 16) launch_cluster<T, 2, 16, EXTRA>(a, B, c.C, s);
-    else if (c.NT == 2) launch_cluster<T, 2, 8, EXTRA>(a, B, c.C, s);
-    else launch_cluster<T, 1, 8, EXTRA>(a, B, c.C, s);
-}
-void launch_cluster_walk(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const ClusterShape& c, cudaStream_t s) {
-    if (dtype == RSD_F32) {
-        if (extra) launch_cluster_shape<float, true>(a, B, c, s);
-        else launch_cluster_shape<float, false>(a, B, c, s);
-    } else {
-        if (extra) launch_cluster_shape<__nv_bfloat16, true>(a, B, c, s);
-        else launch_cluster_shape<__nv_bfloat16, false>(a, B, c, s);
-    }
+void launch_cluster_walk(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const rsd::walk_cluster::Shape& c, cudaStream_t s) {
+    if (dtype == RSD_F32) rsd::walk_cluster::launch_f32(a, extra, B, c, s);
+    else rsd::walk_cluster::launch_bf16(a, extra, B, c, s);
 }
 }  // namespace
 
@@ -149,7 +118,7 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
     // 256 sequences: 73 / 79 against 49 / 84), from about 8 where the last token is drawn by Gumbel-Top-1 (256 / 1024
     // sequences: 147 / 348 against 128 / 392).  For plain walks over other rows the cluster is ahead at every size (32,001
     // entries, 64 / 512 / 1000 sequences: 110 / 296 / 444 against 32 / 180 / 329).
-    const ClusterShape shape = cluster_shape(B, V);
+    const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
     const float most = ring ? 2.0f : plain ? 1e30f : final_sampler == RSD_FINAL_GUMBEL_TOP1 ? 8.0f : 3.0f;
     if (shape.C > 0 && shape.waves <= most) {
         rsd::walk_cluster::ClusterArgs ca;
@@ -196,7 +165,7 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     a.out_token = out_token; a.out_residual = out_residual; a.status = status;
     cudaStream_t s = (cudaStream_t)stream;
     // rows that fit a cluster take it at every batch size (V = 32,000, three rejected tokens: 137 -> 75 us for 256 sequences)
-    const ClusterShape shape = cluster_shape(B, V);
+    const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
     if (shape.C > 0) {
         rsd::walk_cluster::ClusterArgs ca;
         memset(&ca, 0, sizeof(ca));

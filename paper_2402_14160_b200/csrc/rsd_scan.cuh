@@ -16,8 +16,6 @@
 
 namespace rsd {
 
-constexpr int kScanThreads = 128;
-constexpr int kScanWarps = kScanThreads / 32;
 constexpr int kMaxRows = 256;
 constexpr int kIdxNone = 0x7FFFFFFF;
 // Queue sizes of the per-row stages.  Overflow of any of them is handled (general path, raised bound), so a build
@@ -54,6 +52,10 @@ struct ScanArgs {
     int32_t node_row[kMaxRows];
     int32_t child_base[kMaxRows];
 };
+
+// One block of `threads` threads per row, `blocks` rows (defined in rsd_scan_f32.cu and rsd_scan_bf16.cu).
+void launch_scan_f32(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, cudaStream_t s);
+void launch_scan_bf16(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, cudaStream_t s);
 
 // Packed pairs of fp32 (sm_100 executes fma/add on two floats per instruction).
 __device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
@@ -146,6 +148,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return r;
 }
 
+// the 16 bytes that start m bytes into the two neighbouring words a, b (m < 16)
+__device__ __forceinline__ uint4 window16(const uint4& a, const uint4& b, uint32_t m) {
+    uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z, w7 = b.w;
+    if (m & 8u) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = w7; }
+    if (m & 4u) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
+    const uint32_t s = (m & 3u) * 8u;
+    return make_uint4(__funnelshift_r(w0, w1, s), __funnelshift_r(w1, w2, s), __funnelshift_r(w2, w3, s), __funnelshift_r(w3, w4, s));
+}
+
 // The 16 elements of a group as loaded (fp32: four 16-byte words, bf16: two), kept packed while they wait.
 template <typename T>
 struct Packed;
@@ -194,6 +205,17 @@ struct Packed<float> {
     __device__ __forceinline__ void load(const void* row, int g, int V, bool aligned_full, bool wide = false) {
         if (aligned_full) {
             load_aligned((const float*)row + (size_t)g * 16, wide);
+        } else if (g > 0 && (g + 1) * 16 + 4 <= V) {   // the five aligned words around the group, shifted
+            const char* at = (const char*)row + (int64_t)g * 64;
+            const uint32_t m = (uint32_t)(uintptr_t)at & 15u;
+            const uint4* p = (const uint4*)(at - m);
+            uint4 prev = __ldg(p);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint4 next = __ldg(p + i + 1);
+                w[i] = window16(prev, next, m);
+                prev = next;
+            }
         } else {
             uint32_t u[16];
 #pragma unroll
@@ -254,6 +276,13 @@ struct Packed<__nv_bfloat16> {
     __device__ __forceinline__ void load(const void* row, int g, int V, bool aligned_full, bool wide = false) {
         if (aligned_full) {
             load_aligned((const uint16_t*)row + (size_t)g * 16, wide);
+        } else if (g > 0 && (g + 1) * 16 + 8 <= V) {   // the three aligned words around the group, shifted
+            const char* at = (const char*)row + (int64_t)g * 32;
+            const uint32_t m = (uint32_t)(uintptr_t)at & 15u;
+            const uint4* p = (const uint4*)(at - m);
+            const uint4 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+            w[0] = window16(a, b, m);
+            w[1] = window16(b, c, m);
         } else {
             uint32_t u[8];
 #pragma unroll
@@ -387,17 +416,27 @@ __device__ __forceinline__ float slot_element<__nv_bfloat16>(uint32_t addr, uint
     return __uint_as_float(r << 16);
 }
 
+// Shared memory of a block of NT threads: the bounds of the row's groups, then one buffer with two uses: the threads'
+// group slots during the streaming loop, the queues of the stages after it.
+template <typename T, int NT>
+__host__ __device__ constexpr size_t scan_buffer_bytes() {
+    const size_t queues = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap), slots = (size_t)NT * GroupSlot<T>::kStride;
+    return queues > slots ? queues : slots;
+}
+__host__ __device__ inline size_t scan_bounds_bytes(int V) { return 4 * (size_t)((((V + 15) / 16) + 3) / 4 * 4); }   // padded to fours
+
 // One block per row.
-// ALIGNED: rows start on 16-byte boundaries and V is a multiple of 16 (vector loads); WIDE: 32-byte boundaries as well.
+// ALIGNED: rows start on 32-byte boundaries and V is a multiple of 16 (256-bit loads); other rows are read in aligned
+// 16-byte words, shifted.
 // TEMP: a sampling temperature other than 1 applies (otherwise the scale factors are compile-time constants).
-// Nine blocks per SM for 2-byte rows (56 registers: a group in flight is 8 registers), eight for 4-byte rows.
-template <typename T, bool ALIGNED, bool WIDE, bool NEED_LSE, bool TEMP>
-__global__ void __launch_bounds__(kScanThreads, sizeof(T) == 2 ? 9 : 8) scan_topk_kernel(const ScanArgs a) {
-    extern __shared__ float ub[];                    // [n_groups] upper bound of each group's perturbed values
-    // One buffer, two uses: the threads' group slots during the streaming loop, the queues of the stages after it.
-    constexpr int kQueueBytes = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap);
-    constexpr int kSlotBytes = kScanThreads * GroupSlot<T>::kStride;
-    __shared__ __align__(16) unsigned char shared_buf[kQueueBytes > kSlotBytes ? kQueueBytes : kSlotBytes];
+// Blocks of 128 threads: nine per SM for 2-byte rows (56 registers: a group in flight is 8 registers), eight for 4-byte rows.
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT>
+__global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) scan_topk_kernel(const __grid_constant__ ScanArgs a) {
+    constexpr int kScanThreads = NT, kScanWarps = NT / 32;
+    constexpr bool WIDE = ALIGNED;
+    extern __shared__ __align__(16) unsigned char scan_smem[];
+    float* const ub = (float*)scan_smem;             // [n_groups] upper bound of each group's perturbed values
+    unsigned char* const shared_buf = scan_smem + scan_bounds_bytes(a.V);
     int* const cand = (int*)shared_buf;                              // groups whose bound reaches tau
     uint32_t* const tk_x = (uint32_t*)(cand + kCandCap);             // element index | (it carries the group's largest noise) << 31
     float* const tk_base = (float*)(tk_x + kTaskCap);                // lower bound of t(U_M) / 16 of the element's group

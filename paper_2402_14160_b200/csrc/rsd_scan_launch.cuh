@@ -1,0 +1,51 @@
+// Launch of the row scan for one element type; each type is a translation unit of its own (rsd_scan_f32.cu,
+// rsd_scan_bf16.cu), which keeps the compiles short.
+#pragma once
+#include <atomic>
+
+#include "../../include/rsd.h"
+#include "rsd_scan.cuh"
+
+namespace rsd {
+
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT>
+void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
+    const auto kernel = scan_topk_kernel<T, ALIGNED, NEED_LSE, TEMP, NT>;
+    const size_t smem = scan_bounds_bytes(a.V) + scan_buffer_bytes<T, NT>();
+    if (smem > 40 * 1024) {
+        // The attribute belongs to the (function, device) pair: raised once per device to what the longest row needs.
+        static std::atomic<bool> raised[64];
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return;   // the error stays pending: the caller's check_launch() reports it
+        if (dev < 0 || dev >= 64 || !raised[dev].load(std::memory_order_acquire)) {
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + scan_buffer_bytes<T, NT>())) != cudaSuccess)
+                return;
+            if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
+        }
+    }
+    kernel<<<blocks, NT, smem, s>>>(a);
+}
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP>
+void launch_scan_temp(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {
+    if (threads == 512) launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 512>(blocks, a, s);
+    else if (threads == 256) launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 256>(blocks, a, s);
+    else launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 128>(blocks, a, s);
+}
+template <typename T, bool ALIGNED, bool NEED_LSE>
+void launch_scan_lse(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {
+    if (a.temp != 1.0f) launch_scan_temp<T, ALIGNED, NEED_LSE, true>(threads, blocks, a, s);
+    else launch_scan_temp<T, ALIGNED, NEED_LSE, false>(threads, blocks, a, s);
+}
+template <typename T>
+void launch_scan_of(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, cudaStream_t s) {
+    if (need_lse) {
+        if (aligned) launch_scan_lse<T, true, true>(threads, blocks, a, s);
+        else launch_scan_lse<T, false, true>(threads, blocks, a, s);
+    } else {
+        if (aligned) launch_scan_lse<T, true, false>(threads, blocks, a, s);
+        else launch_scan_lse<T, false, false>(threads, blocks, a, s);
+    }
+}
+
+}  // namespace rsd

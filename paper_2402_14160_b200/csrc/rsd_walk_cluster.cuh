@@ -17,7 +17,7 @@
 // bits, so which of them runs (a matter of batch size and vocabulary) does not show in any result.
 // Every wait on an mbarrier is bounded (about a second); a wait that runs out abandons the walk with RSD_ST_TIMEOUT.
 #pragma once
-#include "rsd_verify.cuh"
+#include "rsd_walk_cluster_args.h"
 #include "rsd_walk_ring.cuh"
 
 namespace rsd {
@@ -57,13 +57,6 @@ struct __align__(16) Cmd {
     int flags;
     int node;            // kOpen, kOpenTarget: the node; kDump: the tile; kTop1: the node of the random stream
     float a_hi, a_lo;
-};
-
-struct ClusterArgs {
-    VerifyArgs v;
-    ResampleArgs r;      // resample != 0: the stand-alone draw (v: rows, V and random stream only)
-    int resample;
-    int off_boundaries;  // a base or stride of the rows is not a multiple of 16 bytes
 };
 
 template <int WARPS, int NT>

@@ -1,0 +1,36 @@
+// Launch of the cluster walk for one element type.
+#pragma once
+#include "rsd_walk_cluster.cuh"
+
+namespace rsd {
+namespace walk_cluster {
+
+template <typename T, int NT, int WARPS, bool EXTRA>
+void launch_shape(const ClusterArgs& a, int B, int C, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * C));
+    cfg.blockDim = dim3((WARPS + 1) * 32);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, walk_cluster_kernel<T, NT, WARPS, EXTRA>, a);   // (an error stays pending for check_launch())
+}
+template <typename T, bool EXTRA>
+void launch_extra(const ClusterArgs& a, int B, const Shape& c, cudaStream_t s) {
+    if (c.W == 16) launch_shape<T, 2, 16, EXTRA>(a, B, c.C, s);
+    else if (c.NT == 2) launch_shape<T, 2, 8, EXTRA>(a, B, c.C, s);
+    else launch_shape<T, 1, 8, EXTRA>(a, B, c.C, s);
+}
+template <typename T>
+void launch_of(const ClusterArgs& a, bool extra, int B, const Shape& c, cudaStream_t s) {
+    if (extra) launch_extra<T, true>(a, B, c, s);
+    else launch_extra<T, false>(a, B, c, s);
+}
+
+}  // namespace walk_cluster
+}  // namespace rsd
