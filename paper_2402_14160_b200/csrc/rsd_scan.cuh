@@ -423,20 +423,29 @@ __host__ __device__ constexpr size_t scan_buffer_bytes() {
     const size_t queues = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap), slots = (size_t)NT * GroupSlot<T>::kStride;
     return queues > slots ? queues : slots;
 }
+// blocks of more than 128 threads: a sum and a reference per lane and chunk
+template <int NT>
+__host__ __device__ constexpr size_t scan_partial_bytes(int V) { return NT == 128 ? 0 : (size_t)((V + 2047) / 2048) * 32 * 8; }
 __host__ __device__ inline size_t scan_bounds_bytes(int V) { return 4 * (size_t)((((V + 15) / 16) + 3) / 4 * 4); }   // padded to fours
 
 // One block per row.
 // ALIGNED: rows start on 32-byte boundaries and V is a multiple of 16 (256-bit loads); other rows are read in aligned
 // 16-byte words, shifted.
 // TEMP: a sampling temperature other than 1 applies (otherwise the scale factors are compile-time constants).
-// Blocks of 128 threads: nine per SM for 2-byte rows (56 registers: a group in flight is 8 registers), eight for 4-byte rows.
+// Blocks of 128 threads: nine per SM for 2-byte rows (56 registers: a group in flight is 8 registers), eight for 4-byte rows;
+// fewer for shifted rows, which need registers for the words around a group.
+template <typename T, bool ALIGNED, int NT>
+constexpr int scan_blocks_per_sm() {
+    return ALIGNED ? (NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) : (NT == 128 ? (sizeof(T) == 2 ? 8 : 6) : NT == 256 ? 3 : 2);
+}
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT>
-__global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) scan_topk_kernel(const __grid_constant__ ScanArgs a) {
+__global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan_topk_kernel(const __grid_constant__ ScanArgs a) {
     constexpr int kScanThreads = NT, kScanWarps = NT / 32;
     constexpr bool WIDE = ALIGNED;
     extern __shared__ __align__(16) unsigned char scan_smem[];
     float* const ub = (float*)scan_smem;             // [n_groups] upper bound of each group's perturbed values
     unsigned char* const shared_buf = scan_smem + scan_bounds_bytes(a.V);
+    float2* const partial = (float2*)(shared_buf + scan_buffer_bytes<T, NT>());   // [chunk][lane] (NT > 128)
     int* const cand = (int*)shared_buf;                              // groups whose bound reaches tau
     uint32_t* const tk_x = (uint32_t*)(cand + kCandCap);             // element index | (it carries the group's largest noise) << 31
     float* const tk_base = (float*)(tk_x + kTaskCap);                // lower bound of t(U_M) / 16 of the element's group
@@ -450,7 +459,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
     __shared__ int sv_idx[kSurvCap];
     __shared__ uint32_t bin_max[32];                 // per lane index: largest sample over the warps (ordered encoding)
     __shared__ float red_f[kScanWarps];
-    __shared__ float red_s[kScanWarps];
+    __shared__ float red_s[4];
     __shared__ int n_cand, n_surv, nan_flag;
     __shared__ float lse_sh;
 
@@ -473,13 +482,42 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
     // A warp takes chunks of 128 consecutive groups; lane l meets groups l, l + 32, l + 64, l + 96 of the chunk, whose
     // coarse-stream words are the four words of one Philox call.
     float best = kNegInf;                  // largest exact sample of this thread (value(a) + lower bound of G_max)
-    // Running log-sum-exp of this thread's elements: sum of 2^(value * log2(e) - c) with an integer c, fixed at the
-    // first finite group maximum and moved up only when a group maximum exceeds it by more than 40.
+    // Log-sum-exp: per lane and chunk the sum of 2^(value * log2(e) - c) with an integer c, moved up only when a group
+    // maximum exceeds it by more than 40; the chunks w, w + 4, w + 8, ... of a lane are then added up in that order.  c
+    // starts from the first group of chunk w of the lane (w = chunk mod 4), so every sum is the same whatever the number
+    // of threads, and so are all results.
     const float inv_temp = TEMP ? a.inv_temp : 1.0f, temp = TEMP ? a.temp : 1.0f;   // values enter as value * inv_temp
     const float log2e_t = kLog2e * inv_temp;
+    float lse_thr0 = kNegInf, lse_negc0 = 0.0f;   // every chunk starts with these
     float lse_thr = kNegInf;               // group maxima above this move the reference (-inf: nothing finite yet)
     float lse_negc = 0.0f;                 // -c
     unsigned long long acc0 = f32x2(0.0f, 0.0f), acc1 = acc0;
+    float fold_c = kNegInf, fold_s = 0.0f; // the chunks added up so far (fold_c: reference, -inf: nothing)
+    auto fold = [&](float c, float sum) {
+        if (c == fold_c) {
+            fold_s += sum;
+        } else if (c > kNegInf) {
+            const float m = fmaxf(c, fold_c);
+            fold_s = (fold_c > kNegInf ? fold_s * exp2f(fold_c - m) : 0.0f) + sum * exp2f(c - m);
+            fold_c = m;
+        }
+    };
+    auto begin_chunk = [&] {
+        if (NEED_LSE) {
+            lse_thr = lse_thr0;
+            lse_negc = lse_negc0;
+            acc0 = acc1 = f32x2(0.0f, 0.0f);
+        }
+    };
+    auto end_chunk = [&](int chunk) {
+        if (NEED_LSE) {
+            float s0, s1;
+            split_f32x2(add_f32x2(acc0, acc1), s0, s1);
+            const float c = lse_thr > kNegInf ? -lse_negc : kNegInf, sum = s0 + s1;
+            if (NT == 128) fold(c, sum);
+            else partial[chunk * 32 + lane] = make_float2(sum, c);
+        }
+    };
     const uint32_t slot = (uint32_t)__cvta_generic_to_shared(shared_buf) + (uint32_t)tid * GroupSlot<T>::kStride;
     // work on one group whose 16 values are in `cur`; `word` is the group's coarse-stream word, `ub_g` = &ub[group]
     auto body = [&](Packed<T>& cur, float* ub_g, uint32_t word) {   // may rewrite cur
@@ -532,9 +570,23 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
         int c = warp;
         fetch(q0, c * 128 + lane);
         fetch(q1, c * 128 + 32 + lane);
+        if (NEED_LSE) {
+            Packed<T> qf = q0;
+            const int g_first = (NT == 128 ? c : warp & 3) * 128 + lane;
+            if (NT > 128 && warp >= 4) fetch(qf, g_first);
+            if (g_first < n_groups) {
+                float m = group_max_nan(qf);
+                if (m != m) { qf.clean_nan(); m = group_max_nan(qf); }
+                if (m > kNegInf) {
+                    lse_negc0 = -ceilf(m * log2e_t);
+                    lse_thr0 = fmaf(40.0f, temp, m);   // 40 in scaled units
+                }
+            }
+        }
         for (; c < n_full; c += kScanWarps) {
             const int g0 = c * 128 + lane;
             float* ub_g = ub + g0;
+            begin_chunk();
             const uint4 cw = philox_row(a, pr, (uint32_t)(c * 32 + lane));
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {   // two turns of two groups: keeps the loop's code small
@@ -544,10 +596,12 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
                 body(q1, ub_g + 64 * h + 32, h ? cw.w : cw.y);
                 fetch(q1, g_next + 32);
             }
+            end_chunk(c);
         }
         if (c == n_full && (n_groups & 127)) {   // this warp owns the partial chunk; q0 and q1 are on their way
             const int g0 = c * 128 + lane;
             float* ub_g = ub + g0;
+            begin_chunk();
             const uint4 cw = philox_row(a, pr, (uint32_t)(c * 32 + lane));
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
@@ -557,6 +611,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
                 if (g + 32 < n_groups) body(q1, ub_g + 64 * h + 32, h ? cw.w : cw.y);
                 if (h == 0) fetch(q1, g0 + 96);
             }
+            end_chunk(c);
         }
     }
 
@@ -565,37 +620,43 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
     // warps); the k-th largest bin maximum is at most the k-th largest sample, hence at most the k-th largest
     // perturbed value of the row.  Every warp finds it from the 32 bin maxima itself, so one barrier is enough.
     if (best > kNegInf) atomicMax(&bin_max[lane], float_to_ordered(best));
-    if (NEED_LSE) {
-        // the warp's share of the log-sum-exp: largest reference exponent C_w and sum of s_t * 2^(c_t - C_w) (exact
-        // scaling); the last thread combines the warps' shares after the barrier.  All in fp32: the threads' sums
-        // already are, and double-precision instructions are slow enough to show on every row's critical path.
-        const float lse_c = lse_thr > kNegInf ? -lse_negc : kNegInf;  // this thread's reference exponent
-        const float cw_max = warp_max(lse_c);
-        float s0, s1, s2, s3;
-        split_f32x2(acc0, s0, s1);
-        split_f32x2(acc1, s2, s3);
-        const float d = lse_c - cw_max;   // <= 0, an integer (NaN or -inf when there is nothing to add)
+    // the warp's share of the log-sum-exp: largest reference exponent C_w and sum of s_t * 2^(c_t - C_w) (exact scaling);
+    // the last thread combines the four shares after a barrier.  All in fp32: the threads' sums already are, and
+    // double-precision instructions are slow enough to show on every row's critical path.
+    auto share_of_warp = [&] {
+        const float cw_max = warp_max(fold_c);
+        const float d = fold_c - cw_max;   // <= 0, an integer (NaN or -inf when there is nothing to add)
         float term = 0.0f;
-        if (lse_c > kNegInf && d > -120.0f) term = ((s0 + s1) + (s2 + s3)) * exp2f(d);
+        if (fold_c > kNegInf && d > -120.0f) term = fold_s * exp2f(d);
         if (cw_max == -kNegInf) term = cw_max - cw_max;  // a +inf value: the sum is not a number
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) term += __shfl_xor_sync(0xFFFFFFFFu, term, o);
         if (lane == 0) { red_f[warp] = cw_max; red_s[warp] = term; }
-    }
+    };
+    if (NEED_LSE && NT == 128) share_of_warp();
     __syncthreads();   // also: every thread is done with its group slot, the queues may take the buffer over
-    if (NEED_LSE && tid == kScanThreads - 1) {
+    auto combine_shares = [&] {
         float C = red_f[0];
 #pragma unroll
-        for (int w = 1; w < kScanWarps; ++w) C = fmaxf(C, red_f[w]);
+        for (int w = 1; w < 4; ++w) C = fmaxf(C, red_f[w]);
         float S = 0.0f;
 #pragma unroll
-        for (int w = 0; w < kScanWarps; ++w) {
+        for (int w = 0; w < 4; ++w) {
             const float d = red_f[w] - C;
             if (red_f[w] > kNegInf && d > -120.0f) S += red_s[w] * exp2f(d);
             else if (d != d) S = d;
         }
         // C ln 2 + ln S with ln 2 split so that C * hi is exact (C is a small integer)
         lse_sh = (C > kNegInf && (S > 0.0f || S != S)) ? fmaf(C, 0.693145751953125f, fmaf(C, 1.4286068203094172e-06f, logf(S))) : kNegInf;
+    };
+    if (NEED_LSE && NT == 128 && tid == kScanThreads - 1) combine_shares();
+    if (NEED_LSE && NT > 128 && warp < 4) {
+        const int n_chunks = (n_groups + 127) >> 7;
+        for (int c = warp; c < n_chunks; c += 4) {
+            const float2 f = partial[c * 32 + lane];
+            fold(f.y, f.x);
+        }
+        share_of_warp();
     }
     float tau;
     {
@@ -649,6 +710,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 102
         }
     }
     __syncthreads();
+    if (NEED_LSE && NT > 128 && tid == kScanThreads - 1) combine_shares();
     const int n_queued = n_cand;
 
     // exact perturbed values of the elements of group g that can reach tau

@@ -11,7 +11,7 @@ namespace rsd {
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT>
 void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
     const auto kernel = scan_topk_kernel<T, ALIGNED, NEED_LSE, TEMP, NT>;
-    const size_t smem = scan_bounds_bytes(a.V) + scan_buffer_bytes<T, NT>();
+    const size_t smem = scan_bounds_bytes(a.V) + scan_buffer_bytes<T, NT>() + scan_partial_bytes<NT>(a.V);
     if (smem > 40 * 1024) {
         // The attribute belongs to the (function, device) pair: raised once per device to what the longest row needs.
         static std::atomic<bool> raised[64];
@@ -19,7 +19,7 @@ void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
         if (cudaGetDevice(&dev) != cudaSuccess) return;   // the error stays pending: the caller's check_launch() reports it
         if (dev < 0 || dev >= 64 || !raised[dev].load(std::memory_order_acquire)) {
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + scan_buffer_bytes<T, NT>())) != cudaSuccess)
+                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + scan_buffer_bytes<T, NT>() + scan_partial_bytes<NT>(RSD_MAX_VOCAB))) != cudaSuccess)
                 return;
             if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
         }

@@ -783,7 +783,10 @@ struct Control {
             const double sp_over_sq = Sp * inv_Sq;
             double qpd, px_row, qxd;                  // q(x) / p(x), p(x), q(x)
             auto weigh_children = [&] {
-                qpd = qp_rows.times(sp_over_sq);
+                // Precise weights: the quotient of the very weights that the sums are made of, as long as they are in range, so
+                // that their errors cancel where the token carries much of the residual.
+                if (precise && qh > 1e-30f && ph > 1e-30f) qpd = (double)qh / (double)ph * sp_over_sq;
+                else qpd = qp_rows.times(sp_over_sq);
                 px_row = (double)ph * inv_Sp;
                 qxd = (double)qh * inv_Sq;
             };

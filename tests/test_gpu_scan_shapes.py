@@ -1,0 +1,45 @@
+"""The row scan uses 128, 256 or 512 threads per row, by the number of rows and their length, and reads rows off 32-byte
+boundaries in shifted words.  None of this may show: a few rows scanned alone give the bits they give inside a large
+batch (picks, perturbed values and log-probabilities), at the sizes where the number of threads changes."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads
+from tests.parity import Tally, compare_topk
+
+pytestmark = pytest.mark.gpu
+
+
+def _draft(rows, k, seq_base, is_logprob=False, temperature=1.0):
+    import paper_2402_14160_b200 as rsd
+    out = rsd.rsd_gumbel_topk_draft(rows, [k], [2], 17, 3, seq_base=seq_base, want_values=True, is_logprob=is_logprob, temperature=temperature)
+    return {key: v.cpu().numpy() for key, v in out.items()}
+
+
+@pytest.mark.parametrize("dtype,V,B,off,trouble", [
+    ("bf16", 4096, 700, 0, ""), ("f32", 4080, 300, 0, "jump"), ("bf16", 16384, 500, 0, "jump"), ("f32", 32000, 400, 0, "nan"), ("bf16", 32016, 400, 8, ""),
+    ("bf16", 32001, 400, 0, "nan"), ("f32", 16389, 400, 3, "jump"), ("bf16", 65552, 300, 0, ""), ("f32", 131072, 240, 0, ""),
+    ("bf16", 65537, 300, 1, "")])
+def test_rows_alone_and_in_a_batch_give_the_same_bits(dtype, V, B, off, trouble):
+    gen = torch.Generator(device="cuda").manual_seed(V + B)
+    rows = torch.randn((B, 1, V + off), generator=gen, device="cuda") * 2
+    if trouble == "jump":        # maxima that jump by more than the log-sum-exp's reference allows, and chunks of -inf
+        rows[::2, :, V // 2::97] += 60.0
+        rows[1::3, :, :3000] = float("-inf")
+    elif trouble == "nan":
+        rows[::4, :, V - 1 + off] = float("nan")
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32)[:, :, off:]
+    whole = _draft(rows, 8, 5)
+    for b, n in ((0, 3), (B - 2, 2), (B // 2, 160)):
+        n = min(n, B - b)
+        part = _draft(rows[b:b + n], 8, 5 + b)
+        for key in part:
+            assert np.array_equal(part[key], whole[key][b:b + n], equal_nan=part[key].dtype.kind == "f"), (key, b)
+    n = 2
+    o = oracle.gumbel_topk(workloads.as_oracle_rows(rows[:n].contiguous()), [8], [2], 17, 3, seq_base=5)
+    t = Tally()
+    # an fp32 log-probability is a difference of terms of up to 70: two ulps of that on top of the usual 1e-6
+    compare_topk(t, whole["token"][:n], o, [8], whole["perturbed"][:n], whole["logprob"][:n], logprob_abs_tol=1e-6 + 2 * 70 * 1.2e-7)
+    t.check()
