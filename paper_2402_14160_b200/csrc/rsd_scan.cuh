@@ -417,11 +417,11 @@ __device__ __forceinline__ float slot_element<__nv_bfloat16>(uint32_t addr, uint
 }
 
 // Shared memory of a block of NT threads: the bounds of the row's groups, then one buffer with two uses: the threads'
-// group slots during the streaming loop, the queues of the stages after it.
+// group slots and log-sum-exp references during the streaming loop, the queues of the stages after it.
 template <typename T, int NT>
 __host__ __device__ constexpr size_t scan_buffer_bytes() {
-    const size_t queues = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap), slots = (size_t)NT * GroupSlot<T>::kStride;
-    return queues > slots ? queues : slots;
+    const size_t queues = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap), loop = (size_t)NT * (GroupSlot<T>::kStride + 16);
+    return queues > loop ? queues : loop;
 }
 // blocks of more than 128 threads: a sum and a reference per lane and chunk
 template <int NT>
@@ -488,34 +488,33 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     // of threads, and so are all results.
     const float inv_temp = TEMP ? a.inv_temp : 1.0f, temp = TEMP ? a.temp : 1.0f;   // values enter as value * inv_temp
     const float log2e_t = kLog2e * inv_temp;
-    float lse_thr0 = kNegInf, lse_negc0 = 0.0f;   // every chunk starts with these
     float lse_thr = kNegInf;               // group maxima above this move the reference (-inf: nothing finite yet)
     float lse_negc = 0.0f;                 // -c
     unsigned long long acc0 = f32x2(0.0f, 0.0f), acc1 = acc0;
-    float fold_c = kNegInf, fold_s = 0.0f; // the chunks added up so far (fold_c: reference, -inf: nothing)
-    auto fold = [&](float c, float sum) {
-        if (c == fold_c) {
-            fold_s += sum;
-        } else if (c > kNegInf) {
-            const float m = fmaxf(c, fold_c);
-            fold_s = (fold_c > kNegInf ? fold_s * exp2f(fold_c - m) : 0.0f) + sum * exp2f(c - m);
-            fold_c = m;
-        }
-    };
-    auto begin_chunk = [&] {
-        if (NEED_LSE) {
-            lse_thr = lse_thr0;
-            lse_negc = lse_negc0;
-            acc0 = acc1 = f32x2(0.0f, 0.0f);
-        }
+    // Chunks whose reference stayed where it started are added up in fold_s, the others (rare) in jumped: (reference, sum).
+    // What the loop seldom needs waits in shared memory: at nine blocks per SM every register counts.
+    float fold_s = 0.0f;
+    float2* const ref0 = (float2*)(shared_buf + NT * GroupSlot<T>::kStride) + tid;   // lse_thr, lse_negc at a chunk's start
+    float2* const jumped = ref0 + NT;
+    auto fold = [](float2 into, float c, float sum) {   // (a reference of -inf: nothing)
+        if (c == into.x) return make_float2(c, into.y + sum);
+        if (!(c > kNegInf)) return into;
+        const float m = fmaxf(c, into.x);
+        return make_float2(m, (into.x > kNegInf ? into.y * exp2f(into.x - m) : 0.0f) + sum * exp2f(c - m));
     };
     auto end_chunk = [&](int chunk) {
         if (NEED_LSE) {
             float s0, s1;
             split_f32x2(add_f32x2(acc0, acc1), s0, s1);
-            const float c = lse_thr > kNegInf ? -lse_negc : kNegInf, sum = s0 + s1;
-            if (NT == 128) fold(c, sum);
-            else partial[chunk * 32 + lane] = make_float2(sum, c);
+            acc0 = acc1 = f32x2(0.0f, 0.0f);
+            const float2 r0 = *ref0;
+            if (NT > 128) partial[chunk * 32 + lane] = make_float2(lse_thr > kNegInf ? -lse_negc : kNegInf, s0 + s1);
+            else if (lse_thr == r0.x) fold_s += s0 + s1;
+            else *jumped = fold(*jumped, -lse_negc, s0 + s1);
+            if (lse_thr != r0.x) {
+                lse_thr = r0.x;
+                lse_negc = r0.y;
+            }
         }
     };
     const uint32_t slot = (uint32_t)__cvta_generic_to_shared(shared_buf) + (uint32_t)tid * GroupSlot<T>::kStride;
@@ -578,15 +577,16 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
                 float m = group_max_nan(qf);
                 if (m != m) { qf.clean_nan(); m = group_max_nan(qf); }
                 if (m > kNegInf) {
-                    lse_negc0 = -ceilf(m * log2e_t);
-                    lse_thr0 = fmaf(40.0f, temp, m);   // 40 in scaled units
+                    lse_negc = -ceilf(m * log2e_t);
+                    lse_thr = fmaf(40.0f, temp, m);   // 40 in scaled units
                 }
             }
+            *ref0 = make_float2(lse_thr, lse_negc);
+            if (NT == 128) *jumped = make_float2(kNegInf, 0.0f);
         }
         for (; c < n_full; c += kScanWarps) {
             const int g0 = c * 128 + lane;
             float* ub_g = ub + g0;
-            begin_chunk();
             const uint4 cw = philox_row(a, pr, (uint32_t)(c * 32 + lane));
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {   // two turns of two groups: keeps the loop's code small
@@ -601,7 +601,6 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
         if (c == n_full && (n_groups & 127)) {   // this warp owns the partial chunk; q0 and q1 are on their way
             const int g0 = c * 128 + lane;
             float* ub_g = ub + g0;
-            begin_chunk();
             const uint4 cw = philox_row(a, pr, (uint32_t)(c * 32 + lane));
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
@@ -623,17 +622,23 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     // the warp's share of the log-sum-exp: largest reference exponent C_w and sum of s_t * 2^(c_t - C_w) (exact scaling);
     // the last thread combines the four shares after a barrier.  All in fp32: the threads' sums already are, and
     // double-precision instructions are slow enough to show on every row's critical path.
-    auto share_of_warp = [&] {
-        const float cw_max = warp_max(fold_c);
-        const float d = fold_c - cw_max;   // <= 0, an integer (NaN or -inf when there is nothing to add)
+    float2 start_ref = make_float2(kNegInf, 0.0f);   // .x: this thread's reference at a chunk's start (-inf: none)
+    auto share_of_warp = [&](float2 left) {
+        const float2 mine = fold(make_float2(start_ref.x, fold_s), left.x, left.y);
+        const float cw_max = warp_max(mine.x);
+        const float d = mine.x - cw_max;   // <= 0, an integer (NaN or -inf when there is nothing to add)
         float term = 0.0f;
-        if (fold_c > kNegInf && d > -120.0f) term = fold_s * exp2f(d);
+        if (mine.x > kNegInf && d > -120.0f) term = mine.y * exp2f(d);
         if (cw_max == -kNegInf) term = cw_max - cw_max;  // a +inf value: the sum is not a number
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) term += __shfl_xor_sync(0xFFFFFFFFu, term, o);
         if (lane == 0) { red_f[warp] = cw_max; red_s[warp] = term; }
     };
-    if (NEED_LSE && NT == 128) share_of_warp();
+    if (NEED_LSE) {
+        start_ref = *ref0;
+        start_ref.x = start_ref.x > kNegInf ? -start_ref.y : kNegInf;
+        if (NT == 128) share_of_warp(*jumped);
+    }
     __syncthreads();   // also: every thread is done with its group slot, the queues may take the buffer over
     auto combine_shares = [&] {
         float C = red_f[0];
@@ -652,11 +657,13 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     if (NEED_LSE && NT == 128 && tid == kScanThreads - 1) combine_shares();
     if (NEED_LSE && NT > 128 && warp < 4) {
         const int n_chunks = (n_groups + 127) >> 7;
+        float2 left = make_float2(kNegInf, 0.0f);
         for (int c = warp; c < n_chunks; c += 4) {
             const float2 f = partial[c * 32 + lane];
-            fold(f.y, f.x);
+            if (f.x == start_ref.x) fold_s += f.y;
+            else left = fold(left, f.x, f.y);
         }
-        share_of_warp();
+        share_of_warp(left);
     }
     float tau;
     {
