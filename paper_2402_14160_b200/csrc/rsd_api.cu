@@ -20,21 +20,25 @@ namespace {
 thread_local cudaEvent_t g_scan_before = nullptr, g_scan_after = nullptr;  // one-shot, see rsd_profile_next_scan
 
 // Threads per row.  A block is a row; 128 threads give the most rows in flight and the least work per row (the stages after
-// the streaming loop cost a row the same whatever its threads), but a row then takes 16 us at 32,000 entries, and with few
-// rows most of the chip waits for it.  Measured (us, 32,000 bf16 with log-sum-exp; 128 / 256 / 512 threads): 4 rows 10.0 /
-// 9.0 / 8.0, 192 rows 16.0 / 12.1 / 12.0, 320 rows 16.4 / 14.1 / 18.4, 640 rows 20.2 / 22.3 / 26.4.  Rows of more than
-// 49,152 entries carry over 12 KB of bounds, so that blocks of 128 threads no longer fill an SM: 128,000 bf16, 5000 rows
-// 370 / 247 / 286, 4-byte rows 3000 rows 321 / 284 / 268.
-int scan_threads(int rows, int V, bool f32) {
+// the streaming loop cost a row the same whatever its threads), but with few rows most of the chip waits for the longest.
+// Without a log-sum-exp (us; 128 / 256 / 512 threads, launch included, 32,000 fp32): 32 rows 12.7 / 10.4 / 10.4, 192 rows
+// 17.1 / 14.5 / 14.5, 320 rows 18.6 / 16.6 / 20.4, 640 rows 25.5 / 29.1 / 29.7.  Rows of more than 65,536 entries carry
+// over 16 KB of bounds, so that blocks of 128 threads no longer fill an SM: 128,000 entries, 3000 rows, bf16 196 / 145 / 157,
+// fp32 274 / 262 / 241.
+// A log-sum-exp must come out the same in every launch, and its sums follow the warps: up to 65,536 entries they are those of
+// four warps (few rows: 256 threads with the sums on four warps and the perturbed values on the others), beyond those of
+// eight (256 threads at every size; 128,000 bf16, 192 / 5000 rows: 43 / 370 with 128 threads, 27 / 247 with 256).
+int scan_threads(int rows, int V, bool f32, bool need_lse) {
     static const int sms = [] {
         int dev = 0, n = 0;
         return (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 148;
     }();
-    if (V >= 16384 && rows <= sms + sms / 2) return 512;
+    const bool few = rows <= sms + sms / 2;
+    if (need_lse) return V > rsd::kScanSplitVocab || (V >= 16384 && rows <= 5 * sms / 2) ? 256 : 128;
+    if (V >= 16384 && few) return 512;
     if (V > 65536) return f32 ? 512 : 256;
     if (V >= 16384 && rows <= 5 * sms / 2) return 256;
-    if (V >= 4096 && rows <= sms + sms / 2) return 256;
-    return 128;
+    return V >= 4096 && few ? 256 : 128;
 }
 
 void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs& a, cudaStream_t s) {
@@ -44,7 +48,7 @@ void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs&
         a.rk1[r] = a.seed_hi + (uint32_t)r * 0xBB67AE85u;
     }
     if (g_scan_before) cudaEventRecord(g_scan_before, s);
-    const int threads = scan_threads(blocks, a.V, rows->dtype == RSD_F32);
+    const int threads = scan_threads(blocks, a.V, rows->dtype == RSD_F32, need_lse);
     if (rows->dtype == RSD_F32) rsd::launch_scan_f32(threads, aligned, need_lse, blocks, a, s);
     else rsd::launch_scan_bf16(threads, aligned, need_lse, blocks, a, s);
     if (g_scan_after) cudaEventRecord(g_scan_after, s);

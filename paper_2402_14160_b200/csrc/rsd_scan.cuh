@@ -17,6 +17,7 @@
 namespace rsd {
 
 constexpr int kMaxRows = 256;
+constexpr int kScanSplitVocab = 65536;   // with a log-sum-exp, longer rows always take 256 threads
 constexpr int kIdxNone = 0x7FFFFFFF;
 // Queue sizes of the per-row stages.  Overflow of any of them is handled (general path, raised bound), so a build
 // with tiny sizes (-DRSD_SCAN_SMALL_QUEUES) gives the same results; the tests use one to exercise those paths.
@@ -417,35 +418,35 @@ __device__ __forceinline__ float slot_element<__nv_bfloat16>(uint32_t addr, uint
 }
 
 // Shared memory of a block of NT threads: the bounds of the row's groups, then one buffer with two uses: the threads'
-// group slots and log-sum-exp references during the streaming loop, the queues of the stages after it.
+// group slots during the streaming loop, the queues of the stages after it.
 template <typename T, int NT>
 __host__ __device__ constexpr size_t scan_buffer_bytes() {
-    const size_t queues = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap), loop = (size_t)NT * (GroupSlot<T>::kStride + 16);
-    return queues > loop ? queues : loop;
+    const size_t queues = 4 * (kCandCap + 3 * kTaskCap + 4 * kFinCap), slots = (size_t)NT * GroupSlot<T>::kStride;
+    return queues > slots ? queues : slots;
 }
-// blocks of more than 128 threads: a sum and a reference per lane and chunk
-template <int NT>
-__host__ __device__ constexpr size_t scan_partial_bytes(int V) { return NT == 128 ? 0 : (size_t)((V + 2047) / 2048) * 32 * 8; }
 __host__ __device__ inline size_t scan_bounds_bytes(int V) { return 4 * (size_t)((((V + 15) / 16) + 3) / 4 * 4); }   // padded to fours
 
 // One block per row.
 // ALIGNED: rows start on 32-byte boundaries and V is a multiple of 16 (256-bit loads); other rows are read in aligned
 // 16-byte words, shifted.
 // TEMP: a sampling temperature other than 1 applies (otherwise the scale factors are compile-time constants).
+// SPLIT: the first four warps take the log-sum-exp and nothing else, the others the perturbed values: a few rows are done
+// sooner, and the sums are those of a block of 128 threads to the bit (the loads of the second half hit L2).
 // Blocks of 128 threads: nine per SM for 2-byte rows (56 registers: a group in flight is 8 registers), eight for 4-byte rows;
 // fewer for shifted rows, which need registers for the words around a group.
 template <typename T, bool ALIGNED, int NT>
 constexpr int scan_blocks_per_sm() {
     return ALIGNED ? (NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) : (NT == 128 ? (sizeof(T) == 2 ? 8 : 6) : NT == 256 ? 3 : 2);
 }
-template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT>
-__global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan_topk_kernel(const __grid_constant__ ScanArgs a) {
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
+__global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan_topk_kernel(const ScanArgs a) {
     constexpr int kScanThreads = NT, kScanWarps = NT / 32;
+    constexpr int kLseWarps = SPLIT ? 4 : kScanWarps;      // warps with a share of the log-sum-exp
+    constexpr int kStride = SPLIT ? 4 : kScanWarps;        // a warp's chunks are this far apart
     constexpr bool WIDE = ALIGNED;
     extern __shared__ __align__(16) unsigned char scan_smem[];
     float* const ub = (float*)scan_smem;             // [n_groups] upper bound of each group's perturbed values
     unsigned char* const shared_buf = scan_smem + scan_bounds_bytes(a.V);
-    float2* const partial = (float2*)(shared_buf + scan_buffer_bytes<T, NT>());   // [chunk][lane] (NT > 128)
     int* const cand = (int*)shared_buf;                              // groups whose bound reaches tau
     uint32_t* const tk_x = (uint32_t*)(cand + kCandCap);             // element index | (it carries the group's largest noise) << 31
     float* const tk_base = (float*)(tk_x + kTaskCap);                // lower bound of t(U_M) / 16 of the element's group
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     __shared__ int sv_idx[kSurvCap];
     __shared__ uint32_t bin_max[32];                 // per lane index: largest sample over the warps (ordered encoding)
     __shared__ float red_f[kScanWarps];
-    __shared__ float red_s[4];
+    __shared__ float red_s[kScanWarps];
     __shared__ int n_cand, n_surv, nan_flag;
     __shared__ float lse_sh;
 
@@ -482,51 +483,28 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     // A warp takes chunks of 128 consecutive groups; lane l meets groups l, l + 32, l + 64, l + 96 of the chunk, whose
     // coarse-stream words are the four words of one Philox call.
     float best = kNegInf;                  // largest exact sample of this thread (value(a) + lower bound of G_max)
-    // Log-sum-exp: per lane and chunk the sum of 2^(value * log2(e) - c) with an integer c, moved up only when a group
-    // maximum exceeds it by more than 40; the chunks w, w + 4, w + 8, ... of a lane are then added up in that order.  c
-    // starts from the first group of chunk w of the lane (w = chunk mod 4), so every sum is the same whatever the number
-    // of threads, and so are all results.
+    // Running log-sum-exp of this thread's elements: sum of 2^(value * log2(e) - c) with an integer c, fixed at the
+    // first finite group maximum and moved up only when a group maximum exceeds it by more than 40.
     const float inv_temp = TEMP ? a.inv_temp : 1.0f, temp = TEMP ? a.temp : 1.0f;   // values enter as value * inv_temp
     const float log2e_t = kLog2e * inv_temp;
     float lse_thr = kNegInf;               // group maxima above this move the reference (-inf: nothing finite yet)
     float lse_negc = 0.0f;                 // -c
     unsigned long long acc0 = f32x2(0.0f, 0.0f), acc1 = acc0;
-    // Chunks whose reference stayed where it started are added up in fold_s, the others (rare) in jumped: (reference, sum).
-    // What the loop seldom needs waits in shared memory: at nine blocks per SM every register counts.
-    float fold_s = 0.0f;
-    float2* const ref0 = (float2*)(shared_buf + NT * GroupSlot<T>::kStride) + tid;   // lse_thr, lse_negc at a chunk's start
-    float2* const jumped = ref0 + NT;
-    auto fold = [](float2 into, float c, float sum) {   // (a reference of -inf: nothing)
-        if (c == into.x) return make_float2(c, into.y + sum);
-        if (!(c > kNegInf)) return into;
-        const float m = fmaxf(c, into.x);
-        return make_float2(m, (into.x > kNegInf ? into.y * exp2f(into.x - m) : 0.0f) + sum * exp2f(c - m));
-    };
-    auto end_chunk = [&](int chunk) {
-        if (NEED_LSE) {
-            float s0, s1;
-            split_f32x2(add_f32x2(acc0, acc1), s0, s1);
-            acc0 = acc1 = f32x2(0.0f, 0.0f);
-            const float2 r0 = *ref0;
-            if (NT > 128) partial[chunk * 32 + lane] = make_float2(lse_thr > kNegInf ? -lse_negc : kNegInf, s0 + s1);
-            else if (lse_thr == r0.x) fold_s += s0 + s1;
-            else *jumped = fold(*jumped, -lse_negc, s0 + s1);
-            if (lse_thr != r0.x) {
-                lse_thr = r0.x;
-                lse_negc = r0.y;
-            }
-        }
-    };
     const uint32_t slot = (uint32_t)__cvta_generic_to_shared(shared_buf) + (uint32_t)tid * GroupSlot<T>::kStride;
     // work on one group whose 16 values are in `cur`; `word` is the group's coarse-stream word, `ub_g` = &ub[group]
     auto body = [&](Packed<T>& cur, float* ub_g, uint32_t word) {   // may rewrite cur
-        slot_store(slot, cur);
-        float g_lo, g_hi;
-        group_noise_bounds(word >> 4, g_lo, g_hi);
-        float gmax = group_max_nan(cur);
-        *ub_g = fmaf(gmax, inv_temp, g_hi);                    // NaN if the group holds a NaN: looked at later
-        best = fmaxf(best, fmaf(slot_element<T>(slot, word & 15u), inv_temp, g_lo));  // fmaxf drops NaN
-        if (NEED_LSE) {
+        float gmax = 0.0f;
+        if (!SPLIT || warp >= 4) {
+            slot_store(slot, cur);
+            float g_lo, g_hi;
+            group_noise_bounds(word >> 4, g_lo, g_hi);
+            gmax = group_max_nan(cur);
+            *ub_g = fmaf(gmax, inv_temp, g_hi);                    // NaN if the group holds a NaN: looked at later
+            best = fmaxf(best, fmaf(slot_element<T>(slot, word & 15u), inv_temp, g_lo));  // fmaxf drops NaN
+        } else {
+            gmax = group_max_nan(cur);
+        }
+        if (NEED_LSE && (!SPLIT || warp < 4)) {
             // The sums are taken straight from the packed words, a pair at a time, so that no more than a few unpacked
             // values are alive at once; the rare cases below rewrite the group in place first.
             if (!(gmax <= lse_thr)) {  // rare: a NaN in the group, the first finite group, or a jump of more than 40
@@ -566,37 +544,23 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
             if (g < n_groups) q.load(row, g, V, ALIGNED, WIDE);
         };
         Packed<T> q0, q1;
-        int c = warp;
+        static_assert(!SPLIT || (NT == 256 && NEED_LSE), "four warps for the sums, four for the values");
+        int c = SPLIT ? warp & 3 : warp;
         fetch(q0, c * 128 + lane);
         fetch(q1, c * 128 + 32 + lane);
-        if (NEED_LSE) {
-            Packed<T> qf = q0;
-            const int g_first = (NT == 128 ? c : warp & 3) * 128 + lane;
-            if (NT > 128 && warp >= 4) fetch(qf, g_first);
-            if (g_first < n_groups) {
-                float m = group_max_nan(qf);
-                if (m != m) { qf.clean_nan(); m = group_max_nan(qf); }
-                if (m > kNegInf) {
-                    lse_negc = -ceilf(m * log2e_t);
-                    lse_thr = fmaf(40.0f, temp, m);   // 40 in scaled units
-                }
-            }
-            *ref0 = make_float2(lse_thr, lse_negc);
-            if (NT == 128) *jumped = make_float2(kNegInf, 0.0f);
-        }
-        for (; c < n_full; c += kScanWarps) {
+        for (; c < n_full; c += kStride) {
             const int g0 = c * 128 + lane;
             float* ub_g = ub + g0;
-            const uint4 cw = philox_row(a, pr, (uint32_t)(c * 32 + lane));
+            uint4 cw = make_uint4(0u, 0u, 0u, 0u);
+            if (!SPLIT || warp >= 4) cw = philox_row(a, pr, (uint32_t)(c * 32 + lane));
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {   // two turns of two groups: keeps the loop's code small
-                const int g_next = h ? g0 + kScanWarps * 128 : g0 + 64;   // first turn: inside this chunk
+                const int g_next = h ? g0 + kStride * 128 : g0 + 64;   // first turn: inside this chunk
                 body(q0, ub_g + 64 * h, h ? cw.z : cw.x);
                 fetch(q0, g_next);
                 body(q1, ub_g + 64 * h + 32, h ? cw.w : cw.y);
                 fetch(q1, g_next + 32);
             }
-            end_chunk(c);
         }
         if (c == n_full && (n_groups & 127)) {   // this warp owns the partial chunk; q0 and q1 are on their way
             const int g0 = c * 128 + lane;
@@ -610,7 +574,6 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
                 if (g + 32 < n_groups) body(q1, ub_g + 64 * h + 32, h ? cw.w : cw.y);
                 if (h == 0) fetch(q1, g0 + 96);
             }
-            end_chunk(c);
         }
     }
 
@@ -619,51 +582,37 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     // warps); the k-th largest bin maximum is at most the k-th largest sample, hence at most the k-th largest
     // perturbed value of the row.  Every warp finds it from the 32 bin maxima itself, so one barrier is enough.
     if (best > kNegInf) atomicMax(&bin_max[lane], float_to_ordered(best));
-    // the warp's share of the log-sum-exp: largest reference exponent C_w and sum of s_t * 2^(c_t - C_w) (exact scaling);
-    // the last thread combines the four shares after a barrier.  All in fp32: the threads' sums already are, and
-    // double-precision instructions are slow enough to show on every row's critical path.
-    float2 start_ref = make_float2(kNegInf, 0.0f);   // .x: this thread's reference at a chunk's start (-inf: none)
-    auto share_of_warp = [&](float2 left) {
-        const float2 mine = fold(make_float2(start_ref.x, fold_s), left.x, left.y);
-        const float cw_max = warp_max(mine.x);
-        const float d = mine.x - cw_max;   // <= 0, an integer (NaN or -inf when there is nothing to add)
+    if (NEED_LSE && warp < kLseWarps) {
+        // the warp's share of the log-sum-exp: largest reference exponent C_w and sum of s_t * 2^(c_t - C_w) (exact
+        // scaling); the last thread combines the warps' shares after the barrier.  All in fp32: the threads' sums
+        // already are, and double-precision instructions are slow enough to show on every row's critical path.
+        const float lse_c = lse_thr > kNegInf ? -lse_negc : kNegInf;  // this thread's reference exponent
+        const float cw_max = warp_max(lse_c);
+        float s0, s1, s2, s3;
+        split_f32x2(acc0, s0, s1);
+        split_f32x2(acc1, s2, s3);
+        const float d = lse_c - cw_max;   // <= 0, an integer (NaN or -inf when there is nothing to add)
         float term = 0.0f;
-        if (mine.x > kNegInf && d > -120.0f) term = mine.y * exp2f(d);
+        if (lse_c > kNegInf && d > -120.0f) term = ((s0 + s1) + (s2 + s3)) * exp2f(d);
         if (cw_max == -kNegInf) term = cw_max - cw_max;  // a +inf value: the sum is not a number
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) term += __shfl_xor_sync(0xFFFFFFFFu, term, o);
         if (lane == 0) { red_f[warp] = cw_max; red_s[warp] = term; }
-    };
-    if (NEED_LSE) {
-        start_ref = *ref0;
-        start_ref.x = start_ref.x > kNegInf ? -start_ref.y : kNegInf;
-        if (NT == 128) share_of_warp(*jumped);
     }
     __syncthreads();   // also: every thread is done with its group slot, the queues may take the buffer over
-    auto combine_shares = [&] {
+    if (NEED_LSE && tid == kScanThreads - 1) {
         float C = red_f[0];
 #pragma unroll
-        for (int w = 1; w < 4; ++w) C = fmaxf(C, red_f[w]);
+        for (int w = 1; w < kLseWarps; ++w) C = fmaxf(C, red_f[w]);
         float S = 0.0f;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
+        for (int w = 0; w < kLseWarps; ++w) {
             const float d = red_f[w] - C;
             if (red_f[w] > kNegInf && d > -120.0f) S += red_s[w] * exp2f(d);
             else if (d != d) S = d;
         }
         // C ln 2 + ln S with ln 2 split so that C * hi is exact (C is a small integer)
         lse_sh = (C > kNegInf && (S > 0.0f || S != S)) ? fmaf(C, 0.693145751953125f, fmaf(C, 1.4286068203094172e-06f, logf(S))) : kNegInf;
-    };
-    if (NEED_LSE && NT == 128 && tid == kScanThreads - 1) combine_shares();
-    if (NEED_LSE && NT > 128 && warp < 4) {
-        const int n_chunks = (n_groups + 127) >> 7;
-        float2 left = make_float2(kNegInf, 0.0f);
-        for (int c = warp; c < n_chunks; c += 4) {
-            const float2 f = partial[c * 32 + lane];
-            if (f.x == start_ref.x) fold_s += f.y;
-            else left = fold(left, f.x, f.y);
-        }
-        share_of_warp(left);
     }
     float tau;
     {
@@ -717,7 +666,6 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
         }
     }
     __syncthreads();
-    if (NEED_LSE && NT > 128 && tid == kScanThreads - 1) combine_shares();
     const int n_queued = n_cand;
 
     // exact perturbed values of the elements of group g that can reach tau

@@ -8,10 +8,10 @@
 
 namespace rsd {
 
-template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT>
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
 void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
-    const auto kernel = scan_topk_kernel<T, ALIGNED, NEED_LSE, TEMP, NT>;
-    const size_t smem = scan_bounds_bytes(a.V) + scan_buffer_bytes<T, NT>() + scan_partial_bytes<NT>(a.V);
+    const auto kernel = scan_topk_kernel<T, ALIGNED, NEED_LSE, TEMP, NT, SPLIT>;
+    const size_t smem = scan_bounds_bytes(a.V) + scan_buffer_bytes<T, NT>();
     if (smem > 40 * 1024) {
         // The attribute belongs to the (function, device) pair: raised once per device to what the longest row needs.
         static std::atomic<bool> raised[64];
@@ -19,7 +19,7 @@ void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
         if (cudaGetDevice(&dev) != cudaSuccess) return;   // the error stays pending: the caller's check_launch() reports it
         if (dev < 0 || dev >= 64 || !raised[dev].load(std::memory_order_acquire)) {
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + scan_buffer_bytes<T, NT>() + scan_partial_bytes<NT>(RSD_MAX_VOCAB))) != cudaSuccess)
+                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + scan_buffer_bytes<T, NT>())) != cudaSuccess)
                 return;
             if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
         }
@@ -28,9 +28,15 @@ void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
 }
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP>
 void launch_scan_temp(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {
-    if (threads == 512) launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 512>(blocks, a, s);
-    else if (threads == 256) launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 256>(blocks, a, s);
-    else launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 128>(blocks, a, s);
+    if (NEED_LSE) {   // (512 threads would sum in another order: see scan_threads())
+        if (threads == 256 && a.V <= kScanSplitVocab) launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 256, NEED_LSE>(blocks, a, s);
+        else if (threads == 256) launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 256, false>(blocks, a, s);
+        else launch_scan_threads<T, ALIGNED, NEED_LSE, TEMP, 128, false>(blocks, a, s);
+    } else {
+        if (threads == 512) launch_scan_threads<T, ALIGNED, false, TEMP, 512, false>(blocks, a, s);
+        else if (threads == 256) launch_scan_threads<T, ALIGNED, false, TEMP, 256, false>(blocks, a, s);
+        else launch_scan_threads<T, ALIGNED, false, TEMP, 128, false>(blocks, a, s);
+    }
 }
 template <typename T, bool ALIGNED, bool NEED_LSE>
 void launch_scan_lse(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {
