@@ -203,10 +203,12 @@ struct Packed<float> {
             for (int i = 0; i < 4; ++i) w[i] = ld_stream((const uint4*)group + i);
         }
     }
+    // SHIFTED: a group that is not aligned or full is read in aligned words where they lie inside the row
+    template <bool SHIFTED = true>
     __device__ __forceinline__ void load(const void* row, int g, int V, bool aligned_full, bool wide = false) {
         if (aligned_full) {
             load_aligned((const float*)row + (size_t)g * 16, wide);
-        } else if (g > 0 && (g + 1) * 16 + 4 <= V) {   // the five aligned words around the group, shifted
+        } else if (SHIFTED && g > 0 && (g + 1) * 16 + 4 <= V) {   // the five aligned words around the group, shifted
             const char* at = (const char*)row + (int64_t)g * 64;
             const uint32_t m = (uint32_t)(uintptr_t)at & 15u;
             const uint4* p = (const uint4*)(at - m);
@@ -274,10 +276,12 @@ struct Packed<__nv_bfloat16> {
             w[1] = ld_stream((const uint4*)group + 1);
         }
     }
+    // SHIFTED: a group that is not aligned or full is read in aligned words where they lie inside the row
+    template <bool SHIFTED = true>
     __device__ __forceinline__ void load(const void* row, int g, int V, bool aligned_full, bool wide = false) {
         if (aligned_full) {
             load_aligned((const uint16_t*)row + (size_t)g * 16, wide);
-        } else if (g > 0 && (g + 1) * 16 + 8 <= V) {   // the three aligned words around the group, shifted
+        } else if (SHIFTED && g > 0 && (g + 1) * 16 + 8 <= V) {   // the three aligned words around the group, shifted
             const char* at = (const char*)row + (int64_t)g * 32;
             const uint32_t m = (uint32_t)(uintptr_t)at & 15u;
             const uint4* p = (const uint4*)(at - m);
@@ -446,7 +450,9 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     constexpr bool WIDE = ALIGNED;
     extern __shared__ __align__(16) unsigned char scan_smem[];
     float* const ub = (float*)scan_smem;             // [n_groups] upper bound of each group's perturbed values
-    unsigned char* const shared_buf = scan_smem + scan_bounds_bytes(a.V);
+    // (a static buffer where it fits: with its address known the loop is 2.5 % faster)
+    __shared__ __align__(16) unsigned char static_buf[NT == 128 ? scan_buffer_bytes<T, NT>() : 16];
+    unsigned char* const shared_buf = NT == 128 ? static_buf : scan_smem + scan_bounds_bytes(a.V);
     int* const cand = (int*)shared_buf;                              // groups whose bound reaches tau
     uint32_t* const tk_x = (uint32_t*)(cand + kCandCap);             // element index | (it carries the group's largest noise) << 31
     float* const tk_base = (float*)(tk_x + kTaskCap);                // lower bound of t(U_M) / 16 of the element's group
@@ -541,7 +547,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     {
         const int n_full = n_groups >> 7;                    // whole chunks
         auto fetch = [&](Packed<T>& q, int g) {              // guarded
-            if (g < n_groups) q.load(row, g, V, ALIGNED, WIDE);
+            if (g < n_groups) q.template load<!ALIGNED>(row, g, V, ALIGNED, WIDE);
         };
         Packed<T> q0, q1;
         static_assert(!SPLIT || (NT == 256 && NEED_LSE), "four warps for the sums, four for the values");
@@ -671,7 +677,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     // exact perturbed values of the elements of group g that can reach tau
     auto process_group = [&](int g) {
         Packed<T> grp;
-        grp.load(row, g, V, ALIGNED && (g + 1) * 16 <= V, WIDE);
+        grp.template load<!ALIGNED>(row, g, V, ALIGNED && (g + 1) * 16 <= V, WIDE);
         const uint32_t word = coarse_select(philox_row(a, pr, coarse_index((uint32_t)g)), (uint32_t)g);
         const float base = neg_log_group_uniform_f32(word) * 0.0625f;   // t(U_M) / 16
         const float g_max = -logf(base);
@@ -712,7 +718,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
         for (int i = tid; i < n_queued; i += kScanThreads) {
             const int g = cand[i];
             Packed<T> grp;
-            grp.load(row, g, V, ALIGNED && (g + 1) * 16 <= V, WIDE);
+            grp.template load<!ALIGNED>(row, g, V, ALIGNED && (g + 1) * 16 <= V, WIDE);
             const uint32_t word = coarse_select(philox_row(a, pr, coarse_index((uint32_t)g)), (uint32_t)g);
             const float u = fmaf((float)(word >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f);
             const float t_hat = -__logf(u);

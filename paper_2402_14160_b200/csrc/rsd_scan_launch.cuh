@@ -11,15 +11,16 @@ namespace rsd {
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
 void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
     const auto kernel = scan_topk_kernel<T, ALIGNED, NEED_LSE, TEMP, NT, SPLIT>;
-    const size_t smem = scan_bounds_bytes(a.V) + scan_buffer_bytes<T, NT>();
-    if (smem > 40 * 1024) {
+    constexpr size_t kBuffer = NT == 128 ? 0 : scan_buffer_bytes<T, NT>();   // (128 threads: a static one)
+    const size_t smem = scan_bounds_bytes(a.V) + kBuffer;
+    if (smem > (NT == 128 ? 32 : 40) * 1024) {   // (with the static arrays beside it close to the 48 KB that need no attribute)
         // The attribute belongs to the (function, device) pair: raised once per device to what the longest row needs.
         static std::atomic<bool> raised[64];
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return;   // the error stays pending: the caller's check_launch() reports it
         if (dev < 0 || dev >= 64 || !raised[dev].load(std::memory_order_acquire)) {
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + scan_buffer_bytes<T, NT>())) != cudaSuccess)
+                                     (int)(scan_bounds_bytes(RSD_MAX_VOCAB) + kBuffer)) != cudaSuccess)
                 return;
             if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
         }
