@@ -202,21 +202,21 @@ int rsd_filter_rows(const rsd_rows* rows, int B, int R, int V, int top_k, float 
     a.R = R; a.V = V; a.top_k = top_k; a.top_p = top_p;
     a.log2e_over_t = rsd::kLog2e / temperature_of(rows);
     a.kept = out_kept; a.status = status;
+    // 1024 threads where only one row fits on an SM
+    const bool wide = smem + sizeof(rsd::FilterSmem) + 1024 > 114 * 1024;
+    const int which = (rows->dtype == RSD_F32 ? 0 : 2) + (wide ? 1 : 0);
+    const auto kernel = rows->dtype == RSD_F32 ? (wide ? rsd::filter_rows_kernel<float, 1024> : rsd::filter_rows_kernel<float, 512>)
+                                               : (wide ? rsd::filter_rows_kernel<__nv_bfloat16, 1024> : rsd::filter_rows_kernel<__nv_bfloat16, 512>);
     // the attribute belongs to the (function, device) pair: raised once per device to the largest row that fits
-    static std::atomic<bool> raised[2][64];
+    static std::atomic<bool> raised[4][64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return check_launch("cudaGetDevice");
-    const int which = rows->dtype == RSD_F32 ? 0 : 1;
     if (dev < 0 || dev >= 64 || !raised[which][dev].load(std::memory_order_acquire)) {
-        const int most = (int)(kSharedPerBlock - sizeof(rsd::FilterSmem) - 256);
-        const cudaError_t e = rows->dtype == RSD_F32
-                                  ? cudaFuncSetAttribute(rsd::filter_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
-                                  : cudaFuncSetAttribute(rsd::filter_rows_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e != cudaSuccess) return check_launch("cudaFuncSetAttribute");
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSharedPerBlock - sizeof(rsd::FilterSmem) - 256)) != cudaSuccess)
+            return check_launch("cudaFuncSetAttribute");
         if (dev >= 0 && dev < 64) raised[which][dev].store(true, std::memory_order_release);
     }
-    if (rows->dtype == RSD_F32) rsd::filter_rows_kernel<float><<<B * R, rsd::kFilterThreads, smem, s>>>(a);
-    else rsd::filter_rows_kernel<__nv_bfloat16><<<B * R, rsd::kFilterThreads, smem, s>>>(a);
+    kernel<<<B * R, wide ? 1024 : 512, smem, s>>>(a);
     return check_launch("rsd_filter_rows");
 }
 

@@ -8,28 +8,30 @@
 //
 // One block per row.  The row is copied to shared memory once (NaN turned into -inf on the way); both cuts are then
 // found without sorting, by a search for the value of the last kept token over the ordered bit patterns of the
-// values.  The first step of a search sweeps the row once, 16 bytes at a time, into a histogram of 2048 bins of equal
-// width in value (where the tokens spread evenly): one 64-bit shared-memory addition per token carries both its
-// count and its weight exp(value / T) as a fixed-point number, so the sums are integers and do not depend on the
-// order of the additions.  The bin that brings the tally to what is needed holds a few hundred tokens at most; they
-// are gathered, in token order, and the rest of the search runs over that short list, 16 sub-intervals at a time with
-// bins private to each thread (summed in a fixed order).  The last kept token among equal values comes from a prefix
-// count in token order.
+// values:
+//   sweep   the row once into a histogram of 1024 bins of equal width in value (where the tokens spread evenly).  A token
+//           adds its weight exp(value / T) as a 32-bit fixed-point number, in two halves to two 32-bit counters, so the
+//           sums are integers and do not depend on the order.  (Top-k: it adds 1.)
+//   pick    the bin that brings the tally to what is needed, by a prefix sum over the block
+//   gather  the few hundred tokens of that bin into a list, by tests on whole 16-byte words
+//   finish  by one warp alone, the others waiting at a barrier: 32-way narrowing of the list's code interval down to one
+//           value, then the last kept token among its equals
+// A bin that holds more tokens than the list is swept again, into bins of equal width in code.
+//
+// The kernel is bound by instruction issue: 67,000 instructions per row of 32,000 entries went down to half when every
+// token's work in the sweep was cut from 24 instructions to 14 (no returned atomics, packed arithmetic) and the search
+// behind it was left to one warp.  Three blocks per SM for rows of up to 64,000 bytes, and 1024 threads for rows of which
+// only one fits on an SM.
 #pragma once
 #include "rsd_device.cuh"
-#include "rsd_scan.cuh"   // ex2_approx, better()
+#include "rsd_scan.cuh"   // ex2_approx, packed arithmetic
 
 namespace rsd {
 
-constexpr int kFilterThreads = 512;
-constexpr int kFilterWarps = kFilterThreads / 32;
-constexpr int kFineThreads = 256;                // threads that keep private bins in a search pass over the list
-constexpr int kBins = 16;                        // sub-intervals per search pass over the list
-constexpr int kCoarseBins = 2048;                // bins of the sweep over the row
-constexpr int kCountShift = 47;                  // a histogram entry: count << 47 | weight as fixed point, kept as two 32-bit halves
-constexpr int kListCap = 2048;                   // tokens gathered into a list (indices as 16 bits: rows up to 65,536); sized so
-                                                 // that a 4-byte row of 50,272 entries still fits beside this kernel's other data
-constexpr float kValueRange = 24.0f;             // value-linear bins cover this many nats of value / T below the interval's top
+constexpr int kBins = 1024;                      // bins of a sweep over the row
+constexpr int kListCap = 1024;                   // tokens gathered into a list
+constexpr int kNarrow = 32;                      // sub-intervals per turn of the list's search
+constexpr float kValueRange = 24.0f;             // value-linear bins cover this many nats of value / T below the row's top
 
 struct FilterArgs {
     const void* data;
@@ -46,28 +48,25 @@ struct FilterArgs {
 struct FilterSmem {
     union {
         struct {
-            float mass[kBins][kFineThreads];     // per-thread bins of a search pass over the list
-            uint16_t count[kBins][kFineThreads];
-        } fine;
-        struct {
-            uint32_t lo[kCoarseBins];            // the sweep's histogram: low halves (weights),
-            uint32_t hi[kCoarseBins];            // high halves (count << 15 | the weights' carries)
+            uint32_t lo[kBins];                  // the sweep's histogram: low halves of the weights (or counts),
+            uint32_t hi[kBins];                  // high halves
         } hist;
+        struct {
+            uint32_t lo[kNarrow], hi[kNarrow], count[kNarrow];   // the same for a turn of the list's search
+            uint32_t tie[kListCap];              // tokens equal to the value found
+        } fine;
     };
-    uint32_t bound[kBins + 1];                   // bin q holds the codes bound[q] .. bound[q + 1] - 1 (the last: .. hi)
-    double mass_total[kBins];
-    int count_total[kBins];
-    uint16_t list[kListCap];                     // indices of the tokens still in play, in token order
-    unsigned long long scan_w[kFilterWarps];
-    int red_i[kFilterWarps][2];
-    int scan_i[kFilterWarps];
-    unsigned long long pick_above;               // histogram entries above the picked bin
+    uint32_t list[kListCap];                     // indices of the tokens still in play, in no particular order
+    unsigned long long scan_w[32];
+    unsigned long long pick_above;               // tally above the picked bin
     unsigned long long row_bar;                  // mbarrier of the row's bulk copy
-    int copy_gave_up;
-    int needs_cleaning;
-    int pick_bin;
-    int found;
-    int nan_flag;
+    double above;                                // what the list's search found: the mass or number of the tokens strictly above
+    uint32_t cut_code;                           // the last kept value, its code and
+    int cut_tok;                                 // the last kept token among its equals
+    uint32_t top, ext_lo, ext_hi;                // codes of the row's largest value, of a bin's smallest and largest
+    int pick_bin, n_list, not_finite, n_kept;
+    int copy_gave_up, needs_cleaning, nan_flag;
+    int scan_i[32];
 };
 
 // ordered code of a value's bit pattern: larger value <=> larger code, equal values <=> equal codes; NaN counts as -inf.
@@ -195,6 +194,18 @@ struct RowVec<__nv_bfloat16> {
         }
         return make_uint4(o[0], o[1], o[2], o[3]);
     }
+    // entries of a cleaned word that are not -inf
+    __device__ static __forceinline__ int finite_entries(const uint4& w) {
+        const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+        uint32_t acc = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint32_t gt;
+            asm("set.gt.u32.bf16x2 %0, %1, %2;" : "=r"(gt) : "r"(q[j]), "r"(0xFF80FF80u));
+            acc |= gt & ((1u << (2 * j)) | (1u << (2 * j + 17)));
+        }
+        return __popc(acc);
+    }
 };
 template <>
 struct RowVec<float> {
@@ -217,6 +228,9 @@ struct RowVec<float> {
         }
         return make_uint4(o[0], o[1], o[2], o[3]);
     }
+    __device__ static __forceinline__ int finite_entries(const uint4& w) {
+        return (w.x != 0xFF800000u) + (w.y != 0xFF800000u) + (w.z != 0xFF800000u) + (w.w != 0xFF800000u);
+    }
 };
 
 // A cut in the order (value descending, token ascending): a token is at or before the cut iff its code is larger,
@@ -227,7 +241,8 @@ struct Cut {
 };
 __device__ __forceinline__ bool within(const Cut& c, uint32_t code, int i) { return code > c.code || (code == c.code && i <= c.tok); }
 
-// inclusive prefix sum of a 64-bit word over the block (sm.scan_w as scratch); `total` = the sum over all threads
+// inclusive prefix sum of a 64-bit word over the block; `total` = the sum over all threads
+template <int NT>
 __device__ __forceinline__ unsigned long long block_scan_u64(unsigned long long v, unsigned long long* scratch, unsigned long long& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -237,393 +252,375 @@ __device__ __forceinline__ unsigned long long block_scan_u64(unsigned long long 
     }
     if (lane == 31) scratch[warp] = v;
     __syncthreads();
-    unsigned long long before = 0;
-    total = 0;
+    // every warp adds up the warps' sums by itself
+    const unsigned long long mine = lane < NT / 32 ? scratch[lane] : 0ull;
+    unsigned long long s = mine;
 #pragma unroll
-    for (int w = 0; w < kFilterWarps; ++w) {
-        const unsigned long long s = scratch[w];
-        if (w < warp) before += s;
-        total += s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, s, o);
+        if (lane >= o) s += up;
     }
-    __syncthreads();
-    return v + before;
+    total = __shfl_sync(0xFFFFFFFFu, s, 31);
+    return v + __shfl_sync(0xFFFFFFFFu, s - mine, warp);
 }
 
-template <typename T>
+// Bins over an interval of codes [lo, hi], bin 0 at the top: of equal width in value (values further than the range below
+// hi fall into the last bin), or, where `shift` >= 0, of 2^shift codes each.
+struct BinMap {
+    float scale, offset;     // bin = round(offset - value * scale), at most kBins - 1
+    uint32_t lo, hi;
+    int shift;
+    __device__ __forceinline__ static int of_position(float d) {   // round to nearest, in the low mantissa bits
+        return (int)(__float_as_uint(fminf(d, (float)(kBins - 1)) + 12582912.0f) & (uint32_t)(kBins - 1));
+    }
+    __device__ __forceinline__ int of(float v, uint32_t code) const {
+        return shift >= 0 ? (int)((hi - code) >> shift) : of_position(fmaf(v, -scale, offset));
+    }
+};
+
+template <typename T, int NT>
 struct RowFilter {
     FilterSmem& sm;
     const unsigned char* row;   // shared memory, NaN already turned into -inf
     int V;
     float k, neg_c;             // weight of a value: 2^(value * k + neg_c)
-    int n_list;                 // >= 0: the tokens still in play are sm.list[0 .. n_list); -1: the whole row
+    bool all_finite;            // nothing in the row is -inf
+    int frac_bits, split;       // fixed point of the sweep's weights; bits of a low half
 
-    static constexpr int kPerVec = RowCodes<T>::kPerVec;
+    using Codes = RowCodes<T>;
+    static constexpr int kPerVec = Codes::kPerVec;
 
     __device__ __forceinline__ float weight_of_value(float v) const { return ex2_approx(fmaf(v, k, neg_c)); }
-    __device__ __forceinline__ float weight(uint32_t code) const { return weight_of_value(RowCodes<T>::value_of_code(code)); }
-    __device__ __forceinline__ int items() const { return n_list >= 0 ? n_list : V; }
-    __device__ __forceinline__ int index(int m) const { return n_list >= 0 ? (int)sm.list[m] : m; }
+    __device__ __forceinline__ float weight(uint32_t code) const { return weight_of_value(Codes::value_of_code(code)); }
+    __device__ __forceinline__ float to_fixed() const { return __uint_as_float((uint32_t)(127 + frac_bits) << 23); }
+    __device__ __forceinline__ int words() const { return (V + kPerVec - 1) / kPerVec; }   // (the last one is padded with -inf)
 
-    // What the search found: the code t of the last kept value, the mass and the number of the tokens strictly above it,
-    // and the total mass of the tokens the search started from.
-    struct Found {
-        uint32_t t;
-        double above_mass;
-        int above_count;
-        double total_mass;
-    };
-
-    // f(i, bits) for every token i of the row (the row as 16-byte words, then the few entries past the last whole word)
-    template <typename F>
-    __device__ __forceinline__ void for_each_token(F f) const {
-        const int n_vec = V / kPerVec;
-        for (int m = threadIdx.x; m < n_vec; m += kFilterThreads) {
-            uint32_t h[kPerVec];
-            RowCodes<T>::unpack_bits(((const uint4*)row)[m], h);
-#pragma unroll
-            for (int j = 0; j < kPerVec; ++j) f(m * kPerVec + j, h[j]);
-        }
-        for (int i = n_vec * kPerVec + threadIdx.x; i < V; i += kFilterThreads) f(i, RowCodes<T>::bits(row, i));
+    __device__ __forceinline__ void clear_histogram() {
+        for (int q = threadIdx.x; q < kBins; q += NT) { sm.hist.lo[q] = 0u; sm.hist.hi[q] = 0u; }
     }
 
-    // Bins of equal width in value over [v_lo, v_hi], bin 0 at the top; values below v_lo fall into the last bin.
-    struct Coarse {
-        float v_hi, scale;
-        __device__ __forceinline__ int bin(float v) const {
-            const float d = fminf((v_hi - v) * scale, (float)(kCoarseBins - 1));
-            return (int)(__float_as_uint(d + 12582912.0f) & (uint32_t)(kCoarseBins - 1));   // round to nearest, in the low mantissa bits
-        }
-    };
-
-    // First step of a search over the whole row: one sweep into the histogram, the bin that brings the tally to `need`,
-    // and that bin's tokens gathered into the list.  Returns false (nothing changed but r.total_mass and `need`) when
-    // the interval is too narrow for bins in value or the bin holds more tokens than the list.
+    // Every token of the row into the histogram (cleared): rows without -inf, bins of equal width in value.
     template <bool BY_MASS>
-    __device__ __forceinline__ bool coarse_step(uint32_t& lo, uint32_t& hi, double& need, double need_frac, bool need_is_frac,
-                                                const Cut& inside, bool everything, Found& r) {
-        const int tid = threadIdx.x;
-        Coarse cb;
-        cb.v_hi = RowCodes<T>::value_of_code(hi);
-        const float v_lo = fmaxf(RowCodes<T>::value_of_code(lo), cb.v_hi - kValueRange * kLog2e / k);
-        const float width = cb.v_hi - v_lo;
-        if (!(width > 0.0f) || !(width < 3.0e38f) || hi - lo < 4096u || V > 65536) return false;
-        cb.scale = (float)(kCoarseBins - 1) / width;
-        // Fixed point of the weights: V weights of at most 1 must fit below the count.  32 fraction bits up to 32,767
-        // entries, 31 up to 65,535 (the conversion saturates at 2^32 - 1, which only the row's largest value can reach).
-        // A weight is off by at most half a unit, so the tally is within V 2^-(bits + 1) of the exact sum relative to
-        // the row's largest weight (4e-6 for 32,000 entries in the worst case, around 1e-8 in practice).
-        const int frac_bits = min(32, kCountShift - (32 - __clz(V)));
-        const float to_fixed = __uint_as_float((uint32_t)(127 + frac_bits) << 23);
-        for (int q = tid; q < kCoarseBins; q += kFilterThreads) { sm.hist.lo[q] = 0u; sm.hist.hi[q] = 0u; }
-        __syncthreads();
-        for_each_token([&](int i, uint32_t h) {
-            const float v = RowCodes<T>::value_of_bits(h);
-            if (everything) {
-                if (!(v > kNegInf)) return;                       // -inf (NaN is gone): neither counted nor weighed
+    __device__ __forceinline__ void sweep_all(const BinMap& bm) {
+        const unsigned long long ns = f32x2(-bm.scale, -bm.scale), of = f32x2(bm.offset, bm.offset), magic = f32x2(12582912.0f, 12582912.0f),
+                                 k2 = f32x2(k, k), c2 = f32x2(neg_c, neg_c), fx = f32x2(to_fixed(), to_fixed()), zero = f32x2(0.0f, 0.0f);
+        const uint32_t low_mask = (1u << split) - 1u;
+        auto two = [&](unsigned long long v) {
+            float d0, d1;
+            split_f32x2(fma_f32x2(v, ns, of), d0, d1);
+            split_f32x2(add_f32x2(f32x2(fminf(d0, (float)(kBins - 1)), fminf(d1, (float)(kBins - 1))), magic), d0, d1);
+            const int q0 = (int)(__float_as_uint(d0) & (uint32_t)(kBins - 1)), q1 = (int)(__float_as_uint(d1) & (uint32_t)(kBins - 1));
+            if (BY_MASS) {
+                float x0, x1;
+                split_f32x2(fma_f32x2(v, k2, c2), x0, x1);
+                split_f32x2(fma_f32x2(f32x2(ex2_approx(x0), ex2_approx(x1)), fx, zero), x0, x1);
+                const uint32_t w0 = __float2uint_rn(x0), w1 = __float2uint_rn(x1);
+                atomicAdd(&sm.hist.lo[q0], w0 & low_mask);
+                atomicAdd(&sm.hist.hi[q0], w0 >> split);
+                atomicAdd(&sm.hist.lo[q1], w1 & low_mask);
+                atomicAdd(&sm.hist.hi[q1], w1 >> split);
             } else {
-                const uint32_t code = RowCodes<T>::code_of_bits(h);
-                if (code < lo || code > hi || !within(inside, code, i) || code <= RowCodes<T>::kNegInfCode) return;
+                atomicAdd(&sm.hist.lo[q0], 1u);
+                atomicAdd(&sm.hist.lo[q1], 1u);
             }
-            const int q = cb.bin(v);
-            uint32_t up = 1u << (kCountShift - 32);                // the count's unit in the high half
-            if (BY_MASS) {                                         // a 64-bit addition as two 32-bit ones with the carry
-                const uint32_t w = __float2uint_rn(weight_of_value(v) * to_fixed);
-                const uint32_t old = atomicAdd(&sm.hist.lo[q], w);
-                up += (old + w < old) ? 1u : 0u;
-            }
-            atomicAdd(&sm.hist.hi[q], up);
-        });
-        __syncthreads();
-        // ---- tally from the top bin down: eight bins per thread, then a prefix sum over the threads ---------------------
-        constexpr int kPer = kCoarseBins / kFilterThreads;
-        unsigned long long mine = 0;
-#pragma unroll
-        for (int e = 0; e < kPer; ++e) mine += ((unsigned long long)sm.hist.hi[tid * kPer + e] << 32) | sm.hist.lo[tid * kPer + e];
-        unsigned long long total;
-        const unsigned long long incl = block_scan_u64(mine, sm.scan_w, total);
-        const unsigned long long mass_mask = (1ull << kCountShift) - 1ull;
-        const double from_fixed = 1.0 / (double)(1ull << frac_bits);
-        if (BY_MASS) {
-            r.total_mass = (double)(total & mass_mask) * from_fixed;
-            if (need_is_frac) need = need_frac * r.total_mass;
-        }
-        if (tid == 0) sm.pick_bin = -1;
-        __syncthreads();
-        {
-            unsigned long long run = incl - mine;   // everything above this thread's bins
-            auto tally = [&](unsigned long long w) { return BY_MASS ? (double)(w & mass_mask) * from_fixed : (double)(w >> kCountShift); };
-            if (tally(run) < need && tally(incl) >= need) {
-#pragma unroll
-                for (int e = 0; e < kPer; ++e) {
-                    const unsigned long long w = ((unsigned long long)sm.hist.hi[tid * kPer + e] << 32) | sm.hist.lo[tid * kPer + e];
-                    if (tally(run + w) >= need) { sm.pick_bin = tid * kPer + e; sm.pick_above = run; break; }
-                    run += w;
-                }
-            }
-        }
-        __syncthreads();
-        const int pick = sm.pick_bin;
-        if (pick < 0) return false;                                 // (need beyond the total: left to the search over the row)
-        const unsigned long long above = sm.pick_above;
-        const int population = (int)(sm.hist.hi[pick] >> (kCountShift - 32));
-        __syncthreads();
-        if (population > kListCap) return false;
-        // ---- the codes of the picked bin: the bin index does not increase with the code, so both ends come from a
-        // bisection over the codes with the same arithmetic as the sweep ----------------------------------------------------
-        if (threadIdx.x == 0) {                                      // (two threads of two warps: the others sleep at the barrier)
-            uint32_t a_ = lo, b_ = hi;                               // smallest code with bin <= pick
-            while (a_ < b_) {
-                const uint32_t mid = a_ + ((b_ - a_) >> 1);
-                if (cb.bin(RowCodes<T>::value_of_code(mid)) <= pick) b_ = mid; else a_ = mid + 1u;
-            }
-            sm.bound[0] = a_;
-        } else if (threadIdx.x == 32) {
-            uint32_t a_ = lo, b_ = hi;                               // largest code with bin >= pick
-            while (a_ < b_) {
-                const uint32_t mid = a_ + ((b_ - a_ + 1u) >> 1);
-                if (cb.bin(RowCodes<T>::value_of_code(mid)) >= pick) a_ = mid; else b_ = mid - 1u;
-            }
-            sm.bound[1] = a_;
-        }
-        __syncthreads();
-        const uint32_t first_in = sm.bound[0], last_in = sm.bound[1];   // smallest and largest code of [lo, hi] in the bin
-        __syncthreads();
-        if (first_in > last_in) return false;
-        gather(first_in, last_in, inside, everything);
-        if (n_list < 0) return false;
-        r.above_mass = (double)(above & mass_mask) * from_fixed;
-        r.above_count = (int)(above >> kCountShift);
-        lo = first_in;
-        hi = last_in;
-        return true;
-    }
-
-    // The largest code t in [lo, hi] with F(t) >= need, F(t) = the number (BY_MASS = false) or the weight (BY_MASS = true)
-    // of the tokens within `inside` whose code is >= t.  need = need_abs, or, when need_abs < 0, need_frac times the
-    // total weight of the tokens within `inside` (they all lie in [lo, hi]: the first pass measures it).  F is
-    // non-increasing, F(lo) >= need, nothing within `inside` lies above hi.  `everything`: `inside` holds every finite
-    // token of the row and lo is the smallest finite code (the checks per token then reduce to "finite").
-    template <bool BY_MASS>
-    __device__ __forceinline__ Found search(uint32_t lo, uint32_t hi, double need_abs, double need_frac, const Cut& inside, bool everything) {
-        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-        Found r = {lo, 0.0, 0, 0.0};
-        double need = need_abs;
-        int level = 0;
-        if (n_list < 0 && coarse_step<BY_MASS>(lo, hi, need, need_frac, need_abs < 0.0, inside, everything, r)) {
-            level = 1;
-            if (lo >= hi) { r.t = lo; return r; }
-        } else {
-            r.above_mass = 0.0;
-            r.above_count = 0;
-        }
-        const bool total_known = level > 0;   // (a first step that gave up leaves everything to the passes below)
-        for (;; ++level) {
-            // ---- the 16 sub-intervals ------------------------------------------------------------------------------------------
-            const uint32_t span = hi - lo;
-            const bool by_value = level < 2 && span > 4096u;
-            if (tid <= kBins) {
-                uint32_t bd;
-                if (tid == 0) bd = lo;
-                else if (tid == kBins) bd = hi;          // (unused as a lower bound; bin 15 ends at hi)
-                else if (by_value) {
-                    const float v_hi = RowCodes<T>::value_of_code(hi);
-                    const float v_lo = fmaxf(RowCodes<T>::value_of_code(lo), v_hi - kValueRange * kLog2e / k);
-                    const uint32_t c = RowCodes<T>::code_of_float(v_lo + (v_hi - v_lo) * (float)tid * (1.0f / kBins));
-                    bd = c <= lo ? lo + 1u : (c > hi ? hi : c);
-                } else {
-                    const int shift = max(0, 32 - __clz(span | 1u) - 4);      // (span >> shift) < 16
-                    const uint32_t c = lo + ((uint32_t)tid << shift);
-                    bd = (c < lo || c > hi) ? hi : c;                        // bins past the interval's end are empty:
-                }                                                            // they all start at hi, and only the last holds it
-                sm.bound[tid] = bd;
-            }
-            if (tid < kFineThreads) {
-#pragma unroll
-                for (int q = 0; q < kBins; ++q) { sm.fine.mass[q][tid] = 0.0f; sm.fine.count[q][tid] = 0; }
-            }
-            __syncthreads();
-            // bins that start at the same code: only the last of them is used (the search below takes the largest q)
-            const int n_items = items();
-            for (int m = tid; m < n_items && tid < kFineThreads; m += kFineThreads) {
-                const int i = index(m);
-                const uint32_t code = RowCodes<T>::code(row, i);
-                if (code < lo || code > hi || !within(inside, code, i) || code <= RowCodes<T>::kNegInfCode) continue;
-                int q = code >= sm.bound[8] ? 8 : 0;
-                q += code >= sm.bound[q + 4] ? 4 : 0;
-                q += code >= sm.bound[q + 2] ? 2 : 0;
-                q += code >= sm.bound[q + 1] ? 1 : 0;
-                if (q == kBins) q = kBins - 1;                               // code == hi == bound[16]
-                sm.fine.mass[q][tid] += weight(code);
-                sm.fine.count[q][tid] += 1;
-            }
-            __syncthreads();
-            // ---- totals of the bins: warp w adds up bin w, every lane eight threads' entries in order, then a fixed
-            // tree over the lanes -----------------------------------------------------------------------------------------------
-            static_assert(kFilterWarps == kBins, "one warp per bin");
-            {
-                const int q = warp;
-                double v = 0.0;
-                int c = 0;
-#pragma unroll
-                for (int e = 0; e < kFineThreads / 32; ++e) {
-                    v += (double)sm.fine.mass[q][lane * (kFineThreads / 32) + e];
-                    c += (int)sm.fine.count[q][lane * (kFineThreads / 32) + e];
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-                c = __reduce_add_sync(0xFFFFFFFFu, c);
-                if (lane == 0) { sm.mass_total[q] = v; sm.count_total[q] = c; }
-            }
-            __syncthreads();
-            if (level == 0 && !total_known) {
-                double tot = 0.0;
-                for (int q = 0; q < kBins; ++q) tot += sm.mass_total[q];
-                r.total_mass = tot;
-                if (need_abs < 0.0) need = need_frac * tot;
-            }
-            // ---- from the top bin down: the first bin that brings the tally to `need` holds t ------------------------------
-            double run_m = r.above_mass;
-            int run_c = r.above_count;
-            int pick = 0;
-            for (int q = kBins - 1; q >= 0; --q) {
-                const double f = BY_MASS ? run_m + sm.mass_total[q] : (double)(run_c + sm.count_total[q]);
-                if (f >= need) { pick = q; break; }
-                run_m += sm.mass_total[q];
-                run_c += sm.count_total[q];
-            }
-            r.above_mass = run_m;
-            r.above_count = run_c;
-            const uint32_t new_lo = sm.bound[pick];
-            uint32_t new_hi = hi;
-            if (pick < kBins - 1) {
-                const uint32_t nb = sm.bound[pick + 1];
-                new_hi = nb > new_lo ? nb - 1u : new_lo;          // (an empty bin cannot be picked unless need <= what lies above)
-                if (nb <= new_lo) new_hi = new_lo;
-            }
-            const int population = sm.count_total[pick];
-            __syncthreads();
-            lo = new_lo;
-            hi = new_hi;
-            if (lo >= hi) break;
-            // few enough tokens left: gather them, in token order, and go on over the list
-            if (n_list < 0 && population <= kListCap && V <= 65536) gather(lo, hi, inside, false);
-        }
-        r.t = lo;
-        return r;
-    }
-
-    // The indices of the tokens within `inside` with a code in [lo, hi], in token order, into sm.list (n_list stays -1
-    // when they do not fit).  Threads own consecutive runs of 16-byte words; one prefix count over the block.
-    __device__ __forceinline__ void gather(uint32_t lo, uint32_t hi, const Cut& inside, bool everything) {
-        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-        const int n_vec = (V + kPerVec - 1) / kPerVec;                 // the row's buffer is padded to whole words with -inf
-        const int per = (n_vec + kFilterThreads - 1) / kFilterThreads;
-        const int m0 = min(n_vec, tid * per), m1 = min(n_vec, m0 + per);
-        auto member = [&](int i, uint32_t h) {
-            const uint32_t code = RowCodes<T>::code_of_bits(h);
-            return code >= lo && code <= hi && code > RowCodes<T>::kNegInfCode && (everything || within(inside, code, i)) && i < V;
         };
-        // bit (m - m0) * kPerVec + j of `marks`: entry j of word m may belong (`everything`: a test on the values of
-        // whole words, which is a superset; the passes over the list look at the codes again)
-        const float v_first = RowCodes<T>::value_of_code(lo), v_last = RowCodes<T>::value_of_code(hi);
-        const bool by_word = everything && per * kPerVec <= 128 && lo > RowCodes<T>::kNegInfCode;   // (padding is -inf: never marked)
-        unsigned long long marks[2] = {0ull, 0ull};
-        int mine = 0;
-        for (int m = m0; m < m1; ++m) {
-            if (by_word) {
-                const unsigned long long in = RowVec<T>::between(((const uint4*)row)[m], v_first, v_last);
-                const int at_bit = (m - m0) * kPerVec;               // (a word's bits never straddle the two halves)
-                if (at_bit < 64) marks[0] |= in << at_bit;
-                else marks[1] |= in << (at_bit - 64);
-            } else {
-                uint32_t h[kPerVec];
-                RowCodes<T>::unpack_bits(((const uint4*)row)[m], h);
+        const int n_vec = V / kPerVec;
+        for (int m = threadIdx.x; m < n_vec; m += NT) {
+            uint32_t h[kPerVec];
+            Codes::unpack_bits(((const uint4*)row)[m], h);
 #pragma unroll
-                for (int j = 0; j < kPerVec; ++j) mine += member(m * kPerVec + j, h[j]) ? 1 : 0;
+            for (int j = 0; j < kPerVec; j += 2) two(f32x2(Codes::value_of_bits(h[j]), Codes::value_of_bits(h[j + 1])));
+        }
+        for (int i = n_vec * kPerVec + threadIdx.x; i < V; i += NT) add_one<BY_MASS>(bm.of(Codes::value_of_bits(Codes::bits(row, i)), 0u), Codes::value_of_bits(Codes::bits(row, i)));
+    }
+    template <bool BY_MASS>
+    __device__ __forceinline__ void add_one(int q, float v) {
+        if (BY_MASS) {
+            const uint32_t w = __float2uint_rn(weight_of_value(v) * to_fixed());
+            atomicAdd(&sm.hist.lo[q], w & ((1u << split) - 1u));
+            atomicAdd(&sm.hist.hi[q], w >> split);
+        } else {
+            atomicAdd(&sm.hist.lo[q], 1u);
+        }
+    }
+    // f(i, value, code) for the tokens within `inside` with a code in [bm.lo, bm.hi]
+    template <typename F>
+    __device__ __forceinline__ void for_tokens(const BinMap& bm, const Cut& inside, F f) const {
+        for (int m = threadIdx.x; m < words(); m += NT) {
+            uint32_t h[kPerVec];
+            Codes::unpack_bits(((const uint4*)row)[m], h);
+#pragma unroll
+            for (int j = 0; j < kPerVec; ++j) {
+                const uint32_t code = Codes::code_of_bits(h[j]);
+                const int i = m * kPerVec + j;
+                if (code >= bm.lo && code <= bm.hi && within(inside, code, i) && code > Codes::kNegInfCode) f(i, Codes::value_of_bits(h[j]), code);
             }
         }
-        if (by_word) mine = __popcll(marks[0]) + __popcll(marks[1]);
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += up;
-        }
-        if (lane == 31) sm.scan_i[warp] = incl;
-        __syncthreads();
-        int at = incl - mine, total = 0;
-        for (int w = 0; w < kFilterWarps; ++w) {
-            if (w < warp) at += sm.scan_i[w];
-            total += sm.scan_i[w];
-        }
-        if (total <= kListCap && mine > 0) {
-            if (by_word) {
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    unsigned long long left = marks[half];
-                    while (left) {
-                        const int bit = __ffsll((long long)left) - 1;
-                        left &= left - 1ull;
-                        sm.list[at++] = (uint16_t)(m0 * kPerVec + half * 64 + bit);
-                    }
-                }
-            } else {
-                for (int m = m0; m < m1; ++m) {
-                    uint32_t h[kPerVec];
-                    RowCodes<T>::unpack_bits(((const uint4*)row)[m], h);
-#pragma unroll
-                    for (int j = 0; j < kPerVec; ++j)
-                        if (member(m * kPerVec + j, h[j])) sm.list[at++] = (uint16_t)(m * kPerVec + j);
-                }
-            }
-        }
-        __syncthreads();
-        if (total <= kListCap) n_list = total;
     }
 
-    // Number of the tokens in play that have code `code` and lie within `inside`, and the index of the j-th (1-based) of
-    // them in token order (-1 if there are fewer).  Threads own consecutive runs; one prefix count over the block.
+    // values that may lie in bin `pick`: its edges and a little more (2-byte rows compare against the bounds cut to 16 bits)
+    __device__ __forceinline__ void bin_edges(const BinMap& bm, int pick, float& v_first, float& v_last) const {
+        if (bm.shift >= 0) {
+            const uint32_t hi = bm.hi - ((uint32_t)pick << bm.shift), w = (1u << bm.shift) - 1u;
+            v_first = Codes::value_of_code(hi - bm.lo < w ? bm.lo : hi - w);
+            v_last = Codes::value_of_code(hi);
+        } else {
+            const float slack = 0.5f + 1e-3f + 4e-7f * fabsf(bm.offset);
+            v_last = pick == 0 ? -kNegInf : (bm.offset - ((float)pick - slack)) / bm.scale;
+            v_first = pick == kBins - 1 ? kNegInf : (bm.offset - ((float)pick + slack)) / bm.scale;
+            v_last += fabsf(v_last) * 0.0079f;
+            v_first -= fabsf(v_first) * 0.0079f;
+        }
+    }
+    // The tokens with a value in [v_first, v_last] that f(value, code) accepts (and that are within `inside`) into the list;
+    // sm.n_list counts them, also beyond the list's end.
+    template <typename F>
+    __device__ __forceinline__ void gather(float v_first, float v_last, uint32_t lo, uint32_t hi, const Cut& inside, F f) {
+        if (threadIdx.x == 0) sm.n_list = 0;
+        __syncthreads();
+        for (int m = threadIdx.x; m < words(); m += NT) {
+            const uint4 w = ((const uint4*)row)[m];
+            uint32_t in = RowVec<T>::between(w, v_first, v_last);
+            while (in) {
+                const int j = __ffs(in) - 1;
+                in &= in - 1u;
+                const int i = m * kPerVec + j;
+                const uint32_t h = Codes::bits(row, i), code = Codes::code_of_bits(h);
+                if (code < lo || code > hi || code <= Codes::kNegInfCode || !within(inside, code, i) || !f(Codes::value_of_bits(h), code)) continue;
+                const int at = atomicAdd(&sm.n_list, 1);
+                if (at < kListCap) sm.list[at] = (uint32_t)i;
+            }
+        }
+        __syncthreads();
+    }
+
+    // The j-th (1-based, in token order) of the tokens with code `code` within `inside`, and how many there are: for runs of
+    // equal values that do not fit the list.  Threads own consecutive runs; one prefix count over the block.
     __device__ __forceinline__ int nth_with_code(uint32_t code, int j, const Cut& inside, int& how_many) {
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-        const int n_items = items();
-        const int per = (n_items + kFilterThreads - 1) / kFilterThreads;
-        const int m0 = tid * per, m1 = min(n_items, m0 + per);
+        const int per = (V + NT - 1) / NT;
+        const int m0 = min(V, tid * per), m1 = min(V, m0 + per);
         int mine = 0;
-        for (int m = m0; m < m1; ++m) {
-            const int i = index(m);
-            mine += (RowCodes<T>::code(row, i) == code && within(inside, code, i)) ? 1 : 0;
-        }
+        for (int i = m0; i < m1; ++i) mine += (Codes::code(row, i) == code && within(inside, code, i)) ? 1 : 0;
         int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
             if (lane >= o) incl += up;
         }
+        __syncthreads();
         if (lane == 31) sm.scan_i[warp] = incl;
-        if (tid == 0) sm.found = -1;
+        if (tid == 0) sm.cut_tok = V;
         __syncthreads();
         int before = incl - mine, total = 0;
-        for (int w = 0; w < kFilterWarps; ++w) {
+        for (int w = 0; w < NT / 32; ++w) {
             if (w < warp) before += sm.scan_i[w];
             total += sm.scan_i[w];
         }
         how_many = total;
         if (mine > 0 && before < j && j <= before + mine) {
             int seen = before;
-            for (int m = m0; m < m1; ++m) {
-                const int i = index(m);
-                if (RowCodes<T>::code(row, i) == code && within(inside, code, i) && ++seen == j) { sm.found = i; break; }
-            }
+            for (int i = m0; i < m1; ++i)
+                if (Codes::code(row, i) == code && within(inside, code, i) && ++seen == j) { sm.cut_tok = i; break; }
         }
         __syncthreads();
-        const int r = sm.found;
-        __syncthreads();
-        return r;
+        return sm.cut_tok;
+    }
+
+    // how many of `ties` tokens of code t stay so that the tally reaches `need`
+    template <bool BY_MASS>
+    __device__ __forceinline__ int ties_to_keep(uint32_t t, int ties, double above, double need) const {
+        if (!BY_MASS) return max(1, min(ties, (int)(need - above)));
+        const double w = (double)weight(t);
+        if (!(w > 0.0)) return ties;
+        const double want = ceil((need - above) / w);
+        int j = want < 1.0 ? 1 : (want > (double)ties ? ties : (int)want);
+        while (j > 1 && above + (double)(j - 1) * w >= need) --j;
+        while (j < ties && above + (double)j * w < need) ++j;
+        return j;
+    }
+
+    // The cut within the list (n tokens), by one warp: the largest code t with F(t) >= need, F(t) = `above` plus the number
+    // or weight of the list's tokens whose code is >= t, and the last kept token among its equals.
+    template <bool BY_MASS>
+    __device__ __forceinline__ void finish(int n, double above, double need, const Cut& inside) {
+        const int lane = threadIdx.x & 31;
+        uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+        for (int i = lane; i < n; i += 32) {
+            const uint32_t c = Codes::code(row, (int)sm.list[i]);
+            lo = min(lo, c);
+            hi = max(hi, c);
+        }
+        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+        // weights as 32-bit fixed point relative to the list's largest: exact unless they spread over more than a factor of 128
+        const float w_top = weight(hi);
+        const int e = max((int)((__float_as_uint(w_top) >> 23) & 255u), 1) - 127;
+        const float up_a = __uint_as_float((uint32_t)(127 + (31 - e) / 2) << 23), up_b = __uint_as_float((uint32_t)(127 + (31 - e) - (31 - e) / 2) << 23);
+        const double unit = 1.0 / ((double)up_a * (double)up_b);
+        while (lo < hi) {
+            const int shift = max(0, 32 - __clz(hi - lo) - 5);
+            sm.fine.lo[lane] = 0u;
+            sm.fine.hi[lane] = 0u;
+            sm.fine.count[lane] = 0u;
+            __syncwarp();
+            for (int i = lane; i < n; i += 32) {
+                const uint32_t c = Codes::code(row, (int)sm.list[i]);
+                if (c < lo || c > hi) continue;
+                const int q = (int)((hi - c) >> shift);
+                atomicAdd(&sm.fine.count[q], 1u);
+                if (BY_MASS) {
+                    const uint32_t w = __float2uint_rn((weight(c) * up_a) * up_b);
+                    atomicAdd(&sm.fine.lo[q], w & 0xFFFFu);
+                    atomicAdd(&sm.fine.hi[q], w >> 16);
+                }
+            }
+            __syncwarp();
+            const uint32_t count = sm.fine.count[lane];
+            unsigned long long sum = BY_MASS ? ((unsigned long long)sm.fine.hi[lane] << 16) + sm.fine.lo[lane] : (unsigned long long)count;
+            __syncwarp();
+            const unsigned long long mine = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long s = __shfl_up_sync(0xFFFFFFFFu, sum, o);
+                if (lane >= o) sum += s;
+            }
+            const double per = BY_MASS ? unit : 1.0;
+            const unsigned reached = __ballot_sync(0xFFFFFFFFu, count > 0u && above + (double)sum * per >= need), some = __ballot_sync(0xFFFFFFFFu, count > 0u);
+            const int pick = reached ? __ffs(reached) - 1 : 31 - __clz(some);   // (rounding: the last one that holds anything)
+            above += (double)__shfl_sync(0xFFFFFFFFu, sum - mine, pick) * per;
+            const uint32_t new_hi = hi - ((uint32_t)pick << shift), width = (1u << shift) - 1u;
+            lo = new_hi - lo < width ? lo : new_hi - width;
+            hi = new_hi;
+        }
+        // the tokens equal to the value found, in no particular order
+        int ties = 0;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const uint32_t x = i0 + lane < n ? sm.list[i0 + lane] : 0u;
+            const bool eq = i0 + lane < n && Codes::code(row, (int)x) == lo;
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, eq);
+            if (eq) sm.fine.tie[ties + __popc(m & ((1u << lane) - 1u))] = x;
+            ties += __popc(m);
+        }
+        __syncwarp();
+        const int j = ties_to_keep<BY_MASS>(lo, ties, above, need);
+        int tok = lo == inside.code ? inside.tok : V;      // (all of them stay)
+        if (j < ties) {
+            if (ties <= 32) {
+                const uint32_t x = lane < ties ? sm.fine.tie[lane] : 0xFFFFFFFFu;
+                int rank = 0;
+                for (int i = 0; i < ties; ++i) rank += __shfl_sync(0xFFFFFFFFu, x, i) < x ? 1 : 0;
+                tok = (int)__shfl_sync(0xFFFFFFFFu, x, __ffs(__ballot_sync(0xFFFFFFFFu, lane < ties && rank == j - 1)) - 1);
+            } else {                                       // smallest token with j ties up to it
+                int a_ = 0, b_ = V - 1;
+                while (a_ < b_) {
+                    const int mid = (a_ + b_) >> 1;
+                    int c = 0;
+                    for (int i = lane; i < ties; i += 32) c += (int)sm.fine.tie[i] <= mid ? 1 : 0;
+                    if (__reduce_add_sync(0xFFFFFFFFu, c) >= j) b_ = mid; else a_ = mid + 1;
+                }
+                tok = a_;
+            }
+        }
+        if (lane == 0) { sm.cut_code = lo; sm.cut_tok = tok; }
+    }
+
+    // The cut at which the number (BY_MASS = false) or the weight of the tokens within `inside` reaches need_abs, or, when that
+    // is negative, need_frac of their total weight.  Nothing within `inside` lies above code `top`.  The histogram is clear.
+    template <bool BY_MASS>
+    __device__ __forceinline__ Cut search(uint32_t bottom, uint32_t top, double need_abs, double need_frac, const Cut& inside, bool everything) {
+        const int tid = threadIdx.x;
+        double need = need_abs, above = 0.0;
+        BinMap bm;
+        bm.lo = bottom;
+        bm.hi = top;
+        for (int level = 0;; ++level) {
+            // bins of equal width in value first; in code where the interval is narrow or infinite, and on every further level
+            bm.shift = -1;
+            const float v_hi = Codes::value_of_code(bm.hi);
+            const float width = v_hi - fmaxf(Codes::value_of_code(bm.lo), v_hi - kValueRange * kLog2e / k);
+            bm.scale = (float)(kBins - 1) / width;
+            bm.offset = v_hi * bm.scale;
+            if (level > 0 || bm.hi - bm.lo < (uint32_t)kBins || !(width > 0.0f) || !(width < 3.0e38f) || !(fabsf(bm.offset) < 1.0e6f))   // (rows far from 0: the position's rounding must stay below half a bin)
+                bm.shift = max(0, 32 - __clz(bm.hi - bm.lo) - 10);   // ((hi - lo) >> shift) < 1024
+            if (bm.shift < 0 && everything && all_finite) sweep_all<BY_MASS>(bm);
+            else for_tokens(bm, inside, [&](int, float v, uint32_t code) { add_one<BY_MASS>(bm.of(v, code), v); });
+            __syncthreads();
+            // ---- tally from the top bin down -------------------------------------------------------------------------------
+            constexpr int kPer = kBins / NT;
+            auto bin_sum = [&](int q) { return ((unsigned long long)sm.hist.hi[q] << split) + sm.hist.lo[q]; };
+            unsigned long long mine = 0;
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) mine += bin_sum(tid * kPer + e);
+            unsigned long long total;
+            const unsigned long long incl = block_scan_u64<NT>(mine, sm.scan_w, total);
+            const double unit = BY_MASS ? 1.0 / (double)(1ull << frac_bits) : 1.0;
+            if (level == 0 && need_abs < 0.0) need = need_frac * ((double)total * unit);
+            if (tid == 0) sm.pick_bin = -1;
+            __syncthreads();
+            {
+                unsigned long long run = incl - mine;   // everything above this thread's bins
+                auto tally = [&](unsigned long long w) { return above + (double)w * unit; };
+                if (tally(run) < need && tally(incl) >= need) {
+#pragma unroll
+                    for (int e = 0; e < kPer; ++e) {
+                        const unsigned long long w = bin_sum(tid * kPer + e);
+                        if (tally(run) < need && tally(run + w) >= need) { sm.pick_bin = tid * kPer + e; sm.pick_above = run; }
+                        run += w;
+                    }
+                }
+            }
+            __syncthreads();
+            int pick = sm.pick_bin;
+            if (pick < 0) {                              // (`need` beyond the total by rounding: the last bin that holds anything)
+                unsigned long long run = incl - mine;
+                if (mine > 0 && incl == total) {
+                    for (int e = 0; e < kPer; ++e) {
+                        const unsigned long long w = bin_sum(tid * kPer + e);
+                        if (w > 0) { sm.pick_bin = tid * kPer + e; sm.pick_above = run; }
+                        run += w;
+                    }
+                }
+                __syncthreads();
+                pick = max(sm.pick_bin, 0);
+                if (sm.pick_bin < 0 && tid == 0) sm.pick_above = 0ull;
+                __syncthreads();
+            }
+            above += (double)sm.pick_above * unit;
+            float v_first, v_last;
+            bin_edges(bm, pick, v_first, v_last);
+            gather(v_first, v_last, bm.lo, bm.hi, inside, [&](float v, uint32_t code) { return bm.of(v, code) == pick; });   // (ends with a barrier)
+            const int n = sm.n_list;
+            if (n > 0 && n <= kListCap) {
+                if (tid < 32) finish<BY_MASS>(n, above, need, inside);
+                __syncthreads();
+                return {sm.cut_code, sm.cut_tok};
+            }
+            // ---- more tokens than the list holds: the codes the bin spans, then once more over these ------------------------
+            if (tid == 0) { sm.ext_lo = 0xFFFFFFFFu; sm.ext_hi = 0u; }
+            __syncthreads();
+            uint32_t c_lo = 0xFFFFFFFFu, c_hi = 0u;
+            for_tokens(bm, inside, [&](int, float v, uint32_t code) {
+                if (bm.of(v, code) == pick) { c_lo = min(c_lo, code); c_hi = max(c_hi, code); }
+            });
+            c_lo = __reduce_min_sync(0xFFFFFFFFu, c_lo);
+            c_hi = __reduce_max_sync(0xFFFFFFFFu, c_hi);
+            if ((tid & 31) == 0) { atomicMin(&sm.ext_lo, c_lo); atomicMax(&sm.ext_hi, c_hi); }
+            clear_histogram();
+            __syncthreads();
+            bm.lo = sm.ext_lo;
+            bm.hi = sm.ext_hi;
+            if (bm.lo >= bm.hi) {                        // a run of equal values
+                int ties;
+                nth_with_code(bm.hi, 1, inside, ties);
+                return {bm.hi, nth_with_code(bm.hi, ties_to_keep<BY_MASS>(bm.hi, ties, above, need), inside, ties)};
+            }
+        }
     }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const FilterArgs a) {
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(const FilterArgs a) {
     extern __shared__ __align__(16) unsigned char row_sm[];   // the row, padded with -inf to whole 16-byte words
     __shared__ FilterSmem sm;
     constexpr int kElem = (int)sizeof(T);
@@ -633,6 +630,7 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const Filte
     const unsigned char* src = (const unsigned char*)a.data + ((int64_t)b * a.seq_stride + (int64_t)r * a.row_stride) * kElem;
     unsigned char* dst = (unsigned char*)a.out + ((int64_t)b * a.R + r) * (int64_t)V * kElem;
     const int n_vec = V / kPerVec;                               // whole 16-byte words of the row
+    const int n_all = (V + kPerVec - 1) / kPerVec;               // with the padded word
 
     // ---- the row into shared memory, NaN as -inf; its largest value and the number of finite entries ------------------
     // Rows that start on a 16-byte boundary come in by one bulk copy of the whole words, the others by plain loads.  A
@@ -643,22 +641,31 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const Filte
         sm.nan_flag = 0;
         sm.copy_gave_up = 0;
         sm.needs_cleaning = 0;
+        sm.not_finite = 0;
+        sm.n_kept = 0;
+        sm.top = RowCodes<T>::kNegInfCode;
         if (bulk) {
             mbar_init(&sm.row_bar, 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-    }
-    __syncthreads();
-    if (bulk) {
-        if (tid == 0) {
             // (an mbarrier counts at most 2^20 - 1 bytes per phase, a row has fewer)
             mbar_expect_tx(&sm.row_bar, (uint32_t)n_vec * 16u);
             bulk_load(row_sm, src, (uint32_t)n_vec * 16u, &sm.row_bar);
         }
-    } else {
-        for (int i = tid; i < n_vec * kPerVec; i += kFilterThreads) {
-            if (kElem == 2) ((uint16_t*)row_sm)[i] = (uint16_t)RowCodes<T>::bits(src, i);
-            else ((uint32_t*)row_sm)[i] = RowCodes<T>::bits(src, i);
+    }
+    for (int q = tid; q < kBins; q += NT) { sm.hist.lo[q] = 0u; sm.hist.hi[q] = 0u; }
+    if (!bulk) {
+        const uint32_t m = (uint32_t)(uintptr_t)src & 15u;
+        if (m != 0 && n_vec > 2 && m % kElem == 0) {             // in the aligned words around each, shifted; the ends one by one
+            for (int i = 1 + tid; i < n_vec - 1; i += NT) {
+                const uint4* p = (const uint4*)(src + (size_t)i * 16 - m);
+                ((uint4*)row_sm)[i] = window16(__ldg(p), __ldg(p + 1), m);
+            }
+        }
+        const bool ends = m != 0 && n_vec > 2 && m % kElem == 0;
+        for (int i = tid; i < (ends ? 2 * kPerVec : n_vec * kPerVec); i += NT) {
+            const int x = ends && i >= kPerVec ? (n_vec - 2) * kPerVec + i : i;
+            if (kElem == 2) ((uint16_t*)row_sm)[x] = (uint16_t)RowCodes<T>::bits(src, x);
+            else ((uint32_t*)row_sm)[x] = RowCodes<T>::bits(src, x);
         }
     }
     if (tid < kPerVec && n_vec * kPerVec < V) {                  // the last, partial word, padded with -inf
@@ -667,34 +674,34 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const Filte
         if (kElem == 2) ((uint16_t*)row_sm)[i] = (uint16_t)h;
         else ((uint32_t*)row_sm)[i] = h;
     }
+    __syncthreads();
     if (bulk && warp == 0) wait_bar(&sm.row_bar, 0, &sm.copy_gave_up);   // one warp polls, the others sleep at the barrier
     __syncthreads();
     if (bulk && warp != 0 && !sm.copy_gave_up) wait_bar(&sm.row_bar, 0, &sm.copy_gave_up);   // (done: every thread has now seen the copy's completion itself)
+    {
+        float vtop = kNegInf;
+        bool odd = false;                                        // something is NaN or -inf
+        for (int m = tid; m < n_vec; m += NT) vtop = fmaxf(vtop, RowStats<T>::largest(((const uint4*)row_sm)[m], odd));
+        for (int i = n_vec * kPerVec + tid; i < V; i += NT) {
+            const float v = RowCodes<T>::value_of_bits(RowCodes<T>::bits(row_sm, i));
+            vtop = fmaxf(vtop, v);
+            odd |= !(v > kNegInf);
+        }
+        if (odd) sm.needs_cleaning = 1;
+        // (+0 and -0 are equal as values but not as codes: the larger code stands for both)
+        uint32_t top = vtop == 0.0f ? RowCodes<T>::code_of_float(0.0f) : (vtop > kNegInf ? RowCodes<T>::code_of_float(vtop) : RowCodes<T>::kNegInfCode);
+        top = __reduce_max_sync(0xFFFFFFFFu, top);
+        if (lane == 0) atomicMax(&sm.top, top);
+    }
     __syncthreads();
     if (sm.copy_gave_up) {                                        // the copy never landed: report, write nothing
         if (tid == 0) atomicOr(&a.status[b], 32);                 // RSD_ST_TIMEOUT
         return;
     }
-    uint32_t top = RowCodes<T>::kNegInfCode;
-    int finite = V;
-    {
-        const int n_all = (V + kPerVec - 1) / kPerVec;           // with the padded word
-        float vtop = kNegInf;
-        bool odd = false;                                        // something is NaN or -inf
-        for (int m = tid; m < n_all; m += kFilterThreads) {
-            const uint4 w = ((const uint4*)row_sm)[m];
-            vtop = fmaxf(vtop, RowStats<T>::largest(w, odd));
-        }
-        if (odd) sm.needs_cleaning = 1;
-        // (+0 and -0 are equal as values but not as codes: the larger code stands for both)
-        top = vtop == 0.0f ? RowCodes<T>::code_of_float(0.0f) : (vtop > kNegInf ? RowCodes<T>::code_of_float(vtop) : RowCodes<T>::kNegInfCode);
-    }
-    __syncthreads();
     if (sm.needs_cleaning) {
         bool saw_nan = false;
         int not_finite = 0;
-        const int n_all = (V + kPerVec - 1) / kPerVec;
-        for (int m = tid; m < n_all; m += kFilterThreads) {
+        for (int m = tid; m < n_all; m += NT) {
             uint32_t h[kPerVec];
             RowCodes<T>::unpack_bits(((const uint4*)row_sm)[m], h);
 #pragma unroll
@@ -704,72 +711,71 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const Filte
             }
             ((uint4*)row_sm)[m] = RowCodes<T>::pack_bits(h);
         }
-        finite = -not_finite;                                    // (V is added back after the sum over the block)
+        not_finite = __reduce_add_sync(0xFFFFFFFFu, not_finite);
+        if (lane == 0 && not_finite) atomicAdd(&sm.not_finite, not_finite);
         if (saw_nan) sm.nan_flag = 1;
-    } else {
-        finite = 0;
+        __syncthreads();
     }
-    top = __reduce_max_sync(0xFFFFFFFFu, top);
-    finite = __reduce_add_sync(0xFFFFFFFFu, finite);
-    if (lane == 0) { sm.red_i[warp][0] = (int)top; sm.red_i[warp][1] = finite; }
-    __syncthreads();
-    top = 0u;
-    finite = V;
-    for (int w = 0; w < kFilterWarps; ++w) {
-        top = (uint32_t)sm.red_i[w][0] > top ? (uint32_t)sm.red_i[w][0] : top;
-        finite += sm.red_i[w][1];
-    }
-    __syncthreads();
+    const uint32_t top = sm.top;
+    const int finite = V - sm.not_finite;
 
     const float vmax = RowCodes<T>::value_of_code(top);
     const bool plus_inf = vmax == -kNegInf;                       // a +inf entry: it alone carries the mass
-    RowFilter<T> f = {sm, row_sm, V, a.log2e_over_t, (finite > 0 && !plus_inf) ? -vmax * a.log2e_over_t : 0.0f, -1};
+    // Fixed point of the weights: 32 fraction bits up to 32,767 entries, 31 up to 65,535, 30 beyond (the conversion saturates
+    // at 2^32 - 1, which only the row's largest value can reach); the halves are such that V of them fit 32 bits.  A weight is
+    // off by at most half a unit, so the tally is within V 2^-(bits + 1) of the exact sum relative to the row's largest
+    // weight (4e-6 for 32,000 entries in the worst case, around 1e-8 in practice).
+    const int frac_bits = V < 32768 ? 32 : V < 65536 ? 31 : 30;
+    RowFilter<T, NT> f = {sm, row_sm, V, a.log2e_over_t, (finite > 0 && !plus_inf) ? -vmax * a.log2e_over_t : 0.0f, sm.not_finite == 0, frac_bits,
+                          V < 65536 ? 16 : 15};
     Cut cut = {RowCodes<T>::kNegInfCode, V};                      // everything finite
     int kept = finite;
-    bool everything = true;
+    bool everything = true, count_kept = false;
 
     // ---- top-k: the value of the k-th largest entry, then the last kept token among its equals -------------------------
+    const bool want_p = a.top_p > 0.0f && a.top_p < 1.0f && finite > 0 && !plus_inf;
     if (a.top_k > 0 && a.top_k < V && finite > a.top_k) {
-        const typename RowFilter<T>::Found r = f.template search<false>(RowCodes<T>::kNegInfCode + 1u, top, (double)a.top_k, 0.0, cut, true);
-        int ties;
-        const int tok = f.nth_with_code(r.t, a.top_k - r.above_count, cut, ties);   // that many of the entries equal to t stay
-        cut.code = r.t;
-        cut.tok = tok >= 0 ? tok : V;
+        cut = f.template search<false>(RowCodes<T>::kNegInfCode + 1u, top, (double)a.top_k, 0.0, cut, true);
         kept = a.top_k;
-        f.n_list = -1;                                            // (the list was gathered for the old cut)
         everything = false;
+        if (want_p) {
+            __syncthreads();
+            f.clear_histogram();
+            __syncthreads();
+        }
     }
     // ---- top-p: of what is left, the shortest prefix (value descending, token ascending) whose mass reaches top_p -------
-    if (a.top_p > 0.0f && a.top_p < 1.0f && kept > 0 && !plus_inf) {
-        const typename RowFilter<T>::Found r = f.template search<true>(everything ? RowCodes<T>::kNegInfCode + 1u : cut.code, top, -1.0,
-                                                                       (double)a.top_p, cut, everything);
-        const double need = (double)a.top_p * r.total_mass;
-        // entries equal to t within the cut: each weighs w; the first j of them (token order) complete the prefix
-        int ties;
-        f.nth_with_code(r.t, 1, cut, ties);
-        const double w = (double)f.weight(r.t);
-        int j = ties;
-        if (w > 0.0) {
-            const double want = ceil((need - r.above_mass) / w);
-            j = want < 1.0 ? 1 : (want > (double)ties ? ties : (int)want);
-            while (j > 1 && r.above_mass + (double)(j - 1) * w >= need) --j;
-            while (j < ties && r.above_mass + (double)j * w < need) ++j;
+    if (want_p) {
+        if (!everything && kept <= kListCap) {
+            // the kept tokens all fit the list: one warp does the rest (their total in the sweep's fixed point)
+            f.gather(RowCodes<T>::value_of_code(cut.code), vmax, cut.code, top, cut, [](float, uint32_t) { return true; });
+            if (tid < 32) {
+                unsigned long long total = 0;
+                const int n = sm.n_list;
+                for (int i = lane; i < n; i += 32)
+                    total += __float2uint_rn(f.weight(RowCodes<T>::code(row_sm, (int)sm.list[i])) * f.to_fixed());
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+                f.template finish<true>(n, 0.0, (double)a.top_p * ((double)total / (double)(1ull << frac_bits)), cut);
+            }
+            __syncthreads();
+            cut = {sm.cut_code, sm.cut_tok};
+        } else {
+            cut = f.template search<true>(everything ? RowCodes<T>::kNegInfCode + 1u : cut.code, top, -1.0, (double)a.top_p, cut, everything);
         }
-        const int tok = f.nth_with_code(r.t, j, cut, ties);
-        cut.code = r.t;
-        cut.tok = tok >= 0 ? tok : V;
-        kept = r.above_count + j;
+        count_kept = a.kept != nullptr;
     }
 
     // ---- the row with -inf at the filtered entries ------------------------------------------------------------------------------
     {
-        auto keep_bits = [&](int i, uint32_t h) {
+        auto keeps = [&](int i, uint32_t h) {
             const uint32_t c = RowCodes<T>::code_of_bits(h);
-            return (c > RowCodes<T>::kNegInfCode && within(cut, c, i)) ? h : RowCodes<T>::kNegInfBits;
+            return c > RowCodes<T>::kNegInfCode && within(cut, c, i);
         };
         const bool dst16 = ((uintptr_t)dst & 15u) == 0;
         const float cut_value = RowCodes<T>::value_of_code(cut.code);
-        for (int m = tid; m < n_vec; m += kFilterThreads) {
+        int n_kept = 0;
+        for (int m = tid; m < n_vec; m += NT) {
             const uint4 w = ((const uint4*)row_sm)[m];
             uint32_t any_eq;
             uint4 o = RowVec<T>::at_least(w, cut_value, any_eq);   // right wherever no entry equals the cut's value
@@ -777,9 +783,11 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const Filte
                 uint32_t h[kPerVec];
                 RowCodes<T>::unpack_bits(w, h);
 #pragma unroll
-                for (int j = 0; j < kPerVec; ++j) h[j] = keep_bits(m * kPerVec + j, h[j]);
+                for (int j = 0; j < kPerVec; ++j)
+                    if (!keeps(m * kPerVec + j, h[j])) h[j] = RowCodes<T>::kNegInfBits;
                 o = RowCodes<T>::pack_bits(h);
             }
+            if (count_kept) n_kept += RowVec<T>::finite_entries(o);
             if (dst16) {
                 ((uint4*)dst)[m] = o;
             } else {
@@ -792,10 +800,19 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const Filte
                 }
             }
         }
-        for (int i = n_vec * kPerVec + tid; i < V; i += kFilterThreads) {
-            const uint32_t h = keep_bits(i, RowCodes<T>::bits(row_sm, i));
+        for (int i = n_vec * kPerVec + tid; i < V; i += NT) {
+            const uint32_t h0 = RowCodes<T>::bits(row_sm, i);
+            const bool stays = keeps(i, h0);
+            const uint32_t h = stays ? h0 : RowCodes<T>::kNegInfBits;
+            n_kept += stays ? 1 : 0;
             if (kElem == 2) ((uint16_t*)dst)[i] = (uint16_t)h;
             else ((uint32_t*)dst)[i] = h;
+        }
+        if (count_kept) {
+            n_kept = __reduce_add_sync(0xFFFFFFFFu, n_kept);
+            if (lane == 0) atomicAdd(&sm.n_kept, n_kept);
+            __syncthreads();
+            kept = sm.n_kept;
         }
     }
     if (tid == 0) {

@@ -144,3 +144,17 @@ def test_filtered_rows_through_drafting_and_verification(rsd, dtype, V):
     for b in range(B):
         node = ov["accepted_node"][b, ov["accepted_len"][b] - 1] if ov["accepted_len"][b] > 0 else 0
         assert keep_t[b, node][ov["last_token"][b]]                # the last token comes from the target's nucleus
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 32767), ("bf16", 32768), ("bf16", 49000), ("bf16", 65535), ("bf16", 65537), ("bf16", 100001),
+                                     ("f32", 25600), ("f32", 50003)])
+def test_filter_rows_at_the_edges_of_its_fixed_point_and_block_sizes(rsd, dtype, V):
+    # the weights' fraction bits change at 32,768 and 65,536 entries, the block at about 100 KB of row; top_k on both sides of
+    # the list's 1024 entries, alone and before a nucleus; rows far from 0 and rows too flat for the first sweep's bins
+    rows = _rows((1, 4, V), "f32", 2.0, 90 + V)
+    rows[0, 1] += 700.0
+    rows[0, 2] *= 0.01
+    rows[0, 3, ::7] = float("-inf")
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    for top_k, top_p, T in ((0, 0.95, 1.0), (1024, 0.9, 1.0), (1025, 0.9, 0.7), (2000, 1.0, 1.0)):
+        _check_filter(rsd, rows, top_k, top_p, T, max_borderline=2)
