@@ -104,17 +104,33 @@ __device__ __forceinline__ void send_word(uint32_t addr, float v, uint32_t bar) 
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// the command barrier: the control warp arrives, the working warps wait
+// (every barrier is met by whole warps: the lanes are brought together first)
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int ID, int THREADS>
+__device__ __forceinline__ void named_sync() {
+    __syncwarp();
+    asm volatile("barrier.cta.sync.aligned %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+// The command barrier: the control warp arrives, the working warps wait.  It arrives for a pass only when it has the sums of
+// the pass before, that is when every working warp has met the barrier before: nobody arrives twice at one barrier.
 template <int THREADS>
-__device__ __forceinline__ void cmd_arrive() { asm volatile("barrier.cta.arrive 1, %0;" ::"n"(THREADS) : "memory"); }
+__device__ __forceinline__ void cmd_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cta.arrive.aligned 1, %0;" ::"n"(THREADS) : "memory");
+}
 template <int THREADS>
-__device__ __forceinline__ void cmd_sync() { asm volatile("barrier.cta.sync 1, %0;" ::"n"(THREADS) : "memory"); }
+__device__ __forceinline__ void cmd_sync() { named_sync<1, THREADS>(); }
 template <int THREADS>
-__device__ __forceinline__ void dump_sync() { asm volatile("barrier.cta.sync 3, %0;" ::"n"(THREADS) : "memory"); }
+__device__ __forceinline__ void workers_sync() { named_sync<2, THREADS>(); }
 template <int THREADS>
-__device__ __forceinline__ void workers_sync() { asm volatile("barrier.cta.sync 2, %0;" ::"n"(THREADS) : "memory"); }
+__device__ __forceinline__ void dump_sync() { named_sync<3, THREADS>(); }
 
 // A lane's 16 values of a tile: the 16-byte pieces lane, lane + 32, ... (the order of the ring walk), -inf beyond the
 // row's end.  Rows on 16-byte boundaries take one load a piece.  Others take the two aligned words around it, shifted;
