@@ -2,7 +2,8 @@
 
 Every function takes torch CUDA tensors, passes their device pointers and the current CUDA stream to the entry
 point of the same name, and returns freshly allocated output tensors.  Nothing is computed here.  The library is
-loaded on first use and a missing or unbuilt library raises: there is no CPU fallback.
+loaded on first use and a missing or unbuilt library raises: there is no CPU fallback.  The calls go through a small
+CPython extension (csrc/rsd_bind.cpp); `lib()` is the same library through ctypes.
 """
 from __future__ import annotations
 
@@ -87,17 +88,27 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def _bind():
+    """The extension that reads the tensors and makes the calls.  Raises if it has not been built."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _rsdbind
+        except ImportError as e:
+            raise RsdError("_rsdbind.so is missing or does not load (%s): build it with "
+                           "`python -m paper_2402_14160_b200.build` (there is no fallback path)" % e)
+        _rsdbind.bind(LIB_PATH, RsdError)
+        _native = _rsdbind
+    return _native
+
+
 def _check(code: int):
     if code != 0:
         raise RsdError("librsd error %d: %s" % (code, lib().rsd_last_error().decode()))
-
-
-def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
-
-
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else t.data_ptr()
 
 
 def rows_of(t: torch.Tensor, is_logprob: bool = False, temperature: float = 1.0) -> RsdRows:
@@ -125,25 +136,16 @@ def _new(shape, dtype, device):
     return torch.empty(shape, dtype=dtype, device=device)
 
 
-def _host_i32(values: Sequence[int]):
-    arr = (C.c_int32 * len(values))(*[int(v) for v in values])
-    return arr
-
-
 def rsd_filter_rows(rows: torch.Tensor, top_k: int = 0, top_p: float = 1.0, *, temperature: float = 1.0,
                     out: Optional[dict] = None):
     """rows [B, R, V] -> dict(rows [B, R, V] with -inf at the entries that top-k / nucleus filtering removes, kept [B, R],
     status [B]).  Pass the result to the drafting and verification calls in place of the rows, with the same temperature."""
-    B, R, V = rows.shape
-    dev = rows.device
     if out is None:
+        B, R, V = rows.shape
+        dev = rows.device
         out = dict(rows=_new((B, R, V), rows.dtype, dev), kept=_new((B, R), torch.int32, dev),
                    status=_new((B,), torch.int32, dev))
-    if not out["rows"].is_contiguous() or out["rows"].dtype != rows.dtype:
-        raise RsdError("out rows must be contiguous and of the rows' dtype")
-    r = rows_of(rows, False, temperature)
-    _check(lib().rsd_filter_rows(C.byref(r), B, R, V, int(top_k), float(top_p), _ptr(out["rows"]), _ptr(out["kept"]),
-                                 _ptr(out["status"]), _stream()))
+    (_native or _bind()).filter_rows(rows, temperature, top_k, top_p, out["rows"], out["kept"], out["status"])
     return out
 
 
@@ -156,22 +158,16 @@ def rsd_gumbel_topk_draft(draft: torch.Tensor, k_per_row: Sequence[int], rng_nod
 
     With child_base [R] and node_token [B, N+1] (int32) the picks also land in the tree's per-node token array.
     """
-    B, R, V = draft.shape
     max_k = int(max_k or max(k_per_row))
-    dev = draft.device
     if out is None:
+        B, R, V = draft.shape
+        dev = draft.device
         out = dict(token=_new((B, R, max_k), torch.int32, dev),
                    status=_new((B,), torch.int32, dev),
                    perturbed=_new((B, R, max_k), torch.float32, dev) if want_values else None,
                    logprob=_new((B, R, max_k), torch.float32, dev) if want_values else None)
-    rows = rows_of(draft, is_logprob, temperature)
-    if node_token is not None and (node_token.dtype != torch.int32 or not node_token.is_contiguous()):
-        raise RsdError("node_token must be contiguous int32")
-    _check(lib().rsd_gumbel_topk_draft(C.byref(rows), B, R, V, _host_i32(k_per_row), _host_i32(rng_node), max_k,
-                                       seed, step, seq_base, _ptr(out["token"]), _ptr(out.get("perturbed")),
-                                       _ptr(out.get("logprob")), None if child_base is None else _host_i32(child_base),
-                                       _ptr(node_token), 0 if node_token is None else node_token.shape[1],
-                                       _ptr(out["status"]), _stream()))
+    (_native or _bind()).gumbel_topk_draft(draft, is_logprob, temperature, k_per_row, rng_node, max_k, seed, step, seq_base, out["token"],
+                                           out.get("perturbed"), out.get("logprob"), child_base, node_token, out["status"])
     return out
 
 
@@ -194,25 +190,21 @@ def rsd_sbs_step(draft_level: torch.Tensor, W: int, first_parent_node: int, sum_
     out["token"] / out["parent"] may be [B, W] views into wider [B, N+1] tree arrays (row stride kept); parent_base
     is added to every parent index.
     """
-    B, n_par, V = draft_level.shape
-    dev = draft_level.device
-    need = rsd_sbs_workspace_bytes(B, n_par, W)
-    if workspace is None:
-        workspace = _new((need,), torch.uint8, dev)
-    if out is None:
-        out = dict(token=_new((B, W), torch.int32, dev),
-                   parent=_new((B, W), torch.int32, dev),
-                   sum_logprob=_new((B, W), torch.float32, dev),
-                   trunc_gumbel=_new((B, W), torch.float32, dev),
-                   count=_new((B,), torch.int32, dev),
-                   status=_new((B,), torch.int32, dev))
-    rows = rows_of(draft_level, is_logprob, temperature)
-    if out["token"].stride(0) != out["parent"].stride(0) or out["token"].stride(1) != 1 or out["parent"].stride(1) != 1:
-        raise RsdError("out token/parent must share a row stride and be dense along the picks")
-    _check(lib().rsd_sbs_step(C.byref(rows), B, n_par, V, W, first_parent_node, _ptr(sum_logprob_in),
-                              _ptr(trunc_gumbel_in), seed, step, seq_base, _ptr(out["token"]), _ptr(out["parent"]),
-                              out["token"].stride(0), parent_base, _ptr(out["sum_logprob"]), _ptr(out["trunc_gumbel"]), _ptr(out["count"]),
-                              _ptr(out["status"]), _ptr(workspace), workspace.numel(), _stream()))
+    if workspace is None or out is None:
+        B, n_par, V = draft_level.shape
+        dev = draft_level.device
+        if workspace is None:
+            workspace = _new((rsd_sbs_workspace_bytes(B, n_par, W),), torch.uint8, dev)
+        if out is None:
+            out = dict(token=_new((B, W), torch.int32, dev),
+                       parent=_new((B, W), torch.int32, dev),
+                       sum_logprob=_new((B, W), torch.float32, dev),
+                       trunc_gumbel=_new((B, W), torch.float32, dev),
+                       count=_new((B,), torch.int32, dev),
+                       status=_new((B,), torch.int32, dev))
+    (_native or _bind()).sbs_step(draft_level, is_logprob, temperature, W, first_parent_node, sum_logprob_in, trunc_gumbel_in, seed, step, seq_base,
+                                  out["token"], out["parent"], parent_base, out["sum_logprob"], out["trunc_gumbel"], out["count"],
+                                  out["status"], workspace)
     return out
 
 
@@ -226,24 +218,18 @@ def rsd_sbs_draft_tree(draft: torch.Tensor, W: int, L: int, seed: int, step: int
     """draft [B, 1 + (L - 1) W, V]: every level of one Stochastic Beam Search tree in two launches.  Fills
     node_token / node_parent [B, >= 1 + L W] (the tree arrays rsd_verify_tree reads) and returns
     dict(sum_logprob, trunc_gumbel [B, W] of the last level, count [L, B], status [B])."""
-    B, P, V = draft.shape
-    dev = draft.device
-    if P != 1 + (L - 1) * W:
-        raise RsdError("draft must hold 1 + (L - 1) W = %d rows per sequence, got %d" % (1 + (L - 1) * W, P))
-    if node_token.stride(0) != node_parent.stride(0) or node_token.stride(1) != 1 or node_parent.stride(1) != 1:
-        raise RsdError("node_token / node_parent must share a row stride and be dense along the nodes")
-    if workspace is None:
-        workspace = _new((rsd_sbs_tree_workspace_bytes(B, W, L),), torch.uint8, dev)
-    if out is None:
-        out = dict(sum_logprob=_new((B, W), torch.float32, dev),
-                   trunc_gumbel=_new((B, W), torch.float32, dev),
-                   count=_new((L, B), torch.int32, dev),
-                   status=_new((B,), torch.int32, dev))
-    rows = rows_of(draft, is_logprob, temperature)
-    _check(lib().rsd_sbs_draft_tree(C.byref(rows), B, V, W, L, seed, step, seq_base, _ptr(node_token),
-                                    _ptr(node_parent), node_token.stride(0), _ptr(out["sum_logprob"]),
-                                    _ptr(out["trunc_gumbel"]), _ptr(out["count"]), _ptr(out["status"]),
-                                    _ptr(workspace), workspace.numel(), _stream()))
+    if workspace is None or out is None:
+        B, P, V = draft.shape
+        dev = draft.device
+        if workspace is None:
+            workspace = _new((rsd_sbs_tree_workspace_bytes(B, W, L),), torch.uint8, dev)
+        if out is None:
+            out = dict(sum_logprob=_new((B, W), torch.float32, dev),
+                       trunc_gumbel=_new((B, W), torch.float32, dev),
+                       count=_new((L, B), torch.int32, dev),
+                       status=_new((B,), torch.int32, dev))
+    (_native or _bind()).sbs_draft_tree(draft, is_logprob, temperature, W, L, seed, step, seq_base, node_token, node_parent, out["sum_logprob"],
+                                        out["trunc_gumbel"], out["count"], out["status"], workspace)
     return out
 
 
@@ -260,15 +246,9 @@ def rsd_sbs_step_static(draft_level: torch.Tensor, W: int, first_parent_node: in
     this wrapper allocates nothing either.  Raises RsdError when B * n_par * W is too large for the built-in
     scratch.  Calls that overlap on one GPU share that scratch and race.
     """
-    B, n_par, V = draft_level.shape
-    rows = rows_of(draft_level, is_logprob, temperature)
-    if out["token"].stride(0) != out["parent"].stride(0) or out["token"].stride(1) != 1 or out["parent"].stride(1) != 1:
-        raise RsdError("out token/parent must share a row stride and be dense along the picks")
-    _check(lib().rsd_sbs_step_static(C.byref(rows), B, n_par, V, W, first_parent_node, _ptr(sum_logprob_in),
-                                     _ptr(trunc_gumbel_in), seed, step, seq_base, _ptr(out["token"]),
-                                     _ptr(out["parent"]), out["token"].stride(0), parent_base,
-                                     _ptr(out["sum_logprob"]), _ptr(out["trunc_gumbel"]), _ptr(out["count"]),
-                                     _ptr(out["status"]), _stream()))
+    (_native or _bind()).sbs_step(draft_level, is_logprob, temperature, W, first_parent_node, sum_logprob_in, trunc_gumbel_in, seed, step, seq_base,
+                                  out["token"], out["parent"], parent_base, out["sum_logprob"], out["trunc_gumbel"], out["count"],
+                                  out["status"], None)
     return out
 
 
@@ -279,31 +259,19 @@ def rsd_verify_tree(draft: torch.Tensor, target: torch.Tensor, parent: torch.Ten
     """draft [B, P, V], target [B, N+1, V], parent [N+1] or [B, N+1] int32, token [B, N+1] int32.
     rule = RULE_RRS with final_sampler = FINAL_INVERSE_CDF calls rsd_verify_tree; anything else calls
     rsd_verify_tree_rule."""
-    B, _, V = target.shape
-    dev = target.device
-    n_nodes = token.shape[1]
     L = int(num_levels)
-    if parent.dtype != torch.int32 or token.dtype != torch.int32:
-        raise RsdError("parent and token must be int32")
-    if not (parent.is_contiguous() and token.is_contiguous()):
-        raise RsdError("parent and token must be contiguous")
     if out is None:
+        B, dev = target.shape[0], target.device
         out = dict(accepted_len=_new((B,), torch.int32, dev),
                    accepted_node=_new((B, max(L, 1)), torch.int32, dev)[:, :L],
                    accepted_token=_new((B, max(L, 1)), torch.int32, dev)[:, :L],
                    last_token=_new((B,), torch.int32, dev),
                    stop_reason=_new((B,), torch.int32, dev),
                    status=_new((B,), torch.int32, dev))
-        out["theta"] = _new((B, n_nodes), torch.float32, dev) if want_theta else None
-    tree = RsdTree(L, n_nodes, parent.data_ptr(), token.data_ptr(), 1 if parent.dim() == 1 else 0)
-    d, t = rows_of(draft, False, draft_temperature), rows_of(target, False, target_temperature)
-    outs = (_ptr(out["accepted_len"]), _ptr(out["accepted_node"]), _ptr(out["accepted_token"]),
-            _ptr(out["last_token"]), _ptr(out["stop_reason"]), _ptr(out.get("theta")), _ptr(out["status"]), _stream())
-    if rule == RULE_RRS and final_sampler == FINAL_INVERSE_CDF and not _force_rule_entry:
-        _check(lib().rsd_verify_tree(C.byref(d), C.byref(t), C.byref(tree), B, V, seed, step, seq_base, *outs))
-    else:
-        _check(lib().rsd_verify_tree_rule(C.byref(d), C.byref(t), C.byref(tree), B, V, int(rule), float(gamma),
-                                          int(final_sampler), seed, step, seq_base, *outs))
+        out["theta"] = _new((B, token.shape[1]), torch.float32, dev) if want_theta else None
+    (_native or _bind()).verify_tree(draft, draft_temperature, target, target_temperature, parent, token, L, seed, step, seq_base, rule, gamma,
+                                     final_sampler, _force_rule_entry, out["accepted_len"], out["accepted_node"], out["accepted_token"],
+                                     out["last_token"], out["stop_reason"], out.get("theta"), out["status"])
     return out
 
 
@@ -325,11 +293,6 @@ def rsd_resample_residual(draft_row: Optional[torch.Tensor], target_row: torch.T
     token = _new((B,), torch.int32, dev)
     status = _new((B,), torch.int32, dev)
     residual = _new((B, V), torch.float32, dev) if want_residual else None
-    t = rows_of(target_row, False, target_temperature)
-    d = rows_of(draft_row, False, draft_temperature) if draft_row is not None else t
-    max_k = 0 if rejected is None else rejected.shape[1]
-    if rejected is not None and (rejected.dtype != torch.int32 or not rejected.is_contiguous()):
-        raise RsdError("rejected must be contiguous int32")
-    _check(lib().rsd_resample_residual(C.byref(d), C.byref(t), B, V, _ptr(rejected), max_k, _ptr(rng_node), seed,
-                                       step, seq_base, _ptr(token), _ptr(residual), _ptr(status), _stream()))
+    (_native or _bind()).resample_residual(draft_row, draft_temperature, target_row, target_temperature, rejected, rng_node, seed, step, seq_base,
+                                           token, residual, status)
     return dict(token=token, residual=residual, status=status)
