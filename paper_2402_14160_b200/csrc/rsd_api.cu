@@ -55,6 +55,16 @@ void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs&
     g_scan_before = g_scan_after = nullptr;
 }
 
+// status[0..B) = 0 ahead of a kernel that ORs bits into it, which does not wait for this one until it touches status (a memset
+// in its place kept that kernel back by about 3 us).  Launched in plain stream order: the kernel behind it may read
+// whatever the stream's earlier work wrote.
+__global__ void clear_status_kernel(int32_t* status, int B) {
+    rsd::grid_started();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < B) status[i] = 0;
+}
+void clear_status(int32_t* status, int B, cudaStream_t s) { clear_status_kernel<<<(B + 255) / 256, 256, 0, s>>>(status, B); }
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -99,7 +109,7 @@ int rsd_gumbel_topk_draft(const rsd_rows* draft, int B, int R, int V, const int3
     }
     if (B == 0) return RSD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(status, 0, sizeof(int32_t) * (size_t)B, s) != cudaSuccess) return check_launch("memset(status)");
+    clear_status(status, B, s);
     a.data = draft->data; a.seq_stride = draft->seq_stride; a.row_stride = draft->row_stride;
     a.R = R; a.V = V; a.max_k = max_k;
     a.seed_lo = (uint32_t)seed; a.seed_hi = (uint32_t)(seed >> 32); a.step = step; a.seq_base = seq_base;
@@ -158,6 +168,7 @@ int rsd_sbs_step(const rsd_rows* draft_level, int B, int n_par, int V, int W, in
     a.subtract_lse = 0;
     a.out_token = fin_token; a.out_perturbed = fin_pert; a.out_value = fin_value; a.out_lse = fin_lse;
     a.status = status; a.row_status = row_status;   // status[b] is written by the epilogue
+    a.wait_first = 1;
     a.temp = temperature_of(draft_level); a.inv_temp = 1.0f / a.temp; a.raw_values = 1;
     launch_scan(draft_level, !rows_are_logprob(draft_level), B * n_par, a, s);
     if (int e = check_launch("rsd_sbs_step(scan)")) return e;
@@ -173,7 +184,7 @@ int rsd_sbs_step(const rsd_rows* draft_level, int B, int n_par, int V, int W, in
     e.sum_out = sum_logprob_out; e.gamma_out = trunc_gumbel_out;
     e.out_count = out_count; e.status = status;
     const size_t smem = rsd::sbs_level_scratch_bytes(n_par, W);
-    rsd::sbs_epilogue_kernel<<<B, rsd::kEpilogueThreads, smem, s>>>(e);
+    launch_overlapped(rsd::sbs_epilogue_kernel, (unsigned)B, rsd::kEpilogueThreads, smem, s, 0, e);
     return check_launch("rsd_sbs_step(epilogue)");
 }
 
@@ -196,7 +207,7 @@ int rsd_filter_rows(const rsd_rows* rows, int B, int R, int V, int top_k, float 
                     (kSharedPerBlock - sizeof(rsd::FilterSmem) - 272) / elem);
     if (B == 0) return RSD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(status, 0, sizeof(int32_t) * (size_t)B, s) != cudaSuccess) return check_launch("memset(status)");
+    clear_status(status, B, s);
     rsd::FilterArgs a;
     a.data = rows->data; a.out = out_rows; a.seq_stride = rows->seq_stride; a.row_stride = rows->row_stride;
     a.R = R; a.V = V; a.top_k = top_k; a.top_p = top_p;
@@ -216,7 +227,7 @@ int rsd_filter_rows(const rsd_rows* rows, int B, int R, int V, int top_k, float 
             return check_launch("cudaFuncSetAttribute");
         if (dev >= 0 && dev < 64) raised[which][dev].store(true, std::memory_order_release);
     }
-    kernel<<<B * R, wide ? 1024 : 512, smem, s>>>(a);
+    launch_overlapped(kernel, (unsigned)(B * R), wide ? 1024 : 512, smem, s, 0, a);
     return check_launch("rsd_filter_rows");
 }
 
@@ -271,6 +282,7 @@ int rsd_sbs_draft_tree(const rsd_rows* draft, int B, int V, int W, int L, uint64
     a.subtract_lse = 0;
     a.out_token = fin_token; a.out_perturbed = fin_pert; a.out_value = fin_value; a.out_lse = fin_lse;
     a.status = status; a.row_status = row_status;
+    a.wait_first = 1;
     a.temp = temperature_of(draft); a.inv_temp = 1.0f / a.temp; a.raw_values = 1;
     launch_scan(draft, !rows_are_logprob(draft), (int)(B * P), a, s);
     if (int e = check_launch("rsd_sbs_draft_tree(scan)")) return e;
@@ -289,7 +301,7 @@ int rsd_sbs_draft_tree(const rsd_rows* draft, int B, int V, int W, int L, uint64
     // the finalists of a sequence are staged in shared memory when they fit well inside the default 48 KB
     c.staged = rsd::sbs_chain_smem_bytes(W, (int)P, true) <= 40 * 1024 ? 1 : 0;
     const size_t smem = rsd::sbs_chain_smem_bytes(W, (int)P, c.staged != 0);
-    rsd::sbs_chain_kernel<<<B, rsd::kEpilogueThreads, smem, s>>>(c);
+    launch_overlapped(rsd::sbs_chain_kernel, (unsigned)B, rsd::kEpilogueThreads, smem, s, 0, c);
     return check_launch("rsd_sbs_draft_tree(levels)");
 }
 

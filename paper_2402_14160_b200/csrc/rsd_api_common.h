@@ -26,6 +26,27 @@ inline int check_launch(const char* what) {
     return RSD_OK;
 }
 
+// Launch that may overlap the end of the stream's previous kernel; the kernel orders itself with rsd::grid_wait().  (An error
+// stays pending for check_launch().)
+template <typename... KArgs, typename... Args>
+inline void launch_overlapped(void (*kernel)(KArgs...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, int cluster, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 0 ? 2 : 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 inline int check_rows(const char* name, const rsd_rows* r, int V, bool need_row_stride) {
     if (!r || !r->data) return fail(RSD_ERR_INVALID_ARG, "%s: null rows", name);
     if (r->dtype != RSD_F32 && r->dtype != RSD_BF16) return fail(RSD_ERR_UNSUPPORTED, "%s: unknown dtype %d", name, r->dtype);

@@ -36,7 +36,7 @@ void launch_ring_walk(const rsd::VerifyArgs& a, int B, cudaStream_t s) {
             return;
         if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
     }
-    verify_tree_ring_kernel<T><<<B, kThreads, kRingBytes, s>>>(a);
+    launch_overlapped(verify_tree_ring_kernel<T>, (unsigned)B, kThreads, kRingBytes, s, 0, a);
 }
 
 // The smallest cluster that holds a row, with one tile per warp (three blocks an SM) as long as all sequences are

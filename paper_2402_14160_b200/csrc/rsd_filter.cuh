@@ -695,7 +695,10 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     }
     __syncthreads();
     if (sm.copy_gave_up) {                                        // the copy never landed: report, write nothing
-        if (tid == 0) atomicOr(&a.status[b], 32);                 // RSD_ST_TIMEOUT
+        if (tid == 0) {
+            grid_wait();                                          // (status[] has been cleared)
+            atomicOr(&a.status[b], 32);                           // RSD_ST_TIMEOUT
+        }
         return;
     }
     if (sm.needs_cleaning) {
@@ -766,6 +769,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
         count_kept = a.kept != nullptr;
     }
 
+    grid_started();
     // ---- the row with -inf at the filtered entries ------------------------------------------------------------------------------
     {
         auto keeps = [&](int i, uint32_t h) {
@@ -817,6 +821,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     }
     if (tid == 0) {
         if (a.kept) a.kept[(int64_t)b * a.R + r] = kept;
+        grid_wait();                                              // (status[] has been cleared)
         if (sm.nan_flag) atomicOr(&a.status[b], 1);               // RSD_ST_NAN_INPUT
     }
 }

@@ -48,6 +48,8 @@ struct ScanArgs {
                           // the epilogue assembles status[b], and a row with fewer than k picks is not an event)
     int32_t* node_token;  // [B][node_stride] or null: pick j of row r also goes to node child_base[r] + j
     int node_stride;
+    int wait_first;       // 1: the stream's previous kernel may still run (it may have written the rows); 0: it is the one that
+                          // clears status[], which is not touched before the end
     uint32_t rk0[10], rk1[10];  // Philox round keys: seed_lo + r * 0x9E3779B9, seed_hi + r * 0xBB67AE85
     uint8_t k_row[kMaxRows];
     int32_t node_row[kMaxRows];
@@ -480,6 +482,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     const int n_iter = (n_groups + kScanThreads - 1) / kScanThreads;
     const PhiloxRow pr = philox_row_setup(a, (node & 0x0FFFFFFFu) | (kTagGumbelCoarse << 28), key.seq, key.step);
 
+    if (a.wait_first) grid_wait();
     if (tid == 0) { n_cand = 0; n_surv = 0; nan_flag = 0; n_task = 0; n_fin = 0; }
     if (tid < 32) bin_max[tid] = float_to_ordered(kNegInf);
     if (tid < 4 && n_groups + tid < ((n_groups + 3) & ~3)) ub[n_groups + tid] = kNegInf;   // padding of the bounds
@@ -829,6 +832,8 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
 
     const float lse = NEED_LSE ? lse_sh : 0.0f;   // written before the barriers that end the stages above
 
+    grid_started();
+
     // ---- rank the survivors, write the picks ----------------------------------------------------------------------------
     const int total = ns < k ? ns : k;
     const int64_t o = ((int64_t)b * a.R + r) * a.max_k;
@@ -856,8 +861,12 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
         int st = 0;
         if (nan_flag) st |= 1;       // RSD_ST_NAN_INPUT
         if (total < k) st |= 2;      // RSD_ST_FEWER_THAN_K
-        if (a.row_status) a.row_status[(int64_t)b * a.R + r] = st & 1;
-        else if (st) atomicOr(&a.status[b], st);
+        if (a.row_status) {
+            a.row_status[(int64_t)b * a.R + r] = st & 1;
+        } else {
+            grid_wait();   // (status[] has been cleared)
+            if (st) atomicOr(&a.status[b], st);
+        }
     }
 }
 
@@ -1053,7 +1062,9 @@ __device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, cons
 
 static __global__ void __launch_bounds__(kEpilogueThreads) sbs_epilogue_kernel(const SbsEpilogueArgs a) {
     extern __shared__ double sm_d[];
+    grid_wait();   // the scan's finalists
     sbs_epilogue_body(a, blockIdx.x, sm_d);
+    grid_started();
 }
 
 // All L levels of one Stochastic Beam Search tree (Algorithm 8's level loop around Algorithm 9) for rows that exist
@@ -1086,6 +1097,7 @@ __host__ __device__ inline size_t sbs_chain_smem_bytes(int W, int P, bool staged
 static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(const SbsChainArgs c) {
     extern __shared__ double sm_d[];
     const int b = blockIdx.x, W = c.lvl.W, tid = threadIdx.x, F = c.P * W;
+    grid_wait();   // the scan's finalists
     float* const state = (float*)((unsigned char*)sm_d + sbs_level_scratch_bytes(W, W));   // sum[2][W], gamma[2][W]
     int32_t* const s_tok = (int32_t*)(state + 4 * W);
     float* const s_val = (float*)(s_tok + F);
@@ -1148,6 +1160,7 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(cons
         }
     }
     if (tid == 0) c.status[b] = st;
+    grid_started();
 }
 
 }  // namespace rsd

@@ -4,6 +4,7 @@
 #include <atomic>
 
 #include "../../include/rsd.h"
+#include "rsd_api_common.h"
 #include "rsd_scan.cuh"
 
 namespace rsd {
@@ -25,7 +26,7 @@ void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
             if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
         }
     }
-    kernel<<<blocks, NT, smem, s>>>(a);
+    rsd_host::launch_overlapped(kernel, (unsigned)blocks, NT, smem, s, 0, a);
 }
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP>
 void launch_scan_temp(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {

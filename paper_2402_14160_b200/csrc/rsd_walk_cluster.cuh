@@ -1038,8 +1038,8 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         sm.nan_seen = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __syncwarp();
     cluster_arrive();
+    grid_wait();   // the tree, and whatever else the stream has on the way
     if (threadIdx.x < WARPS * 32) {
         WorkRows rows;
         rows.q = row_ptr<T>(a.target, b, 0);
@@ -1058,6 +1058,7 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         if (EXTRA && ca.resample) control.resample();
         else control.walk();
     }
+    grid_started();
     cluster_arrive();   // nothing is on its way to a block that has left
     cluster_wait();
 }

@@ -1,5 +1,6 @@
 // Launch of the cluster walk for one element type.
 #pragma once
+#include "rsd_api_common.h"
 #include "rsd_walk_cluster.cuh"
 
 namespace rsd {
@@ -7,18 +8,7 @@ namespace walk_cluster {
 
 template <typename T, int NT, int WARPS, bool EXTRA>
 void launch_shape(const ClusterArgs& a, int B, int C, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(B * C));
-    cfg.blockDim = dim3((WARPS + 1) * 32);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, walk_cluster_kernel<T, NT, WARPS, EXTRA>, a);   // (an error stays pending for check_launch())
+    rsd_host::launch_overlapped(walk_cluster_kernel<T, NT, WARPS, EXTRA>, (unsigned)(B * C), (WARPS + 1) * 32, 0, s, C, a);
 }
 template <typename T, bool EXTRA>
 void launch_extra(const ClusterArgs& a, int B, const Shape& c, cudaStream_t s) {

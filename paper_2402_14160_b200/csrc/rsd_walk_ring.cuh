@@ -500,6 +500,7 @@ __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const Ver
         sm.nan_seen = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    grid_wait();   // the tree
     for (int i = tid; i < a.L; i += kThreads) {
         a.accepted_node[(int64_t)b * a.L + i] = -1;
         a.accepted_token[(int64_t)b * a.L + i] = -1;
@@ -841,6 +842,7 @@ __global__ void __launch_bounds__(kThreads, 3) verify_tree_ring_kernel(const Ver
             last = pick_in_tile(w, t);
         }
     }
+    grid_started();
     if (lane == 0) {
         a.accepted_len[b] = len;
         a.last_token[b] = last;
