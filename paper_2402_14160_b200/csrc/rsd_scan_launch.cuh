@@ -26,7 +26,8 @@ void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
             if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
         }
     }
-    rsd_host::launch_overlapped(kernel, (unsigned)blocks, NT, smem, s, 0, a);
+    if (NT == 128 && a.wait_first) kernel<<<blocks, NT, smem, s>>>(a);
+    else rsd_host::launch_overlapped(kernel, (unsigned)blocks, NT, smem, s, 0, a);
 }
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP>
 void launch_scan_temp(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {
