@@ -30,6 +30,10 @@ using walk_ring::warp_sum_f32;
 constexpr int kClasses = 8;              // summation classes: tiles of equal index modulo 8
 constexpr int kMaxListed = 64;           // rejected tokens remembered per node
 
+// What a kernel is compiled for: recursive rejection sampling with the inverse-CDF last draw; the other rules and the
+// Gumbel-Top-1 draw; the stand-alone residual draw.  (One kernel for the last two spilled four times as many registers.)
+enum { kPlainWalk = 0, kRuleWalk = 1, kResample = 2 };
+
 // Cmd::flags: what a pass does (low four bits) and options
 enum {
     kEnd = 0,
@@ -295,8 +299,8 @@ __device__ __forceinline__ void top1_pass(Smem<WARPS, NT>& sm, const Place& pl, 
 }
 
 // The working warps: the passes they are told to run.  The root's rows are asked for before the first command is there.
-// EXTRA: also the passes that only the baseline rules, the Gumbel-Top-1 draw and the stand-alone residual draw need.
-template <typename T, int NT, int WARPS, bool EXTRA>
+// MODE: which of the rarer passes exist.
+template <typename T, int NT, int WARPS, int MODE>
 __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const WorkRows& rows) {
     constexpr int kAll = (WARPS + 1) * 32, kWorkers = WARPS * 32;
     constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
@@ -377,7 +381,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                 }
             }
         } else if (kind == kResidualPass) {
-            if (EXTRA && (flags & kFreeze)) {
+            if (MODE == kResample && (flags & kFreeze)) {
                 const int x = sm.freeze_x;
                 int l_, j_;
                 walk_ring::piece_of<T>(x % kTileElems, l_, j_);
@@ -414,7 +418,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                 for (int j = 0; j < 16; ++j) w[j] = ((gone >> j) & 1u) ? 0.0f : p[k][j];
                 s[k] = tree_sum16(w);
             }
-        } else if (EXTRA && (kind == kOverlapPass || kind == kSeqPass)) {
+        } else if (MODE == kRuleWalk && (kind == kOverlapPass || kind == kSeqPass)) {
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
                 float w[16];
@@ -427,14 +431,14 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
             for (int k = 0; k < NT; ++k)
                 if (tile0 + tile_step * k == node) {
                     float w[16];
-                    mode_weights<EXTRA>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, EXTRA ? sm.c_seq : 0.0f, w);
+                    mode_weights<MODE == kRuleWalk>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, MODE == kRuleWalk ? sm.c_seq : 0.0f, w);
 #pragma unroll
                     for (int i = 0; i < kRuns; ++i)
 #pragma unroll
                         for (int j = 0; j < kPer; ++j) sm.tile_w[(i * 32 + lane) * kPer + j] = w[i * kPer + j];
                 }
             dump_sync<kAll>();
-        } else if (EXTRA && kind == kWrite) {
+        } else if (MODE == kResample && kind == kWrite) {
             dump_sync<kAll>();                  // everyone has read the command
             const double inv = sm.inv_total;
             float* out = rows.out_residual;
@@ -444,7 +448,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                 const int tile = tile0 + tile_step * k;
                 if (tile >= n_tiles) continue;
                 float w[16];
-                mode_weights<EXTRA>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, 0.0f, w);
+                mode_weights<false>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, 0.0f, w);
 #pragma unroll
                 for (int i = 0; i < 16; i += 4) {
                     const int x = tile * kTileElems + ((i / kPer) * 32 + lane) * kPer + i % kPer;
@@ -460,7 +464,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                     }
                 }
             }
-        } else if (EXTRA && kind == kTop1) {
+        } else if (MODE == kRuleWalk && kind == kTop1) {
             top1_pass<T, NT, WARPS>(sm, pl, rows.key, (uint32_t)node, flags, a_hi, a_lo, q, p);
         } else {
             return;                             // kEnd
@@ -521,7 +525,7 @@ __device__ __forceinline__ double class_tree(double v) {
 }
 
 // The control warp: the walk itself, the same in every block of the cluster.
-template <typename T, int NT, int WARPS, bool EXTRA>
+template <typename T, int NT, int WARPS, int MODE>
 struct Control {
     static constexpr int kAll = (WARPS + 1) * 32;
     Smem<WARPS, NT>& sm;
@@ -726,7 +730,7 @@ struct Control {
         const int32_t* par = a.parent + (a.shared_topology ? 0 : (int64_t)b * a.num_nodes);
         const int32_t* tok = a.token + (int64_t)b * a.num_nodes;
         const bool cached = a.num_nodes <= kMaxCachedNodes;
-        const int rule = EXTRA ? a.rule : 0;
+        const int rule = (MODE == kRuleWalk) ? a.rule : 0;
         const int64_t out0 = (int64_t)b * a.L;
         if (cached) {
 #pragma unroll 4
@@ -797,14 +801,15 @@ struct Control {
             inv_Sp = 1.0 / Sp;
             ratio = Sq * inv_Sp;
             const double sp_over_sq = Sp * inv_Sq;
-            double qpd, px_row, qxd;                  // q(x) / p(x), p(x), q(x)
+            double qpd;                               // q(x) / p(x)
+            unsigned none_left, repeats;              // children that the draft cannot produce any more; those among them that repeat
             auto weigh_children = [&] {
                 // Precise weights: the quotient of the very weights that the sums are made of, as long as they are in range, so
                 // that their errors cancel where the token carries much of the residual.
                 if (precise && qh > 1e-30f && ph > 1e-30f) qpd = (double)qh / (double)ph * sp_over_sq;
                 else qpd = qp_rows.times(sp_over_sq);
-                px_row = (double)ph * inv_Sp;
-                qxd = (double)qh * inv_Sq;
+                none_left = __ballot_sync(0xFFFFFFFFu, repeated || p_none);
+                repeats = __ballot_sync(0xFFFFFFFFu, repeated);
             };
             if (mq != 0.0f || mp != 0.0f) child_weights();   // (the references have moved)
             weigh_children();
@@ -812,38 +817,39 @@ struct Control {
             double one_mP = 1.0, one_mP_err = 0.0, inv_1mP = 1.0;
             int j = 0, accepted_lane = -1;            // j: lane of the child under test
             for (;;) {
-                // Eq. 3 in closed form: accept iff U < min(1, (q/p - A)+ (1 - P) / Z); a child the draft cannot produce any more
-                // is taken iff it has residual mass (RSD_ST_ZERO_DRAFT_PROB).  Every lane tests its own child, lane j's counts.
-                const bool no_draft = repeated || p_none;
-                double g;
-                bool take;
-                if (EXTRA && rule == 2) {             // K-SEQ: min(1, q / (gamma p))
-                    g = no_draft ? (qxd > 0.0 ? 1.0 : 0.0) : qpd / (double)a.gamma;
+                // Eq. 3 in closed form: accept iff U < min(1, (q/p - A)+ (1 - P) / Z).  Every lane tests its own child, lane j's
+                // counts.  A child the draft cannot produce any more is taken iff it has residual mass (RSD_ST_ZERO_DRAFT_PROB).
+                double g = fmax(qpd - A, 0.0) * one_mP;
+                bool take = Ud * Z < g;
+                if ((MODE == kRuleWalk) && rule == 2) {   // K-SEQ: min(1, q / (gamma p))
+                    g = qpd / (double)a.gamma;
                     take = Ud < g;
-                } else if (!no_draft) {
-                    g = fmax(qpd - A, 0.0) * one_mP;
-                    take = Ud * Z < g;
-                } else {
-                    take = fmax(qxd - A * px_row, 0.0) > 0.0;
-                    g = take ? Z : 0.0;
                 }
-                const unsigned taken = __ballot_sync(0xFFFFFFFFu, take), none_left = __ballot_sync(0xFFFFFFFFu, no_draft);
-                if ((none_left >> j) & 1u) status |= 8;
+                if ((none_left >> j) & 1u) {
+                    status |= 8;
+                    const double qx = (double)qh * inv_Sq;
+                    const bool any = (MODE == kRuleWalk) && rule == 2 ? qx > 0.0 : fmax(qx - A * ((double)ph * inv_Sp), 0.0) > 0.0;
+                    if (lane == j) {
+                        take = any;
+                        g = any ? ((MODE == kRuleWalk) && rule == 2 ? 1.0 : Z) : 0.0;
+                    }
+                }
+                const unsigned taken = __ballot_sync(0xFFFFFFFFu, take);
                 if (a.dbg_theta && pl.rank == 0 && lane == j)
-                    a.dbg_theta[(int64_t)b * a.num_nodes + child_node] = (float)fmin(1.0, (EXTRA && rule == 2) ? g : g / Z);
+                    a.dbg_theta[(int64_t)b * a.num_nodes + child_node] = (float)fmin(1.0, ((MODE == kRuleWalk) && rule == 2) ? g : g / Z);
                 if ((taken >> j) & 1u) { accepted_lane = j; break; }
                 // rejected.  Eqs. 1-2 in closed form: A_{j+1} = A_j + Z_j / (1 - P_j), Z_{j+1} = sum (q - A_{j+1} p)+
                 const bool more_here = j < 31 && ((kids >> (j + 1)) & 1u);
                 const int more_nodes = (j == 31 && kids == 0xFFFFFFFFu) ? children(cur, __shfl_sync(0xFFFFFFFFu, child_node, 31), par, tok, cached) : -1;
                 const bool more = more_here || __any_sync(0xFFFFFFFFu, more_nodes >= 0);
                 const double A_old = A;
-                if (!(EXTRA && rule == 2)) {
+                if (!((MODE == kRuleWalk) && rule == 2)) {
                     set_a(fma(Z, inv_1mP, A));
                     issue(kResidualPass | (more ? 0 : kStoreTiles), 0, kClasses + (more ? 0 : pl.n_tiles));
                 }
                 const int x = __shfl_sync(0xFFFFFFFFu, child_x, j);
-                const bool rep = (__ballot_sync(0xFFFFFFFFu, repeated) >> j) & 1u;
-                const double px = (EXTRA && rule != 0) ? 0.0 : __shfl_sync(0xFFFFFFFFu, no_draft ? 0.0 : px_row, j);
+                const bool rep = (repeats >> j) & 1u;
+                const double px = ((MODE == kRuleWalk) && rule != 0) || ((none_left >> j) & 1u) ? 0.0 : (double)__shfl_sync(0xFFFFFFFFu, ph, j) * inv_Sp;
                 double one_mP_new = one_mP - px, err_new = one_mP_err + 4e-7 * px;   // (px = 0 for a repeated token)
                 if (!rep && n_removed < kMaxListed) {
                     if (lane == 0) sm.gone_tok[n_removed] = x;
@@ -865,14 +871,14 @@ struct Control {
                     }
                     next_kid = children(__shfl_sync(0xFFFFFFFFu, child_node, j), 0, par, tok, cached);
                 }
-                if (!(EXTRA && rule == 2)) {
+                if (!((MODE == kRuleWalk) && rule == 2)) {
                     const double Z_new = collect() * inv_Sq;
                     if (aborted) break;
                     bool kept;
                     take_in(Z_new, A_old, kept);
                     tiles_valid = kept && !more;
                 }
-                if (!(EXTRA && rule != 0)) {
+                if (!((MODE == kRuleWalk) && rule != 0)) {
                     if (more && err_new > 2e-6 * one_mP_new && n_removed < kMaxListed) {   // (every rejected token is listed)
                         one_mP_new = rest(n_removed);
                         if (aborted) break;
@@ -906,7 +912,7 @@ struct Control {
             ++len;
         }
         int mode = with_draft && A != 0.0 ? (int)kResidual : 0;
-        if (EXTRA && !aborted && rule == 2 && with_draft) {
+        if ((MODE == kRuleWalk) && !aborted && rule == 2 && with_draft) {
             // K-SEQ after all K children were rejected: beta = sum min{p, q / gamma}, then the residual
             // (q - min{p, q / gamma} (1 - (1 - beta)^K) / beta)+
             a_hi = (float)(Sq / Sp);
@@ -923,7 +929,7 @@ struct Control {
             if (tiles_valid) mode = kSeqResidual;
             else status |= 4;                         // RSD_ST_ZERO_RESIDUAL: draw from the target row itself
         }
-        const bool top1 = EXTRA && a.final_sampler == 1;
+        const bool top1 = (MODE == kRuleWalk) && a.final_sampler == 1;
         if (!aborted && !tiles_valid && !top1) refresh_tiles(mode == kResidual);
         int last = -1;
         bool mine = pl.rank == 0;
@@ -1019,7 +1025,7 @@ struct Control {
     }
 };
 
-template <typename T, int NT, int WARPS, bool EXTRA>
+template <typename T, int NT, int WARPS, int MODE>
 __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 2) : 1) walk_cluster_kernel(const __grid_constant__ ClusterArgs ca) {
     __shared__ Smem<WARPS, NT> sm;
     const VerifyArgs& a = ca.v;
@@ -1031,7 +1037,7 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
     pl.n_local = pl.n_tiles > pl.rank ? (pl.n_tiles - pl.rank + pl.C - 1) / pl.C : 0;
     const int b = blockIdx.x / pl.C;
     // Rows off 16-byte boundaries, the baseline rules and the residual draw never take the ring walk: no bits to match.
-    const bool precise = EXTRA || ca.off_boundaries;
+    const bool precise = MODE != kPlainWalk || ca.off_boundaries;
     if (threadIdx.x == WARPS * 32) {
         mbar_init(&sm.red_bar[0], 1);
         mbar_init(&sm.red_bar[1], 1);
@@ -1048,14 +1054,14 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         rows.stride_p = a.draft.row_stride * RowIO<T>::kBytes;
         rows.kq = kLog2e * a.target.inv_temp;
         rows.kp = kLog2e * a.draft.inv_temp;
-        rows.with_draft = EXTRA && ca.resample ? ca.r.max_k > 0 : (a.L > 0 && a.num_nodes > 1);
+        rows.with_draft = MODE == kResample ? ca.r.max_k > 0 : (a.L > 0 && a.num_nodes > 1);
         rows.precise = precise;
         rows.key = RngKey{a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
-        rows.out_residual = EXTRA && ca.resample && ca.r.out_residual ? ca.r.out_residual + (int64_t)b * a.V : nullptr;
-        work<T, NT, WARPS, EXTRA>(sm, pl, rows);
+        rows.out_residual = MODE == kResample && ca.r.out_residual ? ca.r.out_residual + (int64_t)b * a.V : nullptr;
+        work<T, NT, WARPS, MODE>(sm, pl, rows);
     } else {
-        Control<T, NT, WARPS, EXTRA> control(sm, ca, pl, b, precise);
-        if (EXTRA && ca.resample) control.resample();
+        Control<T, NT, WARPS, MODE> control(sm, ca, pl, b, precise);
+        if constexpr (MODE == kResample) control.resample();
         else control.walk();
     }
     grid_started();

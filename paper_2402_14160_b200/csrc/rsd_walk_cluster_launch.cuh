@@ -6,20 +6,21 @@
 namespace rsd {
 namespace walk_cluster {
 
-template <typename T, int NT, int WARPS, bool EXTRA>
+template <typename T, int NT, int WARPS, int MODE>
 void launch_shape(const ClusterArgs& a, int B, int C, cudaStream_t s) {
-    rsd_host::launch_overlapped(walk_cluster_kernel<T, NT, WARPS, EXTRA>, (unsigned)(B * C), (WARPS + 1) * 32, 0, s, C, a);
+    rsd_host::launch_overlapped(walk_cluster_kernel<T, NT, WARPS, MODE>, (unsigned)(B * C), (WARPS + 1) * 32, 0, s, C, a);
 }
-template <typename T, bool EXTRA>
-void launch_extra(const ClusterArgs& a, int B, const Shape& c, cudaStream_t s) {
-    if (c.W == 16) launch_shape<T, 2, 16, EXTRA>(a, B, c.C, s);
-    else if (c.NT == 2) launch_shape<T, 2, 8, EXTRA>(a, B, c.C, s);
-    else launch_shape<T, 1, 8, EXTRA>(a, B, c.C, s);
+template <typename T, int MODE>
+void launch_mode(const ClusterArgs& a, int B, const Shape& c, cudaStream_t s) {
+    if (c.W == 16) launch_shape<T, 2, 16, MODE>(a, B, c.C, s);
+    else if (c.NT == 2) launch_shape<T, 2, 8, MODE>(a, B, c.C, s);
+    else launch_shape<T, 1, 8, MODE>(a, B, c.C, s);
 }
 template <typename T>
 void launch_of(const ClusterArgs& a, bool extra, int B, const Shape& c, cudaStream_t s) {
-    if (extra) launch_extra<T, true>(a, B, c, s);
-    else launch_extra<T, false>(a, B, c, s);
+    if (a.resample) launch_mode<T, kResample>(a, B, c, s);
+    else if (extra) launch_mode<T, kRuleWalk>(a, B, c, s);
+    else launch_mode<T, kPlainWalk>(a, B, c, s);
 }
 
 }  // namespace walk_cluster
