@@ -922,8 +922,16 @@ __device__ __forceinline__ double ordered_to_double(unsigned long long k) {
     return __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
 }
 
+// -ln of the exponential form of a token's Gumbel noise, in double: G(x) = -sbs_log_noise
+__device__ __forceinline__ double sbs_log_noise(const RngKey& key, uint32_t node, uint32_t x) {
+    const uint32_t word = coarse_word(key, node, x >> 4);
+    const double t_elem = ((x & 15u) != (word & 15u)) ? neg_log_uniform_f64(fine_word(key, node, x)) : 0.0;
+    return log(neg_log_group_uniform_f64(word) * 0.0625 + t_elem);
+}
+
 // One level for sequence b, by a block of kEpilogueThreads threads; sm_d: sbs_level_scratch_bytes(n_par, W) bytes.
-__device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, const int b, double* sm_d) {
+// noise: sbs_log_noise of the level's finalists, [n_par][W], or null (then it is taken here).
+__device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, const int b, double* sm_d, const double* noise = nullptr) {
     const int F = a.n_par * a.W;
     // the finalists that pass the first test are gathered in a list; entry i of the arrays below belongs to list[i]
     double* s_pert = sm_d;                   // [F] phi~
@@ -998,11 +1006,8 @@ __device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, cons
         const double sigma = a.sum_in ? (double)a.sum_in[state_off + kpar] : 0.0;
         const double lse = a.is_logprob ? 0.0 : (double)a.fin_lse[row_off + kpar];
         const uint32_t node = (uint32_t)(a.first_parent_node + kpar);
-        const uint32_t word = coarse_word(key, node, (uint32_t)x >> 4);
-        const double t_elem = (((uint32_t)x & 15u) != (word & 15u))
-                                  ? neg_log_uniform_f64(fine_word(key, node, (uint32_t)x)) : 0.0;
         const double phi = sigma + ((double)a.fin_value[fin_off + f] * a.inv_temp - lse);
-        const double pert = phi - log(neg_log_group_uniform_f64(word) * 0.0625 + t_elem);
+        const double pert = phi - (noise ? noise[f] : sbs_log_noise(key, node, (uint32_t)x));
         s_tok[i] = x;
         s_phi[i] = phi;
         s_pert[i] = pert;
@@ -1092,7 +1097,7 @@ struct SbsChainArgs {
 
 // dynamic shared memory of sbs_chain_kernel
 __host__ __device__ inline size_t sbs_chain_smem_bytes(int W, int P, bool staged) {
-    return sbs_level_scratch_bytes(W, W) + (size_t)4 * W * 4 + (staged ? (size_t)P * W * 12 + (size_t)P * 8 : 0);
+    return sbs_level_scratch_bytes(W, W) + (size_t)4 * W * 4 + (staged ? (size_t)P * W * 20 + (size_t)P * 8 + 8 : 0);
 }
 
 static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(const SbsChainArgs c) {
@@ -1105,6 +1110,7 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(cons
     float* const s_pert = s_val + F;
     float* const s_lse = s_pert + F;
     int32_t* const s_rs = (int32_t*)(s_lse + c.P);
+    double* const s_noise = (double*)(((uintptr_t)(s_rs + c.P) + 7) & ~(uintptr_t)7);
     if (c.staged) {
         const int64_t f0 = (int64_t)b * F, r0 = (int64_t)b * c.P;
         for (int i = tid; i < F; i += kEpilogueThreads) {
@@ -1115,6 +1121,13 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(cons
         for (int i = tid; i < c.P; i += kEpilogueThreads) {
             s_lse[i] = c.lvl.fin_lse[r0 + i];
             s_rs[i] = c.lvl.row_status[r0 + i];
+        }
+        // The noise of a finalist does not depend on the levels above it: taken for all of them at once, not for a dozen at a
+        // time inside the chain (three double-precision logarithms and two Philox calls, a third of a level's latency).
+        const RngKey key = {c.lvl.seed_lo, c.lvl.seed_hi, c.lvl.step, c.lvl.seq_base + (uint32_t)b};
+        for (int i = tid; i < F; i += kEpilogueThreads) {
+            const int x = s_tok[i];   // (this thread's own copy)
+            s_noise[i] = x >= 0 ? sbs_log_noise(key, (uint32_t)(i / W), (uint32_t)x) : 0.0;
         }
         __syncthreads();
     }
@@ -1152,7 +1165,7 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(cons
         a.parent_base = first;
         a.out_count = c.level_count + (int64_t)l * c.B;
         a.status = c.level_status + (int64_t)l * c.B;
-        sbs_epilogue_body(a, b, sm_d);
+        sbs_epilogue_body(a, b, sm_d, c.staged ? s_noise + first * W : nullptr);
         __syncthreads();   // the level's outputs are the next level's inputs
         if (tid == 0) st |= a.status[b];
         if (last && tid < W) {
