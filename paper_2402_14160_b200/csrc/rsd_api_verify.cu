@@ -41,8 +41,9 @@ void launch_ring_walk(const rsd::VerifyArgs& a, int B, cudaStream_t s) {
 
 // The smallest cluster that holds a row, with one tile per warp (three blocks an SM) as long as all sequences are
 // resident at once, else with two (two blocks an SM), which costs a sequence about 10 % more time and 25 % fewer SM-cycles
-// (V = 32,000, bf16: 42 against 47 us at 64 sequences, 122 against 102 us at 256).  Rows beyond 65,536 entries take
-// sixteen warps, one block an SM; beyond 131,072 no cluster holds them (C = 0).
+// (V = 32,000, bf16: 42 against 47 us at 64 sequences, 122 against 102 us at 256).  Rows of up to 8192 entries stay with one
+// tile per warp: a cluster of one block has nobody to share with (V = 8096, 492 sequences: two blocks 57 us, one 63 us).
+// Rows beyond 65,536 entries take sixteen warps, one block an SM; beyond 131,072 no cluster holds them (C = 0).
 rsd::walk_cluster::Shape cluster_shape(int B, int V) {
     auto blocks = [&](int per_block) {
         int c = 1;
@@ -51,7 +52,7 @@ rsd::walk_cluster::Shape cluster_shape(int B, int V) {
     };
     const float sms = (float)sm_count();
     int c = blocks(8 * 512);
-    if (c <= 8 && (float)B * (float)c <= 3.0f * sms) return {c, 8, 1, (float)B * (float)c / (3.0f * sms)};
+    if (c <= 2 || (c <= 8 && (float)B * (float)c <= 3.0f * sms)) return {c, 8, 1, (float)B * (float)c / (3.0f * sms)};
     c = blocks(16 * 512);
     if (c <= 8) return {c, 8, 2, (float)B * (float)c / (2.0f * sms)};
     c = blocks(32 * 512);
@@ -113,13 +114,17 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
     const bool ring = plain && aligned && (row_bytes + rsd::walk_ring::kRowChunkBytes - 1) / rsd::walk_ring::kRowChunkBytes <= 64;
     // A cluster per sequence while there are few: its passes are two to three times as short (V = 32,000 bf16: 30 -> 16 us
     // for one sequence, 94 -> 42 for 64), but it takes more SM time per walk.  The kernels with one block per sequence are
-    // ahead from about 2.5 waves of clusters on with rows on 16-byte boundaries (192 / 320 sequences: ring 104 / 116 us,
-    // cluster 79 / 119; V = 50,272: 64 / 128 sequences 59 / 61 against 49 / 81), from about 3 for the baseline rules (128 /
-    // 256 sequences: 73 / 79 against 49 / 84), from about 8 where the last token is drawn by Gumbel-Top-1 (256 / 1024
-    // sequences: 147 / 348 against 128 / 392).  For plain walks over other rows the cluster is ahead at every size (32,001
-    // entries, 64 / 512 / 1000 sequences: 110 / 296 / 444 against 32 / 180 / 329).
+    // ahead from about two waves of clusters on with rows on 16-byte boundaries (V = 32,000, 148 / 200 sequences: ring 63 / 67
+    // us, cluster 59 / 73; V = 16,000, 250 / 300: 57 / 57 against 51 / 61; with clusters of one or two blocks already from 1.3:
+    // V = 8096, 300 / 492: 42 / 53 against 42 / 57).  For the baseline rules (rows of up to 8192 entries: never; else)
+    // from about three waves (V = 32,000, 128 / 256 sequences: 67 / 75 against 49 / 85), from about seven where the last token
+    // is drawn by Gumbel-Top-1 (256 / 512 sequences: 147 / 239 against 128 / 241).  Plain walks over other rows stay with the
+    // cluster (8001 entries, 300 / 1000 sequences: 53 / 143 against 40 / 102; 32,001 entries: 114 / 294 against 120 / 362),
+    // so that their sums do not depend on the batch.
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
-    const float most = ring ? 2.0f : plain ? 1e30f : final_sampler == RSD_FINAL_GUMBEL_TOP1 ? 8.0f : 3.0f;
+    float most = 1e30f;
+    if (ring) most = shape.C <= 2 ? 1.3f : 2.0f;
+    else if (!plain && shape.C > 2) most = final_sampler == RSD_FINAL_GUMBEL_TOP1 ? 7.0f : 3.0f;
     if (shape.C > 0 && shape.waves <= most) {
         rsd::walk_cluster::ClusterArgs ca;
         memset(&ca, 0, sizeof(ca));
