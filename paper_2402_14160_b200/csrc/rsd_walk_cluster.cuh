@@ -231,66 +231,78 @@ struct WorkRows {
 };
 
 // Gumbel-Top-1 draw (Algorithm 6's last step, see gumbel_top1_pick() in rsd_verify_walk.inc): arg min of E(y) / w(y),
-// E(y) = t(U_M) / 16 + [y mod 16 != a] t(U_y).  E >= t(U_M) / 16 with equality at position a: the smallest exact key at
-// the positions a of the block's groups bounds the winner, and only entries whose own lower bound reaches it (a few per
-// cent) need their word of the fine stream.  The result is that of taking every entry.
+// E(y) = t(U_M) / 16 + [y mod 16 != a] t(U_y).  E >= t(U_M) / 16 with equality at position a: the smallest key at the
+// positions a of the block's groups, from fast logarithms rounded up, bounds the winner from above, and only entries whose
+// lower bound reaches it (a few per block) are taken exactly.  The result is that of taking every entry.
+// (Exact logarithms and a second round of Philox calls for every group made this pass 25 us of a walk's 73.)
 template <typename T, int NT, int WARPS>
 __device__ __forceinline__ void top1_pass(Smem<WARPS, NT>& sm, const Place& pl, const RngKey& key, uint32_t node, int flags, float a_hi, float a_lo,
                                           const float (&q)[NT][16], const float (&p)[NT][16]) {
     constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float inf = __int_as_float(0x7F800000);
+    uint32_t cw[NT][kRuns];                      // the groups' coarse-stream words
+    float bound = inf;
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        const int tile = pl.rank + pl.C * (warp + WARPS * k);
+        float w[16];
+        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+#pragma unroll
+        for (int i = 0; i < kRuns; ++i) {
+            const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
+            const uint32_t g = (uint32_t)x0 >> 4;
+            cw[k][i] = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
+            const float t_hat = -__logf(fmaf((float)(cw[k][i] >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f));
+            const float tg_hi = (t_hat + fmaf(t_hat, 1e-6f, 2.5e-7f)) * 0.0625f;
+            const int ja = (int)(cw[k][i] & 15u) - (x0 & 15);
+#pragma unroll
+            for (int j = 0; j < kPer; ++j)
+                if (j == ja && tile < pl.n_tiles && w[i * kPer + j] > 0.0f) bound = fminf(bound, tg_hi / w[i * kPer + j] * 1.00001f);
+        }
+    }
+    bound = -warp_max(-bound);
+    if (lane == 0) sm.warp_top[0][warp] = bound;
+    workers_sync<WARPS * 32>();
+    bound = -warp_max(-(lane < WARPS ? sm.warp_top[0][lane] : inf));
     unsigned long long best = ~0ull;             // key bits << 32 | token: keys are >= 0, so the order is that of (key, token)
-    auto offer = [&](float k, int x) {
-        if (k < inf) best = min(best, ((unsigned long long)__float_as_uint(k) << 32) | (uint32_t)x);
-    };
-#pragma unroll 1
-    for (int turn = 0; turn < 2; ++turn) {       // turn 0: positions a; turn 1: the rest below the block's bound
-        const float bound = best == ~0ull ? inf : __uint_as_float((uint32_t)(best >> 32));
 #pragma unroll
-        for (int k = 0; k < NT; ++k) {
-            const int tile = pl.rank + pl.C * (warp + WARPS * k);
-            if (tile >= pl.n_tiles) continue;
-            float w[16];
-            mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+    for (int k = 0; k < NT; ++k) {
+        const int tile = pl.rank + pl.C * (warp + WARPS * k);
+        float w[16];
+        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
 #pragma unroll
-            for (int i = 0; i < kRuns; ++i) {
-                const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
-                const uint32_t g = (uint32_t)x0 >> 4;
-                const uint32_t cw = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
-                const float tg = neg_log_group_uniform_f32(cw) * 0.0625f;
-                const int ja = (int)(cw & 15u) - (x0 & 15);
-                if (turn == 0) {
+        for (int i = 0; i < kRuns; ++i) {
+            const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
+            const float t_hat = -__logf(fmaf((float)(cw[k][i] >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f));
+            const float tg_lo = fmaxf(t_hat - fmaf(t_hat, 1e-6f, 2.5e-7f), 0.0f) * 0.0625f;
+            uint32_t todo = 0;
 #pragma unroll
-                    for (int j = 0; j < kPer; ++j)
-                        if (j == ja && w[i * kPer + j] > 0.0f) offer(tg / w[i * kPer + j], x0 + j);
-                } else {
-                    uint32_t todo = 0;
+            for (int j = 0; j < kPer; ++j)
+                if (tile < pl.n_tiles && w[i * kPer + j] > 0.0f && tg_lo <= bound * w[i * kPer + j] * 1.00001f) todo |= 1u << j;
+            while (todo) {
+                const int j = __ffs(todo) - 1;
+                todo &= todo - 1;
+                float wj = 0.0f;
 #pragma unroll
-                    for (int j = 0; j < kPer; ++j)
-                        if (w[i * kPer + j] > 0.0f && j != ja && tg <= bound * w[i * kPer + j] * 1.00001f) todo |= 1u << j;
-                    while (todo) {
-                        const int j = __ffs(todo) - 1;
-                        todo &= todo - 1;
-                        float wj = 0.0f;
-#pragma unroll
-                        for (int jj = 0; jj < kPer; ++jj)
-                            if (jj == j) wj = w[i * kPer + jj];
-                        const uint4 fw = rng_draw(key, node, kTagFinalGumbelFine, (uint32_t)(x0 + j) >> 2);
-                        const uint32_t sel = (uint32_t)(x0 + j) & 3u;
-                        const uint32_t word = sel < 2 ? (sel == 0 ? fw.x : fw.y) : (sel == 2 ? fw.z : fw.w);
-                        offer((tg + neg_log_uniform_f32(word)) / wj, x0 + j);
-                    }
+                for (int jj = 0; jj < kPer; ++jj)
+                    if (jj == j) wj = w[i * kPer + jj];
+                float e = neg_log_group_uniform_f32(cw[k][i]) * 0.0625f;
+                if (j != (int)(cw[k][i] & 15u) - (x0 & 15)) {
+                    const uint4 fw = rng_draw(key, node, kTagFinalGumbelFine, (uint32_t)(x0 + j) >> 2);
+                    const uint32_t sel = (uint32_t)(x0 + j) & 3u;
+                    e += neg_log_uniform_f32(sel < 2 ? (sel == 0 ? fw.x : fw.y) : (sel == 2 ? fw.z : fw.w));
                 }
+                const float key_j = e / wj;
+                if (key_j < inf) best = min(best, ((unsigned long long)__float_as_uint(key_j) << 32) | (uint32_t)(x0 + j));
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
-        if (lane == 0) sm.warp_key[warp] = best;
-        workers_sync<WARPS * 32>();
-        for (int w = 0; w < WARPS; ++w) best = min(best, sm.warp_key[w]);
-        workers_sync<WARPS * 32>();
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
+    if (lane == 0) sm.warp_key[warp] = best;
+    workers_sync<WARPS * 32>();
+    for (int w = 0; w < WARPS; ++w) best = min(best, sm.warp_key[w]);
     if (warp == 0 && lane < pl.C) {
         const uint32_t bar = remote_addr(&sm.red_bar[flags & kBuffer ? 1 : 0], lane), at = remote_addr(&sm.top1[pl.rank], lane);
         send_word(at, __uint_as_float((uint32_t)best), bar);
