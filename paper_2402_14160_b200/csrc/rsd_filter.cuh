@@ -18,10 +18,11 @@
 //           value, then the last kept token among its equals
 // A bin that holds more tokens than the list is swept again, into bins of equal width in code.
 //
-// The kernel is bound by instruction issue: 67,000 instructions per row of 32,000 entries went down to half when every
-// token's work in the sweep was cut from 24 instructions to 14 (no returned atomics, packed arithmetic) and the search
-// behind it was left to one warp.  Three blocks per SM for rows of up to 64,000 bytes, and 1024 threads for rows of which
-// only one fits on an SM.
+// Bound by instruction issue (58 %), the histogram's bank conflicts (3.8 wavefronts per addition) and the barriers between
+// a row's serial steps.  A row of 32,000 bf16 entries takes 43,600 warp instructions; it took 67,000 before the sweep went
+// without returned atomics and with packed arithmetic, and before the search behind it was left to one warp: 1344 rows
+// 146 -> 104 us.  Three blocks per SM for rows of up to 64,000 bytes, and 1024 threads for rows of which only one fits on an
+// SM (32 rows of 32,000 fp32 with both cuts 47 -> 23 us).
 #pragma once
 #include "rsd_device.cuh"
 #include "rsd_scan.cuh"   // ex2_approx, packed arithmetic
