@@ -1,0 +1,32 @@
+"""The status words of the drafting and filtering calls are cleared by a kernel of 256-thread blocks that the next kernel
+overlaps: whatever the words held, afterwards they hold this call's bits and nothing else, at the edges of a block."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+NAN_INPUT = 1
+
+
+@pytest.mark.parametrize("B", [1, 255, 256, 257, 513])
+@pytest.mark.parametrize("call", ["draft", "filter"])
+def test_status_words_hold_the_bits_of_their_own_call(call, B):
+    import paper_2402_14160_b200 as rsd
+    clean = torch.randn((B, 2, 640), generator=torch.Generator(device="cuda").manual_seed(B), device="cuda")
+    marked = clean.clone()
+    marked[::3, 1, 600] = float("nan")
+    marked[B - 1, 0, 3] = float("nan")
+
+    def run(rows, out=None):
+        if call == "draft":
+            return rsd.rsd_gumbel_topk_draft(rows, [2, 2], [0, 1], 7, 1, out=out)
+        return rsd.rsd_filter_rows(rows, 20, 0.9, out=out)
+
+    want = torch.isnan(marked).any(dim=2).any(dim=1).to(torch.int32) * NAN_INPUT
+    out = run(clean)
+    out["status"].fill_(-1)
+    got = []
+    for rows in (marked, clean, marked, clean):          # one behind the other, into the same words
+        run(rows, out)
+        got.append(out["status"].clone())
+    for g, w in zip(got, (want, want * 0, want, want * 0)):
+        assert torch.equal(g, w)
