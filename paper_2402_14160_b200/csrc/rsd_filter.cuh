@@ -728,9 +728,12 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     // Fixed point of the weights: 32 fraction bits up to 32,767 entries, 31 up to 65,535, 30 beyond (the conversion saturates
     // at 2^32 - 1, which only the row's largest value can reach); the halves are such that V of them fit 32 bits.  A weight is
     // off by at most half a unit, so the tally is within V 2^-(bits + 1) of the exact sum relative to the row's largest
-    // weight (4e-6 for 32,000 entries in the worst case, around 1e-8 in practice).
+    // weight: in the worst case V 2^-33, V 2^-32 and V 2^-31 in the three ranges (4e-6 for 32,000 entries, 5e-5 for the longest
+    // rows; around 1e-8 in practice).
     const int frac_bits = V < 32768 ? 32 : V < 65536 ? 31 : 30;
-    RowFilter<T, NT> f = {sm, row_sm, V, a.log2e_over_t, (finite > 0 && !plus_inf) ? -vmax * a.log2e_over_t : 0.0f, sm.not_finite == 0, frac_bits,
+    // The reference is rounded down, so that no exponent is above 0: in a row far from 0 the product is off by up to 1e-4, and a
+    // largest weight that much above 1 would saturate while all others keep the factor.
+    RowFilter<T, NT> f = {sm, row_sm, V, a.log2e_over_t, (finite > 0 && !plus_inf) ? __fmul_rd(-vmax, a.log2e_over_t) : 0.0f, sm.not_finite == 0, frac_bits,
                           V < 65536 ? 16 : 15};
     Cut cut = {RowCodes<T>::kNegInfCode, V};                      // everything finite
     int kept = finite;

@@ -158,3 +158,29 @@ def test_filter_rows_at_the_edges_of_its_fixed_point_and_block_sizes(rsd, dtype,
     rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
     for top_k, top_p, T in ((0, 0.95, 1.0), (1024, 0.9, 1.0), (1025, 0.9, 0.7), (2000, 1.0, 1.0)):
         _check_filter(rsd, rows, top_k, top_p, T, max_borderline=2)
+
+
+@pytest.mark.parametrize("dtype,V", [("f32", 20007), ("f32", 32767), ("f32", 32771), ("bf16", 20007)])
+def test_filter_rows_far_from_zero_keep_their_shares(rsd, dtype, V):
+    # The exponents' reference is a rounded product of the row's largest value and log2(e) / T.  Far from 0 its rounding is worth
+    # several 1e-4 of a weight: it must not reach the largest weight alone (a peaked row) or the count of equal values (a flat
+    # one).  The top is put where the product's rounding towards 0 is largest.
+    T = 0.3
+    k = np.float32(1.4426950408889634) / np.float32(T)
+    c = np.arange(2800, 3200, dtype=np.float32) if dtype == "f32" else np.arange(2816, 3200, 16, dtype=np.float32)
+    err = c.astype(np.float64) * np.float64(k) - (c * k).astype(np.float64)
+    top = float(c[np.argmax(err)])
+    assert err.max() > 3e-4
+    rows = torch.full((1, 4, V), top)
+    gap = 3.0 if dtype == "f32" else 16.0                            # (bf16: one step at this size)
+    rows[0, 1, :] = top - gap                                        # one token above 20,000 equal ones
+    rows[0, 1, V // 2] = top
+    rows[0, 2, ::2] = top - gap
+    rows[0, 3, :] = top - 3.5 * gap
+    rows[0, 3, 3::1000] = top
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32).cuda()
+    for top_k, top_p in ((0, 0.8), (0, 0.55), (2000, 0.8)):
+        kept = rsd.rsd_filter_rows(rows, top_k, top_p, temperature=T)["kept"].cpu().numpy()
+        want = oracle.filter_rows(workloads.as_oracle_rows(rows), top_k, top_p, temperature=T)["kept"]
+        # exact to 1e-6 of a row's mass (exponents of up to 50 in fp32), so a cut in a run of equal tokens to less than one of them
+        assert np.abs(kept - want).max() <= 1, (kept, want)
