@@ -557,7 +557,7 @@ struct RowFilter {
             const unsigned long long incl = block_scan_u64<NT>(mine, sm.scan_w, total);
             const double unit = BY_MASS ? 1.0 / (double)(1ull << frac_bits) : 1.0;
             if (level == 0 && need_abs < 0.0) need = need_frac * ((double)total * unit);
-            if (tid == 0) sm.pick_bin = -1;
+            if (tid == 0) { sm.pick_bin = -1; sm.pick_above = 0ull; }
             __syncthreads();
             {
                 unsigned long long run = incl - mine;   // everything above this thread's bins
@@ -572,21 +572,9 @@ struct RowFilter {
                 }
             }
             __syncthreads();
-            int pick = sm.pick_bin;
-            if (pick < 0) {                              // (`need` beyond the total by rounding: the last bin that holds anything)
-                unsigned long long run = incl - mine;
-                if (mine > 0 && incl == total) {
-                    for (int e = 0; e < kPer; ++e) {
-                        const unsigned long long w = bin_sum(tid * kPer + e);
-                        if (w > 0) { sm.pick_bin = tid * kPer + e; sm.pick_above = run; }
-                        run += w;
-                    }
-                }
-                __syncthreads();
-                pick = max(sm.pick_bin, 0);
-                if (sm.pick_bin < 0 && tid == 0) sm.pick_above = 0ull;
-                __syncthreads();
-            }
+            // The tallies are exact sums of integers, and bins of a further level share out the picked bin's, so `need` is
+            // reached; a bin is missing only where nothing in the row has a weight (`need` and all tallies 0): then the first.
+            const int pick = max(sm.pick_bin, 0);
             above += (double)sm.pick_above * unit;
             float v_first, v_last;
             bin_edges(bm, pick, v_first, v_last);
