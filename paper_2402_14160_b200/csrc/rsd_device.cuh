@@ -133,6 +133,17 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t 
         : "memory");
     return ok != 0;
 }
+__device__ __forceinline__ bool mbar_test_wait(unsigned long long* bar, uint32_t parity) {   // (does not suspend the thread)
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 // `bytes` a multiple of 16, both addresses 16-byte aligned; completion counts on `bar`
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -140,10 +151,19 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-constexpr long long kCopyWaitCycles = 1ll << 31;   // about a second: a copy that has not landed by then never will
+// About a second: a copy that has not landed by then never will.  (Negative: a wait runs out unless what it waits for is there; the
+// tests build a library like that to see what a walk reports then.)
+#ifndef RSD_WAIT_CYCLES
+#define RSD_WAIT_CYCLES (1ll << 31)
+#endif
+constexpr long long kCopyWaitCycles = RSD_WAIT_CYCLES;
 // Wait for phase `parity` of `bar`, at most about a second.  A wait that runs out sets *gave_up and returns: the caller
 // goes on with whatever the memory holds and reports RSD_ST_TIMEOUT at its next decision point.
 __device__ __forceinline__ void wait_bar(unsigned long long* bar, uint32_t parity, int* gave_up) {
+    if (kCopyWaitCycles < 0) {
+        if (!mbar_test_wait(bar, parity)) *gave_up = 1;
+        return;
+    }
     if (mbar_try_wait(bar, parity)) return;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {

@@ -66,7 +66,7 @@ struct __align__(16) Cmd {
 template <int WARPS, int NT>
 struct Smem {
     unsigned long long red_bar[2];
-    Cmd cmd;
+    Cmd cmd[2];                              // command n: cmd[n & 1]
     float ref_q, ref_p;                      // references of the exponentials, in units of log2
     float c_seq;                             // K-SEQ's factor of its residual
     int freeze_x;
@@ -79,7 +79,7 @@ struct Smem {
     float lane_sum[2][WARPS * NT][32];       // [target / only sum, draft][local tile][lane]
     float warp_top[2][WARPS];
     int nan_seen;
-    int abort;
+    int gave_up;                             // rank 0: some block's wait ran out
     float tile_sum[kClasses * WARPS * NT];   // of all blocks' tiles
     __align__(16) float tile_w[kTileElems];  // (read as float4)
     int par[kMaxCachedNodes], tok[kMaxCachedNodes];
@@ -117,24 +117,30 @@ __device__ __forceinline__ void cluster_wait() {
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-template <int ID, int THREADS>
-__device__ __forceinline__ void named_sync() {
-    __syncwarp();
-    asm volatile("barrier.cta.sync.aligned %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
-}
-// The command barrier: the control warp arrives, the working warps wait.  It arrives for a pass only when it has the sums of
-// the pass before, that is when every working warp has met the barrier before: nobody arrives twice at one barrier.
-template <int THREADS>
-__device__ __forceinline__ void cmd_arrive() {
-    __syncwarp();
-    asm volatile("barrier.cta.arrive.aligned 1, %0;" ::"n"(THREADS) : "memory");
+__device__ __forceinline__ void store_remote(uint32_t addr, int v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 template <int THREADS>
-__device__ __forceinline__ void cmd_sync() { named_sync<1, THREADS>(); }
+__device__ __forceinline__ void named_sync(int id) {
+    __syncwarp();
+    asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(id), "n"(THREADS) : "memory");
+}
+// The command barriers: for command n the control warp arrives at one, the working warps wait there; commands take two places
+// and two barriers in turn.  Command n + 2 follows the sums (or the dump barrier) of command n + 1, which no working
+// warp runs before it has read command n: nobody arrives twice at one barrier, and no command is overwritten unread.
+// That holds for the end of a walk whose wait for the sums of command n has run out as well: it is command n + 1.
+__device__ __forceinline__ int cmd_barrier(int n) { return n & 1 ? 4 : 1; }
 template <int THREADS>
-__device__ __forceinline__ void workers_sync() { named_sync<2, THREADS>(); }
+__device__ __forceinline__ void cmd_arrive(int n) {
+    __syncwarp();
+    asm volatile("barrier.cta.arrive.aligned %0, %1;" ::"r"(cmd_barrier(n)), "n"(THREADS) : "memory");
+}
 template <int THREADS>
-__device__ __forceinline__ void dump_sync() { named_sync<3, THREADS>(); }
+__device__ __forceinline__ void cmd_sync(int n) { named_sync<THREADS>(cmd_barrier(n)); }
+template <int THREADS>
+__device__ __forceinline__ void workers_sync() { named_sync<THREADS>(2); }
+template <int THREADS>
+__device__ __forceinline__ void dump_sync() { named_sync<THREADS>(3); }
 
 // A lane's 16 values of a tile: the 16-byte pieces lane, lane + 32, ... (the order of the ring walk), -inf beyond the
 // row's end.  Rows on 16-byte boundaries take one load a piece.  Others take the two aligned words around it, shifted;
@@ -327,7 +333,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
         for (int j = 0; j < 16; ++j) q[k][j] = p[k][j] = 0.0f;
     int flags = rows.with_draft ? kOpen : kOpenTarget, node = 0;
     float a_hi = 0.0f, a_lo = 0.0f;
-    bool first = true;
+    int n_cmd = 0;                      // commands read
     for (;;) {
         int kind = flags & kKindMask;
         float s[NT];
@@ -345,12 +351,12 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                     if (kind == kOpen) load_tile<T>(rp[k], rowp, tile, lane, V);
                 }
             }
-            if (first) {
-                first = false;
+            if (n_cmd == 0) {
                 cluster_wait();         // every block's mbarriers are in place
-                cmd_sync<kAll>();
-                flags = sm.cmd.flags;   // the root's rows, with or without the draft row
+                cmd_sync<kAll>(0);
+                flags = sm.cmd[0].flags;   // the root's rows, with or without the draft row
                 kind = flags & kKindMask;
+                n_cmd = 1;
             }
             float cq = 0.0f, cp = 0.0f;
             const bool precise = rows.precise && !(flags & kRelative);
@@ -520,8 +526,9 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                 }
             }
         }
-        cmd_sync<kAll>();
-        const Cmd cmd = sm.cmd;
+        cmd_sync<kAll>(n_cmd);
+        const Cmd cmd = sm.cmd[n_cmd & 1];
+        ++n_cmd;
         flags = cmd.flags;
         node = cmd.node;
         a_hi = cmd.a_hi;
@@ -548,7 +555,7 @@ struct Control {
     const bool precise;
     const int lane;
     const RngKey key;
-    int pass_no, backward;
+    int cmd_no, backward;           // (the passes are the first commands: a walk's dump and end come last)
     bool aborted;
     float kq, kp, mq, mp;           // log2(e) / temperature; references of the exponentials (raw units)
     double Sq, Sp, inv_Sq, inv_Sp, ratio;
@@ -558,30 +565,32 @@ struct Control {
 
     __device__ __forceinline__ Control(Smem<WARPS, NT>& sm_, const ClusterArgs& ca_, const Place& pl_, int b_, bool precise_)
         : sm(sm_), ca(ca_), a(ca_.v), pl(pl_), b(b_), precise(precise_), lane(threadIdx.x & 31),
-          key{ca_.v.seed_lo, ca_.v.seed_hi, ca_.v.step, ca_.v.seq_base + (uint32_t)b_}, pass_no(0), backward(0), aborted(false),
+          key{ca_.v.seed_lo, ca_.v.seed_hi, ca_.v.step, ca_.v.seq_base + (uint32_t)b_}, cmd_no(0), backward(0), aborted(false),
           kq(kLog2e * ca_.v.target.inv_temp), kp(kLog2e * ca_.v.draft.inv_temp), mq(0.0f), mp(0.0f), A(0.0), Z(1.0), a_hi(0.0f), a_lo(0.0f),
           status(0) {}
 
-    // publish a command; the pass reports `words` words to every block
-    __device__ __forceinline__ void issue(int flags, int node, int words) {
-        const int buf = pass_no & 1;
-        ++pass_no;
+    __device__ __forceinline__ void publish(int flags, int node) {
         if (lane == 0) {
             Cmd cmd;
-            cmd.flags = flags | (buf ? kBuffer : 0) | (backward ? kBackward : 0);
+            cmd.flags = flags;
             cmd.node = node;
             cmd.a_hi = a_hi;
             cmd.a_lo = a_lo;
-            sm.cmd = cmd;
-            mbar_expect_tx(&sm.red_bar[buf], 4u * (uint32_t)words);
+            sm.cmd[cmd_no & 1] = cmd;
         }
-        __syncwarp();
-        cmd_arrive<kAll>();
+        cmd_arrive<kAll>(cmd_no);
+        ++cmd_no;
+    }
+    // publish a pass that reports `words` words to every block
+    __device__ __forceinline__ void issue(int flags, int node, int words) {
+        const int buf = cmd_no & 1;
+        if (lane == 0) mbar_expect_tx(&sm.red_bar[buf], 4u * (uint32_t)words);
+        publish(flags | (buf ? kBuffer : 0) | (backward ? kBackward : 0), node);
         backward ^= 1;
     }
     // wait for the words of the latest pass; sets `aborted` when they do not come
     __device__ __forceinline__ int land() {
-        const int n = pass_no - 1, buf = n & 1;
+        const int n = cmd_no - 1, buf = n & 1;
         int late = 0;
         wait_bar(&sm.red_bar[buf], (uint32_t)(n >> 1) & 1u, &late);
         if (__any_sync(0xFFFFFFFFu, late)) aborted = true;
@@ -614,7 +623,7 @@ struct Control {
             issue_open(node, with_draft, kClean);
             collect2(s0, s1);
             if (!with_draft) s1 = 1.0;
-            const int buf = (pass_no - 1) & 1;
+            const int buf = (cmd_no - 1) & 1;
             float top_q = kNegInf, top_p = kNegInf;
             bool saw_nan = false;
             for (int i = 0; i < pl.C; ++i) {
@@ -691,16 +700,7 @@ struct Control {
         walk_ring::pick_tile(sm.tile_sum, pl.n_tiles, u, t);
         if (t.tile < 0) { last = -1; return pl.rank == 0; }
         if (t.tile % pl.C != pl.rank) return false;
-        if (lane == 0) {
-            Cmd cmd;
-            cmd.flags = kDump | (mode << kModeShift);
-            cmd.node = t.tile;
-            cmd.a_hi = a_hi;
-            cmd.a_lo = a_lo;
-            sm.cmd = cmd;
-        }
-        __syncwarp();
-        cmd_arrive<kAll>();
+        publish(kDump | (mode << kModeShift), t.tile);
         dump_sync<kAll>();
         float w[16];
 #pragma unroll
@@ -725,10 +725,23 @@ struct Control {
         return collect();
     }
     __device__ __forceinline__ void end_work() {
-        if (lane == 0) sm.cmd.flags = kEnd;
-        __syncwarp();
-        cmd_arrive<kAll>();
-        if (aborted) status |= 32;   // RSD_ST_TIMEOUT
+        publish(kEnd, 0);
+        if (aborted) {
+            status |= 32;            // RSD_ST_TIMEOUT
+            if (lane == 0) store_remote(remote_addr(&sm.gave_up, 0), 1);
+        }
+    }
+    // Rank 0 when the cluster is through: if a wait ran out in any block, the sequence's outputs say so.  (That block need not be
+    // the one that writes them; the writes so far are ordered before this by the cluster's barrier.)
+    __device__ __forceinline__ void report_timeout() {
+        if (pl.rank != 0 || lane != 0 || !sm.gave_up) return;
+        if (MODE == kResample) {
+            ca.r.out_token[b] = -1;
+            ca.r.status[b] |= 32;
+        } else {
+            a.last_token[b] = -1;
+            a.status[b] |= 32;
+        }
     }
 
     // What is left of the draft once subtraction has lost its accuracy: summed anew without the rejected tokens.
@@ -934,12 +947,14 @@ struct Control {
             double miss = 1.0;
             for (int i = 0; i < seq_kids; ++i) miss *= 1.0 - beta;
             const float c = (float)(beta > 0.0 ? (1.0 - miss) / beta : (double)seq_kids);
-            if (lane == 0) sm.c_seq = c;
-            issue(kSeqPass | kStoreTiles, 0, kClasses + pl.n_tiles);
-            const double t = collect();
-            tiles_valid = t > 0.0 && t < 1.7e308;
-            if (tiles_valid) mode = kSeqResidual;
-            else status |= 4;                         // RSD_ST_ZERO_RESIDUAL: draw from the target row itself
+            if (!aborted) {
+                if (lane == 0) sm.c_seq = c;
+                issue(kSeqPass | kStoreTiles, 0, kClasses + pl.n_tiles);
+                const double t = collect();
+                tiles_valid = t > 0.0 && t < 1.7e308;
+                if (tiles_valid) mode = kSeqResidual;
+                else status |= 4;                     // RSD_ST_ZERO_RESIDUAL: draw from the target row itself
+            }
         }
         const bool top1 = (MODE == kRuleWalk) && a.final_sampler == 1;
         if (!aborted && !tiles_valid && !top1) refresh_tiles(mode == kResidual);
@@ -947,11 +962,13 @@ struct Control {
         bool mine = pl.rank == 0;
         if (!aborted) mine = top1 ? draw_top1(mode, (uint32_t)cur, last) : draw(mode, (uint32_t)cur, last);
         end_work();
-        if (mine && lane == 0) {
-            a.accepted_len[b] = len;
-            a.last_token[b] = last;
-            a.stop_reason[b] = reason;
-            a.status[b] = status;
+        if (lane == 0) {
+            if (mine) a.last_token[b] = last;
+            if (pl.rank == 0) {
+                a.accepted_len[b] = len;
+                a.stop_reason[b] = reason;
+                a.status[b] = status;
+            }
         }
     }
 
@@ -1015,24 +1032,15 @@ struct Control {
         if (!aborted) {
             mine = draw(mode, node, last);
             if (r.out_residual) {
-                if (lane == 0) {
-                    sm.inv_total = total > 0.0 ? 1.0 / total : 0.0;
-                    Cmd cmd;
-                    cmd.flags = kWrite | (mode << kModeShift);
-                    cmd.node = 0;
-                    cmd.a_hi = a_hi;
-                    cmd.a_lo = a_lo;
-                    sm.cmd = cmd;
-                }
-                __syncwarp();
-                cmd_arrive<kAll>();
+                if (lane == 0) sm.inv_total = total > 0.0 ? 1.0 / total : 0.0;
+                publish(kWrite | (mode << kModeShift), 0);
                 dump_sync<kAll>();   // (the command has been read: its place may take the next one)
             }
         }
         end_work();
-        if (mine && lane == 0) {
-            r.out_token[b] = last;
-            r.status[b] = status;
+        if (lane == 0) {
+            if (mine) r.out_token[b] = last;
+            if (pl.rank == 0) r.status[b] = status;
         }
     }
 };
@@ -1054,6 +1062,7 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         mbar_init(&sm.red_bar[0], 1);
         mbar_init(&sm.red_bar[1], 1);
         sm.nan_seen = 0;
+        sm.gave_up = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     cluster_arrive();
@@ -1071,14 +1080,18 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         rows.key = RngKey{a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
         rows.out_residual = MODE == kResample && ca.r.out_residual ? ca.r.out_residual + (int64_t)b * a.V : nullptr;
         work<T, NT, WARPS, MODE>(sm, pl, rows);
+        grid_started();
+        cluster_arrive();   // nothing is on its way to a block that has left
+        cluster_wait();
     } else {
         Control<T, NT, WARPS, MODE> control(sm, ca, pl, b, precise);
         if constexpr (MODE == kResample) control.resample();
         else control.walk();
+        grid_started();
+        cluster_arrive();
+        cluster_wait();
+        control.report_timeout();
     }
-    grid_started();
-    cluster_arrive();   // nothing is on its way to a block that has left
-    cluster_wait();
 }
 
 }  // namespace walk_cluster
