@@ -102,6 +102,14 @@ __device__ __forceinline__ uint4 ld_stream(const void* p) {
     return v;
 }
 
+// The same through L1, for words that two threads need.  (volatile: an __ldg may be moved above grid_wait(), to where the kernel
+// before may still be writing the row)
+__device__ __forceinline__ uint4 ld_shared_word(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // 32 bytes at a 32-byte aligned address in one request (sm_100: 256-bit global loads)
 __device__ __forceinline__ void ld_stream_256(const void* p, uint4& lo, uint4& hi) {
     asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"

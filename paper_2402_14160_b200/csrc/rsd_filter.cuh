@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
         if (m != 0 && n_vec > 2 && m % kElem == 0) {             // in the aligned words around each, shifted; the ends one by one
             for (int i = 1 + tid; i < n_vec - 1; i += NT) {
                 const uint4* p = (const uint4*)(src + (size_t)i * 16 - m);
-                ((uint4*)row_sm)[i] = window16(__ldg(p), __ldg(p + 1), m);
+                ((uint4*)row_sm)[i] = window16(ld_shared_word(p), ld_shared_word(p + 1), m);
             }
         }
         const bool ends = m != 0 && n_vec > 2 && m % kElem == 0;

@@ -215,10 +215,10 @@ struct Packed<float> {
             const char* at = (const char*)row + (int64_t)g * 64;
             const uint32_t m = (uint32_t)(uintptr_t)at & 15u;
             const uint4* p = (const uint4*)(at - m);
-            uint4 prev = __ldg(p);
+            uint4 prev = ld_shared_word(p);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const uint4 next = __ldg(p + i + 1);
+                const uint4 next = ld_shared_word(p + i + 1);
                 w[i] = window16(prev, next, m);
                 prev = next;
             }
@@ -288,7 +288,7 @@ struct Packed<__nv_bfloat16> {
             const char* at = (const char*)row + (int64_t)g * 32;
             const uint32_t m = (uint32_t)(uintptr_t)at & 15u;
             const uint4* p = (const uint4*)(at - m);
-            const uint4 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+            const uint4 a = ld_shared_word(p), b = ld_shared_word(p + 1), c = ld_shared_word(p + 2);
             w[0] = window16(a, b, m);
             w[1] = window16(b, c, m);
         } else {
