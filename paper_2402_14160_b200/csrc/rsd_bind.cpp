@@ -40,25 +40,34 @@ const at::Tensor& tensor(PyObject* o) {
     return THPVariable_Unpack(o);
 }
 void* ptr(PyObject* o) { return o == Py_None ? nullptr : tensor(o).data_ptr(); }
-long long integer(PyObject* o) {
-    PyObject* n = PyNumber_Long(o);
+long long low_bits(PyObject* n) {   // takes the reference
     if (!n) throw Failed();
     const unsigned long long v = PyLong_AsUnsignedLongLongMask(n);
     Py_DECREF(n);
     if (PyErr_Occurred()) throw Failed();
     return (long long)v;
 }
-double real(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw Failed();
+long long integer(PyObject* o) { return low_bits(PyNumber_Index(o)); }       // an integer; a float or a text is refused
+long long as_integer(PyObject* o) { return low_bits(PyNumber_Long(o)); }     // int(o)
+double real(PyObject* o) {   // float(o)
+    if (PyFloat_CheckExact(o)) return PyFloat_AS_DOUBLE(o);
+    PyObject* n = PyNumber_Float(o);
+    if (!n) throw Failed();
+    const double v = PyFloat_AsDouble(n);
+    Py_DECREF(n);
     return v;
+}
+bool truth(PyObject* o) {
+    const int t = PyObject_IsTrue(o);
+    if (t < 0) throw Failed();
+    return t != 0;
 }
 std::vector<int32_t> integers(PyObject* o) {
     PyObject* s = PySequence_Fast(o, "a sequence of integers is expected");
     if (!s) throw Failed();
     std::vector<int32_t> v((size_t)PySequence_Fast_GET_SIZE(s));
     try {
-        for (size_t i = 0; i < v.size(); ++i) v[i] = (int32_t)integer(PySequence_Fast_GET_ITEM(s, i));
+        for (size_t i = 0; i < v.size(); ++i) v[i] = (int32_t)as_integer(PySequence_Fast_GET_ITEM(s, i));
     } catch (Failed&) {
         Py_DECREF(s);
         throw;
@@ -127,7 +136,7 @@ PyObject* filter_rows(PyObject* const* a) {
     want_dims(t, 3);
     if (!out.is_contiguous() || out.scalar_type() != t.scalar_type()) fail("out rows must be contiguous and of the rows' dtype");
     const rsd_rows r = rows_of(t, false, real(a[1]));
-    const int top_k = (int)integer(a[2]);
+    const int top_k = (int)as_integer(a[2]);
     const float top_p = (float)real(a[3]);
     void *rows = out.data_ptr(), *kept = ptr(a[5]), *status = ptr(a[6]);
     const rsd_stream_t s = stream();
@@ -140,7 +149,7 @@ PyObject* filter_rows(PyObject* const* a) {
 PyObject* gumbel_topk_draft(PyObject* const* a) {
     const at::Tensor& t = tensor(a[0]);
     want_dims(t, 3);
-    const rsd_rows r = rows_of(t, PyObject_IsTrue(a[1]) == 1, real(a[2]));
+    const rsd_rows r = rows_of(t, truth(a[1]), real(a[2]));
     const int B = (int)t.size(0), R = (int)t.size(1), V = (int)t.size(2);
     const std::vector<int32_t> k = integers(a[3]), node = integers(a[4]);
     std::vector<int32_t> base;
@@ -174,7 +183,7 @@ void same_stride(const at::Tensor& x, const at::Tensor& y, const char* message) 
 PyObject* sbs_step(PyObject* const* a) {
     const at::Tensor &t = tensor(a[0]), &token = tensor(a[10]), &parent = tensor(a[11]);
     want_dims(t, 3);
-    const rsd_rows r = rows_of(t, PyObject_IsTrue(a[1]) == 1, real(a[2]));
+    const rsd_rows r = rows_of(t, truth(a[1]), real(a[2]));
     const int B = (int)t.size(0), n_par = (int)t.size(1), V = (int)t.size(2), W = (int)integer(a[3]);
     const int32_t first = (int32_t)integer(a[4]), base = (int32_t)integer(a[12]);
     const float *sum_in = (const float*)ptr(a[5]), *gum_in = (const float*)ptr(a[6]);
@@ -208,7 +217,7 @@ PyObject* sbs_draft_tree(PyObject* const* a) {
         throw Failed();
     }
     same_stride(token, parent, "node_token / node_parent must share a row stride and be dense along the nodes");
-    const rsd_rows r = rows_of(t, PyObject_IsTrue(a[1]) == 1, real(a[2]));
+    const rsd_rows r = rows_of(t, truth(a[1]), real(a[2]));
     const uint64_t seed = (uint64_t)integer(a[5]);
     const uint32_t step = (uint32_t)integer(a[6]), seq = (uint32_t)integer(a[7]);
     int32_t *tok = (int32_t*)token.data_ptr(), *par = (int32_t*)parent.data_ptr(), *count = (int32_t*)ptr(a[12]), *status = (int32_t*)ptr(a[13]);
@@ -238,13 +247,13 @@ PyObject* verify_tree(PyObject* const* a) {
     const int B = (int)target.size(0), V = (int)target.size(2);
     const uint64_t seed = (uint64_t)integer(a[7]);
     const uint32_t step = (uint32_t)integer(a[8]), seq = (uint32_t)integer(a[9]);
-    const int rule = (int)integer(a[10]), sampler = (int)integer(a[12]);
+    const int rule = (int)as_integer(a[10]), sampler = (int)as_integer(a[12]);
     const float gamma = (float)real(a[11]);
     int32_t *len = (int32_t*)ptr(a[14]), *node = (int32_t*)ptr(a[15]), *tok = (int32_t*)ptr(a[16]), *last = (int32_t*)ptr(a[17]), *reason = (int32_t*)ptr(a[18]),
             *status = (int32_t*)ptr(a[20]);
     float* theta = (float*)ptr(a[19]);
     const rsd_stream_t s = stream();
-    if (rule == RSD_RULE_RRS && sampler == RSD_FINAL_INVERSE_CDF && PyObject_IsTrue(a[13]) == 0)
+    if (rule == RSD_RULE_RRS && sampler == RSD_FINAL_INVERSE_CDF && !truth(a[13]))
         return call([&] { return p_verify_tree(&d, &t, &tree, B, V, seed, step, seq, len, node, tok, last, reason, theta, status, s); });
     return call([&] { return p_verify_tree_rule(&d, &t, &tree, B, V, rule, gamma, sampler, seed, step, seq, len, node, tok, last, reason, theta, status, s); });
 }
