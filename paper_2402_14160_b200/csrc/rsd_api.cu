@@ -298,9 +298,14 @@ int rsd_sbs_draft_tree(const rsd_rows* draft, int B, int V, int W, int L, uint64
     c.node_token = node_token; c.node_parent = node_parent; c.node_stride = node_stride;
     c.level_count = level_count; c.level_status = level_status; c.status = status;
     c.sum_out = sum_logprob_out; c.gamma_out = trunc_gumbel_out;
-    // the finalists of a sequence are staged in shared memory when they fit well inside the default 48 KB
-    c.staged = rsd::sbs_chain_smem_bytes(W, (int)P, true) <= 40 * 1024 ? 1 : 0;
-    const size_t smem = rsd::sbs_chain_smem_bytes(W, (int)P, c.staged != 0);
+    // The finalists of a sequence are staged in shared memory when they fit well inside the default 48 KB, and their noise with
+    // them when that fits as well and a level's finalists are no more than the block's threads: inside the chain a level takes
+    // the noise of the dozen or so that pass its first test, one per thread, ahead of it W W / 128 per thread and level.
+    // (Noise inside / ahead, us at 32 sequences: 4 x 20 79 / 70, 8 x 8 44.7 / 43.3, 10 x 5 37.1 / 35.8; 12 x 6 45.9 / 46.5,
+    // 16 x 5 49.5 / 54.4, 24 x 2 43.9 / 47.6)
+    c.staged = W * W <= rsd::kEpilogueThreads ? rsd::kStagedNoise : rsd::kStagedFinalists;
+    while (c.staged > 0 && rsd::sbs_chain_smem_bytes(W, (int)P, c.staged) > 40 * 1024) --c.staged;
+    const size_t smem = rsd::sbs_chain_smem_bytes(W, (int)P, c.staged);
     launch_overlapped(rsd::sbs_chain_kernel, (unsigned)B, rsd::kEpilogueThreads, smem, s, 0, c);
     return check_launch("rsd_sbs_draft_tree(levels)");
 }

@@ -1079,12 +1079,14 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_epilogue_kernel(c
 // The sequence log-probabilities and truncated Gumbels (Eqs. 10-12) travel from level to level through two pairs of
 // W-element arrays in shared memory used in turn; level l writes the tokens and parents of flat nodes
 // 1 + l W .. (l + 1) W.  When `staged` is set the sequence's finalists (P W tokens, values and perturbed values, P
-// log-sum-exps and row flags) are copied to shared memory once, so that no level waits for global memory.
+// log-sum-exps and row flags) are copied to shared memory once, so that no level waits for global memory, and, where that
+// fits as well, their noise is taken once beside them.
+enum { kStagedFinalists = 1, kStagedNoise = 2 };
 struct SbsChainArgs {
     SbsEpilogueArgs lvl;        // level-independent fields; the per-level ones are filled in by the kernel
     int L, P;                   // levels; parent rows per sequence, 1 + (L - 1) W
     int B;
-    int staged;                 // 1: the dynamic shared memory also holds the finalists' copies
+    int staged;                 // what the dynamic shared memory holds: 0 nothing of the finalists, or one of the above
     int32_t* node_token;        // [B][node_stride]
     int32_t* node_parent;
     int64_t node_stride;
@@ -1096,8 +1098,8 @@ struct SbsChainArgs {
 };
 
 // dynamic shared memory of sbs_chain_kernel
-__host__ __device__ inline size_t sbs_chain_smem_bytes(int W, int P, bool staged) {
-    return sbs_level_scratch_bytes(W, W) + (size_t)4 * W * 4 + (staged ? (size_t)P * W * 20 + (size_t)P * 8 + 8 : 0);
+__host__ __device__ inline size_t sbs_chain_smem_bytes(int W, int P, int staged) {
+    return sbs_level_scratch_bytes(W, W) + (size_t)4 * W * 4 + (staged ? (size_t)P * W * 12 + (size_t)P * 8 : 0) + (staged == kStagedNoise ? (size_t)P * W * 8 + 8 : 0);
 }
 
 static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(const SbsChainArgs c) {
@@ -1125,7 +1127,7 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(cons
         // The noise of a finalist does not depend on the levels above it: taken for all of them at once, not for a dozen at a
         // time inside the chain (three double-precision logarithms and two Philox calls, a third of a level's latency).
         const RngKey key = {c.lvl.seed_lo, c.lvl.seed_hi, c.lvl.step, c.lvl.seq_base + (uint32_t)b};
-        for (int i = tid; i < F; i += kEpilogueThreads) {
+        for (int i = tid; i < F && c.staged == kStagedNoise; i += kEpilogueThreads) {
             const int x = s_tok[i];   // (this thread's own copy)
             s_noise[i] = x >= 0 ? sbs_log_noise(key, (uint32_t)(i / W), (uint32_t)x) : 0.0;
         }
@@ -1165,7 +1167,7 @@ static __global__ void __launch_bounds__(kEpilogueThreads) sbs_chain_kernel(cons
         a.parent_base = first;
         a.out_count = c.level_count + (int64_t)l * c.B;
         a.status = c.level_status + (int64_t)l * c.B;
-        sbs_epilogue_body(a, b, sm_d, c.staged ? s_noise + first * W : nullptr);
+        sbs_epilogue_body(a, b, sm_d, c.staged == kStagedNoise ? s_noise + first * W : nullptr);
         __syncthreads();   // the level's outputs are the next level's inputs
         if (tid == 0) st |= a.status[b];
         if (last && tid < W) {
