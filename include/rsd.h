@@ -38,8 +38,7 @@
  *              the group's largest noise is known from one word of the coarse stream.
  *       tag 2  acceptance     : index = rank of the child among its siblings; U = (word0 >> 8) / 2^24
  *       tag 3  final token    : index = 0; u = (word0 + 1/2) / 2^32
- *     The same (seed, step, inputs) give bit-identical outputs whatever the launch shape (rsd_verify_tree_rule's baseline
- *     rules: up to fp32 rounding, see there).
+ *     The same (seed, step, inputs) give bit-identical outputs whatever the launch shape.
  */
 #ifndef RSD_H_
 #define RSD_H_
@@ -267,9 +266,6 @@ int rsd_verify_tree(const rsd_rows* draft, const rsd_rows* target, const rsd_tre
  *                        beta = sum_x min{p(x), q(x)/gamma}.  gamma in [1, K]; gamma = K is always admissible
  *                        (smaller values need (1 - (1 - beta)^K) / beta <= gamma, else the clamp at 0 applies)
  * gamma is read only by RSD_RULE_KSEQ (finite, >= 1).
- * Under a baseline rule or the Gumbel-Top-1 draw the sums behind a threshold are taken in an order that depends on the number
- * of sequences: a decision within fp32 rounding of its threshold, and the last digits of dbg_theta, may differ between
- * a batch and its parts.
  * final_sampler chooses how the last token is drawn from its distribution w (a residual or a target row):
  *   RSD_FINAL_INVERSE_CDF  one uniform, smallest y whose running sum of w exceeds u * sum(w): rsd_verify_tree's way
  *   RSD_FINAL_GUMBEL_TOP1  arg max over y of log w(y) + G(y) with fresh standard Gumbel noise G (Algorithm 6's last

@@ -1,5 +1,6 @@
 // C ABI of librsd (declared in include/rsd.h), verification half: rsd_verify_tree, rsd_verify_tree_rule and
 // rsd_resample_residual.  Argument checks and kernel launches, nothing else.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 
@@ -60,9 +61,36 @@ rsd::walk_cluster::Shape cluster_shape(int B, int V) {
     return {0, 0, 0, 0.0f};
 }
 
-void launch_cluster_walk(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const rsd::walk_cluster::Shape& c, cudaStream_t s) {
+// Up to how many waves of clusters the on-chip walk is taken.
+//   Rows that the ring takes (figures: us for so many sequences, bf16): from about two waves on the ring is ahead (V = 32,000, 148 / 200:
+// ring 63 / 67, cluster 59 / 73; V = 16,000, 250 / 300: 57 / 57 against 51 / 61; with clusters of one or two blocks already from 1.3:
+// V = 8096, 300 / 492: 42 / 53 against 42 / 57).
+//   Others: clusters of one or two blocks stay (8001 entries, 300 / 1000: 34 / 89 on chip, 41 / 102 read anew).  Beyond, a launch on
+// chip takes as long as it has waves, one that reads the rows anew as long as they are, up to the 296 or 444 sequences that are
+// resident at once: 20,000 entries, multi-round, 148 / 222: 46 / 66 on chip, 43 / 49 read anew; 32,001, plain, 200 / 250: 68 / 88, 73 / 75;
+// 65,001, 148 / 200: 124 / 160, 134 / 150; 100,000, 80 / 128: 139 / 228, 149 / 151, fp32 128: 270, 275.
+//   Gumbel-Top-1 draws take two rounds of Philox calls when rows are read anew: 32,000 entries, 256 / 400: 104 / 154 on chip, 108 / 132
+// read anew; 100,000, 74 / 128: 141 / 240, 216 / 227; fp32, 400 / 512 of 32,000: 176 / 226, 195 / 220.
+float most_waves(const rsd::walk_cluster::Shape& c, int V, bool f32, bool ring, bool top1) {
+    if (ring) return c.C <= 2 ? 1.3f : 2.0f;
+    if (c.C <= 2) return 1e30f;
+    if (top1) return f32 ? 7.0f : std::min(1.6f + (float)V / 16000.0f, 6.6f);
+    return std::min(1.0f + (float)V / 18000.0f, f32 ? 7.0f : 4.8f);
+}
+
+void launch_on_chip(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const rsd::walk_cluster::Shape& c, cudaStream_t s) {
     if (dtype == RSD_F32) rsd::walk_cluster::launch_f32(a, extra, B, c, s);
     else rsd::walk_cluster::launch_bf16(a, extra, B, c, s);
+}
+
+// Rows that no cluster holds: eight blocks a sequence up to about as many sequences as SMs (151,936 entries, us with eight blocks / one, 148
+// sequences: residual draw fp32 251 / 259, multi-round 153 / 177; 222: 357 / 299, 220 / 194), plain walks up to half as many more
+// (fp32, 222 / 256 sequences: 231 / 249, 262 / 258).  2-byte rows: two blocks an SM while that holds the batch, else three.
+void launch_streamed(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, bool fits_cluster, cudaStream_t s) {
+    const int sms = sm_count();
+    const int C = !fits_cluster && B <= (extra ? sms : sms + sms / 2) ? 8 : 1;
+    if (dtype == RSD_F32) rsd::walk_cluster::launch_stream_f32(a, extra, B, C, 2, s);
+    else rsd::walk_cluster::launch_stream_bf16(a, extra, B, C, B > 2 * sms ? 3 : 2, s);
 }
 }  // namespace
 
@@ -112,38 +140,21 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
     // the ring walk: rows on 16-byte boundaries, of at most 64 chunks (it keeps its chunks as bits of one word)
     const size_t row_bytes = (size_t)V * (draft->dtype == RSD_F32 ? 4 : 2);
     const bool ring = plain && aligned && (row_bytes + rsd::walk_ring::kRowChunkBytes - 1) / rsd::walk_ring::kRowChunkBytes <= 64;
-    // A cluster per sequence while there are few: its passes are two to three times as short (V = 32,000 bf16: 30 -> 16 us
-    // for one sequence, 94 -> 42 for 64), but it takes more SM time per walk.  The kernels with one block per sequence are
-    // ahead from about two waves of clusters on with rows on 16-byte boundaries (V = 32,000, 148 / 200 sequences: ring 63 / 67
-    // us, cluster 59 / 73; V = 16,000, 250 / 300: 57 / 57 against 51 / 61; with clusters of one or two blocks already from 1.3:
-    // V = 8096, 300 / 492: 42 / 53 against 42 / 57).  For the baseline rules (rows of up to 8192 entries: never; else)
-    // from about three waves (V = 32,000, 128 / 256 sequences: 67 / 75 against 49 / 85), from about seven where the last token
-    // is drawn by Gumbel-Top-1 (256 / 512 sequences: 147 / 239 against 128 / 241).  Plain walks over other rows stay with the
-    // cluster (8001 entries, 300 / 1000 sequences: 53 / 143 against 40 / 102; 32,001 entries: 114 / 294 against 120 / 362),
-    // so that their sums do not depend on the batch.
+    // The ring's sums and those of the other two are the same for the rows that it takes (ring_rows), and those of the other two
+    // always: a batch and its parts give the same bits.
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
-    float most = 1e30f;
-    if (ring) most = shape.C <= 2 ? 1.3f : 2.0f;
-    else if (!plain && shape.C > 2) most = final_sampler == RSD_FINAL_GUMBEL_TOP1 ? 7.0f : 3.0f;
-    if (shape.C > 0 && shape.waves <= most) {
-        rsd::walk_cluster::ClusterArgs ca;
-        memset(&ca, 0, sizeof(ca));
-        ca.v = a;
-        ca.off_boundaries = aligned ? 0 : 1;
-        launch_cluster_walk(ca, draft->dtype, !plain, B, shape, s);
-    } else if (ring) {
+    const bool on_chip = shape.C > 0 && shape.waves <= most_waves(shape, V, draft->dtype == RSD_F32, ring, final_sampler == RSD_FINAL_GUMBEL_TOP1);
+    rsd::walk_cluster::ClusterArgs ca;
+    memset(&ca, 0, sizeof(ca));
+    ca.v = a;
+    ca.ring_rows = ring ? 1 : 0;
+    if (on_chip) {
+        launch_on_chip(ca, draft->dtype, !plain, B, shape, s);
+    } else if (!ring) {
+        launch_streamed(ca, draft->dtype, !plain, B, shape.C > 0, s);
+    } else {
         if (draft->dtype == RSD_F32) launch_ring_walk<float>(a, B, s);
         else launch_ring_walk<__nv_bfloat16>(a, B, s);
-    } else {
-        using namespace rsd::walk_narrow;
-        auto launch = [&](auto kernel) { kernel<<<B, kVerifyThreads, 0, s>>>(a); };
-        if (draft->dtype == RSD_F32) {
-            if (plain) launch(aligned ? verify_tree_kernel<float, true, false> : verify_tree_kernel<float, false, false>);
-            else launch(aligned ? verify_tree_kernel<float, true, true> : verify_tree_kernel<float, false, true>);
-        } else {
-            if (plain) launch(verify_tree_kernel<__nv_bfloat16, false, false>);   // (2-byte rows on 16-byte boundaries fit the ring)
-            else launch(aligned ? verify_tree_kernel<__nv_bfloat16, true, true> : verify_tree_kernel<__nv_bfloat16, false, true>);
-        }
     }
     return check_launch("rsd_verify_tree_rule");
 }
@@ -170,27 +181,16 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     a.out_token = out_token; a.out_residual = out_residual; a.status = status;
     cudaStream_t s = (cudaStream_t)stream;
     // rows that fit a cluster take it at every batch size (V = 32,000, three rejected tokens: 137 -> 75 us for 256 sequences)
+    rsd::walk_cluster::ClusterArgs ca;
+    memset(&ca, 0, sizeof(ca));
+    ca.r = a;
+    ca.resample = 1;
+    ca.v.draft = a.draft; ca.v.target = a.target;
+    ca.v.V = V; ca.v.num_nodes = 1;
+    ca.v.seed_lo = a.seed_lo; ca.v.seed_hi = a.seed_hi; ca.v.step = step; ca.v.seq_base = seq_base;
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
-    if (shape.C > 0) {
-        rsd::walk_cluster::ClusterArgs ca;
-        memset(&ca, 0, sizeof(ca));
-        ca.r = a;
-        ca.resample = 1;
-        ca.v.draft = a.draft; ca.v.target = a.target;
-        ca.v.V = V; ca.v.num_nodes = 1;
-        ca.v.seed_lo = a.seed_lo; ca.v.seed_hi = a.seed_hi; ca.v.step = step; ca.v.seq_base = seq_base;
-        launch_cluster_walk(ca, target_row->dtype, true, B, shape, s);
-        return check_launch("rsd_resample_residual");
-    }
-    const bool aligned = rows_aligned(target_row) && (!rejected || rows_aligned(draft_row));
-    using namespace rsd::walk_narrow;
-    if (target_row->dtype == RSD_F32) {
-        if (aligned) resample_residual_kernel<float, true><<<B, kVerifyThreads, 0, s>>>(a);
-        else resample_residual_kernel<float, false><<<B, kVerifyThreads, 0, s>>>(a);
-    } else {
-        if (aligned) resample_residual_kernel<__nv_bfloat16, true><<<B, kVerifyThreads, 0, s>>>(a);
-        else resample_residual_kernel<__nv_bfloat16, false><<<B, kVerifyThreads, 0, s>>>(a);
-    }
+    if (shape.C > 0) launch_on_chip(ca, target_row->dtype, true, B, shape, s);
+    else launch_streamed(ca, target_row->dtype, true, B, false, s);
     return check_launch("rsd_resample_residual");
 }
 

@@ -52,8 +52,9 @@ enum {
     kRelative = 32,      // kOpen, kOpenTarget: exponentials relative to sm.ref_q, sm.ref_p (else to 0)
     kStoreTiles = 64,    // the sum of every tile goes to every block's tile_sum
     kBackward = 128,     // order of the lanes' sums
-    kBuffer = 256,       // which half of class_sum / red_bar the pass reports to
+    kBuffer = 256,       // an odd command: the second place, and the second half of class_sum / red_bar
     kFreeze = 512,       // kResidualPass: first sm.freeze_x leaves the draft and keeps its weight
+    kFirst = 1024,       // (a working warp's own mark: no command yet)
     kModeShift = 12      // kDump, kTop1, kWrite: weights are 0 q, kResidual (q - a p)+, kSeqResidual K-SEQ's residual
 };
 
@@ -63,7 +64,8 @@ struct __align__(16) Cmd {
     float a_hi, a_lo;
 };
 
-template <int WARPS, int NT>
+// WARPS working warps; LISTED tiles of the block whose lanes' sums are kept; TILES tiles of all blocks
+template <int WARPS, int LISTED, int TILES>
 struct Smem {
     unsigned long long red_bar[2];
     Cmd cmd[2];                              // command n: cmd[n & 1]
@@ -76,17 +78,19 @@ struct Smem {
     float extra[2][3][kClasses];             // [buffer][maxima of target and draft, NaN seen][block]
     unsigned long long top1[kClasses];       // [block] smallest key of the Gumbel draw with its token
     unsigned long long warp_key[WARPS];
-    float lane_sum[2][WARPS * NT][32];       // [target / only sum, draft][local tile][lane]
+    float lane_sum[2][LISTED][32];           // [target / only sum, draft][local tile][lane]
     float warp_top[2][WARPS];
     int nan_seen;
     int gave_up;                             // rank 0: some block's wait ran out
-    float tile_sum[kClasses * WARPS * NT];   // of all blocks' tiles
+    float tile_sum[TILES];
     __align__(16) float tile_w[kTileElems];  // (read as float4)
     int par[kMaxCachedNodes], tok[kMaxCachedNodes];
     int kid_node[32];
     int gone_tok[kMaxListed];
     int n_gone_tok;
 };
+template <int WARPS, int NT>
+using ChipSmem = Smem<WARPS, WARPS * NT, kClasses * WARPS * NT>;
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -126,17 +130,17 @@ __device__ __forceinline__ void named_sync(int id) {
     asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(id), "n"(THREADS) : "memory");
 }
 // The command barriers: for command n the control warp arrives at one, the working warps wait there; commands take two places
-// and two barriers in turn.  Command n + 2 follows the sums (or the dump barrier) of command n + 1, which no working
+// and two barriers in turn (kBuffer in its flags: the odd ones).  Command n + 2 follows the sums (or the dump barrier) of command n + 1, which no working
 // warp runs before it has read command n: nobody arrives twice at one barrier, and no command is overwritten unread.
 // That holds for the end of a walk whose wait for the sums of command n has run out as well: it is command n + 1.
-__device__ __forceinline__ int cmd_barrier(int n) { return n & 1 ? 4 : 1; }
+__device__ __forceinline__ int cmd_barrier(int odd) { return odd ? 4 : 1; }
 template <int THREADS>
-__device__ __forceinline__ void cmd_arrive(int n) {
+__device__ __forceinline__ void cmd_arrive(int odd) {
     __syncwarp();
-    asm volatile("barrier.cta.arrive.aligned %0, %1;" ::"r"(cmd_barrier(n)), "n"(THREADS) : "memory");
+    asm volatile("barrier.cta.arrive.aligned %0, %1;" ::"r"(cmd_barrier(odd)), "n"(THREADS) : "memory");
 }
 template <int THREADS>
-__device__ __forceinline__ void cmd_sync(int n) { named_sync<THREADS>(cmd_barrier(n)); }
+__device__ __forceinline__ void cmd_sync(int odd) { named_sync<THREADS>(cmd_barrier(odd)); }
 template <int THREADS>
 __device__ __forceinline__ void workers_sync() { named_sync<THREADS>(2); }
 template <int THREADS>
@@ -158,11 +162,7 @@ __device__ __forceinline__ void load_tile(Packed<T>& pk, const char* row, int ti
 #pragma unroll
         for (int i = 0; i < kPieces; ++i) {
             const uint4 a = *(const uint4*)(at + 512 * i - m), b = *(const uint4*)(at + 512 * i - m + 16);
-            uint32_t w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x, w5 = b.y, w6 = b.z, w7 = b.w;
-            if (m & 8u) { w0 = w2; w1 = w3; w2 = w4; w3 = w5; w4 = w6; w5 = w7; }
-            if (m & 4u) { w0 = w1; w1 = w2; w2 = w3; w3 = w4; w4 = w5; }
-            const uint32_t s = (m & 3u) * 8u;
-            pk.w[i] = make_uint4(__funnelshift_r(w0, w1, s), __funnelshift_r(w1, w2, s), __funnelshift_r(w2, w3, s), __funnelshift_r(w3, w4, s));
+            pk.w[i] = window16(a, b, m);
         }
     } else {
         const int x0 = tile * kTileElems + lane * kPer;
@@ -185,19 +185,27 @@ __device__ __forceinline__ void load_tile(Packed<T>& pk, const char* row, int ti
     }
 }
 
+// the tile's largest value, with NaN turned into -inf (and noted)
+template <typename T>
+__device__ __forceinline__ float clean_tile(Packed<T>& pk, bool& saw_nan) {
+    float m = group_max_nan(pk);
+    if (m != m) { saw_nan = true; pk.clean_nan(); m = group_max_nan(pk); }
+    return m;
+}
+
 // exp16() relative to 0 with the exponents' rounding put back in: v k = x + d with x = fl(v k), 2^(v k) = 2^x (1 + d ln 2).
 // Relative to 0 an exponent of ten or so is rounded by 5e-7, where one relative to the row's maximum would be exact for
 // the entries that matter.  (-inf would make d a NaN: it enters as -1e30, whose weight is 0 as well.)
 __device__ __forceinline__ void exp16_precise(const float (&v)[16], float k, float (&e)[16]) {
-    const unsigned long long k2 = f32x2(k, k), zero = f32x2(0.0f, 0.0f), minus = f32x2(-1.0f, -1.0f), ln2 = f32x2(0.69314718f, 0.69314718f);
+    const unsigned long long k2 = f32x2(k, k), minus_k = f32x2(-k, -k), zero = f32x2(0.0f, 0.0f), minus_ln2 = f32x2(-0.69314718f, -0.69314718f);
 #pragma unroll
     for (int j = 0; j < 16; j += 2) {
         const unsigned long long vv = f32x2(max_nan(v[j], -1e30f), max_nan(v[j + 1], -1e30f));
-        const unsigned long long x = fma_f32x2(vv, k2, zero), d = fma_f32x2(vv, k2, fma_f32x2(x, minus, zero));
+        const unsigned long long x = fma_f32x2(vv, k2, zero), minus_d = fma_f32x2(vv, minus_k, x);
         float a, b;
         split_f32x2(x, a, b);
         const unsigned long long w = f32x2(ex2_approx(a), ex2_approx(b));
-        split_f32x2(fma_f32x2(fma_f32x2(w, ln2, zero), d, w), e[j], e[j + 1]);
+        split_f32x2(fma_f32x2(fma_f32x2(w, minus_ln2, zero), minus_d, w), e[j], e[j + 1]);
     }
 }
 __device__ __forceinline__ float weight_precise(float l, float k) {
@@ -222,6 +230,7 @@ __device__ __forceinline__ void mode_weights(int mode, const float (&q)[16], con
 // A block's place in its cluster and the row's tiles.
 struct Place {
     int rank, C, V, n_tiles, n_local;   // n_local: tiles rank, rank + C, ...
+    int per_block;                      // summation classes of a block
 };
 
 // What the working warps need to know about the sequence.
@@ -236,56 +245,52 @@ struct WorkRows {
     float* out_residual;         // kWrite
 };
 
-// Gumbel-Top-1 draw (Algorithm 6's last step, see gumbel_top1_pick() in rsd_verify_walk.inc): arg min of E(y) / w(y),
-// E(y) = t(U_M) / 16 + [y mod 16 != a] t(U_y).  E >= t(U_M) / 16 with equality at position a: the smallest key at the
-// positions a of the block's groups, from fast logarithms rounded up, bounds the winner from above, and only entries whose
-// lower bound reaches it (a few per block) are taken exactly.  The result is that of taking every entry.
-// (Exact logarithms and a second round of Philox calls for every group made this pass 25 us of a walk's 73.)
-template <typename T, int NT, int WARPS>
-__device__ __forceinline__ void top1_pass(Smem<WARPS, NT>& sm, const Place& pl, const RngKey& key, uint32_t node, int flags, float a_hi, float a_lo,
-                                          const float (&q)[NT][16], const float (&p)[NT][16]) {
-    constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const float inf = __int_as_float(0x7F800000);
-    uint32_t cw[NT][kRuns];                      // the groups' coarse-stream words
-    float bound = inf;
+// Gumbel-Top-1 draw (Algorithm 6's last step): arg max over y of log w(y) + G(y), which is the arg min of E(y) / w(y) with
+// E(y) = exp(-G(y)) = t(U_M) / 16 + [y mod 16 != a] t(U_y), the group-wise noise in its exponential form (streams
+// kTagFinalGumbelCoarse / Fine of the node).  Entries without weight are left out; equal keys go to the smaller token.
+// E >= t(U_M) / 16 with equality at position a: the smallest key at the positions a, from fast logarithms rounded up, bounds
+// the winner from above, and only entries whose lower bound reaches it are taken exactly.  The result is that of taking
+// every entry.  (Exact logarithms and a second round of Philox calls for every group made this pass 25 us of a walk's 73.
+// The fast logarithms lie within the margins below for each of the 2^28 words a group can have.)
+struct Top1 {
+    float bound;
+    unsigned long long best;                     // key bits << 32 | token: keys are >= 0, so the order is that of (key, token)
+
+    __device__ __forceinline__ Top1() : bound(-kNegInf), best(~0ull) {}
+
+    // t(U_M) / 16 of a group's word, down (up = -1) or up (+1) to a bound
+    __device__ __forceinline__ static float group_bound(uint32_t word, float up) {
+        const float t_hat = -__logf(fmaf((float)(word >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f));
+        return fmaxf(fmaf(up, fmaf(t_hat, 1e-6f, 2.5e-7f), t_hat), 0.0f) * 0.0625f;
+    }
+    // the coarse words of a lane's pieces of a tile; `bound` from the pieces' positions a
+    template <typename T, int RUNS>
+    __device__ __forceinline__ void look(const RngKey& key, uint32_t node, int tile, int lane, const float (&w)[16], uint32_t (&words)[RUNS]) {
+        constexpr int kPer = 16 / RUNS;
 #pragma unroll
-    for (int k = 0; k < NT; ++k) {
-        const int tile = pl.rank + pl.C * (warp + WARPS * k);
-        float w[16];
-        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
-#pragma unroll
-        for (int i = 0; i < kRuns; ++i) {
+        for (int i = 0; i < RUNS; ++i) {
             const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
             const uint32_t g = (uint32_t)x0 >> 4;
-            cw[k][i] = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
-            const float t_hat = -__logf(fmaf((float)(cw[k][i] >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f));
-            const float tg_hi = (t_hat + fmaf(t_hat, 1e-6f, 2.5e-7f)) * 0.0625f;
-            const int ja = (int)(cw[k][i] & 15u) - (x0 & 15);
+            words[i] = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
+            const float tg_hi = group_bound(words[i], 1.0f);
+            const int ja = (int)(words[i] & 15u) - (x0 & 15);
 #pragma unroll
             for (int j = 0; j < kPer; ++j)
-                if (j == ja && tile < pl.n_tiles && w[i * kPer + j] > 0.0f) bound = fminf(bound, tg_hi / w[i * kPer + j] * 1.00001f);
+                if (j == ja && w[i * kPer + j] > 0.0f) bound = fminf(bound, tg_hi / w[i * kPer + j] * 1.00001f);
         }
     }
-    bound = -warp_max(-bound);
-    if (lane == 0) sm.warp_top[0][warp] = bound;
-    workers_sync<WARPS * 32>();
-    bound = -warp_max(-(lane < WARPS ? sm.warp_top[0][lane] : inf));
-    unsigned long long best = ~0ull;             // key bits << 32 | token: keys are >= 0, so the order is that of (key, token)
+    // the exact keys of the entries that can reach `bound`
+    template <typename T, int RUNS>
+    __device__ __forceinline__ void take(const RngKey& key, uint32_t node, int tile, int lane, const float (&w)[16], const uint32_t (&words)[RUNS]) {
+        constexpr int kPer = 16 / RUNS;
 #pragma unroll
-    for (int k = 0; k < NT; ++k) {
-        const int tile = pl.rank + pl.C * (warp + WARPS * k);
-        float w[16];
-        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
-#pragma unroll
-        for (int i = 0; i < kRuns; ++i) {
+        for (int i = 0; i < RUNS; ++i) {
             const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
-            const float t_hat = -__logf(fmaf((float)(cw[k][i] >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f));
-            const float tg_lo = fmaxf(t_hat - fmaf(t_hat, 1e-6f, 2.5e-7f), 0.0f) * 0.0625f;
+            const float tg_lo = group_bound(words[i], -1.0f);
             uint32_t todo = 0;
 #pragma unroll
             for (int j = 0; j < kPer; ++j)
-                if (tile < pl.n_tiles && w[i * kPer + j] > 0.0f && tg_lo <= bound * w[i * kPer + j] * 1.00001f) todo |= 1u << j;
+                if (w[i * kPer + j] > 0.0f && tg_lo <= bound * w[i * kPer + j] * 1.00001f) todo |= 1u << j;
             while (todo) {
                 const int j = __ffs(todo) - 1;
                 todo &= todo - 1;
@@ -293,17 +298,22 @@ __device__ __forceinline__ void top1_pass(Smem<WARPS, NT>& sm, const Place& pl, 
 #pragma unroll
                 for (int jj = 0; jj < kPer; ++jj)
                     if (jj == j) wj = w[i * kPer + jj];
-                float e = neg_log_group_uniform_f32(cw[k][i]) * 0.0625f;
-                if (j != (int)(cw[k][i] & 15u) - (x0 & 15)) {
+                float e = neg_log_group_uniform_f32(words[i]) * 0.0625f;
+                if (j != (int)(words[i] & 15u) - (x0 & 15)) {
                     const uint4 fw = rng_draw(key, node, kTagFinalGumbelFine, (uint32_t)(x0 + j) >> 2);
                     const uint32_t sel = (uint32_t)(x0 + j) & 3u;
                     e += neg_log_uniform_f32(sel < 2 ? (sel == 0 ? fw.x : fw.y) : (sel == 2 ? fw.z : fw.w));
                 }
                 const float key_j = e / wj;
-                if (key_j < inf) best = min(best, ((unsigned long long)__float_as_uint(key_j) << 32) | (uint32_t)(x0 + j));
+                if (key_j < __int_as_float(0x7F800000)) best = min(best, ((unsigned long long)__float_as_uint(key_j) << 32) | (uint32_t)(x0 + j));
             }
         }
     }
+};
+// the block's smallest key goes to every block
+template <int WARPS, typename SM>
+__device__ __forceinline__ void top1_report(SM& sm, const Place& pl, int flags, unsigned long long best) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
     if (lane == 0) sm.warp_key[warp] = best;
@@ -315,25 +325,106 @@ __device__ __forceinline__ void top1_pass(Smem<WARPS, NT>& sm, const Place& pl, 
         send_word(at + 4u, __uint_as_float((uint32_t)(best >> 32)), bar);
     }
 }
+// The pass over tiles held in registers: the bound is the block's, from all its tiles.
+template <typename T, int NT, int WARPS>
+__device__ __forceinline__ void top1_pass(ChipSmem<WARPS, NT>& sm, const Place& pl, const RngKey& key, uint32_t node, int flags, float a_hi, float a_lo,
+                                          const float (&q)[NT][16], const float (&p)[NT][16]) {
+    constexpr int kRuns = (int)sizeof(T);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t words[NT][kRuns];
+    Top1 top1;
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        float w[16];
+        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+        const int tile = pl.rank + pl.C * (warp + WARPS * k);    // (beyond the row: no weight)
+        top1.look<T>(key, node, tile, lane, w, words[k]);
+    }
+    top1.bound = -warp_max(-top1.bound);
+    if (lane == 0) sm.warp_top[0][warp] = top1.bound;
+    workers_sync<WARPS * 32>();
+    top1.bound = -warp_max(-(lane < WARPS ? sm.warp_top[0][lane] : top1.bound));
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        float w[16];
+        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+        top1.take<T>(key, node, pl.rank + pl.C * (warp + WARPS * k), lane, w, words[k]);
+    }
+    top1_report<WARPS>(sm, pl, flags, top1.best);
+}
+
+// The lanes' sums in sm.lane_sum, added per summation class in the order of the pass, to every block.
+template <int WARPS, typename SM>
+__device__ __forceinline__ void send_class_sums(SM& sm, const Place& pl, int flags) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per_block = pl.per_block, buf = flags & kBuffer ? 1 : 0;
+    for (int i = warp; i < ((flags & kKindMask) == kOpen ? 2 * per_block : per_block); i += WARPS) {
+        const int which = i >= per_block ? 1 : 0, cl = i - which * per_block;
+        const int n = pl.n_local > cl ? (pl.n_local - cl + per_block - 1) / per_block : 0;
+        const int step = flags & kBackward ? -per_block : per_block, at = flags & kBackward ? cl + per_block * (n - 1) : cl;
+        float acc = 0.0f;
+        for (int m0 = 0; m0 < n; m0 += 8) {
+            float v[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) v[m] = m0 + m < n ? sm.lane_sum[which][at + step * (m0 + m)][lane] : 0.0f;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) acc += v[m];
+        }
+        acc = warp_sum_f32(acc);
+        if (lane < pl.C)
+            send_word(remote_addr(&sm.class_sum[buf][which * kClasses + pl.rank + pl.C * cl], lane), acc, remote_addr(&sm.red_bar[buf], lane));
+    }
+}
+// kClean: the rows' maxima and whether a NaN was met, to every block
+template <int WARPS, typename SM>
+__device__ __forceinline__ void send_tops(SM& sm, const Place& pl, int flags) {
+    const int lane = threadIdx.x & 31, buf = flags & kBuffer ? 1 : 0;
+    if ((threadIdx.x >> 5) != WARPS - 1) return;
+    const float mq = warp_max(lane < WARPS ? sm.warp_top[0][lane] : kNegInf), mp = warp_max(lane < WARPS ? sm.warp_top[1][lane] : kNegInf);
+    if (lane < pl.C) {
+        const uint32_t bar = remote_addr(&sm.red_bar[buf], lane);
+        send_word(remote_addr(&sm.extra[buf][0][pl.rank], lane), mq, bar);
+        send_word(remote_addr(&sm.extra[buf][1][pl.rank], lane), mp, bar);
+        send_word(remote_addr(&sm.extra[buf][2][pl.rank], lane), sm.nan_seen ? 1.0f : 0.0f, bar);
+    }
+}
+// a tile's normalised weights to global memory
+template <typename T>
+__device__ __forceinline__ void write_tile(float* out, int tile, int lane, int V, const float (&w)[16], double inv) {
+    constexpr int kPer = 16 / (int)sizeof(T);
+    const bool vec = ((uintptr_t)out & 15u) == 0;
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) {
+        const int x = tile * kTileElems + ((i / kPer) * 32 + lane) * kPer + i % kPer;
+        float o[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o[j] = (float)((double)w[i + j] * inv);
+        if (vec && x + 4 <= V) {
+            *(float4*)(out + x) = make_float4(o[0], o[1], o[2], o[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (x + j < V) out[x + j] = o[j];
+        }
+    }
+}
 
 // The working warps: the passes they are told to run.  The root's rows are asked for before the first command is there.
 // MODE: which of the rarer passes exist.
 template <typename T, int NT, int WARPS, int MODE>
-__device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const WorkRows& rows) {
+__device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, const WorkRows& rows) {
     constexpr int kAll = (WARPS + 1) * 32, kWorkers = WARPS * 32;
     constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int C = pl.C, V = pl.V, n_tiles = pl.n_tiles;
     const int tile0 = pl.rank + C * warp, tile_step = C * WARPS;   // this warp's tiles: tile0, tile0 + tile_step, ...
-    const int per_block = kClasses / C;                            // summation classes of this block
     float q[NT][16], p[NT][16];
 #pragma unroll
     for (int k = 0; k < NT; ++k)
 #pragma unroll
         for (int j = 0; j < 16; ++j) q[k][j] = p[k][j] = 0.0f;
-    int flags = rows.with_draft ? kOpen : kOpenTarget, node = 0;
+    int flags = (rows.with_draft ? kOpen : kOpenTarget) | kFirst, node = 0;
     float a_hi = 0.0f, a_lo = 0.0f;
-    int n_cmd = 0;                      // commands read
     for (;;) {
         int kind = flags & kKindMask;
         float s[NT];
@@ -351,12 +442,11 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                     if (kind == kOpen) load_tile<T>(rp[k], rowp, tile, lane, V);
                 }
             }
-            if (n_cmd == 0) {
+            if (flags & kFirst) {
                 cluster_wait();         // every block's mbarriers are in place
                 cmd_sync<kAll>(0);
                 flags = sm.cmd[0].flags;   // the root's rows, with or without the draft row
                 kind = flags & kKindMask;
-                n_cmd = 1;
             }
             float cq = 0.0f, cp = 0.0f;
             const bool precise = rows.precise && !(flags & kRelative);
@@ -367,14 +457,8 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                     bool saw_nan = false;
 #pragma unroll
                     for (int k = 0; k < NT; ++k) {
-                        float m = group_max_nan(rq[k]);
-                        if (m != m) { saw_nan = true; rq[k].clean_nan(); m = group_max_nan(rq[k]); }
-                        mq = fmaxf(mq, m);
-                        if (kind == kOpen) {
-                            m = group_max_nan(rp[k]);
-                            if (m != m) { saw_nan = true; rp[k].clean_nan(); m = group_max_nan(rp[k]); }
-                            mp = fmaxf(mp, m);
-                        }
+                        mq = fmaxf(mq, clean_tile(rq[k], saw_nan));
+                        if (kind == kOpen) mp = fmaxf(mp, clean_tile(rp[k], saw_nan));
                     }
                     mq = warp_max(mq);
                     mp = warp_max(mp);
@@ -459,28 +543,13 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
         } else if (MODE == kResample && kind == kWrite) {
             dump_sync<kAll>();                  // everyone has read the command
             const double inv = sm.inv_total;
-            float* out = rows.out_residual;
-            const bool vec = ((uintptr_t)out & 15u) == 0;
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
                 const int tile = tile0 + tile_step * k;
                 if (tile >= n_tiles) continue;
                 float w[16];
                 mode_weights<false>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, 0.0f, w);
-#pragma unroll
-                for (int i = 0; i < 16; i += 4) {
-                    const int x = tile * kTileElems + ((i / kPer) * 32 + lane) * kPer + i % kPer;
-                    float o[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) o[j] = (float)((double)w[i + j] * inv);
-                    if (vec && x + 4 <= V) {
-                        *(float4*)(out + x) = make_float4(o[0], o[1], o[2], o[3]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (x + j < V) out[x + j] = o[j];
-                    }
-                }
+                write_tile<T>(rows.out_residual, tile, lane, V, w, inv);
             }
         } else if (MODE == kRuleWalk && kind == kTop1) {
             top1_pass<T, NT, WARPS>(sm, pl, rows.key, (uint32_t)node, flags, a_hi, a_lo, q, p);
@@ -492,22 +561,7 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
             for (int k = 0; k < NT; ++k) sm.lane_sum[0][warp + WARPS * k][lane] = s[k];
             workers_sync<kWorkers>();           // the lanes' sums are in place
             const int buf = flags & kBuffer ? 1 : 0;
-            for (int i = warp; i < (kind == kOpen ? 2 * per_block : per_block); i += WARPS) {
-                const int which = i >= per_block ? 1 : 0, cl = i - which * per_block;
-                const int n = pl.n_local > cl ? (pl.n_local - cl + per_block - 1) / per_block : 0;
-                const int step = flags & kBackward ? -per_block : per_block, at = flags & kBackward ? cl + per_block * (n - 1) : cl;
-                float acc = 0.0f;
-                for (int m0 = 0; m0 < n; m0 += 8) {
-                    float v[8];
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) v[m] = m0 + m < n ? sm.lane_sum[which][at + step * (m0 + m)][lane] : 0.0f;
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) acc += v[m];
-                }
-                acc = warp_sum_f32(acc);
-                if (lane < C)
-                    send_word(remote_addr(&sm.class_sum[buf][which * kClasses + pl.rank + C * cl], lane), acc, remote_addr(&sm.red_bar[buf], lane));
-            }
+            send_class_sums<WARPS>(sm, pl, flags);
             if (flags & kStoreTiles) {
 #pragma unroll
                 for (int k = 0; k < NT; ++k) {
@@ -516,19 +570,11 @@ __device__ __forceinline__ void work(Smem<WARPS, NT>& sm, const Place& pl, const
                     if (lane < C && tile < n_tiles) send_word(remote_addr(&sm.tile_sum[tile], lane), ts, remote_addr(&sm.red_bar[buf], lane));
                 }
             }
-            if ((flags & kClean) && warp == WARPS - 1) {
-                const float mq = warp_max(lane < WARPS ? sm.warp_top[0][lane] : kNegInf), mp = warp_max(lane < WARPS ? sm.warp_top[1][lane] : kNegInf);
-                if (lane < C) {
-                    const uint32_t bar = remote_addr(&sm.red_bar[buf], lane);
-                    send_word(remote_addr(&sm.extra[buf][0][pl.rank], lane), mq, bar);
-                    send_word(remote_addr(&sm.extra[buf][1][pl.rank], lane), mp, bar);
-                    send_word(remote_addr(&sm.extra[buf][2][pl.rank], lane), sm.nan_seen ? 1.0f : 0.0f, bar);
-                }
-            }
+            if (flags & kClean) send_tops<WARPS>(sm, pl, flags);
         }
-        cmd_sync<kAll>(n_cmd);
-        const Cmd cmd = sm.cmd[n_cmd & 1];
-        ++n_cmd;
+        const int odd = flags & kBuffer ? 0 : 1;   // the next command
+        cmd_sync<kAll>(odd);
+        const Cmd cmd = sm.cmd[odd];
         flags = cmd.flags;
         node = cmd.node;
         a_hi = cmd.a_hi;
@@ -544,10 +590,10 @@ __device__ __forceinline__ double class_tree(double v) {
 }
 
 // The control warp: the walk itself, the same in every block of the cluster.
-template <typename T, int NT, int WARPS, int MODE>
+template <typename T, typename SM, int WARPS, int MODE>
 struct Control {
     static constexpr int kAll = (WARPS + 1) * 32;
-    Smem<WARPS, NT>& sm;
+    SM& sm;
     const ClusterArgs& ca;
     const VerifyArgs& a;
     const Place& pl;
@@ -563,29 +609,29 @@ struct Control {
     float a_hi, a_lo;               // A Sq / Sp as a two-float sum
     int status;
 
-    __device__ __forceinline__ Control(Smem<WARPS, NT>& sm_, const ClusterArgs& ca_, const Place& pl_, int b_, bool precise_)
+    __device__ __forceinline__ Control(SM& sm_, const ClusterArgs& ca_, const Place& pl_, int b_, bool precise_)
         : sm(sm_), ca(ca_), a(ca_.v), pl(pl_), b(b_), precise(precise_), lane(threadIdx.x & 31),
           key{ca_.v.seed_lo, ca_.v.seed_hi, ca_.v.step, ca_.v.seq_base + (uint32_t)b_}, cmd_no(0), backward(0), aborted(false),
           kq(kLog2e * ca_.v.target.inv_temp), kp(kLog2e * ca_.v.draft.inv_temp), mq(0.0f), mp(0.0f), A(0.0), Z(1.0), a_hi(0.0f), a_lo(0.0f),
           status(0) {}
 
     __device__ __forceinline__ void publish(int flags, int node) {
+        const int odd = cmd_no & 1;
         if (lane == 0) {
             Cmd cmd;
-            cmd.flags = flags;
+            cmd.flags = flags | (odd ? kBuffer : 0);
             cmd.node = node;
             cmd.a_hi = a_hi;
             cmd.a_lo = a_lo;
-            sm.cmd[cmd_no & 1] = cmd;
+            sm.cmd[odd] = cmd;
         }
-        cmd_arrive<kAll>(cmd_no);
+        cmd_arrive<kAll>(odd);
         ++cmd_no;
     }
     // publish a pass that reports `words` words to every block
     __device__ __forceinline__ void issue(int flags, int node, int words) {
-        const int buf = cmd_no & 1;
-        if (lane == 0) mbar_expect_tx(&sm.red_bar[buf], 4u * (uint32_t)words);
-        publish(flags | (buf ? kBuffer : 0) | (backward ? kBackward : 0), node);
+        if (lane == 0) mbar_expect_tx(&sm.red_bar[cmd_no & 1], 4u * (uint32_t)words);
+        publish(flags | (backward ? kBackward : 0), node);
         backward ^= 1;
     }
     // wait for the words of the latest pass; sets `aborted` when they do not come
@@ -731,19 +777,6 @@ struct Control {
             if (lane == 0) store_remote(remote_addr(&sm.gave_up, 0), 1);
         }
     }
-    // Rank 0 when the cluster is through: if a wait ran out in any block, the sequence's outputs say so.  (That block need not be
-    // the one that writes them; the writes so far are ordered before this by the cluster's barrier.)
-    __device__ __forceinline__ void report_timeout() {
-        if (pl.rank != 0 || lane != 0 || !sm.gave_up) return;
-        if (MODE == kResample) {
-            ca.r.out_token[b] = -1;
-            ca.r.status[b] |= 32;
-        } else {
-            a.last_token[b] = -1;
-            a.status[b] |= 32;
-        }
-    }
-
     // What is left of the draft once subtraction has lost its accuracy: summed anew without the rejected tokens.
     __device__ __forceinline__ double rest(int n_removed) {
         if (lane == 0) sm.n_gone_tok = n_removed;
@@ -1045,19 +1078,28 @@ struct Control {
     }
 };
 
-template <typename T, int NT, int WARPS, int MODE>
-__global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 2) : 1) walk_cluster_kernel(const __grid_constant__ ClusterArgs ca) {
-    __shared__ Smem<WARPS, NT> sm;
+// By a thread of rank 0 when the cluster is through: a wait ran out in some block, which the sequence's outputs say.  (That block need
+// not be the one that has written them; what was written so far is ordered before this by the cluster's barrier.)
+template <int MODE>
+__device__ __forceinline__ void report_timeout(const ClusterArgs& ca, int b) {
+    (MODE == kResample ? ca.r.out_token : ca.v.last_token)[b] = -1;
+    (MODE == kResample ? ca.r.status : ca.v.status)[b] |= 32;   // RSD_ST_TIMEOUT
+}
+
+// A walk by the blocks of a cluster: `work` is what the working warps do.
+template <typename T, int MODE, int WARPS, typename SM, typename F>
+__device__ __forceinline__ void run_walk(SM& sm, const ClusterArgs& ca, F&& work) {
     const VerifyArgs& a = ca.v;
     Place pl;
     pl.rank = (int)cluster_rank();
     pl.C = (int)cluster_size();
     pl.V = a.V;
     pl.n_tiles = (a.V + kTileElems - 1) / kTileElems;
+    pl.per_block = kClasses / pl.C;
     pl.n_local = pl.n_tiles > pl.rank ? (pl.n_tiles - pl.rank + pl.C - 1) / pl.C : 0;
     const int b = blockIdx.x / pl.C;
-    // Rows off 16-byte boundaries, the baseline rules and the residual draw never take the ring walk: no bits to match.
-    const bool precise = MODE != kPlainWalk || ca.off_boundaries;
+    // Rows that the ring walk does not take, the baseline rules and the residual draw have no bits to match.
+    const bool precise = MODE != kPlainWalk || !ca.ring_rows;
     if (threadIdx.x == WARPS * 32) {
         mbar_init(&sm.red_bar[0], 1);
         mbar_init(&sm.red_bar[1], 1);
@@ -1079,19 +1121,25 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 
         rows.precise = precise;
         rows.key = RngKey{a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
         rows.out_residual = MODE == kResample && ca.r.out_residual ? ca.r.out_residual + (int64_t)b * a.V : nullptr;
-        work<T, NT, WARPS, MODE>(sm, pl, rows);
+        work(pl, rows);
         grid_started();
         cluster_arrive();   // nothing is on its way to a block that has left
         cluster_wait();
     } else {
-        Control<T, NT, WARPS, MODE> control(sm, ca, pl, b, precise);
+        Control<T, SM, WARPS, MODE> control(sm, ca, pl, b, precise);
         if constexpr (MODE == kResample) control.resample();
         else control.walk();
         grid_started();
         cluster_arrive();
         cluster_wait();
-        control.report_timeout();
+        if (threadIdx.x == WARPS * 32 && sm.gave_up) report_timeout<MODE>(ca, blockIdx.x / cluster_size());
     }
+}
+
+template <typename T, int NT, int WARPS, int MODE>
+__global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 2) : 1) walk_cluster_kernel(const __grid_constant__ ClusterArgs ca) {
+    __shared__ ChipSmem<WARPS, NT> sm;
+    run_walk<T, MODE, WARPS>(sm, ca, [&](const Place& pl, const WorkRows& rows) { work<T, NT, WARPS, MODE>(sm, pl, rows); });
 }
 
 }  // namespace walk_cluster

@@ -1,0 +1,7 @@
+#include "rsd_walk_stream_launch.cuh"
+
+namespace rsd {
+namespace walk_cluster {
+void launch_stream_f32(const ClusterArgs& a, bool extra, int B, int C, int per_sm, cudaStream_t s) { launch_stream_of<float>(a, extra, B, C, per_sm, s); }
+}  // namespace walk_cluster
+}  // namespace rsd

@@ -1,0 +1,135 @@
+"""Which kernel walks a sequence is a matter of the batch, the rows and the rule: a cluster that holds the rows on chip (in one of
+several shapes), one block or eight that read them in every pass, or, for plain walks over rows on 16-byte boundaries, the ring.
+None of it may show: a few sequences alone give the bits they give inside a large batch, and all agree with the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads
+from tests.parity import Tally, compare_verify
+from tests.test_gpu_parity import _np
+from tests.test_gpu_walk_cluster import _drafted, _tokens
+
+pytestmark = pytest.mark.gpu
+
+
+def _whole_and_parts(rsd, draft, target, parent, token, L, rule=0, gamma=2.0, sampler=0, n=4):
+    B = draft.shape[0]
+    parent = torch.from_numpy(parent).cuda()
+    whole = rsd.rsd_verify_tree_rule(draft, target, parent, token, L, rule, gamma, sampler, 3, 0, want_theta=True)
+    for b in (0, B // 2, B - n):
+        part = rsd.rsd_verify_tree_rule(draft[b:b + n], target[b:b + n], parent, token[b:b + n].contiguous(), L, rule, gamma, sampler, 3, 0,
+                                        seq_base=b, want_theta=True)
+        for key in part:
+            got, want = part[key].cpu().numpy(), whole[key][b:b + n].cpu().numpy()
+            assert np.array_equal(got, want, equal_nan=got.dtype.kind == "f"), (key, b, got, want)
+    return whole
+
+
+# batches beyond the limits of the on-chip walk, and (rows beyond 131,072 entries) on both sides of eight blocks a sequence
+@pytest.mark.parametrize("dtype,V,B,off,rule,sampler,trouble", [
+    ("bf16", 32001, 300, 1, 0, 0, ""), ("bf16", 32001, 230, 7, 0, 0, "nan"), ("f32", 16389, 600, 3, 0, 0, "nan"), ("bf16", 8201, 800, 1, 0, 0, "far"),
+    ("bf16", 65551, 200, 1, 0, 0, "far"), ("bf16", 32000, 300, 0, 1, 0, ""), ("bf16", 16400, 600, 0, 2, 0, "nan"), ("f32", 8208, 800, 0, 2, 1, "far"),
+    ("bf16", 32000, 560, 0, 1, 1, ""), ("bf16", 32000, 280, 0, 2, 1, "far"), ("f32", 8193, 1600, 1, 0, 1, ""), ("bf16", 131072, 200, 0, 1, 0, "far"),
+    ("f32", 131073, 240, 1, 0, 0, "nan"), ("f32", 151936, 240, 0, 0, 0, "far"), ("bf16", 140001, 160, 1, 2, 0, ""), ("bf16", 262144, 160, 0, 1, 1, "nan")])
+def test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble):
+    import paper_2402_14160_b200 as rsd
+    branching = (3, 2) if B * V < 3e7 else (2, 1)
+    draft, target, _ = _drafted(B, V, dtype, branching, 7000 + V, off=off)
+    if trouble == "nan":
+        draft[::3, 0, V // 2] = float("nan")
+        target[1::5, 0, V - 1] = float("nan")
+    elif trouble == "far":
+        target += 300.0
+        draft[::2] -= 120.0
+    token = _tokens(rsd, draft, branching, 3)
+    _whole_and_parts(rsd, draft, target, workloads.rsdc_parent_array(branching), token, 2, rule, 2.0, sampler)
+
+
+@pytest.mark.parametrize("dtype,V,B", [("f32", 32000, 400), ("bf16", 32001, 400), ("f32", 140001, 160), ("bf16", 262144, 310)])
+@pytest.mark.parametrize("k", [0, 3])
+def test_the_route_of_a_residual_draw_does_not_show(dtype, V, B, k):
+    import paper_2402_14160_b200 as rsd
+    gen = torch.Generator(device="cuda").manual_seed(V + k)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    draft = (torch.randn((B, V), generator=gen, device="cuda") * 2).to(dt)
+    target = (draft.float() + torch.randn((B, V), generator=gen, device="cuda")).to(dt)
+    rejected = torch.randint(0, V, (B, k), generator=gen, device="cuda", dtype=torch.int32) if k else None
+    node = torch.arange(B, dtype=torch.int32, device="cuda")
+    whole = rsd.rsd_resample_residual(draft, target, rejected, node, 5, 1, want_residual=True)
+    n = 3
+    for b in (0, B - n):
+        part = rsd.rsd_resample_residual(draft[b:b + n], target[b:b + n], rejected[b:b + n] if k else None, node[b:b + n], 5, 1, seq_base=b,
+                                         want_residual=True)
+        for key in part:
+            assert torch.equal(part[key], whole[key][b:b + n]), (key, b)
+
+
+@pytest.mark.parametrize("dtype,V,B,off", [("bf16", 140000, 2, 0), ("f32", 140001, 2, 1), ("bf16", 131073, 230, 1), ("f32", 16401, 240, 3), ("bf16", 16401, 300, 1)])
+@pytest.mark.parametrize("rule,sampler", [(0, 0), (1, 0), (2, 0), (0, 1), (2, 1)])
+def test_walks_over_rows_read_in_every_pass_match_oracle(dtype, V, B, off, rule, sampler):
+    import paper_2402_14160_b200 as rsd
+    branching = (2, 2) if V * B < 3e5 else (2, 1)
+    draft, target, _ = _drafted(B, V, dtype, branching, 9000 + V, off=off)
+    token = _tokens(rsd, draft, branching, 11)
+    parent = workloads.rsdc_parent_array(branching)
+    g = _np(rsd.rsd_verify_tree_rule(draft, target, torch.from_numpy(parent).cuda(), token, 2, rule, 2.0, sampler, 11, 0, want_theta=True))
+    n = min(B, 6)                                          # (the rest of a large batch: the test above)
+    o = oracle.verify_tree(workloads.as_oracle_rows(draft[:n].contiguous()), workloads.as_oracle_rows(target[:n].contiguous()), parent,
+                           token[:n].cpu().numpy(), 2, 11, 0, rule=rule, gamma=2.0, final_sampler=sampler)
+    g = {key: v[:n] for key, v in g.items()}
+    t = Tally()
+    compare_verify(t, g, o, parent)
+    t.check()
+    assert np.array_equal(g["status"], o["status"])
+
+
+@pytest.mark.parametrize("dtype,V,B", [("f32", 140001, 3), ("bf16", 262143, 2), ("bf16", 140001, 160)])
+@pytest.mark.parametrize("k", [0, 1, 32])
+def test_residual_draws_over_rows_read_in_every_pass_match_oracle(dtype, V, B, k):
+    import paper_2402_14160_b200 as rsd
+    gen = torch.Generator(device="cuda").manual_seed(V + k)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    draft = (torch.randn((B, V), generator=gen, device="cuda") * 2).to(dt)
+    target = (draft.float() + torch.randn((B, V), generator=gen, device="cuda")).to(dt)
+    rej = None
+    if k:                                                  # both ends of the row and of its tiles, one of them twice; then the draft's favourites
+        edges = [V - 1, 0, 511, 512, V - 513, 4096, 0, 1, 15, 16]
+        rej = np.concatenate([np.tile(np.array(edges[:k], np.int32), (B, 1)),
+                              torch.topk(draft.float(), max(1, k - len(edges)), dim=1).indices.int().cpu().numpy()], axis=1)[:, :k].copy()
+    nodes = torch.arange(B, dtype=torch.int32, device="cuda")
+    g = _np(rsd.rsd_resample_residual(draft, target, None if rej is None else torch.from_numpy(rej).cuda(), nodes, 5, 1, want_residual=True))
+    n = min(B, 3)
+    o = oracle.resample_residual(workloads.as_oracle_rows(draft[:n]), workloads.as_oracle_rows(target[:n]), None if rej is None else rej[:n],
+                                 nodes[:n].cpu().numpy(), 5, 1)
+    assert np.all(np.abs(g["residual"][:n] - o["residual"]) <= 1e-5 * o["residual"].max(axis=1, keepdims=True))
+    assert np.array_equal(g["status"][:n], o["status"])
+    assert np.all(o["margin"][g["token"][:n] != o["token"]] <= 1e-5)
+
+
+# What large batches seldom meet: the ring (rows on 16-byte boundaries) and the streamed walk (off them) against small batches, which the
+# oracle tests cover.
+@pytest.mark.parametrize("V,B", [(512, 1400), (16389, 260)])
+@pytest.mark.parametrize("what", ["repeated", "many_children", "large_tree", "peaked"])
+def test_rare_paths_of_large_batches(what, V, B):
+    import paper_2402_14160_b200 as rsd
+    branching = {"repeated": (4,), "many_children": (32, 2), "large_tree": (20, 20), "peaked": (6, 2)}[what]
+    draft, target, P = _drafted(B, V, "bf16", branching, 60 + V)
+    if what in ("many_children", "large_tree"):
+        target = (-1.5 * torch.cat([draft, draft[:, :1].expand(B, target.shape[1] - P, V)], dim=1).float() + 0.3 * target.float()).to(draft.dtype)
+    if what == "peaked":                                   # the rejected tokens hold all but a sliver of the draft
+        draft[:, :, 7::100] += 18.0
+    token = _tokens(rsd, draft, branching, 3)
+    if what == "repeated":
+        token[:, 3] = token[:, 1]
+        target[:, 0].scatter_add_(1, token[:, 1:3].long(), torch.full((B, 2), -9.0, dtype=target.dtype, device="cuda"))
+    parent = workloads.rsdc_parent_array(branching)
+    if what == "many_children":                            # the last level's 64 nodes become children of the root as well
+        parent[33:] = 0
+    whole = _whole_and_parts(rsd, draft, target, parent, token, len(branching), n=40)
+    tested = (~torch.isnan(whole["theta"])).sum(dim=1)
+    if what == "many_children":
+        assert int(tested.max()) > 64
+    if what == "repeated":
+        assert int((whole["status"] & rsd.ST_ZERO_DRAFT_PROB != 0).sum()) > B // 2
