@@ -845,8 +845,18 @@ struct Control {
                 const uint4 rw = rng_draw(key, (uint32_t)cur, kTagAccept, (uint32_t)(j0 + lane));
                 Ud = (double)(rw.x >> 8) * (1.0 / 16777216.0);
                 // an earlier sibling with the same token: rejected by the time this one is tested, its draft mass is gone (Eq. 1)
-                repeated = (__match_any_sync(0xFFFFFFFFu, child_x) & ((1u << lane) - 1u)) != 0u;
-                for (int i = 0; i < n_removed && j0 > 0; ++i) repeated |= sm.gone_tok[i] == child_x;
+                const unsigned same = __match_any_sync(0xFFFFFFFFu, child_x);
+                repeated = (same & ((1u << lane) - 1u)) != 0u;
+                if (j0 > 0) {
+                    bool listed = false;
+                    for (int i = 0; i < n_removed; ++i) listed |= sm.gone_tok[i] == child_x;
+                    if (n_removed + 32 > kMaxListed) {   // (the ring walk does not know a token again that it has not listed)
+                        const int first = __ffs(same) - 1;
+                        const unsigned fresh = __ballot_sync(0xFFFFFFFFu, !listed && !repeated);
+                        repeated = repeated && n_removed + __popc(fresh & ((1u << first) - 1u)) < kMaxListed;
+                    }
+                    repeated |= listed;
+                }
                 if (rule != 0) repeated = false;      // (the baselines never change the draft)
             };
             fetch_children();
