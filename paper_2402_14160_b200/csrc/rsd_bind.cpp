@@ -289,6 +289,11 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "bind(path, exception class)");
         return nullptr;
     }
+    static PyObject* bound = nullptr;         // one library per process: the entry points below are not per caller
+    if (bound && PyUnicode_Compare(bound, a[0]) != 0) {
+        PyErr_Format(PyExc_RuntimeError, "already bound to %U", bound);
+        return nullptr;
+    }
     void* lib = dlopen(path, RTLD_NOW | RTLD_LOCAL);
     if (!lib) {
         PyErr_SetString(PyExc_OSError, dlerror());
@@ -311,6 +316,10 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!all) {
         PyErr_Format(PyExc_OSError, "%s lacks an entry point", path);
         return nullptr;
+    }
+    if (!bound) {
+        Py_INCREF(a[0]);
+        bound = a[0];
     }
     Py_INCREF(a[1]);
     Py_XDECREF(g_error);

@@ -37,3 +37,11 @@ def test_argument_validation_needs_no_gpu():
     rows = api.RsdRows(16, 0, 0, 8, 8)
     code = lib.rsd_gumbel_topk_draft(ctypes.byref(rows), 1, 1, 0, k, k, 1, 0, 0, 0, None, None, None, None, None, 0, None, None)
     assert code == 2
+
+
+def test_the_binding_serves_one_library():
+    import pytest
+    native = api._bind()
+    native.bind(api.LIB_PATH, api.RsdError)                        # the same one again
+    with pytest.raises(RuntimeError, match="already bound"):
+        native.bind(api.LIB_PATH + ".other", api.RsdError)
