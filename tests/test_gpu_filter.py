@@ -184,3 +184,12 @@ def test_filter_rows_far_from_zero_keep_their_shares(rsd, dtype, V):
         want = oracle.filter_rows(workloads.as_oracle_rows(rows), top_k, top_p, temperature=T)["kept"]
         # exact to 1e-6 of a row's mass (exponents of up to 50 in fp32), so a cut in a run of equal tokens to less than one of them
         assert np.abs(kept - want).max() <= 1, (kept, want)
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 109716), ("f32", 54858)])
+def test_filter_rows_of_the_longest_rows_that_fit(rsd, dtype, V):
+    rows = _rows((1, 2, V + 1), dtype, 2.0, V)
+    for top_k, top_p in ((0, 0.95), (2000, 0.9)):
+        _check_filter(rsd, rows[:, :, :V], top_k, top_p, 1.0)
+    with pytest.raises(rsd.RsdError, match="at most %d entries" % V):
+        rsd.rsd_filter_rows(rows, 0, 0.9)
