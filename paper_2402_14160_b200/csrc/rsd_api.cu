@@ -21,13 +21,18 @@ thread_local cudaEvent_t g_scan_before = nullptr, g_scan_after = nullptr;  // on
 
 // Threads per row.  A block is a row; 128 threads give the most rows in flight and the least work per row (the stages after
 // the streaming loop cost a row the same whatever its threads), but with few rows most of the chip waits for the longest.
-// Without a log-sum-exp (us; 128 / 256 / 512 threads, launch included, 32,000 fp32): 32 rows 12.7 / 10.4 / 10.4, 192 rows
-// 17.1 / 14.5 / 14.5, 320 rows 18.6 / 16.6 / 20.4, 640 rows 25.5 / 29.1 / 29.7.  Rows of more than 65,536 entries carry
-// over 16 KB of bounds, so that blocks of 128 threads no longer fill an SM: 128,000 entries, 3000 rows, bf16 196 / 145 / 157,
-// fp32 274 / 262 / 241.
+// Without a log-sum-exp (us; 128 / 256 / 512 threads, launches back to back, bf16):
+//       rows         64                   222                  300                  600
+//       4,096        6.6 /  6.1 /  6.2    6.8 /  6.4 /  6.8    6.7 /  6.5 /  9.8    8.1 / 11.0 / 16.0
+//       16,384       7.2 /  6.2 /  6.4    9.1 /  7.9 /  8.1    9.3 /  8.1 / 12.2    10.4 / 12.9 / 17.6
+//       49,152       13.6 / 9.8 /  9.1    14.4 / 11.0 / 10.7   14.8 / 11.6 / 16.2   17.4 / 20.9 / 24.4
+// (256 threads would also be 0.1 to 0.3 us ahead for 223 to 370 rows of 4,096 to 16,383 entries, and 512 are as much behind 256 at
+// 16,384.)  Rows of more than 65,536 entries carry over 16 KB of bounds, so that blocks of 128 threads no longer fill an SM:
+// 128,000 entries, 3000 rows, bf16 196 / 145 / 157, fp32 274 / 262 / 241.
 // A log-sum-exp must come out the same in every launch, and its sums follow the warps: up to 65,536 entries they are those of
 // four warps (few rows: 256 threads with the sums on four warps and the perturbed values on the others), beyond those of
-// eight (256 threads at every size; 128,000 bf16, 192 / 5000 rows: 43 / 370 with 128 threads, 27 / 247 with 256).
+// eight, by 256 threads in every launch (bf16, 64 / 222 / 370 / 600 rows of 16,384: 8.4 / 10.5 / 11.1 / 12.3 with 128 threads, 8.1 / 10.0 / 10.8 /
+// 17.0 with 256; 192 / 5000 rows of 128,000: 43 / 370 with 128, 27 / 247 with 256).
 int scan_threads(int rows, int V, bool f32, bool need_lse) {
     static const int sms = [] {
         int dev = 0, n = 0;
