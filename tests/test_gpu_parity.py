@@ -345,9 +345,9 @@ def test_verify_tree_special_trees(rsd):
                                                        ("f32", 51, (40,), False)])
 def test_verify_tree_wide_and_large_trees(rsd, dtype, V, branching, aligned):
     # b = (20, 20): 421 nodes, more than the walk kernels keep in shared memory, so the children are searched in
-    # global memory; b = (40, ...): a node with 40 children, more rejections than a warp has lanes (the row values
-    # of the later children are no longer fetched ahead) and, with the draft far from the target, more removed
-    # tokens than the 32 the register-fed walk remembers.  aligned=False: rows at odd offsets (register-fed walk).
+    # global memory; b = (40, ...): a node with 40 children, more than a warp has lanes (the later ones are fetched in a
+    # second batch of 32) and, with the draft far from the target, more than 32 rejections.  aligned=False: rows at odd offsets.
+    # (24 sequences: clusters; the same in batches that other kernels walk: test_gpu_walk_routes.py)
     B = 24
     L = len(branching)
     parent = workloads.rsdc_parent_array(branching)
@@ -374,7 +374,7 @@ def test_verify_tree_wide_and_large_trees(rsd, dtype, V, branching, aligned):
     assert tested.max() >= branching[0] // 2                       # some walk went through many children of a node
 
 
-@pytest.mark.parametrize("V", [128, 127])      # rows on and off 16-byte boundaries: the two walks
+@pytest.mark.parametrize("V", [128, 127])      # rows on and off 16-byte boundaries
 def test_verify_tree_repeated_sibling_tokens(rsd, V):
     # Two children of a node carry the same token (a caller's tree; Gumbel-Top-k never drafts one): once the first is
     # rejected its draft mass is gone (Eq. 1), so the second is a child the draft could not have produced: threshold 0
@@ -401,7 +401,7 @@ def test_verify_tree_repeated_sibling_tokens(rsd, V):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_verify_tree_rows_far_from_zero_and_nan_logits(rsd, dtype):
-    # The copy-engine walk takes its first pass relative to a reference of 0: rows shifted by +-120 (sums over- or
+    # The walks take their first pass relative to a reference of 0: rows shifted by +-120 (sums over- or
     # underflow), rows of which only one far-away entry is finite, and rows with NaN logits make it fall back on the
     # rows' maxima and on its cleaning passes.
     B, V, branching = 20, 4096 + 40, (3, 2)
@@ -683,8 +683,7 @@ def test_verify_tree_peaked_draft_flat_target(rsd, dtype, V, branching):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_verify_tree_more_sequences_than_sms(rsd, dtype):
-    # batches above one sequence per SM run the walk in blocks of 256 threads, smaller ones in blocks of 512: the
-    # other verification tests here are small batches, this one is not
+    # more sequences than SMs: the other verification tests here are small batches, this one is not
     B, V, branching = 200, 1030, (3, 2, 2)
     L = len(branching)
     parent = workloads.rsdc_parent_array(branching)

@@ -1,6 +1,10 @@
 """The row scan uses 128, 256 or 512 threads per row, by the number of rows and their length, and reads rows off 32-byte
 boundaries in shifted words.  None of this may show: a few rows scanned alone give the bits they give inside a large
-batch (picks, perturbed values and log-probabilities), at the sizes where the number of threads changes."""
+batch (picks, perturbed values and log-probabilities), at the sizes where the number of threads changes.
+
+With a log-sum-exp (the first test) that is 128 threads against 256 with the sums on four warps, from 16,384 to 65,536 entries;
+its other sizes run one kernel whatever the batch and are there for the oracle and the shifted words.  Without one (the second
+test: picks only, or rows of log-probabilities) it is all three."""
 import numpy as np
 import pytest
 import torch
@@ -42,4 +46,41 @@ def test_rows_alone_and_in_a_batch_give_the_same_bits(dtype, V, B, off, trouble)
     t = Tally()
     # an fp32 log-probability is a difference of terms of up to 70: two ulps of that on top of the usual 1e-6
     compare_topk(t, whole["token"][:n], o, [8], whole["perturbed"][:n], whole["logprob"][:n], logprob_abs_tol=1e-6 + 2 * 70 * 1.2e-7)
+    t.check()
+
+
+# rows on both sides of 1.5 and 2.5 per SM (222 and 370 of 148): 128 / 256 threads from 4096 entries, 128 / 256 / 512 from 16,384,
+# 2-byte rows of more than 65,536 entries 256 / 512, 4-byte ones always 512
+@pytest.mark.parametrize("dtype,V,B,off,trouble", [
+    ("bf16", 4096, 380, 0, ""), ("f32", 4111, 240, 1, "nan"), ("bf16", 16383, 380, 3, "jump"), ("f32", 16384, 380, 0, "jump"), ("bf16", 32001, 380, 0, "nan"),
+    ("f32", 32000, 380, 0, ""), ("bf16", 65552, 300, 0, "jump"), ("bf16", 65537, 300, 1, ""), ("f32", 65552, 60, 0, "nan")])
+@pytest.mark.parametrize("form", ["picks", "logprob", "tempered picks"])
+def test_rows_without_log_sum_exp_alone_and_in_a_batch_give_the_same_bits(dtype, V, B, off, trouble, form):
+    import paper_2402_14160_b200 as rsd
+    gen = torch.Generator(device="cuda").manual_seed(3 * V + B)
+    rows = torch.randn((B, 1, V + off), generator=gen, device="cuda") * 2
+    if form == "logprob":
+        rows = torch.log_softmax(rows, -1)
+    if trouble == "jump":
+        rows[::2, :, V // 2::97] += 20.0
+        rows[1::3, :, :3000] = float("-inf")
+    elif trouble == "nan":
+        rows[::4, :, V - 1 + off] = float("nan")
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32)[:, :, off:]
+    T = 0.3 if form == "tempered picks" else 1.0
+
+    def scan(part, seq_base):
+        out = rsd.rsd_gumbel_topk_draft(part, [8], [2], 17, 3, seq_base=seq_base, is_logprob=form == "logprob", want_values=form == "logprob", temperature=T)
+        return {key: v.cpu().numpy() for key, v in out.items() if v is not None}
+
+    whole = scan(rows, 5)
+    for b, n in ((0, 3), (B - 2, 2), (B // 4, 150), (10, 230)):
+        n = min(n, B - b)
+        part = scan(rows[b:b + n], 5 + b)
+        for key in part:
+            assert np.array_equal(part[key], whole[key][b:b + n], equal_nan=part[key].dtype.kind == "f"), (key, b)
+    n = 2
+    o = oracle.gumbel_topk(workloads.as_oracle_rows(rows[:n].contiguous()), [8], [2], 17, 3, seq_base=5, is_logprob=form == "logprob", temperature=T)
+    t = Tally()
+    compare_topk(t, whole["token"][:n], o, [8], *([whole["perturbed"][:n], whole["logprob"][:n]] if form == "logprob" else []))
     t.check()

@@ -1,7 +1,7 @@
 """The walk of a thread block cluster per sequence (small batches) and the walk of one block per sequence (large ones) give
 the same bits, so a batch may be split at will: checked at the edges of the clusters' shapes (a row of exactly so many tiles,
-one entry more), with rows on and off 16-byte boundaries, NaN, far-off rows and more children than lanes; and against the
-oracle where only clusters run."""
+one entry more), with rows on 16-byte boundaries, NaN and far-off rows; and against the oracle with rows off them.  (Other
+rows, rules and trees in large batches: test_gpu_walk_routes.py.)"""
 import numpy as np
 import pytest
 import torch
