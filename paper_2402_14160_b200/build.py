@@ -11,7 +11,7 @@ LIB = os.path.join(HERE, "librsd.so")
 BIND = os.path.join(HERE, "_rsdbind.so")
 BIND_SOURCE = "rsd_bind.cpp"
 SOURCES = ["rsd_api.cu", "rsd_api_verify.cu", "rsd_scan_f32.cu", "rsd_scan_bf16.cu", "rsd_walk_cluster_f32.cu", "rsd_walk_cluster_bf16.cu", "rsd_walk_stream_f32.cu", "rsd_walk_stream_bf16.cu"]
-HEADERS = ["rsd_api_common.h", "rsd_device.cuh", "rsd_scan.cuh", "rsd_filter.cuh", "rsd_verify.cuh", "rsd_walk_ring.cuh", "rsd_walk_cluster.cuh", "rsd_walk_cluster_args.h", "rsd_walk_cluster_launch.cuh", "rsd_walk_stream.cuh", "rsd_walk_stream_launch.cuh", "rsd_scan_launch.cuh", os.path.join("..", "..", "include", "rsd.h")]
+HEADERS = ["rsd_api_common.h", "rsd_device.cuh", "rsd_scan.cuh", "rsd_filter.cuh", "rsd_verify.cuh", "rsd_walk_ring.cuh", "rsd_walk_cluster.cuh", "rsd_walk_cluster_args.h", "rsd_walk_cluster_launch.cuh", "rsd_walk_stream.cuh", "rsd_draw.cuh", "rsd_walk_stream_launch.cuh", "rsd_scan_launch.cuh", os.path.join("..", "..", "include", "rsd.h")]
 
 
 def _stale() -> bool:

@@ -78,6 +78,20 @@ float most_waves(const rsd::walk_cluster::Shape& c, int V, bool f32, bool ring, 
     return std::min(1.0f + (float)V / 18000.0f, f32 ? 7.0f : 4.8f);
 }
 
+// The same for residual draws with rejected tokens (a pass per token, always both rows; us, on chip / read anew).  Where the
+// distribution itself is not asked for: bf16 8,096 entries, 256 sequences: 24 / 20; 32,000, 148 / 256 / 512: 38 / 53 / 103, 40 / 44 / 86; 128,000, 64 / 256: 74 / 259,
+// 105 / 139; fp32 16,000, 512: 55 / 61; 32,000, 256 / 512: 58 / 108, 53 / 102.  The pass that writes it costs reading anew more: bf16
+// 32,000, 256 / 1024: 63 / 237, 59 / 212; 128,000, 64 / 148: 85 / 173, 149 / 151; fp32 32,000, 256 / 1024: 64 / 234, 68 / 279; 64,000, the same on both sides;
+// 128,000, 148 / 256: 190 / 332, 207 / 251.
+float most_waves_resample(const rsd::walk_cluster::Shape& c, int V, bool f32, bool whole) {
+    const float v = (float)V;
+    if (c.C <= 1 || (c.C == 2 && (f32 || whole))) return 1e30f;
+    if (c.C == 2) return 0.2f + v / 9000.0f;
+    if (!whole) return std::min(1.0f + v / 18000.0f, f32 ? 7.0f : 4.8f);
+    if (f32) return V > 65536 ? 9.0f : 1e30f;
+    return std::min(1.5f + v / 16000.0f, 6.5f);
+}
+
 void launch_on_chip(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const rsd::walk_cluster::Shape& c, cudaStream_t s) {
     if (dtype == RSD_F32) rsd::walk_cluster::launch_f32(a, extra, B, c, s);
     else rsd::walk_cluster::launch_bf16(a, extra, B, c, s);
@@ -85,12 +99,15 @@ void launch_on_chip(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool ext
 
 // Rows that no cluster holds: eight blocks a sequence up to about as many sequences as SMs (151,936 entries, us with eight blocks / one, 148
 // sequences: residual draw fp32 251 / 259, multi-round 153 / 177; 222: 357 / 299, 220 / 194), plain walks up to half as many more
-// (fp32, 222 / 256 sequences: 231 / 249, 262 / 258).  2-byte rows: two blocks an SM while that holds the batch, else three.
+// (fp32, 222 / 256 sequences: 231 / 249, 262 / 258).
+// 2-byte rows, one block a sequence: a block takes about 1.2 times as long where three share an SM (rsd_walk_stream.cuh), so three
+// where that saves waves: multi-round over 32,000, 256 / 300 / 500 / 600 sequences 67 / 94 / 103 / 127 with two, 72 / 77 / 112 / 121 with three.
 void launch_streamed(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, bool fits_cluster, cudaStream_t s) {
     const int sms = sm_count();
     const int C = !fits_cluster && B <= (extra ? sms : sms + sms / 2) ? 8 : 1;
+    const int waves2 = (B + 2 * sms - 1) / (2 * sms), waves3 = (B + 3 * sms - 1) / (3 * sms);
     if (dtype == RSD_F32) rsd::walk_cluster::launch_stream_f32(a, extra, B, C, 2, s);
-    else rsd::walk_cluster::launch_stream_bf16(a, extra, B, C, B > 2 * sms ? 3 : 2, s);
+    else rsd::walk_cluster::launch_stream_bf16(a, extra, B, C, 6 * waves3 < 5 * waves2 ? 3 : 2, s);
 }
 }  // namespace
 
@@ -180,7 +197,9 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     a.seed_lo = (uint32_t)seed; a.seed_hi = (uint32_t)(seed >> 32); a.step = step; a.seq_base = seq_base;
     a.out_token = out_token; a.out_residual = out_residual; a.status = status;
     cudaStream_t s = (cudaStream_t)stream;
-    // rows that fit a cluster take it at every batch size (V = 32,000, three rejected tokens: 137 -> 75 us for 256 sequences)
+    // A draw with nothing rejected is one sweep over the target row: a block per sequence, but a cluster for the few sequences of
+    // rows beyond 16,384 entries that are resident at once (us, cluster / block, bf16: 32,000 entries, 1 / 64 / 148 sequences 6.2 / 7.3 / 20,
+    // 6.8 / 7.0 / 7.1; 128,000, 1 / 16 / 64: 7.2 / 15 / 36, 17 / 17 / 17).
     rsd::walk_cluster::ClusterArgs ca;
     memset(&ca, 0, sizeof(ca));
     ca.r = a;
@@ -189,8 +208,15 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     ca.v.V = V; ca.v.num_nodes = 1;
     ca.v.seed_lo = a.seed_lo; ca.v.seed_hi = a.seed_hi; ca.v.step = step; ca.v.seq_base = seq_base;
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
-    if (shape.C > 0) launch_on_chip(ca, target_row->dtype, true, B, shape, s);
-    else launch_streamed(ca, target_row->dtype, true, B, false, s);
+    const bool f32 = target_row->dtype == RSD_F32;
+    if (!a.max_k && !(shape.C > 2 && shape.waves <= 1.0f)) {
+        if (f32) rsd::walk_cluster::launch_draw_f32(a, B, s);
+        else rsd::walk_cluster::launch_draw_bf16(a, B, s);
+    } else if (shape.C > 0 && shape.waves <= most_waves_resample(shape, V, f32, out_residual != nullptr)) {
+        launch_on_chip(ca, target_row->dtype, true, B, shape, s);
+    } else {
+        launch_streamed(ca, target_row->dtype, true, B, shape.C > 0, s);
+    }
     return check_launch("rsd_resample_residual");
 }
 

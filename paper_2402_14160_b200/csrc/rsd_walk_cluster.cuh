@@ -589,6 +589,8 @@ __device__ __forceinline__ double class_tree(double v) {
     return v;
 }
 
+__device__ __forceinline__ bool sum_usable(double s) { return s >= (double)kSumFloor && s < 1e300; }
+
 // The control warp: the walk itself, the same in every block of the cluster.
 template <typename T, typename SM, int WARPS, int MODE>
 struct Control {
@@ -652,7 +654,6 @@ struct Control {
         s0 = __shfl_sync(0xFFFFFFFFu, v, 0);
         s1 = __shfl_sync(0xFFFFFFFFu, v, kClasses);
     }
-    __device__ __forceinline__ static bool usable(double s) { return s >= (double)kSumFloor && s < 1e300; }
 
     __device__ __forceinline__ void issue_open(int node, bool with_draft, int options) {
         issue((with_draft ? kOpen : kOpenTarget | kStoreTiles) | options, node,
@@ -665,7 +666,7 @@ struct Control {
         double s0, s1;
         collect2(s0, s1);
         if (!with_draft) s1 = 1.0;
-        if (!(usable(s0) && usable(s1)) && !aborted) {
+        if (!(sum_usable(s0) && sum_usable(s1)) && !aborted) {
             issue_open(node, with_draft, kClean);
             collect2(s0, s1);
             if (!with_draft) s1 = 1.0;
@@ -678,7 +679,7 @@ struct Control {
                 saw_nan |= sm.extra[buf][2][i] != 0.0f;
             }
             if (saw_nan) status |= 1;              // RSD_ST_NAN_INPUT
-            if (!(usable(s0) && usable(s1)) && !aborted) {
+            if (!(sum_usable(s0) && sum_usable(s1)) && !aborted) {
                 if (top_q > kNegInf) mq = top_q;
                 if (with_draft && top_p > kNegInf) mp = top_p;
                 if (lane == 0) { sm.ref_q = mq * kq; sm.ref_p = mp * kp; }

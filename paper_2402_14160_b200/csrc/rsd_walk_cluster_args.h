@@ -26,5 +26,9 @@ void launch_bf16(const ClusterArgs& a, bool extra, int B, const Shape& c, cudaSt
 void launch_stream_f32(const ClusterArgs& a, bool extra, int B, int C, int per_sm, cudaStream_t s);
 void launch_stream_bf16(const ClusterArgs& a, bool extra, int B, int C, int per_sm, cudaStream_t s);
 
+// The residual draw without a rejected token, one block per sequence (rsd_draw.cuh).
+void launch_draw_f32(const ResampleArgs& a, int B, cudaStream_t s);
+void launch_draw_bf16(const ResampleArgs& a, int B, cudaStream_t s);
+
 }  // namespace walk_cluster
 }  // namespace rsd

@@ -80,7 +80,7 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
     float a_hi = 0.0f, a_lo = 0.0f;
     const char *rowq = rows.q, *rowp = rows.p;       // of the node that was opened last
     bool relative = false, dirty = false;            // its exponentials are relative to sm.ref_q, sm.ref_p; its rows may hold NaN
-    int n_frozen = 0;                                // tokens of sm.gone_tok that keep the weight frozen_w (kResample)
+    int n_frozen = 0, frozen_tile = -1;              // tokens of sm.gone_tok that keep the weight frozen_w (kResample); lane i: the i-th one's tile
     Incoming<T> in_q, in_p;
     int held = -1;                                   // the tile whose rows they hold,
     bool held_p = false;                             // with the draft's
@@ -121,7 +121,10 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
             held = -1;
         }
         if (MODE == kResample && kind == kWrite) dump_sync<kAll>();   // everyone has read the command
-        if (MODE == kResample && kind == kResidualPass && (flags & kFreeze)) ++n_frozen;
+        if (MODE == kResample && kind == kResidualPass && (flags & kFreeze)) {
+            if (lane == n_frozen) frozen_tile = sm.gone_tok[n_frozen] / kTileElems;
+            ++n_frozen;
+        }
         const bool use_p = kind >= kDump ? mode != 0 : kind != kOpenTarget && kind != kPlainPass;
         // the warp's tiles: i, i + way, ... of the block's (a dump: the one that is asked for)
         int todo = n_mine, i = flags & kBackward ? warp + kStreamWarps * (n_mine - 1) : warp;
@@ -149,6 +152,22 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
                 if (lane < C) send_word(remote_addr(&sm.tile_sum[tile], lane), ts, remote_addr(&sm.red_bar[buf], lane));
             }
         };
+        // (kResample) removed tokens keep the weight that they had when they were removed
+        auto freeze = [&](int tile, float (&q)[16], float (&p)[16]) {
+            for (unsigned here = __ballot_sync(0xFFFFFFFFu, frozen_tile == tile); here; here &= here - 1u) {
+                const int f = __ffs(here) - 1, o = sm.gone_tok[f] - tile * kTileElems;
+                int l_, j_;
+                walk_ring::piece_of<T>(o, l_, j_);
+                if (l_ != lane) continue;
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (j == j_) {      // (this lane alone reads and writes its tokens' frozen weights)
+                        if ((flags & kFreeze) && f == n_frozen - 1) frozen_w[f] = residual_weight(q[j], p[j], sm.freeze_hi, sm.freeze_lo);
+                        q[j] = frozen_w[f];
+                        p[j] = 0.0f;
+                    }
+            }
+        };
         // The passes that a walk consists of, each as a loop of its own: nothing of the others holds registers or splits the block of
         // instructions that the next tile's loads travel behind.
         auto sweep = [&](auto which) {
@@ -169,6 +188,7 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
                 } else {
                     float w[16];
                     if (KIND == kResidualPass) {
+                        if (MODE == kResample) freeze(pl.rank + C * i, q, p);
                         residual16(q, p, a_hi, a_lo, w);
                         count(tree_sum16(w), 0.0f, false);
                     } else if (KIND == kOverlapPass) {
@@ -183,7 +203,7 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
                 }
             }
         };
-        if (!relative && !dirty && n_frozen == 0) {
+        if (!relative && !dirty) {
             if (kind == kOpen) sweep(std::integral_constant<int, kOpen>());
             else if (kind == kOpenTarget) sweep(std::integral_constant<int, kOpenTarget>());
             else if (kind == kResidualPass) sweep(std::integral_constant<int, kResidualPass>());
@@ -213,22 +233,7 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
                 if (relative) exp16(p, rows.kp, sm.ref_p, p);
                 else exp16_precise(p, rows.kp, p);
             }
-            if (MODE == kResample) {
-                for (int f = 0; f < n_frozen; ++f) {
-                    const int o = sm.gone_tok[f] - tile * kTileElems;
-                    if (o < 0 || o >= kTileElems) continue;
-                    int l_, j_;
-                    walk_ring::piece_of<T>(o, l_, j_);
-                    if (l_ != lane) continue;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (j == j_) {      // (this lane alone reads and writes its tokens' frozen weights)
-                            if ((flags & kFreeze) && f == n_frozen - 1) frozen_w[f] = residual_weight(q[j], p[j], sm.freeze_hi, sm.freeze_lo);
-                            q[j] = frozen_w[f];
-                            p[j] = 0.0f;
-                        }
-                }
-            }
+            if (MODE == kResample) freeze(tile, q, p);
             if (kind == kResidualPass) {
                 residual16(q, p, a_hi, a_lo, w);
             } else if (kind == kRestPass) {

@@ -1,6 +1,7 @@
 // Launch of the streaming walk for one element type.
 #pragma once
 #include "rsd_api_common.h"
+#include "rsd_draw.cuh"
 #include "rsd_walk_stream.cuh"
 
 namespace rsd {
@@ -22,6 +23,11 @@ void launch_stream_of(const ClusterArgs& a, bool extra, int B, int C, int per_sm
     if (a.resample) launch_stream_mode<T, kResample>(a, B, C, per_sm, s);
     else if (extra) launch_stream_mode<T, kRuleWalk>(a, B, C, per_sm, s);
     else launch_stream_mode<T, kPlainWalk>(a, B, C, per_sm, s);
+}
+
+template <typename T>
+void launch_draw_of(const ResampleArgs& a, int B, cudaStream_t s) {
+    rsd_host::launch_overlapped(draw_target_kernel<T>, (unsigned)B, kDrawWarps * 32, 0, s, 0, a);
 }
 
 }  // namespace walk_cluster
