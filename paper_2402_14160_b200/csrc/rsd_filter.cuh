@@ -65,7 +65,8 @@ struct FilterSmem {
     uint32_t cut_code;                           // the last kept value, its code and
     int cut_tok;                                 // the last kept token among its equals
     uint32_t top, ext_lo, ext_hi;                // codes of the row's largest value, of a bin's smallest and largest
-    int pick_bin, n_list, not_finite, n_kept;
+    float low;                                   // the smallest finite value in a sample of the row
+    int pick_bin, n_list, n_all, not_finite, n_kept;
     int copy_gave_up, needs_cleaning, nan_flag;
     int scan_i[32];
 };
@@ -300,15 +301,17 @@ struct RowFilter {
         for (int q = threadIdx.x; q < kBins; q += NT) { sm.hist.lo[q] = 0u; sm.hist.hi[q] = 0u; }
     }
 
-    // Every token of the row into the histogram (cleared): rows without -inf, bins of equal width in value.
-    template <bool BY_MASS>
+    // Every token of the row into the histogram (cleared), bins of equal width in value.  MASKED: the row holds entries of -inf, left out.
+    template <bool BY_MASS, bool MASKED>
     __device__ __forceinline__ void sweep_all(const BinMap& bm) {
         const unsigned long long ns = f32x2(-bm.scale, -bm.scale), of = f32x2(bm.offset, bm.offset), magic = f32x2(12582912.0f, 12582912.0f),
                                  k2 = f32x2(k, k), c2 = f32x2(neg_c, neg_c), fx = f32x2(to_fixed(), to_fixed()), zero = f32x2(0.0f, 0.0f);
         const uint32_t low_mask = (1u << split) - 1u;
         auto two = [&](unsigned long long v) {
             float d0, d1;
+            bool in0 = true, in1 = true;
             split_f32x2(fma_f32x2(v, ns, of), d0, d1);
+            if (MASKED) { in0 = d0 < -kNegInf; in1 = d1 < -kNegInf; }   // (an entry of -inf lies infinitely far below the top)
             split_f32x2(add_f32x2(f32x2(fminf(d0, (float)(kBins - 1)), fminf(d1, (float)(kBins - 1))), magic), d0, d1);
             const int q0 = (int)(__float_as_uint(d0) & (uint32_t)(kBins - 1)), q1 = (int)(__float_as_uint(d1) & (uint32_t)(kBins - 1));
             if (BY_MASS) {
@@ -316,13 +319,17 @@ struct RowFilter {
                 split_f32x2(fma_f32x2(v, k2, c2), x0, x1);
                 split_f32x2(fma_f32x2(f32x2(ex2_approx(x0), ex2_approx(x1)), fx, zero), x0, x1);
                 const uint32_t w0 = __float2uint_rn(x0), w1 = __float2uint_rn(x1);
-                atomicAdd(&sm.hist.lo[q0], w0 & low_mask);
-                atomicAdd(&sm.hist.hi[q0], w0 >> split);
-                atomicAdd(&sm.hist.lo[q1], w1 & low_mask);
-                atomicAdd(&sm.hist.hi[q1], w1 >> split);
+                if (in0) {
+                    atomicAdd(&sm.hist.lo[q0], w0 & low_mask);
+                    atomicAdd(&sm.hist.hi[q0], w0 >> split);
+                }
+                if (in1) {
+                    atomicAdd(&sm.hist.lo[q1], w1 & low_mask);
+                    atomicAdd(&sm.hist.hi[q1], w1 >> split);
+                }
             } else {
-                atomicAdd(&sm.hist.lo[q0], 1u);
-                atomicAdd(&sm.hist.lo[q1], 1u);
+                if (in0) atomicAdd(&sm.hist.lo[q0], 1u);
+                if (in1) atomicAdd(&sm.hist.lo[q1], 1u);
             }
         };
         const int n_vec = V / kPerVec;
@@ -332,7 +339,10 @@ struct RowFilter {
 #pragma unroll
             for (int j = 0; j < kPerVec; j += 2) two(f32x2(Codes::value_of_bits(h[j]), Codes::value_of_bits(h[j + 1])));
         }
-        for (int i = n_vec * kPerVec + threadIdx.x; i < V; i += NT) add_one<BY_MASS>(bm.of(Codes::value_of_bits(Codes::bits(row, i)), 0u), Codes::value_of_bits(Codes::bits(row, i)));
+        for (int i = n_vec * kPerVec + threadIdx.x; i < V; i += NT) {
+            const float v = Codes::value_of_bits(Codes::bits(row, i));
+            if (!MASKED || v > kNegInf) add_one<BY_MASS>(bm.of(v, 0u), v);
+        }
     }
     template <bool BY_MASS>
     __device__ __forceinline__ void add_one(int q, float v) {
@@ -374,7 +384,7 @@ struct RowFilter {
         }
     }
     // The tokens with a value in [v_first, v_last] that f(value, code) accepts (and that are within `inside`) into the list;
-    // sm.n_list counts them, also beyond the list's end.
+    // sm.n_list is their number, or more than the list holds.
     template <typename F>
     __device__ __forceinline__ void gather(float v_first, float v_last, uint32_t lo, uint32_t hi, const Cut& inside, F f) {
         if (threadIdx.x == 0) sm.n_list = 0;
@@ -388,6 +398,7 @@ struct RowFilter {
                 const int i = m * kPerVec + j;
                 const uint32_t h = Codes::bits(row, i), code = Codes::code_of_bits(h);
                 if (code < lo || code > hi || code <= Codes::kNegInfCode || !within(inside, code, i) || !f(Codes::value_of_bits(h), code)) continue;
+                if (*(volatile int*)&sm.n_list > kListCap) break;   // (thousands of additions to one word would come one by one)
                 const int at = atomicAdd(&sm.n_list, 1);
                 if (at < kListCap) sm.list[at] = (uint32_t)i;
             }
@@ -395,9 +406,9 @@ struct RowFilter {
         __syncthreads();
     }
 
-    // The j-th (1-based, in token order) of the tokens with code `code` within `inside`, and how many there are: for runs of
-    // equal values that do not fit the list.  Threads own consecutive runs; one prefix count over the block.
-    __device__ __forceinline__ int nth_with_code(uint32_t code, int j, const Cut& inside, int& how_many) {
+    // The j-th (1-based, in token order) of the tokens with code `code` within `inside`: for runs of equal values that do not
+    // fit the list.  Threads own consecutive runs; one prefix count over the block.
+    __device__ __forceinline__ int nth_with_code(uint32_t code, int j, const Cut& inside) {
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
         const int per = (V + NT - 1) / NT;
         const int m0 = min(V, tid * per), m1 = min(V, m0 + per);
@@ -413,12 +424,8 @@ struct RowFilter {
         if (lane == 31) sm.scan_i[warp] = incl;
         if (tid == 0) sm.cut_tok = V;
         __syncthreads();
-        int before = incl - mine, total = 0;
-        for (int w = 0; w < NT / 32; ++w) {
-            if (w < warp) before += sm.scan_i[w];
-            total += sm.scan_i[w];
-        }
-        how_many = total;
+        int before = incl - mine;
+        for (int w = 0; w < warp; ++w) before += sm.scan_i[w];
         if (mine > 0 && before < j && j <= before + mine) {
             int seen = before;
             for (int i = m0; i < m1; ++i)
@@ -539,12 +546,15 @@ struct RowFilter {
             // bins of equal width in value first; in code where the interval is narrow or infinite, and on every further level
             bm.shift = -1;
             const float v_hi = Codes::value_of_code(bm.hi);
-            const float width = v_hi - fmaxf(Codes::value_of_code(bm.lo), v_hi - kValueRange * kLog2e / k);
+            float v_lo = fmaxf(Codes::value_of_code(bm.lo), v_hi - kValueRange * kLog2e / k);
+            if (sm.low < v_hi) v_lo = fmaxf(v_lo, v_hi - 1.25f * (v_hi - sm.low));   // (what lies further down falls into the last bin)
+            const float width = v_hi - v_lo;
             bm.scale = (float)(kBins - 1) / width;
             bm.offset = v_hi * bm.scale;
             if (level > 0 || bm.hi - bm.lo < (uint32_t)kBins || !(width > 0.0f) || !(width < 3.0e38f) || !(fabsf(bm.offset) < 1.0e6f))   // (rows far from 0: the position's rounding must stay below half a bin)
                 bm.shift = max(0, 32 - __clz(bm.hi - bm.lo) - 10);   // ((hi - lo) >> shift) < 1024
-            if (bm.shift < 0 && everything && all_finite) sweep_all<BY_MASS>(bm);
+            if (bm.shift < 0 && everything && all_finite) sweep_all<BY_MASS, false>(bm);
+            else if (bm.shift < 0 && everything) sweep_all<BY_MASS, true>(bm);
             else for_tokens(bm, inside, [&](int, float v, uint32_t code) { add_one<BY_MASS>(bm.of(v, code), v); });
             __syncthreads();
             // ---- tally from the top bin down -------------------------------------------------------------------------------
@@ -586,23 +596,23 @@ struct RowFilter {
                 return {sm.cut_code, sm.cut_tok};
             }
             // ---- more tokens than the list holds: the codes the bin spans, then once more over these ------------------------
-            if (tid == 0) { sm.ext_lo = 0xFFFFFFFFu; sm.ext_hi = 0u; }
+            if (tid == 0) { sm.ext_lo = 0xFFFFFFFFu; sm.ext_hi = 0u; sm.n_all = 0; }
             __syncthreads();
             uint32_t c_lo = 0xFFFFFFFFu, c_hi = 0u;
+            int members = 0;
             for_tokens(bm, inside, [&](int, float v, uint32_t code) {
-                if (bm.of(v, code) == pick) { c_lo = min(c_lo, code); c_hi = max(c_hi, code); }
+                if (bm.of(v, code) == pick) { c_lo = min(c_lo, code); c_hi = max(c_hi, code); ++members; }
             });
             c_lo = __reduce_min_sync(0xFFFFFFFFu, c_lo);
             c_hi = __reduce_max_sync(0xFFFFFFFFu, c_hi);
-            if ((tid & 31) == 0) { atomicMin(&sm.ext_lo, c_lo); atomicMax(&sm.ext_hi, c_hi); }
+            members = __reduce_add_sync(0xFFFFFFFFu, members);
+            if ((tid & 31) == 0) { atomicMin(&sm.ext_lo, c_lo); atomicMax(&sm.ext_hi, c_hi); atomicAdd(&sm.n_all, members); }
             clear_histogram();
             __syncthreads();
             bm.lo = sm.ext_lo;
             bm.hi = sm.ext_hi;
             if (bm.lo >= bm.hi) {                        // a run of equal values
-                int ties;
-                nth_with_code(bm.hi, 1, inside, ties);
-                return {bm.hi, nth_with_code(bm.hi, ties_to_keep<BY_MASS>(bm.hi, ties, above, need), inside, ties)};
+                return {bm.hi, nth_with_code(bm.hi, ties_to_keep<BY_MASS>(bm.hi, sm.n_all, above, need), inside)};
             }
         }
     }
@@ -677,6 +687,23 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
             odd |= !(v > kNegInf);
         }
         if (odd) sm.needs_cleaning = 1;
+        // One warp looks at 32 words spread over the row for how far down its values reach: the bins of the first sweep go about as
+        // far.  (A flat row would fall into a few of them: 200 rows of 32,000 bf16 within 0.1 of each other, 81 -> 28 us.  All warps
+        // looking at a word each cost every row 0.4 us.)
+        if (warp == 1) {
+            float low = -kNegInf;
+            if (n_vec > 0) {
+                uint32_t h[kPerVec];
+                RowCodes<T>::unpack_bits(((const uint4*)row_sm)[(int)((unsigned)lane * (unsigned)n_vec / 32u)], h);
+#pragma unroll
+                for (int j = 0; j < kPerVec; ++j) {
+                    const float v = RowCodes<T>::value_of_bits(h[j]);
+                    if (v > kNegInf) low = fminf(low, v);
+                }
+            }
+            low = -warp_max(-low);
+            if (lane == 0) sm.low = low;
+        }
         // (+0 and -0 are equal as values but not as codes: the larger code stands for both)
         uint32_t top = vtop == 0.0f ? RowCodes<T>::code_of_float(0.0f) : (vtop > kNegInf ? RowCodes<T>::code_of_float(vtop) : RowCodes<T>::kNegInfCode);
         top = __reduce_max_sync(0xFFFFFFFFu, top);

@@ -186,10 +186,37 @@ def test_filter_rows_far_from_zero_keep_their_shares(rsd, dtype, V):
         assert np.abs(kept - want).max() <= 1, (kept, want)
 
 
-@pytest.mark.parametrize("dtype,V", [("bf16", 109716), ("f32", 54858)])
+@pytest.mark.parametrize("dtype,V", [("bf16", 109712), ("f32", 54856)])
 def test_filter_rows_of_the_longest_rows_that_fit(rsd, dtype, V):
     rows = _rows((1, 2, V + 1), dtype, 2.0, V)
     for top_k, top_p in ((0, 0.95), (2000, 0.9)):
         _check_filter(rsd, rows[:, :, :V], top_k, top_p, 1.0)
     with pytest.raises(rsd.RsdError, match="at most %d entries" % V):
         rsd.rsd_filter_rows(rows, 0, 0.9)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("V", [31, 5003, 20000])
+def test_filter_rows_that_the_sample_of_the_first_sweep_misjudges(rsd, dtype, V):
+    # the first sweep's bins reach as far down as 32 words spread over the row do: flat rows, rows that are flat where the sample
+    # looks and reach far down or up elsewhere, sorted rows, rows with masked entries, runs of equal values longer than the list
+    per = 4 if dtype == "f32" else 8
+    words = V // per
+    g = torch.Generator(device="cpu").manual_seed(V)
+    rows = torch.randn((1, 9, V), generator=g)
+    rows[0, 0] *= 0.02
+    seen = torch.zeros(V, dtype=torch.bool)
+    for lane in range(32):
+        w = lane * words // 32
+        seen[w * per:(w + 1) * per] = True
+    rows[0, 1] = torch.where(seen, torch.tensor(1.0), rows[0, 1] - 3.0)      # all but the sample far below it
+    rows[0, 2] = torch.where(seen, torch.tensor(-20.0), rows[0, 2])
+    rows[0, 3] = torch.sort(rows[0, 3] * 3).values
+    rows[0, 4] = torch.sort(rows[0, 4] * 3, descending=True).values
+    rows[0, 5, ::3] = float("-inf")
+    rows[0, 6] = torch.where(seen, torch.tensor(float("-inf")), rows[0, 6])  # nothing finite in the sample
+    rows[0, 7] = (rows[0, 7] * 0.7).round()
+    rows[0, 8] = torch.where(seen, torch.tensor(2.0), torch.tensor(1.0))
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32).cuda()
+    for top_k, top_p, T in ((0, 0.95, 1.0), (0, 0.3, 0.5), (min(3000, V), 0.9, 1.0), (7, 1.0, 1.0)):
+        _check_filter(rsd, rows, top_k, top_p, T, max_borderline=2)
