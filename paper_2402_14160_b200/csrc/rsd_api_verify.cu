@@ -62,9 +62,9 @@ rsd::walk_cluster::Shape cluster_shape(int B, int V) {
 }
 
 // Up to how many waves of clusters the on-chip walk is taken.
-//   Rows that the ring takes (figures: us for so many sequences, bf16): from about two waves on the ring is ahead (V = 32,000, 148 / 200:
-// ring 63 / 67, cluster 59 / 73; V = 16,000, 250 / 300: 57 / 57 against 51 / 61; with clusters of one or two blocks already from 1.3:
-// V = 8096, 300 / 492: 42 / 53 against 42 / 57).
+//   Rows that the ring takes (us, ring / cluster): from about two waves on the ring is ahead (trees of (3, 2, 2) / (4, 2, 2, 1, 1) / (3, 2, 1);
+// 32,000 bf16 entries, 130 sequences: 36 / 37, 51 / 49, 41 / 34, 148: 36 / 44, 53 / 59, 41 / 44; fp32, 148: 47 / 48, 71 / 63, 51 / 47; 64,000 bf16, 80:
+// 53 / 51, 78 / 63, 54 / 50), with clusters of one or two blocks from 1.3 (16,000 bf16, 180: 35 / 34, 44 / 41, 32 / 31, 222: 36 / 37, 47 / 49, 33 / 34).
 //   Others: clusters of one or two blocks stay (8001 entries, 300 / 1000: 34 / 89 on chip, 41 / 102 read anew).  Beyond, a launch on
 // chip takes as long as it has waves, one that reads the rows anew as long as they are, up to the 296 or 444 sequences that are
 // resident at once: 20,000 entries, multi-round, 148 / 222: 46 / 66 on chip, 43 / 49 read anew; 32,001, plain, 200 / 250: 68 / 88, 73 / 75;
@@ -72,7 +72,7 @@ rsd::walk_cluster::Shape cluster_shape(int B, int V) {
 //   Gumbel-Top-1 draws take two rounds of Philox calls when rows are read anew: 32,000 entries, 256 / 400: 104 / 154 on chip, 108 / 132
 // read anew; 100,000, 74 / 128: 141 / 240, 216 / 227; fp32, 400 / 512 of 32,000: 176 / 226, 195 / 220.
 float most_waves(const rsd::walk_cluster::Shape& c, int V, bool f32, bool ring, bool top1) {
-    if (ring) return c.C <= 2 ? 1.3f : 2.0f;
+    if (ring) return c.C <= 2 ? 1.3f : (c.C == 4 && !f32 ? 1.8f : 2.0f);
     if (c.C <= 2) return 1e30f;
     if (top1) return f32 ? 7.0f : std::min(1.6f + (float)V / 16000.0f, 6.6f);
     return std::min(1.0f + (float)V / 18000.0f, f32 ? 7.0f : 4.8f);
