@@ -440,10 +440,11 @@ __host__ __device__ inline size_t scan_bounds_bytes(int V) { return 4 * (size_t)
 // SPLIT: the first four warps take the log-sum-exp and nothing else, the others the perturbed values: a few rows are done
 // sooner, and the sums are those of a block of 128 threads to the bit (the loads of the second half hit L2).
 // Blocks of 128 threads: nine per SM for 2-byte rows (56 registers: a group in flight is 8 registers), eight for 4-byte rows;
-// fewer for shifted rows, which need registers for the words around a group.
+// fewer for shifted rows, which need registers for the words around a group: eight and seven (six for 4-byte rows left 1792 of them in
+// 2.02 waves: 70 entries 21.0 -> 17.5 us, 1000 19.8 -> 16.5, 32,001 70.8 -> 64.6; eight blocks of the element loads before them 19.0, 20.1, 135).
 template <typename T, bool ALIGNED, int NT>
 constexpr int scan_blocks_per_sm() {
-    return ALIGNED ? (NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) : (NT == 128 ? (sizeof(T) == 2 ? 8 : 6) : NT == 256 ? 3 : 2);
+    return ALIGNED ? (NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) : (NT == 128 ? (sizeof(T) == 2 ? 8 : 7) : NT == 256 ? 3 : 2);
 }
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
 __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan_topk_kernel(const ScanArgs a) {
