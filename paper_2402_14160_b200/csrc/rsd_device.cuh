@@ -264,18 +264,7 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
-// Block-wide sum of doubles / max of floats; `scratch` holds one slot per warp; all threads get the result.
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* scratch) {
-    v = warp_sum(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < NT / 32; ++w) t += scratch[w];  // fixed order: the same on every thread
-    return t;
-}
+// Block-wide max of floats; `scratch` holds one slot per warp; all threads get the result.
 template <int NT>
 __device__ __forceinline__ float block_max(float v, float* scratch) {
     v = warp_max(v);

@@ -1,5 +1,6 @@
 // Recursive rejection sampling along the draft tree (Eqs. 1-4, Algorithm 1; Section 3.2.2, Algorithm 6) and the
-// stand-alone residual draw.  One thread block walks one sequence and reads only the rows of visited nodes.
+// stand-alone residual draw: what all walks share.  A block or a cluster of blocks walks one sequence and reads only the rows
+// of visited nodes.
 //
 // The chain of residuals is carried in closed form.  With p, q the node's draft and target distributions, x_0, x_1,
 // ... the children in stored order, P_j the draft mass of the first j children and
@@ -13,8 +14,8 @@
 // Eq. 2 no longer lowers it).  After a genuine rejection (theta < 1) that mass is 0 and the formula above is
 // already right; for a caller-supplied list of removals it may be positive, so the passes patch those tokens.
 //
-// Numerics: exponentials in fp32 relative to a per-row reference m (any value near the row maximum), sums of 16
-// in fp32, everything above that and all scalars of the chain in fp64.  The coefficient a = A S_q / S_p is applied
+// Numerics: exponentials in fp32, relative to 0 or, where their sum is out of range, to the row's maximum; sums over a lane's
+// share of a summation class in fp32, everything above that and all scalars of the chain in fp64.  The coefficient a = A S_q / S_p is applied
 // as a two-float sum so that its rounding does not tilt the whole residual.
 #pragma once
 #include "rsd_device.cuh"

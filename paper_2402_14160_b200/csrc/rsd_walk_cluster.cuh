@@ -13,8 +13,11 @@
 // runs, one child per lane: tokens, row values, uniforms, the next node's children.
 //
 // Sums are taken in the order of the ring walk (rsd_walk_ring.cuh): per lane over the tiles of equal index modulo 8, in
-// pass direction, then over the lanes, then a tree over the eight classes in double.  The two walks give the same
-// bits, so which of them runs (a matter of batch size and vocabulary) does not show in any result.
+// pass direction, then over the lanes, then a tree over the eight classes in double.  For the rows that the ring walk takes
+// (plain walks, rows on 16-byte boundaries) the weights are its weights as well, so the two give the same bits; elsewhere the
+// exponentials keep the rounding of their exponents (exp16_precise()), here and in the walk that reads the rows in every pass
+// (rsd_walk_stream.cuh).  Which kernel runs, with how many blocks (a matter of batch size and vocabulary), does not show
+// in any result.
 // Every wait on an mbarrier is bounded (about a second); a wait that runs out abandons the walk with RSD_ST_TIMEOUT.
 #pragma once
 #include "rsd_walk_cluster_args.h"

@@ -22,8 +22,8 @@
 // Every wait on an mbarrier is bounded (about a second); a wait that runs out abandons the walk with RSD_ST_TIMEOUT.
 //
 // Used for rows whose base and strides are multiples of 16 bytes, recursive rejection sampling with the inverse-CDF
-// last draw; smaller batches, other rows and the rules take the cluster walk
-// (rsd_walk_cluster.cuh), what neither takes the register-fed kernels of rsd_verify_walk.inc.
+// last draw, in large batches; smaller batches, other rows and the rules take the cluster walk (rsd_walk_cluster.cuh) or read
+// their rows in every pass under its control (rsd_walk_stream.cuh).
 #pragma once
 #include "rsd_verify.cuh"
 
