@@ -384,11 +384,9 @@ struct RowFilter {
         }
     }
     // The tokens with a value in [v_first, v_last] that f(value, code) accepts (and that are within `inside`) into the list;
-    // sm.n_list is their number, or more than the list holds.
+    // sm.n_list, cleared before, is their number, or more than the list holds.
     template <typename F>
     __device__ __forceinline__ void gather(float v_first, float v_last, uint32_t lo, uint32_t hi, const Cut& inside, F f) {
-        if (threadIdx.x == 0) sm.n_list = 0;
-        __syncthreads();
         for (int m = threadIdx.x; m < words(); m += NT) {
             const uint4 w = ((const uint4*)row)[m];
             uint32_t in = RowVec<T>::between(w, v_first, v_last);
@@ -398,9 +396,9 @@ struct RowFilter {
                 const int i = m * kPerVec + j;
                 const uint32_t h = Codes::bits(row, i), code = Codes::code_of_bits(h);
                 if (code < lo || code > hi || code <= Codes::kNegInfCode || !within(inside, code, i) || !f(Codes::value_of_bits(h), code)) continue;
-                if (*(volatile int*)&sm.n_list > kListCap) break;   // (thousands of additions to one word would come one by one)
                 const int at = atomicAdd(&sm.n_list, 1);
                 if (at < kListCap) sm.list[at] = (uint32_t)i;
+                else in = 0u;                            // (too many: one more addition a word tells)
             }
         }
         __syncthreads();
@@ -567,7 +565,7 @@ struct RowFilter {
             const unsigned long long incl = block_scan_u64<NT>(mine, sm.scan_w, total);
             const double unit = BY_MASS ? 1.0 / (double)(1ull << frac_bits) : 1.0;
             if (level == 0 && need_abs < 0.0) need = need_frac * ((double)total * unit);
-            if (tid == 0) { sm.pick_bin = -1; sm.pick_above = 0ull; }
+            if (tid == 0) { sm.pick_bin = -1; sm.pick_above = 0ull; sm.n_list = 0; }
             __syncthreads();
             {
                 unsigned long long run = incl - mine;   // everything above this thread's bins
@@ -687,10 +685,10 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
             odd |= !(v > kNegInf);
         }
         if (odd) sm.needs_cleaning = 1;
-        // One warp looks at 32 words spread over the row for how far down its values reach: the bins of the first sweep go about as
-        // far.  (A flat row would fall into a few of them: 200 rows of 32,000 bf16 within 0.1 of each other, 81 -> 28 us.  All warps
-        // looking at a word each cost every row 0.4 us.)
-        if (warp == 1) {
+        // The last warp, which may have a word less than the others, looks at 32 words spread over the row for how far down its
+        // values reach: the bins of the first sweep go about as far.  (A flat row would fall into a few of them: 200 rows of 32,000
+        // bf16 within 0.1 of each other, 81 -> 28 us.  All warps looking at a word each cost every row 0.4 us, this one 0.2.)
+        if (warp == NT / 32 - 1) {
             float low = -kNegInf;
             if (n_vec > 0) {
                 uint32_t h[kPerVec];
@@ -701,8 +699,8 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
                     if (v > kNegInf) low = fminf(low, v);
                 }
             }
-            low = -warp_max(-low);
-            if (lane == 0) sm.low = low;
+            const uint32_t lowest = __reduce_min_sync(0xFFFFFFFFu, float_to_ordered(low));
+            if (lane == 0) sm.low = ordered_to_float(lowest);
         }
         // (+0 and -0 are equal as values but not as codes: the larger code stands for both)
         uint32_t top = vtop == 0.0f ? RowCodes<T>::code_of_float(0.0f) : (vtop > kNegInf ? RowCodes<T>::code_of_float(vtop) : RowCodes<T>::kNegInfCode);
@@ -760,16 +758,13 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
         cut = f.template search<false>(RowCodes<T>::kNegInfCode + 1u, top, (double)a.top_k, 0.0, cut, true);
         kept = a.top_k;
         everything = false;
-        if (want_p) {
-            __syncthreads();
-            f.clear_histogram();
-            __syncthreads();
-        }
     }
     // ---- top-p: of what is left, the shortest prefix (value descending, token ascending) whose mass reaches top_p -------
     if (want_p) {
         if (!everything && kept <= kListCap) {
             // the kept tokens all fit the list: one warp does the rest (their total in the sweep's fixed point)
+            if (tid == 0) sm.n_list = 0;
+            __syncthreads();
             f.gather(RowCodes<T>::value_of_code(cut.code), vmax, cut.code, top, cut, [](float, uint32_t) { return true; });
             if (tid < 32) {
                 unsigned long long total = 0;
@@ -783,6 +778,11 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
             __syncthreads();
             cut = {sm.cut_code, sm.cut_tok};
         } else {
+            if (!everything) {
+                __syncthreads();
+                f.clear_histogram();
+                __syncthreads();
+            }
             cut = f.template search<true>(everything ? RowCodes<T>::kNegInfCode + 1u : cut.code, top, -1.0, (double)a.top_p, cut, everything);
         }
         count_kept = a.kept != nullptr;
