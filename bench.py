@@ -31,7 +31,7 @@ import workloads  # noqa: E402
 # together with the SHA-256 of the kernel sources it was measured on: when the sources differ, `traffic` is null.
 SCAN_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.006
 SCAN_TRAFFIC_SOURCES = ("paper_2402_14160_b200/csrc/rsd_scan.cuh", "paper_2402_14160_b200/csrc/rsd_device.cuh")
-SCAN_TRAFFIC_SOURCE_SHA256 = "58b35d74e64ea41f8b36a56af257624b605a762ba30b9c8f0a226c293253148d"
+SCAN_TRAFFIC_SOURCE_SHA256 = "aafb17dd45afc0a2a04de478bb91e16ea1f4aa5ad1be2181e44e83eedac5c867"
 
 
 def _scan_sources_sha256():
