@@ -1,5 +1,6 @@
 // Host-side helpers shared by the translation units of librsd: the per-thread error message and argument checks.
 #pragma once
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
@@ -45,6 +46,19 @@ inline void launch_overlapped(void (*kernel)(KArgs...), unsigned blocks, unsigne
     cfg.attrs = at;
     cfg.numAttrs = cluster > 0 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Raises a kernel's limit of dynamic shared memory.  The attribute belongs to the (function, device) pair and setting it costs host
+// time: once per device.  (An error stays pending for check_launch().)
+template <auto KERNEL>
+inline bool raise_shared_memory(int bytes) {
+    static std::atomic<bool> raised[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (dev >= 0 && dev < 64 && raised[dev].load(std::memory_order_acquire)) return true;
+    if (cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    if (dev >= 0 && dev < 64) raised[dev].store(true, std::memory_order_release);
+    return true;
 }
 
 inline int check_rows(const char* name, const rsd_rows* r, int V, bool need_row_stride) {

@@ -40,56 +40,92 @@ void launch_ring_walk(const rsd::VerifyArgs& a, int B, cudaStream_t s) {
     launch_overlapped(verify_tree_ring_kernel<T>, (unsigned)B, kThreads, kRingBytes, s, 0, a);
 }
 
-// The smallest cluster that holds a row, with one tile per warp (three blocks an SM) as long as all sequences are
-// resident at once, else with two (two blocks an SM), which costs a sequence about 10 % more time and 25 % fewer SM-cycles
-// (V = 32,000, bf16: 42 against 47 us at 64 sequences, 122 against 102 us at 256).  Rows of up to 8192 entries stay with one
-// tile per warp: a cluster of one block has nobody to share with (V = 8096, 492 sequences: two blocks 57 us, one 63 us).
-// Rows beyond 65,536 entries take sixteen warps, one block an SM; beyond 131,072 no cluster holds them (C = 0).
+// The cluster that holds a row on chip.  Fewer tiles per warp walk faster, more leave room for more sequences at a time (148 SMs, 32,000
+// entries; bf16 multi-round rule over (3, 2) trees, us at 40 / 75 / 148 / 222 sequences): one tile per warp, eight blocks, 48 resident: 15.6 / 28 / 48 / 68;
+// two, four blocks, 71 resident: 17.0 / 28 / 41 / 53; four, two blocks, 148 resident: 21 / 23 / 26 / 46.  So the first of them that has all
+// sequences resident, else the one with the most.  Rows of up to 8192 entries are held by one or two blocks with one tile per warp; beyond its
+// residents that one stays ahead (V = 8096, 492 sequences: two blocks 57 us, one 63 us).  Rows beyond 65,536 entries: sixteen warps
+// with two tiles (15 resident; 128,000 entries, 9 / 18 / 32 sequences 21 / 33 / 54 us), eight with four (33 resident; 22 / 25 / 31); beyond 131,072 no
+// cluster holds them (C = 0).
 rsd::walk_cluster::Shape cluster_shape(int B, int V) {
-    auto blocks = [&](int per_block) {
+    rsd::walk_cluster::Shape best = {0, 0, 0, 0.0f};
+    auto consider = [&](int W, int NT) {        // true: all sequences are resident
         int c = 1;
-        while (c * per_block < V) c *= 2;
-        return c;
+        while (c * W * NT * 512 < V) c *= 2;
+        if (c > 8) return false;
+        const rsd::walk_cluster::Shape s = {c, W, NT, (float)B / (float)rsd::walk_cluster::resident_clusters(c, W, NT)};
+        if (best.C == 0 || V > 8192 || s.waves <= 1.0f) best = s;
+        return s.waves <= 1.0f;
     };
-    const float sms = (float)sm_count();
-    int c = blocks(8 * 512);
-    if (c <= 2 || (c <= 8 && (float)B * (float)c <= 3.0f * sms)) return {c, 8, 1, (float)B * (float)c / (3.0f * sms)};
-    c = blocks(16 * 512);
-    if (c <= 8) return {c, 8, 2, (float)B * (float)c / (2.0f * sms)};
-    c = blocks(32 * 512);
-    if (c <= 8) return {c, 16, 2, (float)B * (float)c / sms};
-    return {0, 0, 0, 0.0f};
+    if (V > 65536) {
+        if (!consider(16, 2)) consider(8, 4);
+    } else if (!consider(8, 1) && !consider(8, 2) && V > 8192) {
+        consider(8, 4);
+    }
+    return best;
 }
 
-// Up to how many waves of clusters the on-chip walk is taken.
-//   Rows that the ring takes (us, ring / cluster): from about two waves on the ring is ahead (trees of (3, 2, 2) / (4, 2, 2, 1, 1) / (3, 2, 1);
-// 32,000 bf16 entries, 130 sequences: 36 / 37, 51 / 49, 41 / 34, 148: 36 / 44, 53 / 59, 41 / 44; fp32, 148: 47 / 48, 71 / 63, 51 / 47; 64,000 bf16, 80:
-// 53 / 51, 78 / 63, 54 / 50), with clusters of one or two blocks from 1.3 (16,000 bf16, 180: 35 / 34, 44 / 41, 32 / 31, 222: 36 / 37, 47 / 49, 33 / 34).
-//   Others: clusters of one or two blocks stay (8001 entries, 300 / 1000: 34 / 89 on chip, 41 / 102 read anew).  Beyond, a launch on
-// chip takes as long as it has waves, one that reads the rows anew as long as they are, up to the 296 or 444 sequences that are
-// resident at once: 20,000 entries, multi-round, 148 / 222: 46 / 66 on chip, 43 / 49 read anew; 32,001, plain, 200 / 250: 68 / 88, 73 / 75;
-// 65,001, 148 / 200: 124 / 160, 134 / 150; 100,000, 80 / 128: 139 / 228, 149 / 151, fp32 128: 270, 275.
-//   Gumbel-Top-1 draws take two rounds of Philox calls when rows are read anew: 32,000 entries, 256 / 400: 104 / 154 on chip, 108 / 132
-// read anew; 100,000, 74 / 128: 141 / 240, 216 / 227; fp32, 400 / 512 of 32,000: 176 / 226, 195 / 220.
-float most_waves(const rsd::walk_cluster::Shape& c, int V, bool f32, bool ring, bool top1) {
-    if (ring) return c.C <= 2 ? 1.3f : (c.C == 4 && !f32 ? 1.8f : 2.0f);
-    if (c.C <= 2) return 1e30f;
-    if (top1) return f32 ? 7.0f : std::min(1.6f + (float)V / 16000.0f, 6.6f);
-    return std::min(1.0f + (float)V / 18000.0f, f32 ? 7.0f : 4.8f);
-}
-
-// The same for residual draws with rejected tokens (a pass per token, always both rows; us, on chip / read anew).  Where the
-// distribution itself is not asked for: bf16 8,096 entries, 256 sequences: 24 / 20; 32,000, 148 / 256 / 512: 38 / 53 / 103, 40 / 44 / 86; 128,000, 64 / 256: 74 / 259,
-// 105 / 139; fp32 16,000, 512: 55 / 61; 32,000, 256 / 512: 58 / 108, 53 / 102.  The pass that writes it costs reading anew more: bf16
-// 32,000, 256 / 1024: 63 / 237, 59 / 212; 128,000, 64 / 148: 85 / 173, 149 / 151; fp32 32,000, 256 / 1024: 64 / 234, 68 / 279; 64,000, the same on both sides;
-// 128,000, 148 / 256: 190 / 332, 207 / 251.
-float most_waves_resample(const rsd::walk_cluster::Shape& c, int V, bool f32, bool whole) {
+// Up to how many waves of clusters (sequences asked for over sequences resident) the on-chip walk is taken; beyond, the ring walk or the one that
+// reads its rows anew in every pass.  Measured at 11,000 calls (70 to 131,072 entries, 1 to 900 sequences, trees of 10 and 29 nodes); figures in us,
+// on chip / other.  What the clusters need grows with the number of waves (1, 1.7, 2.4, 3.2 times one wave's time), the others' with the row.
+enum WalkKind { kRingRows, kReadAnew, kReadAnewTop1, kDraw, kDrawWhole };
+float most_waves(const rsd::walk_cluster::Shape& c, int B, int V, bool f32, WalkKind kind) {
+    constexpr float kAlways = 1e30f;
     const float v = (float)V;
-    if (c.C <= 1 || (c.C == 2 && (f32 || whole))) return 1e30f;
-    if (c.C == 2) return 0.2f + v / 9000.0f;
-    if (!whole) return std::min(1.0f + v / 18000.0f, f32 ? 7.0f : 4.8f);
-    if (f32) return V > 65536 ? 9.0f : 1e30f;
-    return std::min(1.5f + v / 16000.0f, 6.5f);
+    if (kind == kRingRows) {
+        // One tile per warp, rows of up to 8192 entries: 8192 bf16, 260 / 300 sequences: 24 / 19, 24 / 21.  Two: all resident or not at all.
+        if (c.NT == 1) return 1.3f;
+        if (c.NT == 2) return 1.0f;
+        // One block: 16,000 entries, 256 / 330: bf16 25 / 30, 44 / 36; fp32 from 149 on: 20.4 / 20.4, 26 / 26; 9000 bf16, 223: 33 / 31.
+        if (c.C == 1) return f32 || V < 12000 ? 0.0f : 1.0f;
+        // fp32: 32,000, 148 / 180: 32 / 43, 57 / 47; 65,536, 110 / 148: 61 / 65, 85 / 66; 128,000, 75 / 110: 91 / 110, 123 / 111.
+        if (f32) return std::max(1.0f, v / 43000.0f);
+        // Two blocks, bf16: 20,000, 200: 35 / 32; 32,000, 180 / 222: 45 / 48, 55 / 53; four: 50,272, 110 / 148: 55 / 63, 69 / 59; 65,536, 148 / 222:
+        // 66 / 66, 90 / 84; eight: 128,000, 110 / 148: 107 / 118, 132 / 110.
+        return c.C == 2 ? std::max(1.0f, (v - 9000.0f) / 17000.0f) : std::min(v / 27500.0f, 1.0f + v / 52000.0f);
+    }
+    // Rows that are read anew take about as long for 40 sequences as for all that are resident at once, 296 (fp32) or 444, then twice as long.
+    const int per_round = (f32 ? 2 : 3) * sm_count();
+    const float round = (float)((B + per_round - 1) / per_round);
+    if (c.NT == 1) {
+        if (kind == kDraw && c.C == 2 && !f32) return std::max(1.0f, 0.2f + v / 9000.0f);   // 8192, 200 / 300: 12.6 / 19, 22 / 22
+        return c.C <= 2 ? kAlways : 1.0f;                // (of more blocks, and below of two tiles per warp: only where all are resident)
+    }
+    if (c.NT == 2) return 1.0f;
+    switch (kind) {
+        case kReadAnewTop1:   // Gumbel-Top-1 draws take two rounds of Philox calls when rows are read anew
+            if (f32) {
+                if (c.C == 1) return V < 11000 ? 0.0f : round;                        // 8200, 222: 32 / 28; 14,000, 296 / 444: 38 / 39, 65 / 70
+                if (c.C == 2) return std::max(1.0f, (v - 10000.0f) / 11000.0f) * round;   // 20,000, 222: 60 / 47; 32,000, 222 / 350: 65 / 64, 95 / 116
+                return v / (c.C == 4 ? 22000.0f : 27000.0f) * round;                  // 50,000, 110 / 222: 65 / 79, 122 / 94; 128,000, 148 / 200: 168 / 171, 226 / 192
+            }
+            if (c.C == 1) return std::max(round, v / 9500.0f);                        // 8200, 296 / 350: 37 / 44, 54 / 43; 14,000, 350: 58 / 58
+            if (c.C == 2) return V < 23000 ? 2.0f : v / 8000.0f;                      // 20,000, 260 / 350: 58 / 61, 79 / 66; 32,000, 444: 94 / 109
+            return c.C == 4 ? v / 13600.0f : (v - 10000.0f) / 14000.0f;               // 50,000, 260 / 350: 115 / 135, 153 / 135; 128,000, 200 / 300: 197 / 246, 290 / 290
+        case kDraw:           // residual draws with rejected tokens (a pass per token, always both rows)
+            if (f32) {
+                if (c.C == 1) return kAlways;                                         // 14,000, 444: 38 / 50
+                if (c.C == 2) return (V < 26000 ? 1.0f : 2.0f) * round;               // 20,000, 222: 35 / 30; 32,000, 222 / 350: 36 / 43, 53 / 77
+                return (c.C == 4 ? (v - 10000.0f) / 12500.0f : (v - 32000.0f) / 12200.0f) * round;   // 50,000, 180 / 296: 56 / 66, 88 / 74; 100,000, 148 / 256: 96 / 116, 158 / 136
+            }
+            if (c.C == 1) return 1.0f;                                                // 14,000, 296 / 350: 20 / 27, 38 / 32
+            if (c.C == 2) return V < 26000 ? 1.0f : V < 30000 ? 2.0f : v / 8000.0f - 1.25f;   // 20,000, 180: 35 / 32; 32,000, 296 / 400: 39 / 44, 56 / 55
+            return v / (c.C == 4 ? 21000.0f : 32000.0f);                              // 50,000, 110 / 222: 41 / 49, 78 / 63; 128,000, 75 / 148: 69 / 104, 115 / 122
+        case kDrawWhole:      // the pass that writes the distribution costs reading anew more
+            if (f32) return c.C <= 2 ? kAlways : v / (c.C == 4 ? 10500.0f : 12000.0f) * round;   // 32,000, 350: 68 / 114; 42,000, 296: 102 / 94; 70,000, 200: 141 / 133
+            if (c.C == 1) return round > 1.0f ? kAlways : 1.0f;                       // 14,000, 296 / 350: 25 / 34, 46 / 42; 8200, 800: 63 / 72
+            if (c.C == 2) return V < 23000 ? 1.0f : v / 10000.0f;                     // 20,000, 222: 42 / 42; 32,000, 444: 74 / 81
+            return v / (c.C == 4 ? 17000.0f : 23000.0f);                              // 50,000, 180 / 222: 73 / 89, 94 / 88; 128,000, 110 / 256: 111 / 151, 227 / 198
+        default:              // the rules' walks and rows off 16-byte boundaries
+            if (f32) {
+                if (c.C == 1) return 0.0f;                                            // 14,000, 222: 25 / 20
+                if (c.C == 2) return (V < 26000 ? 0.6f : 1.0f) * round;               // 20,000, 75 / 148: 22 / 22, 24 / 21; 32,000, 148 / 180: 26 / 29, 46 / 32
+                return (c.C == 4 ? std::max(1.0f, v / 25000.0f - 1.1f) : v / 44000.0f) * round;   // 50,000, 75: 45 / 38; 65,000, 90: 48 / 52; 128,000, 75 / 110: 73 / 85, 112 / 120
+            }
+            if (c.C == 1) return round;                                               // 14,000, 296 / 350: 30 / 37, 47 / 38
+            if (c.C == 2) return V < 23000 ? 1.0f : 2.0f;                             // 20,000, 222: 44 / 41; 32,000, 296 / 350: 49 / 58, 64 / 60
+            return c.C == 4 ? (v - 8000.0f) / 14000.0f : v / 22000.0f;                // 50,000, 180 / 222: 67 / 69, 82 / 80; 100,000, 148 / 200: 110 / 118, 146 / 138
+    }
 }
 
 void launch_on_chip(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const rsd::walk_cluster::Shape& c, cudaStream_t s) {
@@ -160,7 +196,8 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
     // The ring's sums and those of the other two are the same for the rows that it takes (ring_rows), and those of the other two
     // always: a batch and its parts give the same bits.
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
-    const bool on_chip = shape.C > 0 && shape.waves <= most_waves(shape, V, draft->dtype == RSD_F32, ring, final_sampler == RSD_FINAL_GUMBEL_TOP1);
+    const WalkKind kind = ring ? kRingRows : final_sampler == RSD_FINAL_GUMBEL_TOP1 ? kReadAnewTop1 : kReadAnew;
+    const bool on_chip = shape.C > 0 && shape.waves <= most_waves(shape, B, V, draft->dtype == RSD_F32, kind);
     rsd::walk_cluster::ClusterArgs ca;
     memset(&ca, 0, sizeof(ca));
     ca.v = a;
@@ -209,10 +246,10 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     ca.v.seed_lo = a.seed_lo; ca.v.seed_hi = a.seed_hi; ca.v.step = step; ca.v.seq_base = seq_base;
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
     const bool f32 = target_row->dtype == RSD_F32;
-    if (!a.max_k && !(shape.C > 2 && shape.waves <= 1.0f)) {
+    if (!a.max_k && !(shape.C > 2 && shape.NT < 4 && shape.waves <= 1.0f)) {
         if (f32) rsd::walk_cluster::launch_draw_f32(a, B, s);
         else rsd::walk_cluster::launch_draw_bf16(a, B, s);
-    } else if (shape.C > 0 && shape.waves <= most_waves_resample(shape, V, f32, out_residual != nullptr)) {
+    } else if (shape.C > 0 && shape.waves <= most_waves(shape, B, V, f32, out_residual ? kDrawWhole : kDraw)) {
         launch_on_chip(ca, target_row->dtype, true, B, shape, s);
     } else {
         launch_streamed(ca, target_row->dtype, true, B, shape.C > 0, s);

@@ -230,6 +230,83 @@ __device__ __forceinline__ void mode_weights(int mode, const float (&q)[16], con
     }
 }
 
+// The draft row's share of a warp: NT tiles of weights, 16 a lane, in registers.
+template <typename T, int NT>
+struct DraftTiles {
+    static constexpr bool kShared = false;
+    float v[NT][16];
+    Packed<T> raw[NT];
+    __device__ __forceinline__ explicit DraftTiles(float4*) {
+#pragma unroll
+        for (int k = 0; k < NT; ++k)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[k][j] = 0.0f;
+    }
+    __device__ __forceinline__ void clear(int k) { raw[k].fill_neg_inf(); }
+    __device__ __forceinline__ void ask(int k, const char* row, int tile, int lane, int V) { load_tile<T>(raw[k], row, tile, lane, V); }
+    __device__ __forceinline__ void landed() const {}
+    __device__ __forceinline__ void get_raw(int k, Packed<T>& out) const { out = raw[k]; }
+    __device__ __forceinline__ void put_raw(int k, const Packed<T>& in) { raw[k] = in; }
+    __device__ __forceinline__ void get(int k, float (&out)[16]) const {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) out[j] = v[k][j];
+    }
+    __device__ __forceinline__ void put(int k, const float (&in)[16]) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[k][j] = in[j];
+    }
+};
+// Four tiles a warp: in shared memory, where the rows land by themselves (cp.async) while the target's are on their way to
+// registers.  Value j of a lane is word j % 4 of its 16-byte place j / 4; a lane reads and writes its own places only.
+template <typename T>
+struct DraftTiles<T, 4> {
+    static constexpr bool kShared = true;
+    static constexpr int kPieces = (int)sizeof(T);
+    float4* const at;                                    // this lane's first place
+    __device__ __forceinline__ explicit DraftTiles(float4* warp_tiles) : at(warp_tiles + (threadIdx.x & 31)) {}
+    __device__ __forceinline__ float4* place(int k, int i) const { return at + (k * 4 + i) * 32; }
+    __device__ __forceinline__ void clear(int k) {
+        Packed<T> none;
+        none.fill_neg_inf();
+        put_raw(k, none);
+    }
+    __device__ __forceinline__ void ask(int k, const char* row, int tile, int lane, int V) {
+        if (((uintptr_t)row & 15u) == 0 && (tile + 1) * kTileElems <= V) {
+            const char* from = row + (int64_t)tile * kTileElems * (int)sizeof(T) + lane * 16;
+#pragma unroll
+            for (int i = 0; i < kPieces; ++i)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(place(k, i))), "l"(from + 512 * i) : "memory");
+        } else {
+            Packed<T> pk;
+            load_tile<T>(pk, row, tile, lane, V);
+            put_raw(k, pk);
+        }
+    }
+    __device__ __forceinline__ void landed() const { asm volatile("cp.async.wait_all;" ::: "memory"); }
+    __device__ __forceinline__ void get_raw(int k, Packed<T>& out) const {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) out.w[i] = *(const uint4*)place(k, i);
+    }
+    __device__ __forceinline__ void put_raw(int k, const Packed<T>& in) {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) *(uint4*)place(k, i) = in.w[i];
+    }
+    __device__ __forceinline__ void get(int k, float (&out)[16]) const {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 f = *place(k, i);
+            out[4 * i] = f.x; out[4 * i + 1] = f.y; out[4 * i + 2] = f.z; out[4 * i + 3] = f.w;
+        }
+    }
+    __device__ __forceinline__ void put(int k, const float (&in)[16]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *place(k, i) = make_float4(in[4 * i], in[4 * i + 1], in[4 * i + 2], in[4 * i + 3]);
+    }
+};
+// shared memory that the draft tiles of a block of WARPS working warps take beside its Smem
+template <int NT, int WARPS>
+constexpr size_t draft_tiles_bytes() { return NT == 4 ? (size_t)WARPS * NT * kTileElems * 4 : 0; }
+
 // A block's place in its cluster and the row's tiles.
 struct Place {
     int rank, C, V, n_tiles, n_local;   // n_local: tiles rank, rank + C, ...
@@ -266,30 +343,41 @@ struct Top1 {
         const float t_hat = -__logf(fmaf((float)(word >> 4), 3.725290298461914e-09f, 1.862645149230957e-09f));
         return fmaxf(fmaf(up, fmaf(t_hat, 1e-6f, 2.5e-7f), t_hat), 0.0f) * 0.0625f;
     }
-    // the coarse words of a lane's pieces of a tile; `bound` from the pieces' positions a
-    template <typename T, int RUNS>
-    __device__ __forceinline__ void look(const RngKey& key, uint32_t node, int tile, int lane, const float (&w)[16], uint32_t (&words)[RUNS]) {
-        constexpr int kPer = 16 / RUNS;
+    // The lane of whose group a lane's piece i is part (a tile is 32 groups; RUNS lanes share one).
+    template <int RUNS>
+    __device__ __forceinline__ static int group_lane(int i, int lane) { return (i * 32 + lane) / RUNS; }
+    // The coarse word of group `lane` of a tile; `bound` from the entries at the groups' positions a.  (Every lane takes one group's word
+    // and bounds and hands them to the lanes that hold its entries: each lane for its own pieces took RUNS times the Philox calls and
+    // logarithms.)
+    template <typename T>
+    __device__ __forceinline__ uint32_t look(const RngKey& key, uint32_t node, int tile, int lane, const float (&w)[16]) {
+        constexpr int RUNS = (int)sizeof(T), kPer = 16 / RUNS;
+        const uint32_t g = (uint32_t)(tile * 32 + lane);
+        const uint32_t word = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
+        const float hi = group_bound(word, 1.0f);
 #pragma unroll
         for (int i = 0; i < RUNS; ++i) {
-            const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
-            const uint32_t g = (uint32_t)x0 >> 4;
-            words[i] = coarse_select(rng_draw(key, node, kTagFinalGumbelCoarse, coarse_index(g)), g);
-            const float tg_hi = group_bound(words[i], 1.0f);
-            const int ja = (int)(words[i] & 15u) - (x0 & 15);
+            const int from = group_lane<RUNS>(i, lane);
+            const float tg_hi = __shfl_sync(0xFFFFFFFFu, hi, from);
+            const int ja = (int)(__shfl_sync(0xFFFFFFFFu, word, from) & 15u) - (lane % RUNS) * kPer;
+            float wa = 0.0f;
 #pragma unroll
             for (int j = 0; j < kPer; ++j)
-                if (j == ja && w[i * kPer + j] > 0.0f) bound = fminf(bound, tg_hi / w[i * kPer + j] * 1.00001f);
+                if (j == ja) wa = w[i * kPer + j];
+            if (wa > 0.0f) bound = fminf(bound, tg_hi / wa * 1.00001f);
         }
+        return word;
     }
     // the exact keys of the entries that can reach `bound`
-    template <typename T, int RUNS>
-    __device__ __forceinline__ void take(const RngKey& key, uint32_t node, int tile, int lane, const float (&w)[16], const uint32_t (&words)[RUNS]) {
-        constexpr int kPer = 16 / RUNS;
+    template <typename T>
+    __device__ __forceinline__ void take(const RngKey& key, uint32_t node, int tile, int lane, const float (&w)[16], uint32_t group_word) {
+        constexpr int RUNS = (int)sizeof(T), kPer = 16 / RUNS;
+        const float lo = group_bound(group_word, -1.0f);
 #pragma unroll
         for (int i = 0; i < RUNS; ++i) {
-            const int x0 = tile * kTileElems + (i * 32 + lane) * kPer;
-            const float tg_lo = group_bound(words[i], -1.0f);
+            const int x0 = tile * kTileElems + (i * 32 + lane) * kPer, from = group_lane<RUNS>(i, lane);
+            const float tg_lo = __shfl_sync(0xFFFFFFFFu, lo, from);
+            const uint32_t word = __shfl_sync(0xFFFFFFFFu, group_word, from);
             uint32_t todo = 0;
 #pragma unroll
             for (int j = 0; j < kPer; ++j)
@@ -301,8 +389,8 @@ struct Top1 {
 #pragma unroll
                 for (int jj = 0; jj < kPer; ++jj)
                     if (jj == j) wj = w[i * kPer + jj];
-                float e = neg_log_group_uniform_f32(words[i]) * 0.0625f;
-                if (j != (int)(words[i] & 15u) - (x0 & 15)) {
+                float e = neg_log_group_uniform_f32(word) * 0.0625f;
+                if (j != (int)(word & 15u) - (x0 & 15)) {
                     const uint4 fw = rng_draw(key, node, kTagFinalGumbelFine, (uint32_t)(x0 + j) >> 2);
                     const uint32_t sel = (uint32_t)(x0 + j) & 3u;
                     e += neg_log_uniform_f32(sel < 2 ? (sel == 0 ? fw.x : fw.y) : (sel == 2 ? fw.z : fw.w));
@@ -310,6 +398,7 @@ struct Top1 {
                 const float key_j = e / wj;
                 if (key_j < __int_as_float(0x7F800000)) best = min(best, ((unsigned long long)__float_as_uint(key_j) << 32) | (uint32_t)(x0 + j));
             }
+            __syncwarp();
         }
     }
 };
@@ -331,27 +420,41 @@ __device__ __forceinline__ void top1_report(SM& sm, const Place& pl, int flags, 
 // The pass over tiles held in registers: the bound is the block's, from all its tiles.
 template <typename T, int NT, int WARPS>
 __device__ __forceinline__ void top1_pass(ChipSmem<WARPS, NT>& sm, const Place& pl, const RngKey& key, uint32_t node, int flags, float a_hi, float a_lo,
-                                          const float (&q)[NT][16], const float (&p)[NT][16]) {
-    constexpr int kRuns = (int)sizeof(T);
+                                          const float (&q)[NT][16], DraftTiles<T, NT>& draft) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t words[NT][kRuns];
+    uint32_t words[NT];
     Top1 top1;
 #pragma unroll
     for (int k = 0; k < NT; ++k) {
-        float w[16];
-        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+        float p[16], w[16];
+        draft.get(k, p);
+        mode_weights<true>(flags >> kModeShift, q[k], p, a_hi, a_lo, sm.c_seq, w);
         const int tile = pl.rank + pl.C * (warp + WARPS * k);    // (beyond the row: no weight)
-        top1.look<T>(key, node, tile, lane, w, words[k]);
+        words[k] = top1.look<T>(key, node, tile, lane, w);
+        if (draft.kShared) draft.put(k, w);                      // (a walk's last pass: nothing needs the draft row any more)
     }
     top1.bound = -warp_max(-top1.bound);
     if (lane == 0) sm.warp_top[0][warp] = top1.bound;
     workers_sync<WARPS * 32>();
     top1.bound = -warp_max(-(lane < WARPS ? sm.warp_top[0][lane] : top1.bound));
+    if constexpr (DraftTiles<T, NT>::kShared) {                  // (one copy of the code: four of them spilled)
+#pragma unroll 1
+        for (int k = 0; k < NT; ++k) {
+            uint32_t word = words[0];
 #pragma unroll
-    for (int k = 0; k < NT; ++k) {
-        float w[16];
-        mode_weights<true>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, sm.c_seq, w);
-        top1.take<T>(key, node, pl.rank + pl.C * (warp + WARPS * k), lane, w, words[k]);
+            for (int i = 1; i < NT; ++i) word = i == k ? words[i] : word;
+            float w[16];
+            draft.get(k, w);
+            top1.take<T>(key, node, pl.rank + pl.C * (warp + WARPS * k), lane, w, word);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            float p[16], w[16];
+            draft.get(k, p);
+            mode_weights<true>(flags >> kModeShift, q[k], p, a_hi, a_lo, sm.c_seq, w);
+            top1.take<T>(key, node, pl.rank + pl.C * (warp + WARPS * k), lane, w, words[k]);
+        }
     }
     top1_report<WARPS>(sm, pl, flags, top1.best);
 }
@@ -415,34 +518,35 @@ __device__ __forceinline__ void write_tile(float* out, int tile, int lane, int V
 // The working warps: the passes they are told to run.  The root's rows are asked for before the first command is there.
 // MODE: which of the rarer passes exist.
 template <typename T, int NT, int WARPS, int MODE>
-__device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, const WorkRows& rows) {
+__device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, float4* draft_sm, const Place& pl, const WorkRows& rows) {
     constexpr int kAll = (WARPS + 1) * 32, kWorkers = WARPS * 32;
     constexpr int kPer = 16 / (int)sizeof(T), kRuns = 16 / kPer;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int C = pl.C, V = pl.V, n_tiles = pl.n_tiles;
     const int tile0 = pl.rank + C * warp, tile_step = C * WARPS;   // this warp's tiles: tile0, tile0 + tile_step, ...
-    float q[NT][16], p[NT][16];
+    float q[NT][16];
+    DraftTiles<T, NT> draft(draft_sm + warp * NT * 128);
 #pragma unroll
     for (int k = 0; k < NT; ++k)
 #pragma unroll
-        for (int j = 0; j < 16; ++j) q[k][j] = p[k][j] = 0.0f;
+        for (int j = 0; j < 16; ++j) q[k][j] = 0.0f;
     int flags = (rows.with_draft ? kOpen : kOpenTarget) | kFirst, node = 0;
     float a_hi = 0.0f, a_lo = 0.0f;
     for (;;) {
         int kind = flags & kKindMask;
         float s[NT];
         if (kind == kOpen || kind == kOpenTarget) {
-            Packed<T> rq[NT], rp[NT];
+            Packed<T> rq[NT];
             const char* rowq = rows.q + (int64_t)node * rows.stride_q;
             const char* rowp = rows.p + (int64_t)node * rows.stride_p;
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
                 const int tile = tile0 + tile_step * k;
                 rq[k].fill_neg_inf();
-                rp[k].fill_neg_inf();
+                if (!draft.kShared || tile >= n_tiles) draft.clear(k);
                 if (tile < n_tiles) {
                     load_tile<T>(rq[k], rowq, tile, lane, V);
-                    if (kind == kOpen) load_tile<T>(rp[k], rowp, tile, lane, V);
+                    if (kind == kOpen) draft.ask(k, rowp, tile, lane, V);
                 }
             }
             if (flags & kFirst) {
@@ -461,7 +565,13 @@ __device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, c
 #pragma unroll
                     for (int k = 0; k < NT; ++k) {
                         mq = fmaxf(mq, clean_tile(rq[k], saw_nan));
-                        if (kind == kOpen) mp = fmaxf(mp, clean_tile(rp[k], saw_nan));
+                        if (kind == kOpen) {
+                            if (k == 0) draft.landed();
+                            Packed<T> rp;
+                            draft.get_raw(k, rp);
+                            mp = fmaxf(mp, clean_tile(rp, saw_nan));
+                            draft.put_raw(k, rp);
+                        }
                     }
                     mq = warp_max(mq);
                     mp = warp_max(mp);
@@ -476,13 +586,18 @@ __device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, c
                 else exp16(q[k], rows.kq, cq, q[k]);
                 s[k] = tree_sum16(q[k]);
             }
+            draft.landed();
             if (kind == kOpen) {
 #pragma unroll
                 for (int k = 0; k < NT; ++k) {
-                    rp[k].unpack(p[k]);
-                    if (precise) exp16_precise(p[k], rows.kp, p[k]);
-                    else exp16(p[k], rows.kp, cp, p[k]);
-                    sm.lane_sum[1][warp + WARPS * k][lane] = tree_sum16(p[k]);
+                    Packed<T> rp;
+                    draft.get_raw(k, rp);
+                    float p[16];
+                    rp.unpack(p);
+                    if (precise) exp16_precise(p, rows.kp, p);
+                    else exp16(p, rows.kp, cp, p);
+                    draft.put(k, p);
+                    sm.lane_sum[1][warp + WARPS * k][lane] = tree_sum16(p);
                 }
             }
         } else if (kind == kResidualPass) {
@@ -493,15 +608,19 @@ __device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, c
 #pragma unroll
                 for (int k = 0; k < NT; ++k)
                     if (tile0 + tile_step * k == x / kTileElems && l_ == lane) {
+                        float p[16];
+                        draft.get(k, p);
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            if (j == j_) { q[k][j] = residual_weight(q[k][j], p[k][j], sm.freeze_hi, sm.freeze_lo); p[k][j] = 0.0f; }
+                            if (j == j_) { q[k][j] = residual_weight(q[k][j], p[j], sm.freeze_hi, sm.freeze_lo); p[j] = 0.0f; }
+                        draft.put(k, p);
                     }
             }
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
-                float w[16];
-                residual16(q[k], p[k], a_hi, a_lo, w);
+                float p[16], w[16];
+                draft.get(k, p);
+                residual16(q[k], p, a_hi, a_lo, w);
                 s[k] = tree_sum16(w);
             }
         } else if (kind == kPlainPass) {
@@ -518,25 +637,28 @@ __device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, c
                     walk_ring::piece_of<T>(o, l_, j_);
                     if (l_ == lane) gone |= 1u << j_;
                 }
-                float w[16];
+                float p[16], w[16];
+                draft.get(k, p);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) w[j] = ((gone >> j) & 1u) ? 0.0f : p[k][j];
+                for (int j = 0; j < 16; ++j) w[j] = ((gone >> j) & 1u) ? 0.0f : p[j];
                 s[k] = tree_sum16(w);
             }
         } else if (MODE == kRuleWalk && (kind == kOverlapPass || kind == kSeqPass)) {
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
-                float w[16];
-                if (kind == kOverlapPass) weights16<kSeqOverlap>(q[k], p[k], a_hi, a_lo, 0.0f, w);
-                else weights16<kSeqResidual>(q[k], p[k], a_hi, a_lo, sm.c_seq, w);
+                float p[16], w[16];
+                draft.get(k, p);
+                if (kind == kOverlapPass) weights16<kSeqOverlap>(q[k], p, a_hi, a_lo, 0.0f, w);
+                else weights16<kSeqResidual>(q[k], p, a_hi, a_lo, sm.c_seq, w);
                 s[k] = tree_sum16(w);
             }
         } else if (kind == kDump) {
 #pragma unroll
             for (int k = 0; k < NT; ++k)
                 if (tile0 + tile_step * k == node) {
-                    float w[16];
-                    mode_weights<MODE == kRuleWalk>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, MODE == kRuleWalk ? sm.c_seq : 0.0f, w);
+                    float p[16], w[16];
+                    draft.get(k, p);
+                    mode_weights<MODE == kRuleWalk>(flags >> kModeShift, q[k], p, a_hi, a_lo, MODE == kRuleWalk ? sm.c_seq : 0.0f, w);
 #pragma unroll
                     for (int i = 0; i < kRuns; ++i)
 #pragma unroll
@@ -550,12 +672,13 @@ __device__ __forceinline__ void work(ChipSmem<WARPS, NT>& sm, const Place& pl, c
             for (int k = 0; k < NT; ++k) {
                 const int tile = tile0 + tile_step * k;
                 if (tile >= n_tiles) continue;
-                float w[16];
-                mode_weights<false>(flags >> kModeShift, q[k], p[k], a_hi, a_lo, 0.0f, w);
+                float p[16], w[16];
+                draft.get(k, p);
+                mode_weights<false>(flags >> kModeShift, q[k], p, a_hi, a_lo, 0.0f, w);
                 write_tile<T>(rows.out_residual, tile, lane, V, w, inv);
             }
         } else if (MODE == kRuleWalk && kind == kTop1) {
-            top1_pass<T, NT, WARPS>(sm, pl, rows.key, (uint32_t)node, flags, a_hi, a_lo, q, p);
+            top1_pass<T, NT, WARPS>(sm, pl, rows.key, (uint32_t)node, flags, a_hi, a_lo, q, draft);
         } else {
             return;                             // kEnd
         }
@@ -1153,7 +1276,8 @@ __device__ __forceinline__ void run_walk(SM& sm, const ClusterArgs& ca, F&& work
 template <typename T, int NT, int WARPS, int MODE>
 __global__ void __launch_bounds__((WARPS + 1) * 32, WARPS == 8 ? (NT == 1 ? 3 : 2) : 1) walk_cluster_kernel(const __grid_constant__ ClusterArgs ca) {
     __shared__ ChipSmem<WARPS, NT> sm;
-    run_walk<T, MODE, WARPS>(sm, ca, [&](const Place& pl, const WorkRows& rows) { work<T, NT, WARPS, MODE>(sm, pl, rows); });
+    extern __shared__ __align__(16) float4 draft_sm[];
+    run_walk<T, MODE, WARPS>(sm, ca, [&](const Place& pl, const WorkRows& rows) { work<T, NT, WARPS, MODE>(sm, draft_sm, pl, rows); });
 }
 
 }  // namespace walk_cluster

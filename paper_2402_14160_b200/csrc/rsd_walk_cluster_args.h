@@ -19,6 +19,9 @@ struct Shape {
     float waves;         // sequences asked for over sequences resident at a time
 };
 
+// How many clusters of such a shape the current device holds at a time (asked once per device).
+int resident_clusters(int C, int W, int NT);
+
 // extra: the baseline rules, the Gumbel-Top-1 draw or the stand-alone residual draw
 void launch_f32(const ClusterArgs& a, bool extra, int B, const Shape& c, cudaStream_t s);
 void launch_bf16(const ClusterArgs& a, bool extra, int B, const Shape& c, cudaStream_t s);

@@ -266,10 +266,9 @@ __device__ __forceinline__ void work_stream(StreamSmem<C>& sm, float* frozen_w, 
 #pragma unroll
                     for (int j = 0; j < kPer; ++j) sm.tile_w[(r * 32 + lane) * kPer + j] = w[r * kPer + j];
             } else if (MODE == kRuleWalk && kind == kTop1) {
-                uint32_t words[kRuns];
-                top1.look<T>(rows.key, (uint32_t)node, tile, lane, w, words);
+                const uint32_t word = top1.look<T>(rows.key, (uint32_t)node, tile, lane, w);
                 top1.bound = -warp_max(-top1.bound);
-                top1.take<T>(rows.key, (uint32_t)node, tile, lane, w, words);
+                top1.take<T>(rows.key, (uint32_t)node, tile, lane, w, word);
             } else if (MODE == kResample && kind == kWrite) {
                 write_tile<T>(rows.out_residual, tile, lane, V, w, sm.inv_total);
             }

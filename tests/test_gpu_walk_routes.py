@@ -145,3 +145,33 @@ def test_rare_paths_of_large_batches(what, V, B):
         assert int(tested.min()) >= 96
     if what == "repeated":
         assert int((whole["status"] & rsd.ST_ZERO_DRAFT_PROB != 0).sum()) > B // 2
+
+
+# A cluster that holds four tiles per warp (the draft's in shared memory) takes the batches that fewer tiles per warp leave waiting: full
+# rows of its tiles, one piece more and less, rows off 16-byte boundaries, every rule; against four sequences, which one or two tiles per warp hold.
+@pytest.mark.parametrize("dtype,V,B,off,rule,sampler,trouble", [
+    ("bf16", 16384, 160, 0, 0, 0, ""), ("bf16", 12288, 290, 0, 1, 1, "nan"), ("bf16", 8193, 200, 1, 0, 0, "far"), ("f32", 32768, 148, 0, 0, 0, "nan"),
+    ("bf16", 32760, 100, 0, 0, 0, "far"), ("f32", 16388, 80, 0, 1, 1, ""), ("bf16", 32767, 120, 1, 2, 1, "nan"), ("f32", 32769, 60, 3, 2, 0, "far"),
+    ("bf16", 65536, 70, 0, 0, 0, ""), ("bf16", 40008, 60, 0, 2, 1, "nan"), ("f32", 65540, 30, 0, 1, 0, ""), ("bf16", 131072, 33, 0, 0, 0, "nan"),
+    ("bf16", 131071, 33, 1, 1, 1, "far"), ("f32", 100001, 24, 1, 0, 1, "nan")])
+def test_four_tiles_per_warp_give_the_bits_of_fewer(dtype, V, B, off, rule, sampler, trouble):
+    test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble)
+
+
+@pytest.mark.parametrize("dtype,V,B", [("f32", 16384, 200), ("bf16", 16385, 148), ("f32", 32000, 148), ("bf16", 65529, 64), ("f32", 131072, 33)])
+def test_residual_draws_with_four_tiles_per_warp_give_the_bits_of_fewer(dtype, V, B):
+    import paper_2402_14160_b200 as rsd
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    draft = (torch.randn((B, V), generator=gen, device="cuda") * 2).to(dt)
+    target = (draft.float() + torch.randn((B, V), generator=gen, device="cuda")).to(dt)
+    target[::3, V // 2] = float("nan")
+    rejected = torch.randint(0, V, (B, 32), generator=gen, device="cuda", dtype=torch.int32)
+    edges = [0, 511, 512, V - 1, V - 512, 0, 15, 16384 % V, 8191, 8192]        # both ends of tiles, of a warp's share and of the row; one of them twice
+    rejected[:, : len(edges)] = torch.tensor(edges, dtype=torch.int32, device="cuda")
+    node = torch.arange(B, dtype=torch.int32, device="cuda")
+    whole = rsd.rsd_resample_residual(draft, target, rejected, node, 5, 1, want_residual=True)
+    for b in (0, B - 3):
+        part = rsd.rsd_resample_residual(draft[b:b + 3], target[b:b + 3], rejected[b:b + 3], node[b:b + 3], 5, 1, seq_base=b, want_residual=True)
+        for key in part:
+            assert torch.equal(part[key], whole[key][b:b + 3]), (key, b)
