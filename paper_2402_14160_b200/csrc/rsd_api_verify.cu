@@ -114,7 +114,7 @@ float most_waves(const rsd::walk_cluster::Shape& c, int B, int V, bool f32, Walk
         case kDrawWhole:      // the pass that writes the distribution costs reading anew more
             if (f32) return c.C <= 2 ? kAlways : v / (c.C == 4 ? 10500.0f : 12000.0f) * round;   // 32,000, 350: 68 / 114; 42,000, 296: 102 / 94; 70,000, 200: 141 / 133
             if (c.C == 1) return round > 1.0f ? kAlways : 1.0f;                       // 14,000, 296 / 350: 25 / 34, 46 / 42; 8200, 800: 63 / 72
-            if (c.C == 2) return V < 23000 ? 1.0f : v / 10000.0f;                     // 20,000, 222: 42 / 42; 32,000, 444: 74 / 81
+            if (c.C == 2) return V < 25000 ? 1.0f : v / 10000.0f;                     // 20,000, 222: 42 / 42; 24,000, 320: 65 / 61; 32,000, 444: 74 / 81
             return v / (c.C == 4 ? 17000.0f : 23000.0f);                              // 50,000, 180 / 222: 73 / 89, 94 / 88; 128,000, 110 / 256: 111 / 151, 227 / 198
         default:              // the rules' walks and rows off 16-byte boundaries
             if (f32) {

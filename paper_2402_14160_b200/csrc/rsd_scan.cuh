@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
 // For a fixed parent psi is increasing in phi~ (Theorem 3.2's argument), so the W best pairs over all parents are
 // among each parent's own W best by phi~.  The scan above leaves those n_par * W finalists in scratch; this kernel
 // recomputes their noise in double, applies the truncation T of Eq. 11 in the stable form
-//   w = log1p(-exp(phi~ - Z)),  v = Gamma - phi~ + w,  psi = Gamma - max(v, 0) - log1p(exp(-|v|)),
+//   psi = Gamma - log1p(exp(Gamma - phi~) (1 - exp(phi~ - Z))),
 // and keeps the W best by (psi desc, parent asc, token asc).
 // ---------------------------------------------------------------------------------------------------------
 struct SbsEpilogueArgs {
@@ -1023,9 +1023,9 @@ __device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, cons
         const double d = pert - z;
         double psi = gamma;
         if (!(d >= 0.0)) {
-            const double w = log1p(-exp(d));
-            const double v = gamma - pert + w;
-            psi = gamma - fmax(v, 0.0) - log1p(exp(-fabs(v)));
+            // (two functions one after the other instead of four: the levels' latency is that of dependent double-precision code)
+            const double x = -expm1(d), t = gamma - pert;
+            psi = t < 700.0 ? gamma - log1p(exp(t) * x) : pert - log(x);
         }
         s_psi[i] = psi;
     }
