@@ -46,7 +46,7 @@ int scan_threads(int rows, int V, bool f32, bool need_lse) {
     return V >= 4096 && few ? 256 : 128;
 }
 
-void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs& a, cudaStream_t s) {
+void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs& a, cudaStream_t s, const rsd::SbsEpilogueArgs* level = nullptr) {
     const bool aligned = a.V % 16 == 0 && rows_aligned(rows, 32);   // rows made of whole groups that start on 32-byte boundaries
     for (int r = 0; r < 10; ++r) {
         a.rk0[r] = a.seed_lo + (uint32_t)r * 0x9E3779B9u;
@@ -54,10 +54,20 @@ void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs&
     }
     if (g_scan_before) cudaEventRecord(g_scan_before, s);
     const int threads = scan_threads(blocks, a.V, rows->dtype == RSD_F32, need_lse);
-    if (rows->dtype == RSD_F32) rsd::launch_scan_f32(threads, aligned, need_lse, blocks, a, s);
+    if (level && rows->dtype == RSD_F32) rsd::launch_level_f32(threads, aligned, need_lse, blocks, a, *level, s);
+    else if (level) rsd::launch_level_bf16(threads, aligned, need_lse, blocks, a, *level, s);
+    else if (rows->dtype == RSD_F32) rsd::launch_scan_f32(threads, aligned, need_lse, blocks, a, s);
     else rsd::launch_scan_bf16(threads, aligned, need_lse, blocks, a, s);
     if (g_scan_after) cudaEventRecord(g_scan_after, s);
     g_scan_before = g_scan_after = nullptr;
+}
+
+// A level of few rows runs in one launch, the rows of a sequence as a cluster; its blocks stay until the longest of them is through, so
+// that many or long rows are better scanned by themselves (us, one launch / two; bf16 32,000 entries, 4 / 224 / 368 rows: 13.4 / 14.9, 18.6 / 19.6, 21.0 / 23.5;
+// fp32 65,536, 192 / 224 / 368: 25.1 / 25.0, 27.9 / 26.6, 37.3 / 35.5; 128,000, 8 / 64 / 192: 17.2 / 19.2, 19.7 / 18.7, 27.4 / 27.1; fp32 4096, 300 / 592: 12.8 / 16.1, 16.9 / 14.6).
+bool level_in_one_launch(int B, int n_par, int V) {
+    const int64_t rows = (int64_t)B * n_par;
+    return n_par <= rsd::kMaxLevelRows && rows <= 370 && rows * V <= (V > 65536 ? 6000000 : 12000000);
 }
 
 // status[0..B) = 0 ahead of a kernel that ORs bits into it, which does not wait for this one until it touches status (a memset
@@ -175,9 +185,6 @@ int rsd_sbs_step(const rsd_rows* draft_level, int B, int n_par, int V, int W, in
     a.status = status; a.row_status = row_status;   // status[b] is written by the epilogue
     a.wait_first = 1;
     a.temp = temperature_of(draft_level); a.inv_temp = 1.0f / a.temp; a.raw_values = 1;
-    launch_scan(draft_level, !rows_are_logprob(draft_level), B * n_par, a, s);
-    if (int e = check_launch("rsd_sbs_step(scan)")) return e;
-
     rsd::SbsEpilogueArgs e;
     e.n_par = n_par; e.W = W; e.is_logprob = rows_are_logprob(draft_level);
     e.fin_seq_stride = (int64_t)n_par * W; e.row_seq_stride = n_par; e.state_stride = n_par; e.out_state_stride = W; e.inv_temp = 1.0 / (double)temperature_of(draft_level); e.first_parent_node = first_parent_node;
@@ -188,6 +195,13 @@ int rsd_sbs_step(const rsd_rows* draft_level, int B, int n_par, int V, int W, in
     e.out_token = out_token; e.out_parent = out_parent; e.out_stride = out_stride; e.parent_base = parent_base;
     e.sum_out = sum_logprob_out; e.gamma_out = trunc_gumbel_out;
     e.out_count = out_count; e.status = status;
+    const bool need_lse = !rows_are_logprob(draft_level);
+    if (level_in_one_launch(B, n_par, V)) {
+        launch_scan(draft_level, need_lse, B * n_par, a, s, &e);
+        return check_launch("rsd_sbs_step(level)");
+    }
+    launch_scan(draft_level, need_lse, B * n_par, a, s);
+    if (int err = check_launch("rsd_sbs_step(scan)")) return err;
     const size_t smem = rsd::sbs_level_scratch_bytes(n_par, W);
     launch_overlapped(rsd::sbs_epilogue_kernel, (unsigned)B, rsd::kEpilogueThreads, smem, s, 0, e);
     return check_launch("rsd_sbs_step(epilogue)");

@@ -12,6 +12,8 @@
 #pragma once
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "rsd_device.cuh"
 
 namespace rsd {
@@ -60,6 +62,10 @@ struct ScanArgs {
 // One block of `threads` threads per row, `blocks` rows (defined in rsd_scan_f32.cu and rsd_scan_bf16.cu).
 void launch_scan_f32(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, cudaStream_t s);
 void launch_scan_bf16(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, cudaStream_t s);
+// The same with the level ended by the rows' cluster (a.R blocks a sequence).
+struct SbsEpilogueArgs;
+void launch_level_f32(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, const SbsEpilogueArgs& e, cudaStream_t s);
+void launch_level_bf16(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, const SbsEpilogueArgs& e, cudaStream_t s);
 
 // Packed pairs of fp32 (sm_100 executes fma/add on two floats per instruction).
 __device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
@@ -433,6 +439,225 @@ __host__ __device__ constexpr size_t scan_buffer_bytes() {
 }
 __host__ __device__ inline size_t scan_bounds_bytes(int V) { return 4 * (size_t)((((V + 15) / 16) + 3) / 4 * 4); }   // padded to fours
 
+// ---------------------------------------------------------------------------------------------------------
+// Stochastic Beam Search level, per-sequence epilogue.
+// For a fixed parent psi is increasing in phi~ (Theorem 3.2's argument), so the W best pairs over all parents are
+// among each parent's own W best by phi~.  The scan above leaves those n_par * W finalists in scratch; this kernel
+// recomputes their noise in double, applies the truncation T of Eq. 11 in the stable form
+//   psi = Gamma - log1p(exp(Gamma - phi~) (1 - exp(phi~ - Z))),
+// and keeps the W best by (psi desc, parent asc, token asc).
+// ---------------------------------------------------------------------------------------------------------
+struct SbsEpilogueArgs {
+    int n_par, W, is_logprob;
+    int64_t fin_seq_stride;    // elements between sequences in fin_token / fin_value / fin_pert (n_par * W for one level)
+    int64_t row_seq_stride;    // elements between sequences in fin_lse / row_status (n_par for one level)
+    int64_t state_stride;      // elements between sequences in sum_in / gamma_in (n_par for one level)
+    int64_t out_state_stride;  // elements between sequences in sum_out / gamma_out (W; 0 when they hold one sequence)
+    double inv_temp;           // 1 / temperature of the parents' rows (1: none)
+    int32_t first_parent_node;
+    uint32_t seed_lo, seed_hi, step, seq_base;
+    const int32_t* fin_token;  // [B][n_par][W]
+    const float* fin_value;    // [B][n_par][W] the row's own value at the finalist
+    const float* fin_pert;     // [B][n_par][W] value + noise in fp32 (decreasing within a parent)
+    const float* fin_lse;      // [B][n_par]
+    const int32_t* row_status; // [B][n_par] status bits of the row scans
+    const float* sum_in;       // [B][n_par] or null
+    const float* gamma_in;     // [B][n_par] or null
+    int32_t* out_token;   // [B][out_stride]
+    int32_t* out_parent;  // [B][out_stride], parent_base added
+    int64_t out_stride;
+    int32_t parent_base;
+    float* sum_out;
+    float* gamma_out;
+    int32_t* out_count;
+    int32_t* status;
+};
+
+constexpr int kEpilogueThreads = 128;
+
+// bytes of shared memory one level needs in sbs_epilogue_body, rounded up to 16
+__host__ __device__ inline size_t sbs_level_scratch_bytes(int n_par, int W) {
+    return (((size_t)n_par * W * 32 + (size_t)n_par * 12) + 15) & ~(size_t)15;
+}
+
+// order-preserving map of a double to an unsigned integer (for an atomic maximum), and back; 0 stands for "none"
+__device__ __forceinline__ unsigned long long double_to_ordered(double v) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double ordered_to_double(unsigned long long k) {
+    if (k == 0) return -__longlong_as_double(0x7FF0000000000000LL);
+    return __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
+}
+
+// -ln of the exponential form of a token's Gumbel noise, in double: G(x) = -sbs_log_noise
+__device__ __forceinline__ double sbs_log_noise(const RngKey& key, uint32_t node, uint32_t x) {
+    const uint32_t word = coarse_word(key, node, x >> 4);
+    const double t_elem = ((x & 15u) != (word & 15u)) ? neg_log_uniform_f64(fine_word(key, node, x)) : 0.0;
+    return log(neg_log_group_uniform_f64(word) * 0.0625 + t_elem);
+}
+
+// One level for sequence b, by a block of THREADS threads; sm_d: sbs_level_scratch_bytes(n_par, W) bytes.
+// noise: sbs_log_noise of the level's finalists, [n_par][W], or null (then it is taken here).
+template <int THREADS = kEpilogueThreads>
+__device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, const int b, double* sm_d, const double* noise = nullptr) {
+    const int F = a.n_par * a.W;
+    // the finalists that pass the first test are gathered in a list; entry i of the arrays below belongs to list[i]
+    double* s_pert = sm_d;                   // [F] phi~
+    double* s_phi = sm_d + F;                // [F] phi
+    double* s_psi = sm_d + 2 * F;            // [F] psi
+    unsigned long long* s_z = (unsigned long long*)(sm_d + 3 * F);   // [n_par] largest phi~ of the parent, ordered
+    int* s_list = (int*)(s_z + a.n_par);     // [F] finalist index f = parent * W + place
+    int* s_tok = s_list + F;                 // [F] its token
+    float* s_gam = (float*)(s_tok + F);      // [n_par]
+    const int tid = threadIdx.x;
+    const int64_t fin_off = (int64_t)b * a.fin_seq_stride, row_off = (int64_t)b * a.row_seq_stride,
+                  state_off = (int64_t)b * a.state_stride;
+    const RngKey key = {a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
+
+    // A child enters the beam only if its psi reaches the W-th best psi of the level.  The best child of parent j has
+    // psi = Gamma_j exactly, so that bound is at least L = the W-th largest Gamma among the parents that deliver a
+    // child (valid parent, at least one finalist); L = -inf when fewer than W do.  Finalists that a cheap fp32 test
+    // shows to lie clearly below L are dropped before the double-precision work; a parent's best finalist is
+    // always kept.
+    __shared__ float s_L;
+    __shared__ int s_row_bits, s_n;
+    if (tid == 0) { s_L = kNegInf; s_row_bits = 0; s_n = 0; }
+    for (int kp = tid; kp < a.n_par; kp += THREADS) {
+        const float sg = a.sum_in ? a.sum_in[state_off + kp] : 0.0f;
+        const float gm = a.gamma_in ? a.gamma_in[state_off + kp] : 0.0f;
+        // a parent slot that the level above left empty (its sum or truncated Gumbel is -inf) has no children
+        const bool delivers = a.fin_token[fin_off + (int64_t)kp * a.W] >= 0 && sg > kNegInf && gm > kNegInf;
+        s_gam[kp] = delivers ? gm : kNegInf;
+        s_z[kp] = 0;
+    }
+    __syncthreads();
+    for (int kp = tid; kp < a.n_par; kp += THREADS) {
+        if (const int bits = a.row_status[row_off + kp]) atomicOr(&s_row_bits, bits);
+        const float g = s_gam[kp];
+        int rank = 0;
+        for (int j = 0; j < a.n_par; ++j) {
+            const float o = s_gam[j];
+            rank += (o > g || (o == g && j < kp)) ? 1 : 0;
+        }
+        if (rank == a.W - 1 && g > kNegInf) s_L = g;
+    }
+    __syncthreads();
+    const float L = s_L;
+
+    for (int f = tid; f < F; f += THREADS) {
+        const int kpar = f / a.W;
+        int x = a.fin_token[fin_off + f];
+        if (s_gam[kpar] == kNegInf) x = -1;   // s_gam is -inf exactly for the slots that deliver nothing
+        if (x >= 0 && L > kNegInf && f != kpar * a.W) {
+            // psi_f < L  <=>  exp(-phi~_f) - exp(-Z) > exp(-L) - exp(-Gamma_k), with Z - phi~_f = the gap d between
+            // the parent's best and this finalist's fp32 perturbed values; margins cover the fp32 arithmetic
+            const float sg = a.sum_in ? a.sum_in[state_off + kpar] : 0.0f;
+            const float gm = a.gamma_in ? a.gamma_in[state_off + kpar] : 0.0f;
+            const float lse = a.is_logprob ? 0.0f : a.fin_lse[row_off + kpar];
+            const float u0 = a.fin_pert[fin_off + (int64_t)kpar * a.W];
+            const float d_lo = (u0 - a.fin_pert[fin_off + f]) - 1e-4f;
+            if (d_lo > 0.0f) {
+                const float z = sg - lse + u0;
+                const float rhs = expf(-L + 1e-3f) - expf(-gm);
+                if (rhs <= 0.0f || -z + logf(expm1f(d_lo)) > logf(rhs) + 1e-2f) x = -1;   // cannot reach the beam
+            }
+        }
+        if (x >= 0) s_list[atomicAdd(&s_n, 1)] = f;   // the order of the list does not matter below
+    }
+    __syncthreads();
+    const int n = s_n;
+
+    // phi and phi~ of the listed finalists, with the noise recomputed in double; Z = the parent's largest phi~
+    for (int i = tid; i < n; i += THREADS) {
+        const int f = s_list[i], kpar = f / a.W;
+        const int x = a.fin_token[fin_off + f];
+        const double sigma = a.sum_in ? (double)a.sum_in[state_off + kpar] : 0.0;
+        const double lse = a.is_logprob ? 0.0 : (double)a.fin_lse[row_off + kpar];
+        const uint32_t node = (uint32_t)(a.first_parent_node + kpar);
+        const double phi = sigma + ((double)a.fin_value[fin_off + f] * a.inv_temp - lse);
+        const double pert = phi - (noise ? noise[f] : sbs_log_noise(key, node, (uint32_t)x));
+        s_tok[i] = x;
+        s_phi[i] = phi;
+        s_pert[i] = pert;
+        atomicMax(&s_z[kpar], double_to_ordered(pert));
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += THREADS) {
+        const int kpar = s_list[i] / a.W;
+        const double z = ordered_to_double(s_z[kpar]);
+        const double gamma = a.gamma_in ? (double)a.gamma_in[state_off + kpar] : 0.0;
+        const double pert = s_pert[i];
+        const double d = pert - z;
+        double psi = gamma;
+        if (!(d >= 0.0)) {
+            // (two functions one after the other instead of four: the levels' latency is that of dependent double-precision code)
+            const double x = -expm1(d), t = gamma - pert;
+            psi = t < 700.0 ? gamma - log1p(exp(t) * x) : pert - log(x);
+        }
+        s_psi[i] = psi;
+    }
+    __syncthreads();
+    // Rank by (psi desc, parent asc, token asc); the finalists of a parent are neighbours in f, so f orders the
+    // parents, and within a parent the token decides.
+    for (int i = tid; i < n; i += THREADS) {
+        const double psi = s_psi[i];
+        const int f = s_list[i], x = s_tok[i], kpar = f / a.W;
+        const int own = kpar * a.W;   // first finalist of f's parent
+        int rank = 0;
+#pragma unroll 4
+        for (int e = 0; e < n; ++e) {
+            const double pe = s_psi[e];
+            const int fe = s_list[e];
+            const bool tie_first = fe < own || (fe < own + a.W && s_tok[e] < x);   // earlier parent, or same parent and smaller token
+            rank += (pe > psi || (pe == psi && tie_first)) ? 1 : 0;
+        }
+        if (rank < a.W) {
+            const int64_t o = (int64_t)b * a.out_state_stride + rank;
+            a.out_token[(int64_t)b * a.out_stride + rank] = x;
+            a.out_parent[(int64_t)b * a.out_stride + rank] = a.parent_base + kpar;
+            a.sum_out[o] = (float)s_phi[i];
+            a.gamma_out[o] = (float)psi;
+        }
+    }
+    const int cnt = n < a.W ? n : a.W;
+    if (tid >= cnt && tid < a.W) {
+        const int64_t o = (int64_t)b * a.out_state_stride + tid;
+        a.out_token[(int64_t)b * a.out_stride + tid] = -1;
+        a.out_parent[(int64_t)b * a.out_stride + tid] = -1;
+        a.sum_out[o] = kNegInf;
+        a.gamma_out[o] = kNegInf;
+    }
+    if (tid == 0) {
+        a.status[b] = (s_row_bits & 1) | (cnt < a.W ? 2 : 0);  // RSD_ST_NAN_INPUT, RSD_ST_FEWER_THAN_K
+        a.out_count[b] = cnt;
+    }
+}
+
+
+// A level in one launch: the rows of a sequence are scanned by the blocks of a cluster, which leave their picks in the first block's shared
+// memory, and that block ends the level.
+constexpr int kMaxLevelRows = 8;                         // the largest cluster that every device takes
+constexpr int kMaxLevelPicks = kMaxLevelRows * 32;
+struct LevelSmem {
+    double noise[kMaxLevelPicks];                        // sbs_log_noise of the picks
+    double scratch[(kMaxLevelPicks * 32 + kMaxLevelRows * 12 + 15) / 16 * 2];   // sbs_level_scratch_bytes()
+    int32_t token[kMaxLevelPicks];
+    float value[kMaxLevelPicks], pert[kMaxLevelPicks];
+    float lse[kMaxLevelRows];
+    int32_t row_status[kMaxLevelRows];
+};
+struct NoLevelSmem {};
+// the same place in the first block of the cluster
+template <typename P>
+__device__ __forceinline__ P* in_first_block(P* p) {
+    uint64_t r;
+    asm volatile("mapa.u64 %0, %1, 0;" : "=l"(r) : "l"(p));
+    return (P*)r;
+}
+__device__ __forceinline__ void level_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void level_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // One block per row.
 // ALIGNED: rows start on 32-byte boundaries and V is a multiple of 16 (256-bit loads); other rows are read in aligned
 // 16-byte words, shifted.
@@ -446,8 +671,9 @@ template <typename T, bool ALIGNED, int NT>
 constexpr int scan_blocks_per_sm() {
     return ALIGNED ? (NT == 128 ? (sizeof(T) == 2 ? 9 : 8) : 1024 / NT) : (NT == 128 ? (sizeof(T) == 2 ? 8 : 7) : NT == 256 ? 3 : 2);
 }
-template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
-__global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan_topk_kernel(const ScanArgs a) {
+// LEVEL: the block is one of a cluster that runs a beam search level (see LevelSmem).
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT, bool LEVEL>
+__device__ __forceinline__ void scan_row(const ScanArgs& a, const SbsEpilogueArgs* level) {
     constexpr int kScanThreads = NT, kScanWarps = NT / 32;
     constexpr int kLseWarps = SPLIT ? 4 : kScanWarps;      // warps with a share of the log-sum-exp
     constexpr int kStride = SPLIT ? 4 : kScanWarps;        // a warp's chunks are this far apart
@@ -473,6 +699,7 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     __shared__ float red_s[kScanWarps];
     __shared__ int n_cand, n_surv, nan_flag;
     __shared__ float lse_sh;
+    __shared__ typename std::conditional<LEVEL, LevelSmem, NoLevelSmem>::type level_sm;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x / a.R, r = blockIdx.x % a.R;
@@ -484,7 +711,8 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
     const int n_iter = (n_groups + kScanThreads - 1) / kScanThreads;
     const PhiloxRow pr = philox_row_setup(a, (node & 0x0FFFFFFFu) | (kTagGumbelCoarse << 28), key.seq, key.step);
 
-    if (NT > 128 && a.wait_first) grid_wait();   // (large launches start in plain stream order instead)
+    if (LEVEL) level_arrive();                   // (the first block has started when its shared memory is written to)
+    if ((NT > 128 || LEVEL) && a.wait_first) grid_wait();   // (large launches start in plain stream order instead)
     if (tid == 0) { n_cand = 0; n_surv = 0; nan_flag = 0; n_task = 0; n_fin = 0; }
     if (tid < 32) bin_max[tid] = float_to_ordered(kNegInf);
     if (tid < 4 && n_groups + tid < ((n_groups + 3) & ~3)) ub[n_groups + tid] = kNegInf;   // padding of the bounds
@@ -836,6 +1064,47 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
 
     grid_started();
 
+    if constexpr (LEVEL) {
+        // ---- rank the survivors into the first block's shared memory; that block ends the level -----------------------------
+        const int W = a.max_k;
+        __syncwarp();
+        level_wait();
+        LevelSmem* const to = in_first_block(&level_sm);
+        for (int e = tid; e < ns; e += kScanThreads) {
+            const float mv = sv_val[e];
+            const int mi = sv_idx[e];
+            int rnk = 0;
+            for (int f = 0; f < ns; ++f) rnk += better(sv_val[f], sv_idx[f], mv, mi) ? 1 : 0;
+            if (rnk >= k) continue;
+            const int at = r * W + rnk;
+            to->token[at] = mi;
+            to->value[at] = sv_raw[e];
+            to->pert[at] = mv;
+            to->noise[at] = sbs_log_noise(key, node, (uint32_t)mi);
+        }
+        if (tid >= (ns < k ? ns : k) && tid < W) {
+            to->token[r * W + tid] = -1;
+            to->value[r * W + tid] = to->pert[r * W + tid] = kNegInf;
+        }
+        if (tid == 0) {
+            to->lse[r] = lse;
+            to->row_status[r] = nan_flag ? 1 : 0;
+        }
+        __syncwarp();
+        level_arrive();
+        level_wait();
+        if (r == 0) {
+            SbsEpilogueArgs e = *level;
+            e.fin_seq_stride = e.row_seq_stride = 0;
+            e.fin_token = level_sm.token;
+            e.fin_value = level_sm.value;
+            e.fin_pert = level_sm.pert;
+            e.fin_lse = level_sm.lse;
+            e.row_status = level_sm.row_status;
+            sbs_epilogue_body<NT>(e, b, level_sm.scratch, level_sm.noise);
+        }
+        return;
+    } else {
     // ---- rank the survivors, write the picks ----------------------------------------------------------------------------
     const int total = ns < k ? ns : k;
     const int64_t o = ((int64_t)b * a.R + r) * a.max_k;
@@ -870,202 +1139,16 @@ __global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan
             if (st) atomicOr(&a.status[b], st);
         }
     }
-}
-
-// ---------------------------------------------------------------------------------------------------------
-// Stochastic Beam Search level, per-sequence epilogue.
-// For a fixed parent psi is increasing in phi~ (Theorem 3.2's argument), so the W best pairs over all parents are
-// among each parent's own W best by phi~.  The scan above leaves those n_par * W finalists in scratch; this kernel
-// recomputes their noise in double, applies the truncation T of Eq. 11 in the stable form
-//   psi = Gamma - log1p(exp(Gamma - phi~) (1 - exp(phi~ - Z))),
-// and keeps the W best by (psi desc, parent asc, token asc).
-// ---------------------------------------------------------------------------------------------------------
-struct SbsEpilogueArgs {
-    int n_par, W, is_logprob;
-    int64_t fin_seq_stride;    // elements between sequences in fin_token / fin_value / fin_pert (n_par * W for one level)
-    int64_t row_seq_stride;    // elements between sequences in fin_lse / row_status (n_par for one level)
-    int64_t state_stride;      // elements between sequences in sum_in / gamma_in (n_par for one level)
-    int64_t out_state_stride;  // elements between sequences in sum_out / gamma_out (W; 0 when they hold one sequence)
-    double inv_temp;           // 1 / temperature of the parents' rows (1: none)
-    int32_t first_parent_node;
-    uint32_t seed_lo, seed_hi, step, seq_base;
-    const int32_t* fin_token;  // [B][n_par][W]
-    const float* fin_value;    // [B][n_par][W] the row's own value at the finalist
-    const float* fin_pert;     // [B][n_par][W] value + noise in fp32 (decreasing within a parent)
-    const float* fin_lse;      // [B][n_par]
-    const int32_t* row_status; // [B][n_par] status bits of the row scans
-    const float* sum_in;       // [B][n_par] or null
-    const float* gamma_in;     // [B][n_par] or null
-    int32_t* out_token;   // [B][out_stride]
-    int32_t* out_parent;  // [B][out_stride], parent_base added
-    int64_t out_stride;
-    int32_t parent_base;
-    float* sum_out;
-    float* gamma_out;
-    int32_t* out_count;
-    int32_t* status;
-};
-
-constexpr int kEpilogueThreads = 128;
-
-// bytes of shared memory one level needs in sbs_epilogue_body, rounded up to 16
-__host__ __device__ inline size_t sbs_level_scratch_bytes(int n_par, int W) {
-    return (((size_t)n_par * W * 32 + (size_t)n_par * 12) + 15) & ~(size_t)15;
-}
-
-// order-preserving map of a double to an unsigned integer (for an atomic maximum), and back; 0 stands for "none"
-__device__ __forceinline__ unsigned long long double_to_ordered(double v) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-    return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double ordered_to_double(unsigned long long k) {
-    if (k == 0) return -__longlong_as_double(0x7FF0000000000000LL);
-    return __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
-}
-
-// -ln of the exponential form of a token's Gumbel noise, in double: G(x) = -sbs_log_noise
-__device__ __forceinline__ double sbs_log_noise(const RngKey& key, uint32_t node, uint32_t x) {
-    const uint32_t word = coarse_word(key, node, x >> 4);
-    const double t_elem = ((x & 15u) != (word & 15u)) ? neg_log_uniform_f64(fine_word(key, node, x)) : 0.0;
-    return log(neg_log_group_uniform_f64(word) * 0.0625 + t_elem);
-}
-
-// One level for sequence b, by a block of kEpilogueThreads threads; sm_d: sbs_level_scratch_bytes(n_par, W) bytes.
-// noise: sbs_log_noise of the level's finalists, [n_par][W], or null (then it is taken here).
-__device__ __forceinline__ void sbs_epilogue_body(const SbsEpilogueArgs& a, const int b, double* sm_d, const double* noise = nullptr) {
-    const int F = a.n_par * a.W;
-    // the finalists that pass the first test are gathered in a list; entry i of the arrays below belongs to list[i]
-    double* s_pert = sm_d;                   // [F] phi~
-    double* s_phi = sm_d + F;                // [F] phi
-    double* s_psi = sm_d + 2 * F;            // [F] psi
-    unsigned long long* s_z = (unsigned long long*)(sm_d + 3 * F);   // [n_par] largest phi~ of the parent, ordered
-    int* s_list = (int*)(s_z + a.n_par);     // [F] finalist index f = parent * W + place
-    int* s_tok = s_list + F;                 // [F] its token
-    float* s_gam = (float*)(s_tok + F);      // [n_par]
-    const int tid = threadIdx.x;
-    const int64_t fin_off = (int64_t)b * a.fin_seq_stride, row_off = (int64_t)b * a.row_seq_stride,
-                  state_off = (int64_t)b * a.state_stride;
-    const RngKey key = {a.seed_lo, a.seed_hi, a.step, a.seq_base + (uint32_t)b};
-
-    // A child enters the beam only if its psi reaches the W-th best psi of the level.  The best child of parent j has
-    // psi = Gamma_j exactly, so that bound is at least L = the W-th largest Gamma among the parents that deliver a
-    // child (valid parent, at least one finalist); L = -inf when fewer than W do.  Finalists that a cheap fp32 test
-    // shows to lie clearly below L are dropped before the double-precision work; a parent's best finalist is
-    // always kept.
-    __shared__ float s_L;
-    __shared__ int s_row_bits, s_n;
-    if (tid == 0) { s_L = kNegInf; s_row_bits = 0; s_n = 0; }
-    for (int kp = tid; kp < a.n_par; kp += kEpilogueThreads) {
-        const float sg = a.sum_in ? a.sum_in[state_off + kp] : 0.0f;
-        const float gm = a.gamma_in ? a.gamma_in[state_off + kp] : 0.0f;
-        // a parent slot that the level above left empty (its sum or truncated Gumbel is -inf) has no children
-        const bool delivers = a.fin_token[fin_off + (int64_t)kp * a.W] >= 0 && sg > kNegInf && gm > kNegInf;
-        s_gam[kp] = delivers ? gm : kNegInf;
-        s_z[kp] = 0;
-    }
-    __syncthreads();
-    for (int kp = tid; kp < a.n_par; kp += kEpilogueThreads) {
-        if (const int bits = a.row_status[row_off + kp]) atomicOr(&s_row_bits, bits);
-        const float g = s_gam[kp];
-        int rank = 0;
-        for (int j = 0; j < a.n_par; ++j) {
-            const float o = s_gam[j];
-            rank += (o > g || (o == g && j < kp)) ? 1 : 0;
-        }
-        if (rank == a.W - 1 && g > kNegInf) s_L = g;
-    }
-    __syncthreads();
-    const float L = s_L;
-
-    for (int f = tid; f < F; f += kEpilogueThreads) {
-        const int kpar = f / a.W;
-        int x = a.fin_token[fin_off + f];
-        if (s_gam[kpar] == kNegInf) x = -1;   // s_gam is -inf exactly for the slots that deliver nothing
-        if (x >= 0 && L > kNegInf && f != kpar * a.W) {
-            // psi_f < L  <=>  exp(-phi~_f) - exp(-Z) > exp(-L) - exp(-Gamma_k), with Z - phi~_f = the gap d between
-            // the parent's best and this finalist's fp32 perturbed values; margins cover the fp32 arithmetic
-            const float sg = a.sum_in ? a.sum_in[state_off + kpar] : 0.0f;
-            const float gm = a.gamma_in ? a.gamma_in[state_off + kpar] : 0.0f;
-            const float lse = a.is_logprob ? 0.0f : a.fin_lse[row_off + kpar];
-            const float u0 = a.fin_pert[fin_off + (int64_t)kpar * a.W];
-            const float d_lo = (u0 - a.fin_pert[fin_off + f]) - 1e-4f;
-            if (d_lo > 0.0f) {
-                const float z = sg - lse + u0;
-                const float rhs = expf(-L + 1e-3f) - expf(-gm);
-                if (rhs <= 0.0f || -z + logf(expm1f(d_lo)) > logf(rhs) + 1e-2f) x = -1;   // cannot reach the beam
-            }
-        }
-        if (x >= 0) s_list[atomicAdd(&s_n, 1)] = f;   // the order of the list does not matter below
-    }
-    __syncthreads();
-    const int n = s_n;
-
-    // phi and phi~ of the listed finalists, with the noise recomputed in double; Z = the parent's largest phi~
-    for (int i = tid; i < n; i += kEpilogueThreads) {
-        const int f = s_list[i], kpar = f / a.W;
-        const int x = a.fin_token[fin_off + f];
-        const double sigma = a.sum_in ? (double)a.sum_in[state_off + kpar] : 0.0;
-        const double lse = a.is_logprob ? 0.0 : (double)a.fin_lse[row_off + kpar];
-        const uint32_t node = (uint32_t)(a.first_parent_node + kpar);
-        const double phi = sigma + ((double)a.fin_value[fin_off + f] * a.inv_temp - lse);
-        const double pert = phi - (noise ? noise[f] : sbs_log_noise(key, node, (uint32_t)x));
-        s_tok[i] = x;
-        s_phi[i] = phi;
-        s_pert[i] = pert;
-        atomicMax(&s_z[kpar], double_to_ordered(pert));
-    }
-    __syncthreads();
-    for (int i = tid; i < n; i += kEpilogueThreads) {
-        const int kpar = s_list[i] / a.W;
-        const double z = ordered_to_double(s_z[kpar]);
-        const double gamma = a.gamma_in ? (double)a.gamma_in[state_off + kpar] : 0.0;
-        const double pert = s_pert[i];
-        const double d = pert - z;
-        double psi = gamma;
-        if (!(d >= 0.0)) {
-            // (two functions one after the other instead of four: the levels' latency is that of dependent double-precision code)
-            const double x = -expm1(d), t = gamma - pert;
-            psi = t < 700.0 ? gamma - log1p(exp(t) * x) : pert - log(x);
-        }
-        s_psi[i] = psi;
-    }
-    __syncthreads();
-    // Rank by (psi desc, parent asc, token asc); the finalists of a parent are neighbours in f, so f orders the
-    // parents, and within a parent the token decides.
-    for (int i = tid; i < n; i += kEpilogueThreads) {
-        const double psi = s_psi[i];
-        const int f = s_list[i], x = s_tok[i], kpar = f / a.W;
-        const int own = kpar * a.W;   // first finalist of f's parent
-        int rank = 0;
-#pragma unroll 4
-        for (int e = 0; e < n; ++e) {
-            const double pe = s_psi[e];
-            const int fe = s_list[e];
-            const bool tie_first = fe < own || (fe < own + a.W && s_tok[e] < x);   // earlier parent, or same parent and smaller token
-            rank += (pe > psi || (pe == psi && tie_first)) ? 1 : 0;
-        }
-        if (rank < a.W) {
-            const int64_t o = (int64_t)b * a.out_state_stride + rank;
-            a.out_token[(int64_t)b * a.out_stride + rank] = x;
-            a.out_parent[(int64_t)b * a.out_stride + rank] = a.parent_base + kpar;
-            a.sum_out[o] = (float)s_phi[i];
-            a.gamma_out[o] = (float)psi;
-        }
-    }
-    const int cnt = n < a.W ? n : a.W;
-    if (tid >= cnt && tid < a.W) {
-        const int64_t o = (int64_t)b * a.out_state_stride + tid;
-        a.out_token[(int64_t)b * a.out_stride + tid] = -1;
-        a.out_parent[(int64_t)b * a.out_stride + tid] = -1;
-        a.sum_out[o] = kNegInf;
-        a.gamma_out[o] = kNegInf;
-    }
-    if (tid == 0) {
-        a.status[b] = (s_row_bits & 1) | (cnt < a.W ? 2 : 0);  // RSD_ST_NAN_INPUT, RSD_ST_FEWER_THAN_K
-        a.out_count[b] = cnt;
     }
 }
-
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
+__global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>()) scan_topk_kernel(const ScanArgs a) {
+    scan_row<T, ALIGNED, NEED_LSE, TEMP, NT, SPLIT, false>(a, nullptr);
+}
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
+__global__ void __launch_bounds__(NT, scan_blocks_per_sm<T, ALIGNED, NT>() < 4 ? scan_blocks_per_sm<T, ALIGNED, NT>() : 4) scan_level_kernel(const __grid_constant__ ScanArgs a, const __grid_constant__ SbsEpilogueArgs level) {
+    scan_row<T, ALIGNED, NEED_LSE, TEMP, NT, SPLIT, true>(a, &level);
+}
 
 static __global__ void __launch_bounds__(kEpilogueThreads) sbs_epilogue_kernel(const SbsEpilogueArgs a) {
     extern __shared__ double sm_d[];

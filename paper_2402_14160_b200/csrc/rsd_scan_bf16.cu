@@ -4,4 +4,7 @@ namespace rsd {
 void launch_scan_bf16(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, cudaStream_t s) {
     launch_scan_of<__nv_bfloat16>(threads, aligned, need_lse, blocks, a, s);
 }
+void launch_level_bf16(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, const SbsEpilogueArgs& e, cudaStream_t s) {
+    launch_level_of<__nv_bfloat16>(threads, aligned, need_lse, blocks, a, e, s);
+}
 }  // namespace rsd

@@ -57,4 +57,33 @@ void launch_scan_of(int threads, bool aligned, bool need_lse, int blocks, const 
     }
 }
 
+// A beam search level: rows few enough for one of the kernels of few rows.
+template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP, int NT, bool SPLIT>
+void launch_level_threads(int blocks, const ScanArgs& a, const SbsEpilogueArgs& e, cudaStream_t s) {
+    constexpr size_t kBuffer = NT == 128 ? 0 : scan_buffer_bytes<T, NT>();
+    constexpr auto kernel = scan_level_kernel<T, ALIGNED, NEED_LSE, TEMP, NT, SPLIT>;
+    if (!rsd_host::raise_shared_memory<kernel>((int)(scan_bounds_bytes(RSD_MAX_VOCAB) + kBuffer))) return;
+    rsd_host::launch_overlapped(kernel, (unsigned)blocks, NT, scan_bounds_bytes(a.V) + kBuffer, s, a.R, a, e);
+}
+template <typename T, bool ALIGNED>
+void launch_level_aligned(int threads, bool need_lse, int blocks, const ScanArgs& a, const SbsEpilogueArgs& e, cudaStream_t s) {
+    if (!need_lse) {                                     // (log-probabilities as they are: no temperature)
+        if (threads == 512) launch_level_threads<T, ALIGNED, false, false, 512, false>(blocks, a, e, s);
+        else launch_level_threads<T, ALIGNED, false, false, 256, false>(blocks, a, e, s);
+    } else if (a.temp != 1.0f) {
+        if (threads == 256 && a.V > kScanSplitVocab) launch_level_threads<T, ALIGNED, true, true, 256, false>(blocks, a, e, s);
+        else if (threads == 256) launch_level_threads<T, ALIGNED, true, true, 256, true>(blocks, a, e, s);
+        else launch_level_threads<T, ALIGNED, true, true, 128, false>(blocks, a, e, s);
+    } else {
+        if (threads == 256 && a.V > kScanSplitVocab) launch_level_threads<T, ALIGNED, true, false, 256, false>(blocks, a, e, s);
+        else if (threads == 256) launch_level_threads<T, ALIGNED, true, false, 256, true>(blocks, a, e, s);
+        else launch_level_threads<T, ALIGNED, true, false, 128, false>(blocks, a, e, s);
+    }
+}
+template <typename T>
+void launch_level_of(int threads, bool aligned, bool need_lse, int blocks, const ScanArgs& a, const SbsEpilogueArgs& e, cudaStream_t s) {
+    if (aligned) launch_level_aligned<T, true>(threads, need_lse, blocks, a, e, s);
+    else launch_level_aligned<T, false>(threads, need_lse, blocks, a, e, s);
+}
+
 }  // namespace rsd

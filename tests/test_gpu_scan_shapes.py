@@ -84,3 +84,37 @@ def test_rows_without_log_sum_exp_alone_and_in_a_batch_give_the_same_bits(dtype,
     t = Tally()
     compare_topk(t, whole["token"][:n], o, [8], *([whole["perturbed"][:n], whole["logprob"][:n]] if form == "logprob" else []))
     t.check()
+
+
+# A level of few rows runs in one launch (the rows of a sequence as a cluster, 128 to 512 threads a row), one of many rows in two.
+@pytest.mark.parametrize("dtype,V,n_par,W,B,off,form,trouble", [
+    ("bf16", 70, 8, 8, 200, 0, "", "few"), ("f32", 4096, 3, 5, 200, 0, "", "nan"), ("bf16", 16383, 8, 32, 60, 1, "tempered", ""), ("f32", 16384, 2, 2, 300, 0, "", "dead"),
+    ("bf16", 32000, 4, 4, 140, 0, "", "nan"), ("f32", 32000, 6, 6, 80, 0, "logprob", "dead"), ("f32", 1001, 7, 3, 90, 1, "logprob", "few"),
+    ("bf16", 65552, 8, 8, 64, 0, "", "dead"), ("f32", 70001, 5, 8, 90, 3, "tempered", "nan"), ("bf16", 131072, 1, 8, 400, 0, "", "")])
+def test_levels_alone_and_in_a_batch_give_the_same_bits(dtype, V, n_par, W, B, off, form, trouble):
+    import paper_2402_14160_b200 as rsd
+    gen = torch.Generator(device="cuda").manual_seed(V + B)
+    rows = torch.randn((B, n_par, V + off), generator=gen, device="cuda") * 2
+    if form == "logprob":
+        rows = torch.log_softmax(rows, -1)
+    if trouble == "nan":
+        rows[::4, n_par - 1, V - 1 + off] = float("nan")
+    elif trouble == "few":       # fewer entries than children
+        rows[::2, :, off + 2:] = float("-inf")
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32)[:, :, off:]
+    total = -torch.rand((B, n_par), generator=gen, device="cuda")
+    gumbel = torch.randn((B, n_par), generator=gen, device="cuda")
+    if trouble == "dead":        # parent slots that the level above left empty
+        total[::3, n_par - 1] = gumbel[::3, n_par - 1] = float("-inf")
+    T = 0.4 if form == "tempered" else 1.0
+
+    def level(b, n):
+        sums = (None, None) if n_par == 1 else (total[b:b + n].contiguous(), gumbel[b:b + n].contiguous())
+        return rsd.rsd_sbs_step(rows[b:b + n], W, 3, *sums, 17, 3, is_logprob=form == "logprob", seq_base=5 + b, temperature=T)
+
+    whole = level(0, B)
+    for b, n in ((0, 1), (B // 2, 3), (B - 2, 2)):
+        part = level(b, n)
+        for key in part:
+            got, want = part[key].cpu().numpy(), whole[key][b:b + n].cpu().numpy()
+            assert np.array_equal(got, want, equal_nan=got.dtype.kind == "f"), (key, b)
