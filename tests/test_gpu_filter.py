@@ -220,3 +220,24 @@ def test_filter_rows_that_the_sample_of_the_first_sweep_misjudges(rsd, dtype, V)
     rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32).cuda()
     for top_k, top_p, T in ((0, 0.95, 1.0), (0, 0.3, 0.5), (min(3000, V), 0.9, 1.0), (7, 1.0, 1.0)):
         _check_filter(rsd, rows, top_k, top_p, T, max_borderline=2)
+
+
+@pytest.mark.parametrize("dtype,V,top_k", [("bf16", 16384, 256), ("bf16", 16384, 257), ("bf16", 16383, 256), ("f32", 8192, 256), ("f32", 8195, 100), ("f32", 8195, 1),
+                                           ("bf16", 65601, 512), ("bf16", 32000, 129), ("f32", 33001, 50), ("f32", 50000, 513)])
+def test_top_k_bounded_by_the_threads_largest_values(rsd, dtype, V, top_k):
+    # up to half as many tokens as threads (512, or 1024 where a row fills an SM) from rows of four words a thread on; lists of up to 128 tokens
+    # are ended in registers
+    g = torch.Generator(device="cpu").manual_seed(V + top_k)
+    rows = torch.randn((1, 7, V), generator=g) * 2
+    rows[0, 1] = (rows[0, 1] * 4).round() / 4                     # ties at every cut
+    rows[0, 2, : V // 2 : 4096] = 40.0                            # the largest in words of one thread
+    rows[0, 2, 3 : V // 2 : 4096] = 41.0
+    rows[0, 3] = float("-inf")                                    # hardly more entries than asked for, in runs
+    rows[0, 3, 1000 : 1000 + top_k + 3] = torch.randn((top_k + 3,), generator=g)
+    rows[0, 4, ::7] = float("nan")
+    rows[0, 5] = torch.arange(V).float() / V                      # the largest at the end
+    rows[0, 6] = torch.where(torch.rand(V, generator=g) < 0.5, 0.0, -0.0)
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32).cuda()
+    # (equal weights put cumulative masses on round fractions: such rows may be borderline)
+    for top_p in (1.0, 0.9, 0.37):
+        _check_filter(rsd, rows, top_k, top_p, 1.0, max_borderline=0 if top_p == 1.0 else 3)
