@@ -181,32 +181,19 @@ struct RowVec<__nv_bfloat16> {
         }
         return (acc | (acc >> 16)) & 0xFFu;
     }
-    // the word with -inf at the entries below `cut`; any_eq != 0 when an entry equals `cut`
-    __device__ static __forceinline__ uint4 at_least(const uint4& w, float cut, uint32_t& any_eq) {
+    // the word with -inf at the entries below `cut`; `kept`: the number of the others
+    __device__ static __forceinline__ uint4 at_least(const uint4& w, float cut, int& kept) {
         const uint32_t q[4] = {w.x, w.y, w.z, w.w}, c2 = twice(cut);
-        uint32_t o[4];
-        any_eq = 0;
+        uint32_t o[4], acc = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            uint32_t ge, eq;
+            uint32_t ge;
             asm("set.ge.u32.bf16x2 %0, %1, %2;" : "=r"(ge) : "r"(q[j]), "r"(c2));
-            asm("set.eq.u32.bf16x2 %0, %1, %2;" : "=r"(eq) : "r"(q[j]), "r"(c2));
             o[j] = (q[j] & ge) | (0xFF80FF80u & ~ge);
-            any_eq |= eq;
+            acc |= ge & ((1u << (2 * j)) | (1u << (2 * j + 17)));
         }
+        kept = __popc(acc);
         return make_uint4(o[0], o[1], o[2], o[3]);
-    }
-    // entries of a cleaned word that are not -inf
-    __device__ static __forceinline__ int finite_entries(const uint4& w) {
-        const uint32_t q[4] = {w.x, w.y, w.z, w.w};
-        uint32_t acc = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            uint32_t gt;
-            asm("set.gt.u32.bf16x2 %0, %1, %2;" : "=r"(gt) : "r"(q[j]), "r"(0xFF80FF80u));
-            acc |= gt & ((1u << (2 * j)) | (1u << (2 * j + 17)));
-        }
-        return __popc(acc);
     }
 };
 template <>
@@ -218,20 +205,17 @@ struct RowVec<float> {
         for (int j = 0; j < 4; ++j) acc |= (v[j] >= first && v[j] <= last) ? 1u << j : 0u;
         return acc;
     }
-    __device__ static __forceinline__ uint4 at_least(const uint4& w, float cut, uint32_t& any_eq) {
+    __device__ static __forceinline__ uint4 at_least(const uint4& w, float cut, int& kept) {
         const uint32_t q[4] = {w.x, w.y, w.z, w.w};
         uint32_t o[4];
-        any_eq = 0;
+        kept = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float v = __uint_as_float(q[j]);
-            o[j] = v >= cut ? q[j] : 0xFF800000u;
-            any_eq |= v == cut ? 1u : 0u;
+            const bool ge = __uint_as_float(q[j]) >= cut;
+            o[j] = ge ? q[j] : 0xFF800000u;
+            kept += ge ? 1 : 0;
         }
         return make_uint4(o[0], o[1], o[2], o[3]);
-    }
-    __device__ static __forceinline__ int finite_entries(const uint4& w) {
-        return (w.x != 0xFF800000u) + (w.y != 0xFF800000u) + (w.z != 0xFF800000u) + (w.w != 0xFF800000u);
     }
 };
 
@@ -908,21 +892,27 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
             return c > RowCodes<T>::kNegInfCode && within(cut, c, i);
         };
         const bool dst16 = ((uintptr_t)dst & 15u) == 0;
-        const float cut_value = RowCodes<T>::value_of_code(cut.code);
+        // Entries that equal the cut's value stay up to the cut's token: words ahead of its word keep what is at least the value, words
+        // behind it what is at least the next larger one (as values +0 and -0 are one here, as they are one code).  In its word the tokens decide.
+        const float cut_value = RowCodes<T>::value_of_code(cut.code), next_value = RowCodes<T>::value_of_code(cut.code + 1u);
+        const int cut_word = cut.tok / kPerVec;
         int n_kept = 0;
         for (int m = tid; m < n_vec; m += NT) {
             const uint4 w = ((const uint4*)row_sm)[m];
-            uint32_t any_eq;
-            uint4 o = RowVec<T>::at_least(w, cut_value, any_eq);   // right wherever no entry equals the cut's value
-            if (any_eq) {                                          // there the codes and the tokens decide
+            int n_here;
+            uint4 o = RowVec<T>::at_least(w, m <= cut_word ? cut_value : next_value, n_here);
+            if (m == cut_word) {
                 uint32_t h[kPerVec];
                 RowCodes<T>::unpack_bits(w, h);
+                n_here = 0;
 #pragma unroll
-                for (int j = 0; j < kPerVec; ++j)
-                    if (!keeps(m * kPerVec + j, h[j])) h[j] = RowCodes<T>::kNegInfBits;
+                for (int j = 0; j < kPerVec; ++j) {
+                    if (keeps(m * kPerVec + j, h[j])) ++n_here;
+                    else h[j] = RowCodes<T>::kNegInfBits;
+                }
                 o = RowCodes<T>::pack_bits(h);
             }
-            if (count_kept) n_kept += RowVec<T>::finite_entries(o);
+            n_kept += n_here;
             if (dst16) {
                 ((uint4*)dst)[m] = o;
             } else {
