@@ -226,7 +226,7 @@ int rsd_filter_rows(const rsd_rows* rows, int B, int R, int V, int top_k, float 
                     (kSharedPerBlock - sizeof(rsd::FilterSmem) - 272) / elem);
     if (B == 0) return RSD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    clear_status(status, B, s);
+    if (R > 1) clear_status(status, B, s);   // (where a row is all there is, its block stores the status: 1 us of a call over 32 rows)
     rsd::FilterArgs a;
     a.data = rows->data; a.out = out_rows; a.seq_stride = rows->seq_stride; a.row_stride = rows->row_stride;
     a.R = R; a.V = V; a.top_k = top_k; a.top_p = top_p;

@@ -43,7 +43,7 @@ struct FilterArgs {
     float top_p;                                 // >= 1: none
     float log2e_over_t;                          // log2(e) / temperature
     int32_t* kept;                               // [B][R] or null
-    int32_t* status;                             // [B], OR-ed into
+    int32_t* status;                             // [B], OR-ed into, or (one row a sequence) written
 };
 
 struct FilterSmem {
@@ -710,6 +710,16 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     const int n_vec = V / kPerVec;                               // whole 16-byte words of the row
     const int n_all = (V + kPerVec - 1) / kPerVec;               // with the padded word
 
+    const bool only_row = a.R == 1;                              // (its status is stored; no kernel ahead clears it)
+    if (only_row) grid_wait();
+    auto report = [&](int bits) {
+        if (only_row) {
+            a.status[b] = bits;
+        } else {
+            grid_wait();                                         // (status[] has been cleared)
+            if (bits) atomicOr(&a.status[b], bits);
+        }
+    };
     // ---- the row into shared memory, NaN as -inf; its largest value and the number of finite entries ------------------
     // Rows that start on a 16-byte boundary come in by one bulk copy of the whole words, the others by plain loads.  A
     // first look takes the largest value and notes whether anything is NaN or -inf; only then is the row gone over
@@ -790,10 +800,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     }
     __syncthreads();
     if (sm.copy_gave_up) {                                        // the copy never landed: report, write nothing
-        if (tid == 0) {
-            grid_wait();                                          // (status[] has been cleared)
-            atomicOr(&a.status[b], 32);                           // RSD_ST_TIMEOUT
-        }
+        if (tid == 0) report(32);                                 // RSD_ST_TIMEOUT
         return;
     }
     if (sm.needs_cleaning) {
@@ -942,8 +949,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     }
     if (tid == 0) {
         if (a.kept) a.kept[(int64_t)b * a.R + r] = kept;
-        grid_wait();                                              // (status[] has been cleared)
-        if (sm.nan_flag) atomicOr(&a.status[b], 1);               // RSD_ST_NAN_INPUT
+        report(sm.nan_flag ? 1 : 0);                              // RSD_ST_NAN_INPUT
     }
 }
 

@@ -30,3 +30,15 @@ def test_status_words_hold_the_bits_of_their_own_call(call, B):
         got.append(out["status"].clone())
     for g, w in zip(got, (want, want * 0, want, want * 0)):
         assert torch.equal(g, w)
+
+
+@pytest.mark.parametrize("B", [1, 3, 300])
+def test_status_of_sequences_of_one_row_is_stored(B):
+    # no kernel ahead clears it: every sequence's word is written, whatever it held
+    import paper_2402_14160_b200 as rsd
+    rows = torch.randn((B, 1, 9000), device="cuda")
+    rows[::2, 0, 5] = float("nan")
+    out = rsd.rsd_filter_rows(rows, 0, 0.9)
+    out["status"].fill_(77)
+    rsd.rsd_filter_rows(rows, 0, 0.9, out=out)
+    assert out["status"].cpu().tolist() == [rsd.ST_NAN_INPUT if b % 2 == 0 else 0 for b in range(B)]
