@@ -124,7 +124,6 @@ int rsd_gumbel_topk_draft(const rsd_rows* draft, int B, int R, int V, const int3
     }
     if (B == 0) return RSD_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    clear_status(status, B, s);
     a.data = draft->data; a.seq_stride = draft->seq_stride; a.row_stride = draft->row_stride;
     a.R = R; a.V = V; a.max_k = max_k;
     a.seed_lo = (uint32_t)seed; a.seed_hi = (uint32_t)(seed >> 32); a.step = step; a.seq_base = seq_base;
@@ -133,6 +132,10 @@ int rsd_gumbel_topk_draft(const rsd_rows* draft, int B, int R, int V, const int3
     a.status = status; a.node_token = node_token; a.node_stride = node_stride;
     a.temp = temperature_of(draft); a.inv_temp = 1.0f / a.temp;
     const bool need_lse = !rows_are_logprob(draft) && (out_perturbed || out_logprob);
+    // (a cluster per sequence gathers its rows' status; otherwise they are OR-ed into cleared words)
+    a.cluster_status = level_in_one_launch(B, R, V) && scan_threads(B * R, V, draft->dtype == RSD_F32, need_lse) > 128;
+    if (a.cluster_status) a.wait_first = 1;
+    else clear_status(status, B, s);
     launch_scan(draft, need_lse, B * R, a, s);
     return check_launch("rsd_gumbel_topk_draft");
 }

@@ -57,6 +57,7 @@ struct ScanArgs {
     int wait_first;       // 1: the stream's previous kernel may still run (it may have written the rows); 0: it is the one that
                           // clears status[], which is not touched before the end
                           // (last: with the round keys four bytes further on the large launches lose 1.5 %)
+    int cluster_status;   // 1: the sequence's rows are a cluster (kernels of more than 128 threads): its first block stores status[b]
 };
 
 // One block of `threads` threads per row, `blocks` rows (defined in rsd_scan_f32.cu and rsd_scan_bf16.cu).
@@ -805,7 +806,13 @@ __device__ __forceinline__ void scan_row(const ScanArgs& a, const SbsEpilogueArg
         if (tid < 2) level_sm.counters[tid] = 0;
         __syncwarp();
     }
-    if (LEVEL) level_arrive();                   // (the first block has started when its shared memory is written to)
+    __shared__ int seq_status;                   // first block of a cluster: the sequence's status
+    const bool gather_status = !LEVEL && NT > 128 && a.cluster_status;
+    if (gather_status) {
+        if (tid == 0) seq_status = 0;
+        __syncwarp();
+    }
+    if (LEVEL || gather_status) level_arrive();  // (the first block has started when its shared memory is written to)
     if ((NT > 128 || LEVEL) && a.wait_first) grid_wait();   // (large launches start in plain stream order instead)
     if (tid == 0) { n_cand = 0; n_surv = 0; nan_flag = 0; n_task = 0; n_fin = 0; }
     if (tid < 32) bin_max[tid] = float_to_ordered(kNegInf);
@@ -1222,6 +1229,7 @@ __device__ __forceinline__ void scan_row(const ScanArgs& a, const SbsEpilogueArg
         if (a.out_perturbed) a.out_perturbed[o + tid] = kNegInf;
         if (a.out_value) a.out_value[o + tid] = kNegInf;
     }
+    if (gather_status) { __syncwarp(); level_wait(); }
     if (tid == 0) {
         if (a.out_lse) a.out_lse[(int64_t)b * a.R + r] = NEED_LSE ? lse : 0.0f;
         int st = 0;
@@ -1229,10 +1237,18 @@ __device__ __forceinline__ void scan_row(const ScanArgs& a, const SbsEpilogueArg
         if (total < k) st |= 2;      // RSD_ST_FEWER_THAN_K
         if (a.row_status) {
             a.row_status[(int64_t)b * a.R + r] = st & 1;
+        } else if (gather_status) {
+            if (st) atomicOr(in_first_block(&seq_status), st);
         } else {
             grid_wait();   // (status[] has been cleared)
             if (st) atomicOr(&a.status[b], st);
         }
+    }
+    if (gather_status) {
+        __syncwarp();
+        level_arrive();
+        level_wait();
+        if (r == 0 && tid == 0) a.status[b] = seq_status;
     }
     }
 }

@@ -27,7 +27,7 @@ void launch_scan_threads(int blocks, const ScanArgs& a, cudaStream_t s) {
         }
     }
     if (NT == 128 && a.wait_first) kernel<<<blocks, NT, smem, s>>>(a);
-    else rsd_host::launch_overlapped(kernel, (unsigned)blocks, NT, smem, s, 0, a);
+    else rsd_host::launch_overlapped(kernel, (unsigned)blocks, NT, smem, s, a.cluster_status ? a.R : 0, a);
 }
 template <typename T, bool ALIGNED, bool NEED_LSE, bool TEMP>
 void launch_scan_temp(int threads, int blocks, const ScanArgs& a, cudaStream_t s) {

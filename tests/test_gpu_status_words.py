@@ -42,3 +42,23 @@ def test_status_of_sequences_of_one_row_is_stored(B):
     out["status"].fill_(77)
     rsd.rsd_filter_rows(rows, 0, 0.9, out=out)
     assert out["status"].cpu().tolist() == [rsd.ST_NAN_INPUT if b % 2 == 0 else 0 for b in range(B)]
+
+
+@pytest.mark.parametrize("B,R,V", [(1, 1, 20000), (1, 7, 32000), (3, 8, 5000), (3, 9, 5000), (46, 8, 17000), (47, 8, 17000), (2, 8, 70000)])
+def test_status_of_few_rows_gathered_by_their_cluster(B, R, V):
+    # up to eight rows a sequence, few in all: a cluster's first block stores the OR of their bits; the other sizes clear and OR
+    import paper_2402_14160_b200 as rsd
+    rows = torch.randn((B, R, V), device="cuda")
+    want = [0] * B
+    rows[0, R - 1, V - 1] = float("nan")
+    want[0] |= NAN_INPUT
+    if B > 1:
+        rows[B - 1, 0, 2:] = float("-inf")               # fewer entries than picks
+        want[B - 1] |= rsd.ST_FEWER_THAN_K
+        rows[B - 1, R - 1, 7] = float("nan")
+        want[B - 1] |= NAN_INPUT
+    for values in (False, True):
+        out = rsd.rsd_gumbel_topk_draft(rows, [3] * R, list(range(R)), 1, 0, want_values=values)
+        out["status"].fill_(77)
+        rsd.rsd_gumbel_topk_draft(rows, [3] * R, list(range(R)), 1, 0, want_values=values, out=out)
+        assert out["status"].cpu().tolist() == want
