@@ -23,6 +23,8 @@
 // without returned atomics and with packed arithmetic, and before the search behind it was left to one warp: 1344 rows
 // 146 -> 104 us.  Three blocks per SM for rows of up to 64,000 bytes, and 1024 threads for rows of which only one fits on an
 // SM (32 rows of 32,000 fp32 with both cuts 47 -> 23 us).
+// Since then, with lists in registers, a thread's words tested before its tokens, top-k from the threads' largest values and an output that compares once a word:
+// 1500 rows of 32,000 bf16, top-p 0.95, 106 -> 90 us, the 32 rows 23 -> 14.
 #pragma once
 #include "rsd_device.cuh"
 #include "rsd_scan.cuh"   // ex2_approx, packed arithmetic
