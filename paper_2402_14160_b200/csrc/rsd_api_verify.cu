@@ -2,6 +2,7 @@
 // rsd_resample_residual.  Argument checks and kernel launches, nothing else.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 
 #include "rsd_api_common.h"
@@ -65,67 +66,33 @@ rsd::walk_cluster::Shape cluster_shape(int B, int V) {
     return best;
 }
 
-// Up to how many waves of clusters (sequences asked for over sequences resident) the on-chip walk is taken; beyond, the ring walk or the one that
-// reads its rows anew in every pass.  Measured at 11,000 calls (70 to 131,072 entries, 1 to 900 sequences, trees of 10 and 29 nodes); figures in us,
-// on chip / other.  What the clusters need grows with the number of waves (1, 1.7, 2.4, 3.2 times one wave's time), the others' with the row.
+// Whether the on-chip walk is taken, or else the ring walk or the one that reads its rows anew in every pass.
+// Where fewer than four tiles per warp hold all sequences at a time it always is: in 7,500 such calls the other route took 1.02 to 15 times
+// as long.  Rows of up to 8192 entries (a cluster of one or two blocks with one tile per warp) stay on chip, but where the ring takes them it is ahead
+// from 1.3 waves on (8192 bf16, 260 / 300 sequences: 24 / 19 us on chip / ring, 24 / 21), and residual draws over 2-byte rows with two blocks a
+// sequence meet a wave's end (8192, 200 / 300: 12.6 / 19 on chip / read anew, 22 / 22).
+// With four tiles per warp two costs are compared.  A launch on chip takes as long as it has waves of clusters, each about the same whatever the row
+// (sequences asked for over sequences resident); the other route as long as it has rounds of blocks (three or, for 4-byte rows read anew, two
+// per SM), each in proportion to a constant and the row.  Sequences end at different times, so that half of a wave counts by its
+// share and half as a whole one.  A round's cost in waves is a + b V / 10,000; a residual draw's pass over its rejected tokens raises it with the fourth root
+// of their number.  Fitted to 12,100 calls with both routes timed (8,193 to 131,072 entries, 8 to 900 sequences, trees of 4 to 29 nodes, 1 to 32
+// rejected tokens): the route taken is 0.7 % slower than the faster one in geometric mean (the limits per cluster size before: 2.7 %), and 54
+// calls are more than a tenth slower than in the walks without a four-tile shape (222 before).
 enum WalkKind { kRingRows, kReadAnew, kReadAnewTop1, kDraw, kDrawWhole };
-float most_waves(const rsd::walk_cluster::Shape& c, int B, int V, bool f32, WalkKind kind) {
-    constexpr float kAlways = 1e30f;
-    const float v = (float)V;
-    if (kind == kRingRows) {
-        // One tile per warp, rows of up to 8192 entries: 8192 bf16, 260 / 300 sequences: 24 / 19, 24 / 21.  Two: all resident or not at all.
-        if (c.NT == 1) return 1.3f;
-        if (c.NT == 2) return 1.0f;
-        // One block: 16,000 entries, 256 / 330: bf16 25 / 30, 44 / 36; fp32 from 149 on: 20.4 / 20.4, 26 / 26; 9000 bf16, 223: 33 / 31.
-        if (c.C == 1) return f32 || V < 12000 ? 0.0f : 1.0f;
-        // fp32: 32,000, 148 / 180: 32 / 43, 57 / 47; 65,536, 110 / 148: 61 / 65, 85 / 66; 128,000, 75 / 110: 91 / 110, 123 / 111.
-        if (f32) return std::max(1.0f, v / 43000.0f);
-        // Two blocks, bf16: 20,000, 200: 35 / 32; 32,000, 180 / 222: 45 / 48, 55 / 53; four: 50,272, 110 / 148: 55 / 63, 69 / 59; 65,536, 148 / 222:
-        // 66 / 66, 90 / 84; eight: 128,000, 110 / 148: 107 / 118, 132 / 110.
-        return c.C == 2 ? std::max(1.0f, (v - 9000.0f) / 17000.0f) : std::min(v / 27500.0f, 1.0f + v / 52000.0f);
+bool on_chip_pays(const rsd::walk_cluster::Shape& c, int B, int V, bool f32, WalkKind kind, int rejected) {
+    if (c.C == 0) return false;
+    if (c.NT == 1 && V <= 8192) {
+        if (kind == kRingRows) return c.waves <= 1.3f;
+        if (kind == kDraw && c.C == 2 && !f32) return c.waves <= std::max(1.0f, 0.2f + (float)V / 9000.0f);
+        return true;
     }
-    // Rows that are read anew take about as long for 40 sequences as for all that are resident at once, 296 (fp32) or 444, then twice as long.
-    const int per_round = (f32 ? 2 : 3) * sm_count();
-    const float round = (float)((B + per_round - 1) / per_round);
-    if (c.NT == 1) {
-        if (kind == kDraw && c.C == 2 && !f32) return std::max(1.0f, 0.2f + v / 9000.0f);   // 8192, 200 / 300: 12.6 / 19, 22 / 22
-        return c.C <= 2 ? kAlways : 1.0f;                // (of more blocks, and below of two tiles per warp: only where all are resident)
-    }
-    if (c.NT == 2) return 1.0f;
-    switch (kind) {
-        case kReadAnewTop1:   // Gumbel-Top-1 draws take two rounds of Philox calls when rows are read anew
-            if (f32) {
-                if (c.C == 1) return V < 11000 ? 0.0f : round;                        // 8200, 222: 32 / 28; 14,000, 296 / 444: 38 / 39, 65 / 70
-                if (c.C == 2) return std::max(1.0f, (v - 10000.0f) / 11000.0f) * round;   // 20,000, 222: 60 / 47; 32,000, 222 / 350: 65 / 64, 95 / 116
-                return v / (c.C == 4 ? 22000.0f : 27000.0f) * round;                  // 50,000, 110 / 222: 65 / 79, 122 / 94; 128,000, 148 / 200: 168 / 171, 226 / 192
-            }
-            if (c.C == 1) return std::max(round, v / 9500.0f);                        // 8200, 296 / 350: 37 / 44, 54 / 43; 14,000, 350: 58 / 58
-            if (c.C == 2) return V < 23000 ? 2.0f : v / 8000.0f;                      // 20,000, 260 / 350: 58 / 61, 79 / 66; 32,000, 444: 94 / 109
-            return c.C == 4 ? v / 13600.0f : (v - 10000.0f) / 14000.0f;               // 50,000, 260 / 350: 115 / 135, 153 / 135; 128,000, 200 / 300: 197 / 246, 290 / 290
-        case kDraw:           // residual draws with rejected tokens (a pass per token, always both rows)
-            if (f32) {
-                if (c.C == 1) return kAlways;                                         // 14,000, 444: 38 / 50
-                if (c.C == 2) return (V < 26000 ? 1.0f : 2.0f) * round;               // 20,000, 222: 35 / 30; 32,000, 222 / 350: 36 / 43, 53 / 77
-                return (c.C == 4 ? (v - 10000.0f) / 12500.0f : (v - 32000.0f) / 12200.0f) * round;   // 50,000, 180 / 296: 56 / 66, 88 / 74; 100,000, 148 / 256: 96 / 116, 158 / 136
-            }
-            if (c.C == 1) return 1.0f;                                                // 14,000, 296 / 350: 20 / 27, 38 / 32
-            if (c.C == 2) return V < 26000 ? 1.0f : V < 30000 ? 2.0f : v / 8000.0f - 1.25f;   // 20,000, 180: 35 / 32; 32,000, 296 / 400: 39 / 44, 56 / 55
-            return v / (c.C == 4 ? 21000.0f : 32000.0f);                              // 50,000, 110 / 222: 41 / 49, 78 / 63; 128,000, 75 / 148: 69 / 104, 115 / 122
-        case kDrawWhole:      // the pass that writes the distribution costs reading anew more
-            if (f32) return c.C <= 2 ? kAlways : v / (c.C == 4 ? 10500.0f : 12000.0f) * round;   // 32,000, 350: 68 / 114; 42,000, 296: 102 / 94; 70,000, 200: 141 / 133
-            if (c.C == 1) return round > 1.0f ? kAlways : 1.0f;                       // 14,000, 296 / 350: 25 / 34, 46 / 42; 8200, 800: 63 / 72
-            if (c.C == 2) return V < 25000 ? 1.0f : v / 10000.0f;                     // 20,000, 222: 42 / 42; 24,000, 320: 65 / 61; 32,000, 444: 74 / 81
-            return v / (c.C == 4 ? 17000.0f : 23000.0f);                              // 50,000, 180 / 222: 73 / 89, 94 / 88; 128,000, 110 / 256: 111 / 151, 227 / 198
-        default:              // the rules' walks and rows off 16-byte boundaries
-            if (f32) {
-                if (c.C == 1) return 0.0f;                                            // 14,000, 222: 25 / 20
-                if (c.C == 2) return (V < 26000 ? 0.6f : 1.0f) * round;               // 20,000, 75 / 148: 22 / 22, 24 / 21; 32,000, 148 / 180: 26 / 29, 46 / 32
-                return (c.C == 4 ? std::max(1.0f, v / 25000.0f - 1.1f) : v / 44000.0f) * round;   // 50,000, 75: 45 / 38; 65,000, 90: 48 / 52; 128,000, 75 / 110: 73 / 85, 112 / 120
-            }
-            if (c.C == 1) return round;                                               // 14,000, 296 / 350: 30 / 37, 47 / 38
-            if (c.C == 2) return V < 23000 ? 1.0f : 2.0f;                             // 20,000, 222: 44 / 41; 32,000, 296 / 350: 49 / 58, 64 / 60
-            return c.C == 4 ? (v - 8000.0f) / 14000.0f : v / 22000.0f;                // 50,000, 180 / 222: 67 / 69, 82 / 80; 100,000, 148 / 200: 110 / 118, 146 / 138
-    }
+    if (c.NT < 4) return c.waves <= 1.0f;
+    static const float cost[5][2][2] = {                 // [kind][4-byte rows]: a, b
+        {{0.75f, 0.22f}, {0.60f, 0.40f}}, {{0.55f, 0.36f}, {0.30f, 0.52f}}, {{0.65f, 0.68f}, {0.80f, 0.60f}}, {{1.05f, 0.28f}, {0.65f, 0.68f}}, {{1.10f, 0.46f}, {0.75f, 1.00f}}};
+    auto counted = [](float n) { return 0.5f * (std::ceil(n) + std::max(n, 1.0f)); };
+    const float rounds = counted((float)B / (float)((f32 && kind != kRingRows ? 2 : 3) * sm_count()));
+    const float passes = kind >= kDraw ? std::sqrt(std::sqrt((float)rejected / 3.0f)) : 1.0f;
+    return counted(c.waves) <= rounds * passes * (cost[kind][f32][0] + cost[kind][f32][1] * (float)V / 10000.0f);
 }
 
 void launch_on_chip(const rsd::walk_cluster::ClusterArgs& a, int dtype, bool extra, int B, const rsd::walk_cluster::Shape& c, cudaStream_t s) {
@@ -197,7 +164,7 @@ int rsd_verify_tree_rule(const rsd_rows* draft, const rsd_rows* target, const rs
     // always: a batch and its parts give the same bits.
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
     const WalkKind kind = ring ? kRingRows : final_sampler == RSD_FINAL_GUMBEL_TOP1 ? kReadAnewTop1 : kReadAnew;
-    const bool on_chip = shape.C > 0 && shape.waves <= most_waves(shape, B, V, draft->dtype == RSD_F32, kind);
+    const bool on_chip = on_chip_pays(shape, B, V, draft->dtype == RSD_F32, kind, 0);
     rsd::walk_cluster::ClusterArgs ca;
     memset(&ca, 0, sizeof(ca));
     ca.v = a;
@@ -249,7 +216,7 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     if (!a.max_k && !(shape.C > 2 && shape.NT < 4 && shape.waves <= 1.0f)) {
         if (f32) rsd::walk_cluster::launch_draw_f32(a, B, s);
         else rsd::walk_cluster::launch_draw_bf16(a, B, s);
-    } else if (shape.C > 0 && shape.waves <= most_waves(shape, B, V, f32, out_residual ? kDrawWhole : kDraw)) {
+    } else if (on_chip_pays(shape, B, V, f32, out_residual ? kDrawWhole : kDraw, a.max_k)) {
         launch_on_chip(ca, target_row->dtype, true, B, shape, s);
     } else {
         launch_streamed(ca, target_row->dtype, true, B, shape.C > 0, s);

@@ -7,6 +7,7 @@ import torch
 
 import oracle
 import workloads
+from tests.launches import launched
 from tests.parity import Tally, compare_verify
 from tests.test_gpu_parity import _np
 from tests.test_gpu_walk_cluster import _drafted, _tokens
@@ -175,3 +176,37 @@ def test_residual_draws_with_four_tiles_per_warp_give_the_bits_of_fewer(dtype, V
         part = rsd.rsd_resample_residual(draft[b:b + 3], target[b:b + 3], rejected[b:b + 3], node[b:b + 3], 5, 1, seq_base=b, want_residual=True)
         for key in part:
             assert torch.equal(part[key], whole[key][b:b + 3]), (key, b)
+
+
+# Where the two costs of a walk that four tiles per warp could hold lie clearly apart (us, on chip / the other route): the faster one is taken.
+@pytest.mark.parametrize("dtype,V,B,off,rule,expected", [
+    ("f32", 130695, 101, 0, 0, "walk_cluster"),            # (3, 2) tree: about 150 / 296
+    ("f32", 46630, 79, 0, 0, "walk_cluster"),              # 57 / 98
+    ("f32", 65840, 59, 1, 0, "walk_cluster"),              # 62 / 101
+    ("f32", 118688, 102, 1, 0, "walk_cluster"),            # 184 / 289
+    ("bf16", 110439, 180, 0, 2, "walk_stream"), ("bf16", 32000, 148, 0, 0, "walk_cluster"), ("bf16", 32000, 444, 0, 0, "verify_tree_ring"),
+    ("f32", 16389, 900, 3, 0, "walk_stream"), ("bf16", 131073, 4, 0, 0, "walk_stream"), ("bf16", 262144, 4, 0, 0, "verify_tree_ring")])
+def test_walks_take_the_faster_route(dtype, V, B, off, rule, expected):
+    import paper_2402_14160_b200 as rsd
+    draft, target, _ = _drafted(B, V, dtype, (2, 1), 5, off=off)
+    token = _tokens(rsd, draft, (2, 1), 3)
+    parent = torch.from_numpy(workloads.rsdc_parent_array((2, 1))).cuda()
+    assert [l.kernel for l in launched(lambda: rsd.rsd_verify_tree_rule(draft, target, parent, token, 2, rule, 2.0, 0, 3, 0))] == [expected]
+
+
+def _draw_launches(dtype, V, B, k, whole):
+    import paper_2402_14160_b200 as rsd
+    rows = torch.randn((B, V), device="cuda").to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    rejected = torch.randint(0, V, (B, k), device="cuda", dtype=torch.int32) if k else None
+    node = torch.zeros(B, dtype=torch.int32, device="cuda")
+    return launched(lambda: rsd.rsd_resample_residual(rows, rows, rejected, node, 5, 1, want_residual=whole))
+
+
+@pytest.mark.parametrize("dtype,V,B,k,whole,expected", [
+    ("bf16", 104256, 106, 1, False, "walk_stream"),        # 67 / 52
+    ("f32", 48448, 216, 1, False, "walk_stream"),          # 52 / 40
+    ("bf16", 31296, 285, 1, False, "walk_stream"),         # 41 / 31
+    ("f32", 110336, 207, 1, False, "walk_stream"),         # 101 / 79
+    ("bf16", 104256, 106, 16, False, "walk_cluster"), ("f32", 32000, 256, 3, True, "walk_cluster"), ("bf16", 8000, 900, 3, True, "walk_cluster")])
+def test_residual_draws_take_the_faster_route(dtype, V, B, k, whole, expected):
+    assert [l.kernel for l in _draw_launches(dtype, V, B, k, whole)] == [expected]
