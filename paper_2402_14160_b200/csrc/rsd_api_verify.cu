@@ -203,7 +203,8 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     cudaStream_t s = (cudaStream_t)stream;
     // A draw with nothing rejected is one sweep over the target row: a block per sequence, but a cluster for the few sequences of
     // rows beyond 16,384 entries that are resident at once (us, cluster / block, bf16: 32,000 entries, 1 / 64 / 148 sequences 6.2 / 7.3 / 20,
-    // 6.8 / 7.0 / 7.1; 128,000, 1 / 16 / 64: 7.2 / 15 / 36, 17 / 17 / 17).
+    // 6.8 / 7.0 / 7.1; 128,000, 1 / 16 / 64: 7.2 / 15 / 36, 17 / 17 / 17).  So, too, with four tiles per warp: eight blocks 0.34 to 0.67 of the block's time
+    // (90,624 entries with the distribution, 16 sequences, bf16: 13 / 36), four 0.6 to 0.75 with the distribution, without it 0.9 for 4-byte rows and 1.2 for 2-byte ones.
     rsd::walk_cluster::ClusterArgs ca;
     memset(&ca, 0, sizeof(ca));
     ca.r = a;
@@ -213,10 +214,11 @@ int rsd_resample_residual(const rsd_rows* draft_row, const rsd_rows* target_row,
     ca.v.seed_lo = a.seed_lo; ca.v.seed_hi = a.seed_hi; ca.v.step = step; ca.v.seq_base = seq_base;
     const rsd::walk_cluster::Shape shape = cluster_shape(B, V);
     const bool f32 = target_row->dtype == RSD_F32;
-    if (!a.max_k && !(shape.C > 2 && shape.NT < 4 && shape.waves <= 1.0f)) {
+    const bool draw_on_chip = shape.C > 2 && shape.waves <= 1.0f && (shape.NT < 4 || shape.C == 8 || f32 || out_residual);
+    if (!a.max_k && !draw_on_chip) {
         if (f32) rsd::walk_cluster::launch_draw_f32(a, B, s);
         else rsd::walk_cluster::launch_draw_bf16(a, B, s);
-    } else if (on_chip_pays(shape, B, V, f32, out_residual ? kDrawWhole : kDraw, a.max_k)) {
+    } else if (!a.max_k || on_chip_pays(shape, B, V, f32, out_residual ? kDrawWhole : kDraw, a.max_k)) {
         launch_on_chip(ca, target_row->dtype, true, B, shape, s);
     } else {
         launch_streamed(ca, target_row->dtype, true, B, shape.C > 0, s);

@@ -159,6 +159,23 @@ def test_four_tiles_per_warp_give_the_bits_of_fewer(dtype, V, B, off, rule, samp
     test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble)
 
 
+@pytest.mark.parametrize("dtype,V,B", [("f32", 131072, 33), ("bf16", 65537, 33), ("f32", 32769, 71), ("bf16", 50272, 40)])
+@pytest.mark.parametrize("whole", [False, True])
+def test_draws_with_nothing_rejected_give_the_same_bits_with_four_tiles_per_warp(dtype, V, B, whole):
+    # (one sequence: fewer tiles per warp; the largest batch: the kernel of a block per sequence)
+    import paper_2402_14160_b200 as rsd
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    rows = (torch.randn((4 * B, V), generator=gen, device="cuda") * 2).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    rows[::3, V // 2] = float("nan")
+    node = torch.arange(4 * B, dtype=torch.int32, device="cuda")
+    all_ = rsd.rsd_resample_residual(rows, rows, None, node, 5, 1, want_residual=whole)
+    for b, n in ((0, B), (B - 1, 1), (3 * B, B)):
+        part = rsd.rsd_resample_residual(rows[b:b + n], rows[b:b + n], None, node[b:b + n], 5, 1, seq_base=b, want_residual=whole)
+        for key in part:
+            if part[key] is not None:
+                assert torch.equal(part[key], all_[key][b:b + n]), (key, b, n)
+
+
 @pytest.mark.parametrize("dtype,V,B", [("f32", 16384, 200), ("bf16", 16385, 148), ("f32", 32000, 148), ("bf16", 65529, 64), ("f32", 131072, 33)])
 def test_residual_draws_with_four_tiles_per_warp_give_the_bits_of_fewer(dtype, V, B):
     import paper_2402_14160_b200 as rsd
@@ -207,6 +224,8 @@ def _draw_launches(dtype, V, B, k, whole):
     ("f32", 48448, 216, 1, False, "walk_stream"),          # 52 / 40
     ("bf16", 31296, 285, 1, False, "walk_stream"),         # 41 / 31
     ("f32", 110336, 207, 1, False, "walk_stream"),         # 101 / 79
+    ("bf16", 90624, 16, 0, True, "walk_cluster"), ("f32", 69744, 18, 0, False, "walk_cluster"), ("f32", 50591, 34, 0, True, "walk_cluster"),   # 13 / 36, 9 / 19, 17 / 29
+    ("bf16", 122904, 34, 0, False, "draw_target"), ("bf16", 60000, 34, 0, False, "draw_target"), ("bf16", 32000, 148, 0, True, "draw_target"),
     ("bf16", 104256, 106, 16, False, "walk_cluster"), ("f32", 32000, 256, 3, True, "walk_cluster"), ("bf16", 8000, 900, 3, True, "walk_cluster")])
 def test_residual_draws_take_the_faster_route(dtype, V, B, k, whole, expected):
     assert [l.kernel for l in _draw_launches(dtype, V, B, k, whole)] == [expected]
