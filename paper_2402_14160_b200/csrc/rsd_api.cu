@@ -33,11 +33,15 @@ thread_local cudaEvent_t g_scan_before = nullptr, g_scan_after = nullptr;  // on
 // four warps (few rows: 256 threads with the sums on four warps and the perturbed values on the others), beyond those of
 // eight, by 256 threads in every launch (bf16, 64 / 222 / 370 / 600 rows of 16,384: 8.4 / 10.5 / 11.1 / 12.3 with 128 threads, 8.1 / 10.0 / 10.8 /
 // 17.0 with 256; 192 / 5000 rows of 128,000: 43 / 370 with 128, 27 / 247 with 256).
-int scan_threads(int rows, int V, bool f32, bool need_lse) {
+int sm_count() {
     static const int sms = [] {
         int dev = 0, n = 0;
         return (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 148;
     }();
+    return sms;
+}
+int scan_threads(int rows, int V, bool f32, bool need_lse) {
+    const int sms = sm_count();
     const bool few = rows <= sms + sms / 2;
     if (need_lse) return V > rsd::kScanSplitVocab || (V >= 16384 && rows <= 5 * sms / 2) ? 256 : 128;
     if (V >= 16384 && few) return 512;
@@ -46,8 +50,25 @@ int scan_threads(int rows, int V, bool f32, bool need_lse) {
     return V >= 4096 && few ? 256 : 128;
 }
 
+// Whether the rows of a sequence are scanned as a cluster, whose first block gathers their status, without a kernel ahead that clears it: up to eight rows,
+// few in all (14,100 drafts of 1 to 370 rows: 0.81 to 0.98 of the time with that kernel in every group of types, row offsets, threads and rows, a fifth of the
+// smallest).  Blocks of a cluster stay within a GPC, two on an SM where the launch alone would give each its own: 4-byte rows off 32-byte boundaries
+// feel that with 512 threads where they come close to one an SM (us, cluster / cleared, 90 x 63,983 / 112 x 58,589 / 126 x 38,920 / 148 x 28,504 entries:
+// 18.3 / 17.1, 21.5 / 16.7, 18.1 / 15.3, 14.3 / 12.5; 80 x 62,296: 15.2 / 16.1; beyond one row an SM 0.94 again; rows of a sequence of their own 0.95).
+bool status_by_cluster(int B, int R, int V, bool f32, bool aligned, bool need_lse) {
+    const int sms = sm_count();
+    const int64_t rows = (int64_t)B * R;
+    if (R > rsd::kMaxLevelRows || rows > 5 * sms / 2 || rows * V > (V > 65536 ? 6000000 : 12000000)) return false;
+    const int threads = scan_threads((int)rows, V, f32, need_lse);
+    if (threads == 512 && f32 && !aligned && R > 1 && rows > 3 * sms / 5 && rows <= sms) return false;
+    return threads > 128;                                // (smaller blocks: rows of less than 4096 entries)
+}
+
+// Rows made of whole groups that start on 32-byte boundaries.
+bool whole_groups(const rsd_rows* rows, int V) { return V % 16 == 0 && rows_aligned(rows, 32); }
+
 void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs& a, cudaStream_t s, const rsd::SbsEpilogueArgs* level = nullptr) {
-    const bool aligned = a.V % 16 == 0 && rows_aligned(rows, 32);   // rows made of whole groups that start on 32-byte boundaries
+    const bool aligned = whole_groups(rows, a.V);
     for (int r = 0; r < 10; ++r) {
         a.rk0[r] = a.seed_lo + (uint32_t)r * 0x9E3779B9u;
         a.rk1[r] = a.seed_hi + (uint32_t)r * 0xBB67AE85u;
@@ -133,7 +154,7 @@ int rsd_gumbel_topk_draft(const rsd_rows* draft, int B, int R, int V, const int3
     a.temp = temperature_of(draft); a.inv_temp = 1.0f / a.temp;
     const bool need_lse = !rows_are_logprob(draft) && (out_perturbed || out_logprob);
     // (a cluster per sequence gathers its rows' status; otherwise they are OR-ed into cleared words)
-    a.cluster_status = level_in_one_launch(B, R, V) && scan_threads(B * R, V, draft->dtype == RSD_F32, need_lse) > 128;
+    a.cluster_status = status_by_cluster(B, R, V, draft->dtype == RSD_F32, whole_groups(draft, V), need_lse);
     if (a.cluster_status) a.wait_first = 1;
     else clear_status(status, B, s);
     launch_scan(draft, need_lse, B * R, a, s);

@@ -3,6 +3,8 @@ overlaps: whatever the words held, afterwards they hold this call's bits and not
 import pytest
 import torch
 
+from tests.launches import launched
+
 pytestmark = pytest.mark.gpu
 NAN_INPUT = 1
 
@@ -62,3 +64,19 @@ def test_status_of_few_rows_gathered_by_their_cluster(B, R, V):
         out["status"].fill_(77)
         rsd.rsd_gumbel_topk_draft(rows, [3] * R, list(range(R)), 1, 0, want_values=values, out=out)
         assert out["status"].cpu().tolist() == want
+
+
+# Close to one row an SM (148) the blocks of a cluster share SMs: 4-byte rows off 32-byte boundaries with 512 threads have their words cleared.
+@pytest.mark.parametrize("dtype,B,R,V,clusters", [
+    ("f32", 16, 7, 58589, False), ("f32", 34, 4, 36910, False), ("f32", 11, 8, 20001, True), ("f32", 30, 5, 20001, True), ("f32", 140, 1, 20001, True),
+    ("f32", 16, 7, 32000, True), ("bf16", 16, 7, 58589, True), ("f32", 12, 9, 20001, False)])
+def test_rows_that_would_share_an_sm_as_clusters_have_their_words_cleared(dtype, B, R, V, clusters):
+    import paper_2402_14160_b200 as rsd
+    rows = torch.randn((B, R, V), device="cuda").to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    rows[::2, R - 1, V - 1] = float("nan")
+    out = rsd.rsd_gumbel_topk_draft(rows, [3] * R, list(range(R)), 1, 0)
+    out["status"].fill_(77)
+    got = launched(lambda: rsd.rsd_gumbel_topk_draft(rows, [3] * R, list(range(R)), 1, 0, out=out))
+    assert [l.kernel for l in got] == (["scan_topk"] if clusters else ["clear_status", "scan_topk"])
+    assert got[-1].cluster == (R if clusters else 0)
+    assert out["status"].cpu().tolist() == [NAN_INPUT if b % 2 == 0 else 0 for b in range(B)]
