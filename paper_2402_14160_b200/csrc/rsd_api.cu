@@ -85,10 +85,20 @@ void launch_scan(const rsd_rows* rows, bool need_lse, int blocks, rsd::ScanArgs&
 
 // A level of few rows runs in one launch, the rows of a sequence as a cluster; its blocks stay until the longest of them is through, so
 // that many or long rows are better scanned by themselves (us, one launch / two; bf16 32,000 entries, 4 / 224 / 368 rows: 13.4 / 14.9, 18.6 / 19.6, 21.0 / 23.5;
-// fp32 65,536, 192 / 224 / 368: 25.1 / 25.0, 27.9 / 26.6, 37.3 / 35.5; 128,000, 8 / 64 / 192: 17.2 / 19.2, 19.7 / 18.7, 27.4 / 27.1; fp32 4096, 300 / 592: 12.8 / 16.1, 16.9 / 14.6).
-bool level_in_one_launch(int B, int n_par, int V) {
+// fp32 128,000, 8 / 64 / 192: 17.2 / 19.2, 19.7 / 18.7, 27.4 / 27.1; fp32 4096, 300 / 592: 12.8 / 16.1, 16.9 / 14.6).  So are
+//   more than 16 children: half as many as the scan's lanes; the bound of more lets so many entries through that their stages decide, which the larger
+// kernel is slower at (16 / 24 / 32 children, rows of 16,384 to 65,536 entries with a log-sum-exp: 0.93 / 1.00 / 1.15 of two launches, at most 1.05 / 1.16 /
+// 1.42; rows of up to 2048 entries have few: 0.95 to 0.99);
+//   4-byte rows of 48,000 to 65,536 entries with a log-sum-exp, more than half as many as SMs (58,816, 198 rows 32.0 / 27.6; 61,376, 119: 30.8 / 26.9;
+// 60,000, 74: 0.93 of two launches), those off 32-byte boundaries beyond that (131,000: 1.03), and what status_by_cluster() leaves out.
+bool level_in_one_launch(int B, int n_par, int V, int W, bool f32, bool aligned, bool need_lse) {
+    const int sms = sm_count();
     const int64_t rows = (int64_t)B * n_par;
-    return n_par <= rsd::kMaxLevelRows && rows <= 370 && rows * V <= (V > 65536 ? 6000000 : 12000000);
+    if (n_par > rsd::kMaxLevelRows || rows > 5 * sms / 2 || rows * V > (V > 65536 ? 6000000 : 12000000)) return false;
+    if (W > 16 && V > 2048) return false;
+    if (!f32) return true;
+    if (need_lse) return V <= 48000 || (V > 65536 ? aligned : 2 * rows <= sms);
+    return V < 16384 || aligned || status_by_cluster(B, n_par, V, f32, aligned, need_lse);
 }
 
 // status[0..B) = 0 ahead of a kernel that ORs bits into it, which does not wait for this one until it touches status (a memset
@@ -220,7 +230,7 @@ int rsd_sbs_step(const rsd_rows* draft_level, int B, int n_par, int V, int W, in
     e.sum_out = sum_logprob_out; e.gamma_out = trunc_gumbel_out;
     e.out_count = out_count; e.status = status;
     const bool need_lse = !rows_are_logprob(draft_level);
-    if (level_in_one_launch(B, n_par, V)) {
+    if (level_in_one_launch(B, n_par, V, W, draft_level->dtype == RSD_F32, whole_groups(draft_level, V), need_lse)) {
         launch_scan(draft_level, need_lse, B * n_par, a, s, &e);
         return check_launch("rsd_sbs_step(level)");
     }

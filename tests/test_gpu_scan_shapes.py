@@ -11,6 +11,7 @@ import torch
 
 import oracle
 import workloads
+from tests.launches import launched
 from tests.parity import Tally, compare_topk
 
 pytestmark = pytest.mark.gpu
@@ -90,7 +91,8 @@ def test_rows_without_log_sum_exp_alone_and_in_a_batch_give_the_same_bits(dtype,
 @pytest.mark.parametrize("dtype,V,n_par,W,B,off,form,trouble", [
     ("bf16", 70, 8, 8, 200, 0, "", "few"), ("f32", 4096, 3, 5, 200, 0, "", "nan"), ("bf16", 16383, 8, 32, 60, 1, "tempered", ""), ("f32", 16384, 2, 2, 300, 0, "", "dead"),
     ("bf16", 32000, 4, 4, 140, 0, "", "nan"), ("f32", 32000, 6, 6, 80, 0, "logprob", "dead"), ("f32", 1001, 7, 3, 90, 1, "logprob", "few"),
-    ("bf16", 65552, 8, 8, 64, 0, "", "dead"), ("f32", 70001, 5, 8, 90, 3, "tempered", "nan"), ("bf16", 131072, 1, 8, 400, 0, "", "")])
+    ("bf16", 65552, 8, 8, 64, 0, "", "dead"), ("f32", 70001, 5, 8, 90, 3, "tempered", "nan"), ("bf16", 131072, 1, 8, 400, 0, "", ""),
+    ("bf16", 2047, 8, 32, 60, 1, "tempered", ""), ("bf16", 40001, 8, 16, 60, 1, "", "nan"), ("f32", 58816, 2, 2, 99, 0, "", "dead"), ("f32", 58589, 7, 7, 16, 3, "logprob", "nan")])
 def test_levels_alone_and_in_a_batch_give_the_same_bits(dtype, V, n_par, W, B, off, form, trouble):
     import paper_2402_14160_b200 as rsd
     gen = torch.Generator(device="cuda").manual_seed(V + B)
@@ -118,3 +120,18 @@ def test_levels_alone_and_in_a_batch_give_the_same_bits(dtype, V, n_par, W, B, o
         for key in part:
             got, want = part[key].cpu().numpy(), whole[key][b:b + n].cpu().numpy()
             assert np.array_equal(got, want, equal_nan=got.dtype.kind == "f"), (key, b)
+
+
+# Up to 16 children of longer rows; 4-byte rows with a log-sum-exp up to half as many as SMs from 48,000 to 65,536 entries, beyond that only whole groups.
+@pytest.mark.parametrize("dtype,V,n_par,W,B,logprob,one", [
+    ("bf16", 32000, 4, 16, 8, False, True), ("bf16", 32000, 4, 17, 8, False, False), ("bf16", 2048, 4, 32, 8, False, True), ("bf16", 2049, 4, 32, 8, False, False),
+    ("f32", 58816, 2, 2, 99, False, False), ("f32", 58816, 2, 2, 37, False, True), ("f32", 48000, 2, 2, 99, False, True), ("f32", 58816, 2, 2, 99, True, True),
+    ("f32", 70001, 5, 5, 10, False, False), ("f32", 70000, 5, 5, 10, False, True), ("f32", 58589, 7, 7, 16, True, False), ("f32", 58592, 7, 7, 16, True, True),
+    ("bf16", 65535, 6, 6, 24, False, True), ("bf16", 32000, 9, 8, 2, False, False)])
+def test_levels_take_the_faster_route(dtype, V, n_par, W, B, logprob, one):
+    import paper_2402_14160_b200 as rsd
+    rows = torch.randn((B, n_par, V), device="cuda")
+    rows = (torch.log_softmax(rows, -1) if logprob else rows).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    sums = torch.zeros((B, n_par), device="cuda")
+    got = launched(lambda: rsd.rsd_sbs_step(rows, W, 3, sums, sums, 17, 3, is_logprob=logprob))
+    assert [l.kernel for l in got] == (["scan_level"] if one else ["scan_topk", "sbs_epilogue"])
