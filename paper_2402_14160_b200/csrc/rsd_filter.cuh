@@ -551,6 +551,14 @@ struct RowFilter {
         if (lane == 0) { sm.cut_code = lo; sm.cut_tok = tok; }
     }
 
+    // The reach of top_few()'s bins below the row's largest value, and whether the part of the slack in bin_edges() that follows the value
+    // itself is at most a twelfth of it.
+    __device__ __forceinline__ float few_width(float v_hi) const { return fminf(kValueRange * kLog2e / k, sm.low < v_hi ? 1.25f * (v_hi - sm.low) : 3.0e38f); }
+    __device__ __forceinline__ bool slack_is_small(uint32_t top) const {
+        const float v_hi = Codes::value_of_code(top);
+        return fabsf(v_hi) * (0.0079f * 12.0f) <= few_width(v_hi);
+    }
+
     // Top-k for few tokens, and top-p among them (top_p < 1), without a histogram of the row: the threads' largest values (of distinct tokens)
     // go into the bins, the n-th largest of them bounds the n-th largest token from below, and what reaches it fits the list
     // (n = 50 of 1024 threads: about 55 tokens).  false: it does not; nothing is decided.  The histogram is clear; mine_top: this thread's largest value.
@@ -561,7 +569,7 @@ struct RowFilter {
         bm.shift = -1;
         bm.lo = Codes::kNegInfCode + 1u;
         bm.hi = top;
-        const float v_hi = Codes::value_of_code(top), width = fminf(kValueRange * kLog2e / k, sm.low < v_hi ? 1.25f * (v_hi - sm.low) : 3.0e38f);
+        const float v_hi = Codes::value_of_code(top), width = few_width(v_hi);
         bm.scale = (float)(kBins - 1) / width;
         bm.offset = v_hi * bm.scale;
         if (!(width > 0.0f) || !(width < 3.0e38f) || !(fabsf(bm.offset) < 1.0e6f)) return false;
@@ -846,9 +854,12 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
     const bool want_p = a.top_p > 0.0f && a.top_p < 1.0f && finite > 0 && !plus_inf;
     bool found_p = false;
     if (a.top_k > 0 && a.top_k < V && finite > a.top_k) {
-        // Half as many tokens as threads: the list's size is sure to do for ordinary rows.  Rows of four words a thread on: top-k 50, top-p 0.9, 1500 rows of
-        // 32,000 bf16 87 -> 60 us, 32 rows of 8000 fp32 1.19 times as fast; single rows of 4100 fp32 with top-k alone 6.2 -> 8.1.
-        const bool few = a.top_k <= NT / 2 && n_vec >= 4 * NT;
+        // (top_few() pays while what reaches the bound, a few more tokens than asked for, stays in the registers of finish(); 512 threads, rows of 8,192 to
+        // 50,000 entries, 4-byte with top-k alone, 64 / 100 / 128 / 256 tokens: 0.87 / 0.92 / 1.08 / 1.38 of the time of a histogram of the row; with a nucleus behind
+        // it 0.81 / 0.74 / 0.89 / 1.13; 2-byte top-k alone 0.82 / 0.88 / 0.94 / 1.06; 1024 threads, 160 / 256: 0.89 / 0.93, 4-byte 1.00 / 1.13, with a nucleus 0.94 / 0.97.  Rows of four words a
+        // thread on: from 16,384 2-byte or 8192 4-byte entries, 32 rows of 8192 fp32, top-k 50 and top-p 0.9 14.6 -> 10.9 us.  And while the slack that bin_edges() gives the bound,
+        // which follows the values' distance from 0, is small beside the bins' reach: 110 rows of 11,336 fp32 around 300 take 33.2 us where it is not heeded, 14.6 here.)
+        const bool few = a.top_k <= (kElem == 2 || want_p ? NT / 4 : NT / 8) && n_vec >= 4 * NT && f.slack_is_small(top);
         if (few && f.top_few(top, vtop, a.top_k, want_p ? a.top_p : 1.0f, cut)) {
             found_p = want_p;
         } else {

@@ -223,10 +223,12 @@ def test_filter_rows_that_the_sample_of_the_first_sweep_misjudges(rsd, dtype, V)
 
 
 @pytest.mark.parametrize("dtype,V,top_k", [("bf16", 16384, 256), ("bf16", 16384, 257), ("bf16", 16383, 256), ("f32", 8192, 256), ("f32", 8195, 100), ("f32", 8195, 1),
-                                           ("bf16", 65601, 512), ("bf16", 32000, 129), ("f32", 33001, 50), ("f32", 50000, 513)])
+                                           ("bf16", 65601, 512), ("bf16", 32000, 129), ("f32", 33001, 50), ("f32", 50000, 513),
+                                           ("bf16", 16384, 128), ("bf16", 16391, 129), ("f32", 8195, 64), ("f32", 8192, 65), ("f32", 8197, 128), ("f32", 8192, 129),
+                                           ("bf16", 65601, 256), ("bf16", 65600, 257), ("f32", 33001, 128), ("f32", 33000, 129), ("f32", 33003, 256), ("f32", 33000, 257)])
 def test_top_k_bounded_by_the_threads_largest_values(rsd, dtype, V, top_k):
-    # up to half as many tokens as threads (512, or 1024 where a row fills an SM) from rows of four words a thread on; lists of up to 128 tokens
-    # are ended in registers
+    # up to a quarter as many tokens as threads (512, or 1024 where a row fills an SM; 4-byte rows with top-k alone an eighth) from rows of four words a
+    # thread on; lists of up to 128 tokens are ended in registers
     g = torch.Generator(device="cpu").manual_seed(V + top_k)
     rows = torch.randn((1, 7, V), generator=g) * 2
     rows[0, 1] = (rows[0, 1] * 4).round() / 4                     # ties at every cut
@@ -241,3 +243,15 @@ def test_top_k_bounded_by_the_threads_largest_values(rsd, dtype, V, top_k):
     # (equal weights put cumulative masses on round fractions: such rows may be borderline)
     for top_p in (1.0, 0.9, 0.37):
         _check_filter(rsd, rows, top_k, top_p, 1.0, max_borderline=0 if top_p == 1.0 else 3)
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 17003), ("f32", 9001), ("f32", 33001)])
+def test_top_k_of_rows_near_and_far_from_zero(rsd, dtype, V):
+    # the slack of the bound follows the values: rows on both sides of where the threads' largest values still serve, and beyond the bins' precision
+    g = torch.Generator(device="cpu").manual_seed(V)
+    rows = torch.randn((1, 8, V), generator=g) * 2
+    for r, shift in enumerate((20.0, 90.0, 160.0, 220.0, 250.0, 300.0, -200.0, -3000.0)):
+        rows[0, r] += shift
+    rows = rows.to(torch.bfloat16 if dtype == "bf16" else torch.float32).cuda()
+    for top_k, top_p, T in ((50, 1.0, 1.0), (50, 0.9, 1.0), (64, 0.9, 0.3)):
+        _check_filter(rsd, rows, top_k, top_p, T, max_borderline=3)
