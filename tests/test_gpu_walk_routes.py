@@ -28,13 +28,18 @@ def _whole_and_parts(rsd, draft, target, parent, token, L, rule=0, gamma=2.0, sa
     return whole
 
 
-# batches beyond the limits of the on-chip walk, and (rows beyond 131,072 entries) on both sides of eight blocks a sequence
-@pytest.mark.parametrize("dtype,V,B,off,rule,sampler,trouble", [
-    ("bf16", 32001, 300, 1, 0, 0, ""), ("bf16", 32001, 230, 7, 0, 0, "nan"), ("f32", 16389, 600, 3, 0, 0, "nan"), ("bf16", 8201, 800, 1, 0, 0, "far"),
-    ("bf16", 65551, 200, 1, 0, 0, "far"), ("bf16", 32000, 300, 0, 1, 0, ""), ("bf16", 16400, 600, 0, 2, 0, "nan"), ("f32", 8208, 800, 0, 2, 1, "far"),
-    ("bf16", 32000, 560, 0, 1, 1, ""), ("bf16", 32000, 280, 0, 2, 1, "far"), ("f32", 8193, 1600, 1, 0, 1, ""), ("bf16", 131072, 200, 0, 1, 0, "far"),
-    ("f32", 131073, 240, 1, 0, 0, "nan"), ("f32", 151936, 240, 0, 0, 0, "far"), ("bf16", 140001, 160, 1, 2, 0, ""), ("bf16", 262144, 160, 0, 1, 1, "nan")])
-def test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble):
+# Batches beyond the limits of the on-chip walk, those that four tiles per warp hold, and (rows beyond 131,072 entries) both sides of eight blocks a
+# sequence, with the kernel that the whole batch takes; the parts take another, or another shape of it.
+@pytest.mark.parametrize("dtype,V,B,off,rule,sampler,trouble,kernel", [
+    ("bf16", 32001, 300, 1, 0, 0, "", "walk_stream"), ("bf16", 32001, 230, 7, 0, 0, "nan", "walk_stream"), ("f32", 16389, 600, 3, 0, 0, "nan", "walk_stream"),
+    ("bf16", 8201, 800, 1, 0, 0, "far", "walk_stream"), ("bf16", 65551, 200, 1, 0, 0, "far", "walk_stream"), ("bf16", 32000, 300, 0, 1, 0, "", "walk_stream"),
+    ("bf16", 16400, 600, 0, 2, 0, "nan", "walk_stream"), ("f32", 8208, 800, 0, 2, 1, "far", "walk_cluster"), ("bf16", 32000, 560, 0, 1, 1, "", "walk_cluster"),
+    ("bf16", 32000, 280, 0, 2, 1, "far", "walk_cluster"), ("f32", 8193, 1600, 1, 0, 1, "", "walk_cluster"), ("bf16", 131072, 200, 0, 1, 0, "far", "walk_stream"),
+    ("f32", 131073, 240, 1, 0, 0, "nan", "walk_stream"), ("f32", 151936, 240, 0, 0, 0, "far", "walk_stream"), ("bf16", 140001, 160, 1, 2, 0, "", "walk_stream"),
+    ("bf16", 262144, 160, 0, 1, 1, "nan", "walk_stream"),
+    ("bf16", 32000, 440, 0, 1, 1, "", "walk_stream"), ("bf16", 24001, 440, 1, 2, 1, "far", "walk_stream"), ("f32", 16400, 592, 0, 2, 1, "far", "walk_stream"),
+    ("f32", 16401, 592, 1, 0, 1, "nan", "walk_stream"), ("f32", 32004, 290, 0, 2, 0, "", "walk_stream"), ("bf16", 32001, 440, 1, 0, 0, "nan", "walk_stream")])
+def test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble, kernel):
     import paper_2402_14160_b200 as rsd
     branching = (3, 2) if B * V < 3e7 else (2, 1)
     draft, target, _ = _drafted(B, V, dtype, branching, 7000 + V, off=off)
@@ -45,10 +50,16 @@ def test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trou
         target += 300.0
         draft[::2] -= 120.0
     token = _tokens(rsd, draft, branching, 3)
-    _whole_and_parts(rsd, draft, target, workloads.rsdc_parent_array(branching), token, 2, rule, 2.0, sampler)
+    parent = workloads.rsdc_parent_array(branching)
+    _whole_and_parts(rsd, draft, target, parent, token, 2, rule, 2.0, sampler)
+    parent = torch.from_numpy(parent).cuda()
+    routes = [launched(lambda: rsd.rsd_verify_tree_rule(draft[:n], target[:n], parent, token[:n], 2, rule, 2.0, sampler, 3, 0)) for n in (B, 4)]
+    (whole,), (part,) = routes
+    assert whole.kernel == kernel and whole._replace(blocks=0) != part._replace(blocks=0), routes
 
 
-@pytest.mark.parametrize("dtype,V,B", [("f32", 32000, 400), ("bf16", 32001, 230), ("bf16", 8201, 330), ("f32", 1000, 700), ("f32", 140001, 160), ("bf16", 262144, 310)])
+@pytest.mark.parametrize("dtype,V,B", [("f32", 32000, 400), ("bf16", 32001, 230), ("bf16", 8201, 330), ("f32", 1000, 700), ("f32", 140001, 160), ("bf16", 262144, 310),
+                                       ("f32", 16389, 1000), ("bf16", 32001, 440)])
 @pytest.mark.parametrize("k", [0, 3])
 @pytest.mark.parametrize("trouble", ["", "nan", "far"])
 @pytest.mark.parametrize("want_residual", [False, True])
@@ -67,6 +78,12 @@ def test_the_route_of_a_residual_draw_does_not_show(dtype, V, B, k, trouble, wan
     node = torch.arange(B, dtype=torch.int32, device="cuda")
     whole = rsd.rsd_resample_residual(draft, target, rejected, node, 5, 1, want_residual=want_residual)
     n = 3
+
+    def kernel(m):
+        return [l._replace(blocks=0) for l in launched(lambda: rsd.rsd_resample_residual(draft[:m], target[:m], rejected[:m] if k else None, node[:m], 5, 1, want_residual=want_residual))]
+
+    # (short rows, and long ones of which nothing is rejected, are drawn from by one kernel whatever the batch)
+    assert (kernel(B) != kernel(n)) == (V > 1000 and (k > 0 or V <= 131072))
     for b in (0, B - n):
         for again in (want_residual, not want_residual):          # (asking for the distribution changes the route as well)
             part = rsd.rsd_resample_residual(draft[b:b + n], target[b:b + n], rejected[b:b + n] if k else None, node[b:b + n], 5, 1, seq_base=b,
@@ -119,9 +136,9 @@ def test_residual_draws_over_rows_read_in_every_pass_match_oracle(dtype, V, B, k
     assert np.all(o["margin"][g["token"][:n] != o["token"]] <= 1e-5)
 
 
-# What large batches seldom meet: the ring (rows on 16-byte boundaries) and the streamed walk (off them) against small batches, which the
-# oracle tests cover.
-@pytest.mark.parametrize("V,B", [(512, 1400), (16389, 260)])
+# What large batches seldom meet: the ring (rows on 16-byte boundaries), the streamed walk (off them) and the cluster walk with four tiles per warp against
+# small batches, which the oracle tests cover.
+@pytest.mark.parametrize("V,B", [(512, 1400), (16389, 260), (16389, 140), (16392, 140)])   # (140 sequences: four tiles per warp; the parts of 40 fewer)
 @pytest.mark.parametrize("what", ["repeated", "many_children", "large_tree", "peaked"])
 def test_rare_paths_of_large_batches(what, V, B):
     import paper_2402_14160_b200 as rsd
@@ -140,7 +157,7 @@ def test_rare_paths_of_large_batches(what, V, B):
         parent[33:] = 0
         token[::2, 60], token[:, 80], token[::2, 90] = token[::2, 3], token[:, 75], token[::2, 12]
         target[:, 0].scatter_(1, token[:, 1:].long(), -30.0)       # (all of them rejected)
-    whole = _whole_and_parts(rsd, draft, target, parent, token, len(branching), n=100)
+    whole = _whole_and_parts(rsd, draft, target, parent, token, len(branching), n=100 if B != 140 else 40)
     tested = (~torch.isnan(whole["theta"])).sum(dim=1)
     if what == "many_children":
         assert int(tested.min()) >= 96
@@ -156,7 +173,7 @@ def test_rare_paths_of_large_batches(what, V, B):
     ("bf16", 65536, 70, 0, 0, 0, ""), ("bf16", 40008, 60, 0, 2, 1, "nan"), ("f32", 65540, 30, 0, 1, 0, ""), ("bf16", 131072, 33, 0, 0, 0, "nan"),
     ("bf16", 131071, 33, 1, 1, 1, "far"), ("f32", 100001, 24, 1, 0, 1, "nan")])
 def test_four_tiles_per_warp_give_the_bits_of_fewer(dtype, V, B, off, rule, sampler, trouble):
-    test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble)
+    test_the_route_of_a_walk_does_not_show(dtype, V, B, off, rule, sampler, trouble, "walk_stream" if V == 8193 else "walk_cluster")
 
 
 @pytest.mark.parametrize("dtype,V,B", [("f32", 131072, 33), ("bf16", 65537, 33), ("f32", 32769, 71), ("bf16", 50272, 40)])
