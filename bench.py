@@ -29,9 +29,9 @@ import workloads  # noqa: E402
 # DRAM bytes moved per algorithmic byte by the scan kernel, from the committed ncu summary of the scan kernel
 # (dram__bytes_read + dram__bytes_write over rows x V x 2 bytes; the traffic grows in proportion to the rows scanned),
 # together with the SHA-256 of the kernel sources it was measured on: when the sources differ, `traffic` is null.
-SCAN_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.007
+SCAN_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.006
 SCAN_TRAFFIC_SOURCES = ("paper_2402_14160_b200/csrc/rsd_scan.cuh", "paper_2402_14160_b200/csrc/rsd_device.cuh")
-SCAN_TRAFFIC_SOURCE_SHA256 = "9b09653ba61a787a42eaae3ba09385b348ec033a4200f97dce0238c0c4c8c513"
+SCAN_TRAFFIC_SOURCE_SHA256 = "f9f2a0ec5a69fbcca548f4dbb2e410d76f5770757264beb4f0296f442b0ff231"
 
 
 def _scan_sources_sha256():

@@ -107,7 +107,8 @@ const char* rsd_last_error(void);
 /*
  * Timing aid (the paper has no counterpart).  The next rsd_gumbel_topk_draft or rsd_sbs_step call made by this host
  * thread records the CUDA event `before` right before and `after` right after its row-scan kernel, on that call's
- * stream; the request is then cleared.  Either may be NULL.  Host handles (cudaEvent_t) owned by the caller.
+ * stream; the request is then cleared.  (A beam search level of few rows is one kernel: the events then enclose all of
+ * it.)  Either may be NULL.  Host handles (cudaEvent_t) owned by the caller.
  */
 int rsd_profile_next_scan(void* before, void* after);
 

@@ -18,13 +18,13 @@
 //           value, then the last kept token among its equals
 // A bin that holds more tokens than the list is swept again, into bins of equal width in code.
 //
-// Bound by instruction issue (58 %), the histogram's bank conflicts (3.8 wavefronts per addition) and the barriers between
-// a row's serial steps.  A row of 32,000 bf16 entries takes 43,600 warp instructions; it took 67,000 before the sweep went
-// without returned atomics and with packed arithmetic, and before the search behind it was left to one warp: 1344 rows
+// Bound by instruction issue (58 %), the histogram's bank conflicts (3.6 wavefronts per addition) and the barriers between
+// a row's serial steps.  A row of 32,000 bf16 entries takes 37,400 warp instructions; it took 67,000 before the sweep went
+// without returned atomics and with packed arithmetic, and before the search behind it was left to one warp: 43,600, 1344 rows
 // 146 -> 104 us.  Three blocks per SM for rows of up to 64,000 bytes, and 1024 threads for rows of which only one fits on an
 // SM (32 rows of 32,000 fp32 with both cuts 47 -> 23 us).
 // Since then, with lists in registers, a thread's words tested before its tokens, top-k from the threads' largest values and an output that compares once a word:
-// 1500 rows of 32,000 bf16, top-p 0.95, 106 -> 90 us, the 32 rows 23 -> 14.
+// 1500 rows of 32,000 bf16, top-p 0.95, 107 -> 90 us, the 1344 98 -> 84, the 32 rows 22 -> 14.7.
 #pragma once
 #include "rsd_device.cuh"
 #include "rsd_scan.cuh"   // ex2_approx, packed arithmetic
@@ -163,8 +163,9 @@ struct RowStats<float> {
     }
 };
 
-// Tests on a whole 16-byte word of the row.  They compare values, so +0 and -0 count as equal although their codes
-// differ: callers treat the answers as a superset and look at the codes where that matters.
+// Tests on a whole 16-byte word of the row.  They compare values; as values and as codes +0 and -0 are one.  between() is a superset (2-byte
+// rows: bounds cut to 16 bits) that gather() checks by code.  at_least() is final: outside the cut's word the output and the number of the kept are
+// what it says, so its bound is a value of the rows' type, and a bound of NaN (the code behind +inf) keeps nothing.
 template <typename T>
 struct RowVec;
 template <>
@@ -803,7 +804,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 3 : 1) filter_rows_kernel(cons
             const uint32_t lowest = __reduce_min_sync(0xFFFFFFFFu, float_to_ordered(low));
             if (lane == 0) sm.low = ordered_to_float(lowest);
         }
-        // (+0 and -0 are equal as values but not as codes: the larger code stands for both)
+        // (a largest value of -0 has the code of +0)
         uint32_t top = vtop == 0.0f ? RowCodes<T>::code_of_float(0.0f) : (vtop > kNegInf ? RowCodes<T>::code_of_float(vtop) : RowCodes<T>::kNegInfCode);
         top = __reduce_max_sync(0xFFFFFFFFu, top);
         if (lane == 0) atomicMax(&sm.top, top);

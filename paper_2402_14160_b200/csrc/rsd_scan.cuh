@@ -443,7 +443,7 @@ __host__ __device__ inline size_t scan_bounds_bytes(int V) { return 4 * (size_t)
 // ---------------------------------------------------------------------------------------------------------
 // Stochastic Beam Search level, per-sequence epilogue.
 // For a fixed parent psi is increasing in phi~ (Theorem 3.2's argument), so the W best pairs over all parents are
-// among each parent's own W best by phi~.  The scan above leaves those n_par * W finalists in scratch; this kernel
+// among each parent's own W best by phi~.  The row scan (scan_row() below) leaves those n_par * W finalists in scratch; this kernel
 // recomputes their noise in double, applies the truncation T of Eq. 11 in the stable form
 //   psi = Gamma - log1p(exp(Gamma - phi~) (1 - exp(phi~ - Z))),
 // and keeps the W best by (psi desc, parent asc, token asc).
