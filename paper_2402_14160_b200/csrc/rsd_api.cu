@@ -33,13 +33,6 @@ thread_local cudaEvent_t g_scan_before = nullptr, g_scan_after = nullptr;  // on
 // four warps (few rows: 256 threads with the sums on four warps and the perturbed values on the others), beyond those of
 // eight, by 256 threads in every launch (bf16, 64 / 222 / 370 / 600 rows of 16,384: 8.4 / 10.5 / 11.1 / 12.3 with 128 threads, 8.1 / 10.0 / 10.8 /
 // 17.0 with 256; 192 / 5000 rows of 128,000: 43 / 370 with 128, 27 / 247 with 256).
-int sm_count() {
-    static const int sms = [] {
-        int dev = 0, n = 0;
-        return (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 148;
-    }();
-    return sms;
-}
 int scan_threads(int rows, int V, bool f32, bool need_lse) {
     const int sms = sm_count();
     const bool few = rows <= sms + sms / 2;

@@ -48,6 +48,18 @@ inline void launch_overlapped(void (*kernel)(KArgs...), unsigned blocks, unsigne
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// SMs of the current device (asked once per device; 148 if the query fails)
+inline int sm_count() {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+    int n = known[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    n = (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 148;
+    known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 // Raises a kernel's limit of dynamic shared memory.  The attribute belongs to the (function, device) pair and setting it costs host
 // time: once per device.  (An error stays pending for check_launch().)
 template <auto KERNEL>

@@ -13,18 +13,6 @@
 using namespace rsd_host;
 
 namespace {
-// SMs of the current device (asked once per device; 148 if the query fails)
-int sm_count() {
-    static int cached[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-    if (cached[dev] == 0) {
-        int n = 0;
-        cached[dev] = (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 148;
-    }
-    return cached[dev];
-}
-
 // The walk fed by the copy engine (rsd_walk_ring.cuh); a launch error stays pending for check_launch().
 template <typename T>
 void launch_ring_walk(const rsd::VerifyArgs& a, int B, cudaStream_t s) {

@@ -37,9 +37,7 @@ int resident_clusters(int C, int W, int NT) {
     n = shape == 3 ? ask_resident<2, 16>(C) : shape == 2 ? ask_resident<4, 8>(C) : shape == 1 ? ask_resident<2, 8>(C) : ask_resident<1, 8>(C);
     if (n <= 0) {
         (void)cudaGetLastError();                        // (a rule of thumb, not an error of the call)
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
-        n = std::max(sms * (shape == 3 ? 1 : shape == 0 ? 3 : 2) / C, 1);
+        n = std::max(rsd_host::sm_count() * (shape == 3 ? 1 : shape == 0 ? 3 : 2) / C, 1);
     }
     if (keep) known[dev][shape][size].store(n, std::memory_order_relaxed);
     return n;
