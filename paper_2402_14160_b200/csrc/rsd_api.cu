@@ -275,9 +275,10 @@ int rsd_filter_rows(const rsd_rows* rows, int B, int R, int V, int top_k, float 
     }
     // A lone row's block waits for the stream's earlier work where it starts.  Moved in ahead of that work's end, the blocks of a launch that comes close to one
     // or two rows an SM pile up on the SMs that have room first, so that it starts in plain stream order (back to back, us, overlapped / plain: bf16 19,632
-    // entries, 106 / 148 / 290 rows 35.0 / 27.6, 35.3 / 27.6, 62 / 49; 80 27 to 35 / 27.6; 200 / 1500 48.6 / 49.1, 248 / 249).
+    // entries, 106 / 148 / 290 rows 35.0 / 27.6, 35.3 / 27.6, 62 / 49; 80 27 to 35 / 27.6; 200 / 1500 48.6 / 49.1, 248 / 249;
+    // 277 rows of 500 6.8 / 7.3, 108 of 1920 6.1 / 6.6: short rows are over too soon).
     const int sms = sm_count(), over = (B - 1) % sms + 1;   // rows beyond whole ones an SM
-    if (R == 1 && B <= 2 * sms && over > sms / 2) kernel<<<(unsigned)B, wide ? 1024 : 512, smem, s>>>(a);
+    if (R == 1 && V > 4096 && B <= 2 * sms && over > sms / 2) kernel<<<(unsigned)B, wide ? 1024 : 512, smem, s>>>(a);
     else launch_overlapped(kernel, (unsigned)(B * R), wide ? 1024 : 512, smem, s, 0, a);
     return check_launch("rsd_filter_rows");
 }

@@ -82,11 +82,13 @@ def test_rows_that_would_share_an_sm_as_clusters_have_their_words_cleared(dtype,
     assert out["status"].cpu().tolist() == [NAN_INPUT if b % 2 == 0 else 0 for b in range(B)]
 
 
-# Lone rows: launches that come close to one or two rows an SM (148) start in plain stream order, the others overlap the end of what is ahead.
+# Lone rows: launches of rows beyond 4096 entries that come close to one or two an SM (148) start in plain stream order, the others overlap the end of
+# what is ahead.
 @pytest.mark.parametrize("B", [74, 75, 148, 149, 222, 223, 296, 297])
-def test_filter_calls_behind_each_other_read_what_the_one_before_wrote(B):
+@pytest.mark.parametrize("V", [4096, 9001])
+def test_filter_calls_behind_each_other_read_what_the_one_before_wrote(B, V):
     import paper_2402_14160_b200 as rsd
-    rows = torch.randn((B, 1, 9001), device="cuda")
+    rows = torch.randn((B, 1, V), device="cuda")
     rows[::2, 0, 5] = float("nan")
     outs = [rsd.rsd_filter_rows(rows, 0, 1.0) for _ in range(4)]
     torch.cuda.synchronize()
@@ -96,7 +98,7 @@ def test_filter_calls_behind_each_other_read_what_the_one_before_wrote(B):
         for out in outs:
             out["status"].fill_(77)
             out["rows"].fill_(1.0)
-        for i, (top_k, top_p) in enumerate(((4000, 0.99), (700, 0.95), (90, 0.9), (0, 0.5))):
+        for i, (top_k, top_p) in enumerate(((3000, 0.99), (700, 0.95), (90, 0.9), (0, 0.5))):
             if wait:
                 torch.cuda.synchronize()
             rsd.rsd_filter_rows(src, top_k, top_p, out=outs[i])
